@@ -150,7 +150,7 @@ gemm_w4a4_decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
   if (warp < kConvBWarp0) reg_dec<kRegsCtl>();
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    if (elect_one()) {
       int s = 0; uint32_t ph = 0;
       uint32_t armed = 0, armed_par = 0;
       bool ok = true;
@@ -173,7 +173,7 @@ gemm_w4a4_decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t idesc = umma_idesc_i8(HR, D.npad, true, !P.a_unsigned);
       int s = 0; uint32_t ph = 0; int seg = 0;
       long long g = g_begin;

@@ -104,7 +104,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    if (elect_one()) {
       int s = 0; uint32_t ph = 0;
       uint32_t armed = 0, armed_par = 0;          // per stage: a copy was issued / parity of its phase
       bool ok = true;
@@ -131,7 +131,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    if (elect_one()) {                     // (not `lane == 0`: see the CTA-pair kernel)
       const uint32_t idesc = umma_idesc_i8(BM, BN, !P.a_unsigned, true);
       int s = 0; uint32_t ph = 0; int it = 0;
       for (int tile = blockIdx.x; tile < P.num_tiles; tile += gridDim.x, ++it) {

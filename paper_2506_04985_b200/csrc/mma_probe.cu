@@ -23,13 +23,12 @@ constexpr int kAStageCol = 480;                    // 32 columns hold 128 int8 p
 struct Params {
   int n;                   // columns of one instruction (multiple of 16, 16..256)
   int n_acc;               // accumulators in rotation: n_acc * n <= 448 columns
-  int a_in_tmem;           // A operand from tensor memory (else from shared memory)
   int iters;               // groups of four instructions
   uint32_t* status;
   unsigned long long* cycles;   // [CTAs] clock64 ticks from the first issue to the last completion (leaders only)
 };
 
-template <bool kPair>
+template <bool kPair, bool kATmem>
 __global__ void __launch_bounds__(kThreads, 1) mma_probe_kernel(const Params P) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -37,7 +36,7 @@ __global__ void __launch_bounds__(kThreads, 1) mma_probe_kernel(const Params P) 
   const uint32_t bar = sbase + kBarOff;
   volatile uint32_t* misc = reinterpret_cast<volatile uint32_t*>(smem + kBarOff + 16);
   volatile uint32_t* abort_flag = misc + 1;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5;
   const uint32_t rank = kPair ? cluster_ctarank() : 0u;
 
   // operand tiles: bytes from a counter hash (the values do not matter, their toggling does)
@@ -76,27 +75,29 @@ __global__ void __launch_bounds__(kThreads, 1) mma_probe_kernel(const Params P) 
   if (kPair) cluster_sync_all(); else __syncthreads();
   tc_fence_after();
 
-  if (warp == 0 && lane == 0 && rank == 0) {
+  // One ELECTED thread issues, the operand kind is a template parameter and the accumulator address is the only
+  // thing the loop computes: with `lane == 0` and branches on the parameters the loop itself took 103 cycles an
+  // instruction, which hid that small instructions finish in 9 (128 x 16) to 64 cycles (128 x 128).
+  if (warp == 0 && rank == 0 && elect_one()) {
     const uint32_t idesc = umma_idesc_i8(kPair ? 256 : 128, P.n, true, true);
     const uint64_t adesc = umma_desc_kmajor_sw128(sbase);
     const uint64_t bdesc = umma_desc_kmajor_sw128(sbase + kATile);
     const uint32_t a_tmem = tmem_base + kAStageCol;
-    const int n = P.n, n_acc = P.n_acc, iters = P.iters;
-    const bool a_tm = P.a_in_tmem != 0;
-    int acc = 0;
+    const uint32_t n = (uint32_t)P.n, d_end = tmem_base + (uint32_t)(P.n_acc * P.n);
+    const int iters = P.iters;
+    uint32_t d = tmem_base;
     const long long t0 = clock64();
     for (int it = 0; it < iters; ++it) {
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk) {
-        const uint32_t d = tmem_base + (uint32_t)(acc * n);
         if (kPair) {
-          if (a_tm) umma_i8_ts_pair(d, a_tmem + 8u * kk, bdesc + 2u * kk, idesc, 1u);
+          if (kATmem) umma_i8_ts_pair(d, a_tmem + 8u * kk, bdesc + 2u * kk, idesc, 1u);
           else umma_i8_pair(d, adesc + 2u * kk, bdesc + 2u * kk, idesc, 1u);
         } else {
-          if (a_tm) umma_i8_ts(d, a_tmem + 8u * kk, bdesc + 2u * kk, idesc, 1u);
+          if (kATmem) umma_i8_ts(d, a_tmem + 8u * kk, bdesc + 2u * kk, idesc, 1u);
           else umma_i8(d, adesc + 2u * kk, bdesc + 2u * kk, idesc, 1u);
         }
-        if (++acc == n_acc) acc = 0;
+        d = d + n == d_end ? tmem_base : d + n;
       }
     }
     if (kPair) umma_commit_pair(bar, 1); else umma_commit(bar);
@@ -146,6 +147,15 @@ extern "C" int fpt_selftest_wait_timeout(void* stream, void* workspace, unsigned
   return cudaGetLastError() == cudaSuccess ? FPT_OK : FPT_ERR_CUDA;
 }
 
+template <bool kPair, bool kATmem>
+static int launch_probe(cudaStream_t st, int ctas, const probe::Params& P) {
+  using namespace probe;
+  auto kern = mma_probe_kernel<kPair, kATmem>;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kAlloc) != cudaSuccess) return FPT_ERR_CUDA;
+  return launch_kernel_cluster(kern, dim3(ctas), dim3(kThreads), kAlloc, st, false, kPair ? 2 : 1, P) == cudaSuccess
+             ? FPT_OK : FPT_ERR_CUDA;
+}
+
 extern "C" int fpt_probe_mma(void* stream, int pair, int n, int n_acc, int a_in_tmem, int iters, int ctas,
                              unsigned long long* cycles, void* workspace) {
   using namespace probe;
@@ -154,27 +164,10 @@ extern "C" int fpt_probe_mma(void* stream, int pair, int n, int n_acc, int a_in_
   if (pair && (ctas & 1)) return FPT_ERR_BAD_ARG;
   if ((uintptr_t)workspace & 15) return FPT_ERR_ALIGNMENT;
   Params P;
-  P.n = n; P.n_acc = n_acc; P.a_in_tmem = a_in_tmem; P.iters = iters;
+  P.n = n; P.n_acc = n_acc; P.iters = iters;
   P.status = reinterpret_cast<uint32_t*>(workspace);
   P.cycles = cycles;
   cudaStream_t st = (cudaStream_t)stream;
-  if (pair) {
-    if (cudaFuncSetAttribute(mma_probe_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAlloc) != cudaSuccess)
-      return FPT_ERR_CUDA;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(ctas, 1, 1);
-    cfg.blockDim = dim3(kThreads, 1, 1);
-    cfg.dynamicSmemBytes = kAlloc;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, mma_probe_kernel<true>, P) != cudaSuccess) return FPT_ERR_CUDA;
-  } else {
-    if (cudaFuncSetAttribute(mma_probe_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAlloc) != cudaSuccess)
-      return FPT_ERR_CUDA;
-    mma_probe_kernel<false><<<ctas, kThreads, kAlloc, st>>>(P);
-  }
-  return cudaGetLastError() == cudaSuccess ? FPT_OK : FPT_ERR_CUDA;
+  if (pair) return a_in_tmem ? launch_probe<true, true>(st, ctas, P) : launch_probe<true, false>(st, ctas, P);
+  return a_in_tmem ? launch_probe<false, true>(st, ctas, P) : launch_probe<false, false>(st, ctas, P);
 }
