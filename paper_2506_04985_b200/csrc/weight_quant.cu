@@ -1,27 +1,73 @@
 // Offline weight quantiser: per-output-channel symmetric INT4 grid, round-to-nearest,
 // min-max or L_p range setting (Sec. 4 "Quantization Setup"; App. D "Quantizer range
-// setting"), packed two codes per byte (App. J).  Not on the timed path: one CTA per row.
+// setting"), packed two codes per byte (App. J).  One CTA per row.
+//
+// The L_p search is bound by arithmetic: 81 candidate scales x K values, each a division, a rounding and a
+// float64 power.  A thread keeps sixteen values in registers (float32 and float64) and walks over the candidates,
+// so that sixteen independent chains hide the float64 latency (nine candidates per value instead: 7.0 ms on the
+// shape below, with half the warps); the division is a multiply that is redone as a division only where the
+// quotient lies so close to a tie that the two could round differently, one branch for the sixteen values; |e|^3
+// (the method's p) is two float64 multiplies; sums meet once per warp and candidate.
+// 14336 x 4096, p = 3, f16 scales: 38.6 -> 2.74 ms; min-max 95 -> 83 us (the row is read once, 16 bytes a load).
 #include "fpt_common.cuh"
 
 namespace fpt {
 
 constexpr int kWqThreads = 256;
+constexpr int kLpFirst = 20, kLpCount = 81;                        // candidate scales a * i / 100, i = 20 .. 100
+constexpr int kLpHold = 16;                                        // values a thread holds during the search
 
-template <typename T> __device__ __forceinline__ float wload(const T* p, size_t i);
-template <> __device__ __forceinline__ float wload<__nv_bfloat16>(const __nv_bfloat16* p, size_t i) { return __bfloat162float(p[i]); }
-template <> __device__ __forceinline__ float wload<float>(const float* p, size_t i) { return p[i]; }
+// eight consecutive weights as float
+__device__ __forceinline__ void wload8(const __nv_bfloat16* p, float* w) {
+  const uint4 v = *reinterpret_cast<const uint4*>(p);
+  w[0] = bf16lo_to_f32(v.x); w[1] = bf16hi_to_f32(v.x); w[2] = bf16lo_to_f32(v.y); w[3] = bf16hi_to_f32(v.y);
+  w[4] = bf16lo_to_f32(v.z); w[5] = bf16hi_to_f32(v.z); w[6] = bf16lo_to_f32(v.w); w[7] = bf16hi_to_f32(v.w);
+}
+__device__ __forceinline__ void wload8(const float* p, float* w) {
+  const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
+  w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w; w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
+}
 
 __device__ __forceinline__ float store_round(float d, int scale_dtype) {
   return scale_dtype == FPT_DTYPE_F16 ? __half2float(__float2half_rn(d)) : d;
 }
 
-__device__ __forceinline__ int quant_code(float w, float d) {
-  float u = rintf(__fdiv_rn(w, d));
-  u = fminf(fmaxf(u, -8.0f), 7.0f);              // NaN -> -8
-  return (int)u;
+// A grid step with what the multiply-instead-of-divide form needs.  `inv` is 0 where that form is not used: a
+// step whose reciprocal is not an ordinary number.
+struct Step {
+  float d, inv;
+};
+__device__ __forceinline__ Step make_step(float d) {
+  Step s;
+  s.d = d;
+  s.inv = (d > 0x1p-100f && d < 0x1p100f) ? __fdiv_rn(1.0f, d) : 0.0f;
+  return s;
 }
 
-template <typename V>
+// clamp(rne(w / d), -8, 7) + 8, w / d rounded to float32 (IEEE division); a NaN gives 0.
+__device__ __forceinline__ int biased_div(float w, float d) {
+  return (int)fminf(fmaxf(rintf(__fdiv_rn(w, d)), -8.0f), 7.0f) + 8;
+}
+// The same through w * (1/d), for quotients below 2^22.  `far` returns how far the product is from its rounded
+// value: the product is within 2^-23 of the quotient, relatively, and the float32 quotient within 2^-24, so for
+// |quotient| < 9 the two are closer than 2e-6 and round alike unless they lie that close to k + 1/2, i.e. unless
+// `far` is above kTieClose (beyond 9 both clamp alike).  A NaN must not come here.
+constexpr float kTieClose = 0.5f - 4e-6f;
+__device__ __forceinline__ int biased_mul(float w, float inv, float& far) {
+  const float t = __fmul_rn(w, inv);
+  const float r = __fadd_rn(t, 12582912.0f);                       // 1.5 * 2^23 + rne(t)
+  far = fabsf(__fsub_rn(t, __fsub_rn(r, 12582912.0f)));
+  return __viaddmin_s32_relu(__float_as_int(r), -0x4B400000 + 8, 15);
+}
+__device__ __forceinline__ int quant_code(float w, const Step& s, bool fast) {
+  float far = 0.0f;
+  int u = fast ? biased_mul(w, s.inv, far) : 0;
+  if (!fast || far > kTieClose) u = biased_div(w, s.d);
+  return u - 8;
+}
+
+// Sum (or maximum) over the CTA, the same in every thread.
+template <int NT, typename V>
 __device__ __forceinline__ V block_reduce(V v, V* scratch, bool is_max) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -32,59 +78,180 @@ __device__ __forceinline__ V block_reduce(V v, V* scratch, bool is_max) {
   if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = v;
   __syncthreads();
   V r = scratch[0];
-  for (int w = 1; w < kWqThreads / 32; ++w) r = is_max ? (scratch[w] > r ? scratch[w] : r) : r + scratch[w];
+  for (int w = 1; w < NT / 32; ++w) r = is_max ? (scratch[w] > r ? scratch[w] : r) : r + scratch[w];
   return r;
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kWqThreads) weight_quant_kernel(const T* __restrict__ W, int N, int K, int range_mode,
-                                                                  float p, int scale_dtype, uint8_t* __restrict__ Wq,
-                                                                  void* __restrict__ sw, int32_t* __restrict__ wsum) {
-  __shared__ double scratch_d[kWqThreads / 32];
-  __shared__ float scratch_f[kWqThreads / 32];
-  __shared__ int scratch_i[kWqThreads / 32];
-  const int n = blockIdx.x;
-  const size_t base = (size_t)n * (size_t)K;
-  const int tid = threadIdx.x;
+// The search: the candidate with the least sum_k |w - D q|^p, equal sums to the larger scale, sums that are not
+// numbers left out; `fallback` where none is left.  Every thread returns the same step.
+template <typename T, int NT, bool kCube>
+__device__ float lp_search(const T* row, int chunks, float a, bool no_nan, float p, int scale_dtype, float fallback) {
+  __shared__ Step step[kLpCount];
+  __shared__ double part[kLpCount][NT / 32];
+  __shared__ float found;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int i = tid; i < kLpCount; i += NT) {
+    float d = store_round(__fdiv_rn(__fmul_rn(a, __fdiv_rn((float)(kLpFirst + i), 100.0f)), 7.0f), scale_dtype);
+    if (a == 0.0f || d == 0.0f) d = 1.0f;
+    step[i] = make_step(d);
+  }
+  for (int i = tid; i < kLpCount * (NT / 32); i += NT) (&part[0][0])[i] = 0.0;
+  __syncthreads();
+  for (int c0 = 0; c0 < chunks; c0 += NT * (kLpHold / 8)) {
+    float w[kLpHold];
+    double w64[kLpHold];
+#pragma unroll
+    for (int h = 0; h < kLpHold / 8; ++h) {
+      const int c = c0 + h * NT + tid;
+      if (c < chunks) wload8(row + 8 * (size_t)c, w + 8 * h);
+      else
+#pragma unroll
+        for (int j = 0; j < 8; ++j) w[8 * h + j] = 0.0f;   // a zero costs no error on any grid
+    }
+#pragma unroll
+    for (int j = 0; j < kLpHold; ++j) w64[j] = (double)w[j];
+    for (int i = 0; i < kLpCount; ++i) {
+      const Step s = step[i];
+      const double neg_d = -(double)s.d;
+      const bool fast = no_nan && s.inv != 0.0f;
+      int u[kLpHold];
+      float close = 0.0f;
+#pragma unroll
+      for (int j = 0; j < kLpHold; ++j) {
+        float far;
+        u[j] = biased_mul(w[j], s.inv, far);
+        close = fmaxf(close, far);
+      }
+      if (!fast || close > kTieClose) {                    // rare
+#pragma unroll
+        for (int j = 0; j < kLpHold; ++j) u[j] = biased_div(w[j], s.d);
+      }
+      double err[2] = {0.0, 0.0};
+#pragma unroll
+      for (int j = 0; j < kLpHold; ++j) {
+        // 2^52 + u as float64 by its bit pattern, then q = u - 8: one exact add instead of a conversion
+        const double q = __hiloint2double(0x43300000, u[j]) - (4503599627370496.0 + 8.0);
+        // |w - D q|: the product of a 24-bit and a 4-bit number is exact in float64
+        const double e = fabs(fma(neg_d, q, w64[j]));
+        err[j & 1] = kCube ? fma(__dmul_rn(e, e), e, err[j & 1]) : err[j & 1] + pow(e, (double)p);
+      }
+      double sum = err[0] + err[1];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      if (lane == 0) part[i][warp] += sum;
+    }
+  }
+  __syncthreads();
+  if (warp == 0) {
+    double best = 1.0 / 0.0;
+    int at = -1;
+    for (int i = lane; i < kLpCount; i += 32) {
+      double e = 0.0;
+      for (int v = 0; v < NT / 32; ++v) e += part[i][v];
+      if (e <= best) { best = e; at = i; }                 // i grows: ties to the larger scale
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double e2 = __shfl_xor_sync(0xffffffffu, best, o);
+      const int a2 = __shfl_xor_sync(0xffffffffu, at, o);
+      if (a2 >= 0 && (at < 0 || e2 < best || (e2 == best && a2 > at))) { best = e2; at = a2; }
+    }
+    if (lane == 0) found = at >= 0 ? step[at].d : fallback;
+  }
+  __syncthreads();
+  return found;
+}
+
+// NT threads; V > 0: the row (at most NT * 8 * V values) is held in registers; V = 0: it is read again (from L1 or
+// L2) in each pass.  kRange: 0 min-max, 1 L_p, 2 L_3; separate kernels, the search needs twice the registers of the rest.
+template <typename T, int NT, int V, int kRange>
+__global__ void __launch_bounds__(NT, kRange == 2 ? 768 / NT : 1) weight_quant_kernel(const T* __restrict__ W, int K, float p, int scale_dtype,
+                                                          uint8_t* __restrict__ Wq, void* __restrict__ sw,
+                                                          int32_t* __restrict__ wsum) {
+  __shared__ float scratch_f[NT / 32];
+  __shared__ int scratch_i[NT / 32];
+  const int n = blockIdx.x, tid = threadIdx.x;
+  const T* row = W + (size_t)n * (size_t)K;
+  const int chunks = K >> 3;
+  constexpr int R = V > 0 ? V : 1;
+  float w[R][8];
+  if constexpr (V > 0) {
+#pragma unroll
+    for (int i = 0; i < V; ++i) {
+      const int c = i * NT + tid;
+      if (c < chunks) wload8(row + 8 * c, w[i]);
+      else
+#pragma unroll
+        for (int j = 0; j < 8; ++j) w[i][j] = 0.0f;      // a zero costs no error on any grid
+    }
+  }
+  // f(values of a chunk, chunk index) over this thread's part of the row
+  auto each_chunk = [&](auto f) {
+    if constexpr (V > 0) {
+#pragma unroll
+      for (int i = 0; i < V; ++i) f(w[i], i * NT + tid);
+    } else {
+      for (int c = tid; c < chunks; c += NT) { wload8(row + 8 * c, w[0]); f(w[0], c); }
+    }
+  };
 
   float a = 0.0f;
-  for (int k = tid; k < K; k += kWqThreads) a = fmaxf(a, fabsf(wload(W, base + k)));
-  a = block_reduce<float>(a, scratch_f, true);
+  bool nan = false;
+  each_chunk([&](const float (&x)[8], int) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) { a = fmaxf(a, fabsf(x[j])); nan = nan || x[j] != x[j]; }
+  });
+  const bool no_nan = __syncthreads_or(nan) == 0;
+  a = block_reduce<NT>(a, scratch_f, true);
 
   float delta = store_round(__fdiv_rn(a, 7.0f), scale_dtype);
   if (a == 0.0f || delta == 0.0f) delta = 1.0f;
-  if (range_mode == FPT_RANGE_LP) {
-    double best = 1.0 / 0.0;   // +inf
-    for (int i = 20; i <= 100; ++i) {
-      const float frac = __fdiv_rn((float)i, 100.0f);
-      float d = store_round(__fdiv_rn(__fmul_rn(a, frac), 7.0f), scale_dtype);
-      if (a == 0.0f || d == 0.0f) d = 1.0f;
-      double err = 0.0;
-      for (int k = tid; k < K; k += kWqThreads) {
-        const float w = wload(W, base + k);
-        const double e = fabs((double)w - (double)d * (double)quant_code(w, d));
-        err += pow(e, (double)p);
-      }
-      err = block_reduce<double>(err, scratch_d, false);
-      if (err <= best) { best = err; delta = d; }
-    }
-  }
+  if constexpr (kRange != 0) delta = lp_search<T, NT, kRange == 2>(row, chunks, a, no_nan, p, scale_dtype, delta);
   if (tid == 0) {
     if (scale_dtype == FPT_DTYPE_F16) reinterpret_cast<__half*>(sw)[n] = __float2half_rn(delta);
     else reinterpret_cast<float*>(sw)[n] = delta;
   }
   int sum = 0;
-  uint8_t* out = Wq + (size_t)n * (size_t)(K / 2);
-  for (int j = tid; j < K / 2; j += kWqThreads) {
-    const int q0 = quant_code(wload(W, base + 2 * j), delta);
-    const int q1 = quant_code(wload(W, base + 2 * j + 1), delta);
-    sum += q0 + q1;
-    out[j] = (uint8_t)((q0 & 0xF) | ((q1 & 0xF) << 4));
-  }
+  const Step fin = make_step(delta);
+  const bool fast = no_nan && fin.inv != 0.0f;
+  uint32_t* out = reinterpret_cast<uint32_t*>(Wq + (size_t)n * (size_t)(K / 2));
+  each_chunk([&](const float (&x)[8], int c) {
+    if (c >= chunks) return;
+    uint32_t word = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int q = quant_code(x[j], fin, fast);
+      sum += q;
+      word |= (uint32_t)(q & 0xF) << (4 * j);
+    }
+    out[c] = word;
+  });
   if (wsum) {
-    sum = block_reduce<int>(sum, scratch_i, false);
+    sum = block_reduce<NT>(sum, scratch_i, false);
     if (tid == 0) wsum[n] = sum;
   }
+}
+
+// Threads by the row's length: sixteen values a thread up to 4096 values, then more passes of the same CTA.  The
+// min-max kernel holds up to 8192 values in registers.
+template <typename T, int kRange>
+static void launch_weight_quant(cudaStream_t st, const T* W, int N, int K, float p, int scale_dtype, uint8_t* Wq,
+                                void* sw, int32_t* wsum) {
+  constexpr int V = kRange == 0 ? 2 : 0;
+  auto go = [&](auto kern, int threads) { kern<<<N, threads, 0, st>>>(W, K, p, scale_dtype, Wq, sw, wsum); };
+  if (K <= 1024) go(weight_quant_kernel<T, 64, V, kRange>, 64);
+  else if (K <= 2048) go(weight_quant_kernel<T, 128, V, kRange>, 128);
+  else if (K <= 4096) go(weight_quant_kernel<T, kWqThreads, V, kRange>, kWqThreads);
+  else if (K <= 8192) go(weight_quant_kernel<T, kWqThreads, 2 * V, kRange>, kWqThreads);
+  else go(weight_quant_kernel<T, kWqThreads, 0, kRange>, kWqThreads);
+}
+template <typename T>
+static void quantize_rows(cudaStream_t st, const void* W, int N, int K, int range_mode, float p, int scale_dtype,
+                          uint8_t* Wq, void* sw, int32_t* wsum) {
+  const T* w = reinterpret_cast<const T*>(W);
+  if (range_mode == FPT_RANGE_MINMAX) launch_weight_quant<T, 0>(st, w, N, K, p, scale_dtype, Wq, sw, wsum);
+  else if (p == 3.0f) launch_weight_quant<T, 2>(st, w, N, K, p, scale_dtype, Wq, sw, wsum);
+  else launch_weight_quant<T, 1>(st, w, N, K, p, scale_dtype, Wq, sw, wsum);
 }
 
 }  // namespace fpt
@@ -100,12 +267,8 @@ extern "C" int fpt_quantize_weights(void* stream, const void* W, int w_dtype, in
   if (range_mode == FPT_RANGE_LP && !(p > 0.0f)) return FPT_ERR_BAD_ARG;
   if (((uintptr_t)W | (uintptr_t)Wq | (uintptr_t)sw) & 15) return FPT_ERR_ALIGNMENT;
   cudaStream_t st = (cudaStream_t)stream;
-  if (w_dtype == FPT_DTYPE_BF16)
-    fpt::weight_quant_kernel<__nv_bfloat16><<<N, fpt::kWqThreads, 0, st>>>(
-        reinterpret_cast<const __nv_bfloat16*>(W), N, K, range_mode, p, scale_dtype, Wq, sw, wsum);
-  else
-    fpt::weight_quant_kernel<float><<<N, fpt::kWqThreads, 0, st>>>(reinterpret_cast<const float*>(W), N, K,
-                                                                    range_mode, p, scale_dtype, Wq, sw, wsum);
+  if (w_dtype == FPT_DTYPE_BF16) fpt::quantize_rows<__nv_bfloat16>(st, W, N, K, range_mode, p, scale_dtype, Wq, sw, wsum);
+  else fpt::quantize_rows<float>(st, W, N, K, range_mode, p, scale_dtype, Wq, sw, wsum);
   return cudaGetLastError() == cudaSuccess ? FPT_OK : FPT_ERR_CUDA;
 }
 

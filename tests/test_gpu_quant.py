@@ -113,6 +113,36 @@ def test_weight_quant_bit_exact(N, K, mode):
     assert np.array_equal(host(wsum), ws)
 
 
+@pytest.mark.parametrize("K", [32, 1024, 1056, 2080, 4128, 8224])       # either side of each thread count and of a second pass
+def test_weight_quant_range_search_at_ties_and_odd_rows(K):
+    rng = np.random.default_rng(K)
+    w = rng.standard_normal((12, K)).astype(np.float32) * 0.02
+    w[0] = rng.integers(-14, 15, K) * 0.5                # quotients that are k + 1/2 on the min-max grid
+    w[0, 0] = 7.0
+    w[1] = rng.integers(-14, 15, K) * np.float32(0.35)   # ... and on the candidate at 70 %, up to rounding
+    w[1, 0] = 7.0
+    w[2] *= 1e-6                                         # float16 scales that underflow
+    w[3] *= 1e7                                          # ... that overflow
+    w[4] *= 1e-37                                        # reciprocals out of range
+    w[5, 3] = np.inf
+    w[6, 5] = np.nan
+    for dt in (torch.bfloat16, torch.float32):
+        wd = torch.from_numpy(w).to(dt)
+        for sd, name in ((torch.float16, "fp16"), (torch.float32, "fp32")):
+            with np.errstate(all="ignore"):
+                codes, d, sums = OQ.quantize_weights(wd.float().numpy()[:5], range_mode=OQ.RANGE_LP, p=3.0, scale_dtype=name)
+            wq, sw, wsum = B.fpt_quantize_weights(dev(wd), None, B.RANGE_LP, 3.0, sd)
+            assert np.array_equal(host(sw.float())[:5].view(np.uint32), d.view(np.uint32))
+            assert np.array_equal(host(wq)[:5], OQ.pack_int4(codes))
+            assert np.array_equal(host(wsum)[:5], sums)
+            # an infinite row has no finite candidate, a NaN compares with none: both keep the min-max step
+            assert np.isinf(host(sw.float())[5])
+            finite = wd.float().numpy()[6]
+            want = np.float32(np.nanmax(np.abs(finite))) / np.float32(7.0)
+            assert host(sw.float())[6] == (np.float32(np.float16(want)) if name == "fp16" else want)
+            assert host(wq)[6, 2] >> 4 == 8              # a NaN takes the lowest code
+
+
 def test_interleave_gate_up_layout():
     d_ff, K = 384, 256
     rng = np.random.default_rng(0)
