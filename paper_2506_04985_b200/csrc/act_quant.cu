@@ -1,8 +1,7 @@
 // Step (1) of the path: RMSNorm-derived per-token scale + static INT4 quantise + pack
 // (Sec. 3.1.3, Eq. 6-7; App. B "Static quantization"), and the SiLU*mul variant that
-// feeds the down projection.  Memory-bound: one CTA per token, the row is read once
-// with 128-bit loads, kept in registers across the reduction, and written as packed
-// nibbles.
+// feeds the down projection.  Memory-bound: the row is read once with 128-bit loads, kept in
+// registers across the reduction, and written as packed nibbles.
 #include "fpt_internal.cuh"
 #include "quant_math.cuh"
 
@@ -24,7 +23,7 @@ struct ActQuantParams {
   uint32_t flip;       // see quant_word
 };
 
-// T threads per token, up to V 16-byte chunks (8 elements) per thread held in registers.
+// RMSNorm: T threads per token, up to V 16-byte chunks (8 elements) per thread held in registers.
 template <int T, int V>
 __global__ void __launch_bounds__(T, V <= 4 ? 2048 / T : 1) act_quant_kernel(const ActQuantParams P) {
   __shared__ double warp_part[T / 32];
@@ -35,69 +34,50 @@ __global__ void __launch_bounds__(T, V <= 4 ? 2048 / T : 1) act_quant_kernel(con
   const int tid = threadIdx.x;
   const int chunks = P.K >> 3;                   // 16-byte chunks per row
   const size_t row = (size_t)t * (size_t)(P.ldx >> 3);
-  const bool silu = (P.flags & FPT_SILU_MUL) != 0;
-  const bool inter = (P.flags & FPT_GU_INTERLEAVED) != 0;
-
   uint4 v[V];
 #pragma unroll
   for (int i = 0; i < V; ++i) {
     const int c = i * T + tid;
-    if (c < chunks) {
-      if (!silu) {
-        v[i] = __ldg(P.X + row + c);
-      } else {
-        // gate column of logical chunk c: groups of 8 chunks (64 columns), gate then up
-        const int gc = inter ? ((c >> 3) << 4) + (c & 7) : c;
-        const uint4 g = __ldg(P.X + row + gc);
-        const uint4 u = inter ? __ldg(P.X + row + gc + 8) : __ldg(P.X2 + row + c);
-        v[i].x = silu_mul_pair(g.x, u.x);
-        v[i].y = silu_mul_pair(g.y, u.y);
-        v[i].z = silu_mul_pair(g.z, u.z);
-        v[i].w = silu_mul_pair(g.w, u.w);
-      }
-    }
+    if (c < chunks) v[i] = __ldg(P.X + row + c);
   }
 
-  float r = 1.0f;
-  if (P.flags & FPT_RMSNORM) {
-    double acc = 0.0;
+  double acc = 0.0;
+#pragma unroll
+  for (int i = 0; i < V; ++i)
+    if (i * T + tid < chunks) acc = sumsq(v[i], acc);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((tid & 31) == 0) warp_part[tid >> 5] = acc;
+  __syncthreads();
+  if (tid == 0) {
+    double s = 0.0;
+#pragma unroll
+    for (int w = 0; w < T / 32; ++w) s += warp_part[w];
+    bcast = (float)s;
+  }
+  __syncthreads();
+  if (!(bcast <= 3.4028234e38f)) {               // Inf / NaN in the row (or a genuine overflow): by the definition
+    __syncthreads();
+    acc = 0.0;
 #pragma unroll
     for (int i = 0; i < V; ++i)
-      if (i * T + tid < chunks) acc = sumsq(v[i], acc);
+      if (i * T + tid < chunks) acc = sumsq_exact(v[i], acc);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if ((tid & 31) == 0) warp_part[tid >> 5] = acc;
-    __syncthreads();
-    if (tid == 0) {
-      double s = 0.0;
-#pragma unroll
-      for (int w = 0; w < T / 32; ++w) s += warp_part[w];
-      bcast = (float)s;
-    }
-    __syncthreads();
-    if (!(bcast <= 3.4028234e38f)) {               // Inf / NaN in the row (or a genuine overflow): by the definition
-      __syncthreads();
-      acc = 0.0;
-#pragma unroll
-      for (int i = 0; i < V; ++i)
-        if (i * T + tid < chunks) acc = sumsq_exact(v[i], acc);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      if ((tid & 31) == 0) warp_part[tid >> 5] = acc;
-    }
-    __syncthreads();
-    if (tid == 0) {
-      double s = 0.0;
-#pragma unroll
-      for (int w = 0; w < T / 32; ++w) s += warp_part[w];
-      const float ss = (float)s;                                        // one rounding to float32
-      const float ms = __fdiv_rn(ss, (float)P.K);
-      const float rho = __fsqrt_rn(__fadd_rn(ms, P.eps));
-      bcast = __fdiv_rn(1.0f, rho);
-    }
-    __syncthreads();
-    r = bcast;
   }
+  __syncthreads();
+  if (tid == 0) {
+    double s = 0.0;
+#pragma unroll
+    for (int w = 0; w < T / 32; ++w) s += warp_part[w];
+    const float ss = (float)s;                                        // one rounding to float32
+    const float ms = __fdiv_rn(ss, (float)P.K);
+    const float rho = __fsqrt_rn(__fadd_rn(ms, P.eps));
+    bcast = __fdiv_rn(1.0f, rho);
+  }
+  __syncthreads();
+  const float r = bcast;
   const float s = P.s_in ? __ldg(P.s_in + t) : 1.0f;
   const float rs = P.s_in ? __fmul_rn(r, s) : r;
   const float p = (P.flags & FPT_SCALE_INPUT) ? rs : r;
@@ -115,7 +95,41 @@ __global__ void __launch_bounds__(T, V <= 4 ? 2048 / T : 1) act_quant_kernel(con
   }
 }
 
-// One warp per token for rows of up to 256 * V elements: the row lives in registers, the
+// Without the RMSNorm nothing is reduced over a token (the multiplier is s_in or 1), so a thread takes one 16-byte
+// chunk of any token and the grid covers the chip whatever the number of tokens.  One CTA per token left 37 tokens
+// to 37 CTAs, which, started early behind a matmul that fills the SMs, pile up on the first few SMs to come free:
+// the SwiGLU pass of 37 x 14336 took 21 us there (5.8 us by itself), now 7 us.
+constexpr int kFlatThreads = 256;
+template <bool kSilu>
+__global__ void __launch_bounds__(kFlatThreads) act_quant_flat_kernel(const ActQuantParams P, int ctas_per_row) {
+  pdl_wait();
+  pdl_launch_dependents();
+  const int chunks = P.K >> 3;
+  const int t = blockIdx.x / ctas_per_row;
+  const int c = (blockIdx.x - t * ctas_per_row) * kFlatThreads + threadIdx.x;
+  if (c >= chunks) return;
+  const uint4* row = P.X + (size_t)t * (size_t)(P.ldx >> 3);
+  uint4 v;
+  if constexpr (kSilu) {
+    const bool inter = (P.flags & FPT_GU_INTERLEAVED) != 0;
+    const int gc = inter ? ((c >> 3) << 4) + (c & 7) : c;          // groups of 8 chunks (64 columns), gate then up
+    const uint4 g = __ldg(row + gc);
+    const uint4 u = inter ? __ldg(row + gc + 8) : __ldg(P.X2 + (size_t)t * (size_t)(P.ldx >> 3) + c);
+    v = make_uint4(silu_mul_pair(g.x, u.x), silu_mul_pair(g.y, u.y), silu_mul_pair(g.z, u.z), silu_mul_pair(g.w, u.w));
+  } else {
+    v = __ldg(row + c);
+  }
+  const float rs = P.s_in ? __ldg(P.s_in + t) : 1.0f;
+  const float p = (P.flags & FPT_SCALE_INPUT) ? rs : 1.0f;
+  if (c == 0) {
+    if (P.s_out) P.s_out[t] = rs;
+    if (P.post_inv) P.post_inv[t] = __fdiv_rn(1.0f, p);
+    if (P.r_out) P.r_out[t] = 1.0f;
+  }
+  P.Xq[(size_t)t * (size_t)chunks + c] = quant_word(v, quant_consts(p, P.inv_delta, P.qmax_minus_z, P.flip));
+}
+
+// RMSNorm, one warp per token for rows of up to 256 * V elements: the row lives in registers, the
 // reduction is a warp shuffle, no shared memory and no block-wide barrier.  W warps per CTA.
 template <int V, int W>
 __global__ void __launch_bounds__(W * 32) act_quant_warp_kernel(const ActQuantParams P) {
@@ -132,29 +146,26 @@ __global__ void __launch_bounds__(W * 32) act_quant_warp_kernel(const ActQuantPa
     const int c = i * 32 + lane;
     if (c < chunks) v[i] = __ldg(row + c);
   }
-  float r = 1.0f;
-  if (P.flags & FPT_RMSNORM) {
-    double acc0 = 0.0, acc1 = 0.0;                 // two chains: the float64 adds are latency-bound otherwise
+  double acc0 = 0.0, acc1 = 0.0;                 // two chains: the float64 adds are latency-bound otherwise
+#pragma unroll
+  for (int i = 0; i < V; ++i)
+    if (i * 32 + lane < chunks) { if (i & 1) acc1 = sumsq(v[i], acc1); else acc0 = sumsq(v[i], acc0); }
+  double acc = acc0 + acc1;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (!((float)acc <= 3.4028234e38f)) {          // Inf / NaN in the row (or a genuine overflow): by the definition
+    acc0 = 0.0;
 #pragma unroll
     for (int i = 0; i < V; ++i)
-      if (i * 32 + lane < chunks) { if (i & 1) acc1 = sumsq(v[i], acc1); else acc0 = sumsq(v[i], acc0); }
-    double acc = acc0 + acc1;
+      if (i * 32 + lane < chunks) acc0 = sumsq_exact(v[i], acc0);
+    acc = acc0;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (!((float)acc <= 3.4028234e38f)) {          // Inf / NaN in the row (or a genuine overflow): by the definition
-      acc0 = 0.0;
-#pragma unroll
-      for (int i = 0; i < V; ++i)
-        if (i * 32 + lane < chunks) acc0 = sumsq_exact(v[i], acc0);
-      acc = acc0;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    }
-    const float ss = (float)acc;                   // one rounding to float32 (every lane holds the same sum)
-    const float ms = __fdiv_rn(ss, (float)P.K);
-    const float rho = __fsqrt_rn(__fadd_rn(ms, P.eps));
-    r = __fdiv_rn(1.0f, rho);
   }
+  const float ss = (float)acc;                   // one rounding to float32 (every lane holds the same sum)
+  const float ms = __fdiv_rn(ss, (float)P.K);
+  const float rho = __fsqrt_rn(__fadd_rn(ms, P.eps));
+  const float r = __fdiv_rn(1.0f, rho);
   const float s = P.s_in ? __ldg(P.s_in + t) : 1.0f;
   const float rs = P.s_in ? __fmul_rn(r, s) : r;
   const float p = (P.flags & FPT_SCALE_INPUT) ? rs : r;
@@ -215,26 +226,23 @@ __global__ void __launch_bounds__(1024) act_quant_stream_kernel(const ActQuantPa
       if (!__all_sync(0xffffffffu, ok)) return;
     }
     const uint4* row = reinterpret_cast<const uint4*>(buf0 + (size_t)b * row_bytes);
-    float r = 1.0f;
-    if (P.flags & FPT_RMSNORM) {
-      double acc0 = 0.0, acc1 = 0.0;
-      int c = lane;
-      for (; c + 32 < chunks; c += 64) { acc0 = sumsq(row[c], acc0); acc1 = sumsq(row[c + 32], acc1); }
-      if (c < chunks) acc0 = sumsq(row[c], acc0);
-      double acc = acc0 + acc1;
+    double acc0 = 0.0, acc1 = 0.0;
+    int c = lane;
+    for (; c + 32 < chunks; c += 64) { acc0 = sumsq(row[c], acc0); acc1 = sumsq(row[c + 32], acc1); }
+    if (c < chunks) acc0 = sumsq(row[c], acc0);
+    double acc = acc0 + acc1;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (!((float)acc <= 3.4028234e38f)) {        // Inf / NaN in the row (or a genuine overflow): by the definition
+      acc = 0.0;
+      for (int c2 = lane; c2 < chunks; c2 += 32) acc = sumsq_exact(row[c2], acc);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      if (!((float)acc <= 3.4028234e38f)) {        // Inf / NaN in the row (or a genuine overflow): by the definition
-        acc = 0.0;
-        for (int c2 = lane; c2 < chunks; c2 += 32) acc = sumsq_exact(row[c2], acc);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      }
-      const float ss = (float)acc;                 // one rounding to float32
-      const float ms = __fdiv_rn(ss, (float)P.K);
-      const float rho = __fsqrt_rn(__fadd_rn(ms, P.eps));
-      r = __fdiv_rn(1.0f, rho);
     }
+    const float ss = (float)acc;                 // one rounding to float32
+    const float ms = __fdiv_rn(ss, (float)P.K);
+    const float rho = __fsqrt_rn(__fadd_rn(ms, P.eps));
+    const float r = __fdiv_rn(1.0f, rho);
     const float s = P.s_in ? __ldg(P.s_in + t) : 1.0f;
     const float rs = P.s_in ? __fmul_rn(r, s) : r;
     const float p = (P.flags & FPT_SCALE_INPUT) ? rs : r;
@@ -314,29 +322,30 @@ cudaError_t act_quant_launch(cudaStream_t st, const void* X, int M, int K, int l
   P.qmax_minus_z = qmax - z;
   P.flip = qp->symmetric ? 0x77777777u : 0xFFFFFFFFu;
   const int chunks = K / 8;
+  if (!(flags & FPT_RMSNORM)) {
+    const int per_row = (chunks + kFlatThreads - 1) / kFlatThreads;      // (a grid of 2^31 CTAs would read terabytes)
+    auto kern = (flags & FPT_SILU_MUL) ? act_quant_flat_kernel<true> : act_quant_flat_kernel<false>;
+    return launch_kernel(kern, dim3((unsigned)per_row * (unsigned)M), dim3(kFlatThreads), 0, st, true, P, per_row);
+  }
   // Many tokens: long rows do best with one CTA per token and many CTAs per SM (measured: 2048 x 8192 in
   // 13 us against 19 us for the streaming kernel); short rows with the persistent streaming kernel
   // (16384 x 2048: 20 us against 23 us).
-  if (!(flags & FPT_SILU_MUL) && M >= 512) {
+  if (M >= 512) {
     if (chunks >= 128 && chunks < 512) return launch_stream(P, st);
     if (chunks == 512) return launch<128, 4>(P, st);
     if (chunks > 512 && chunks <= 1024) return launch<256, 4>(P, st);
     if (chunks > 1024 && chunks <= 2048) return launch<512, 4>(P, st);
   }
-  if (!(flags & FPT_SILU_MUL)) {
-    if (chunks <= 64)        return launch_warp<2, 4>(P, st);
-    else if (chunks <= 128)  return launch_warp<4, 4>(P, st);
-    else if (chunks <= 256)  return launch_warp<8, 4>(P, st);
-    else if (chunks <= 512)  return launch_warp<16, 4>(P, st);
-    else if (chunks <= 1024) return launch_warp<32, 4>(P, st);
-  }
-  if (chunks <= 128)        return launch<128, 1>(P, st);
-  else if (chunks <= 256)   return launch<128, 2>(P, st);
-  else if (chunks <= 512)   return launch<256, 2>(P, st);
-  else if (chunks <= 1024)  return launch<256, 4>(P, st);
-  else if (chunks <= 2048)  return launch<512, 4>(P, st);
-  else if (chunks <= 4096)  return launch<512, 8>(P, st);
-  else if (chunks <= 8192)  return launch<1024, 8>(P, st);
+  // Few tokens: the latency of one row is what counts, so as many threads as the row has chunks (one warp per
+  // token instead: 4.4 against 2.1 us at 1 .. 120 tokens of 4096, 3.1 us at 333: the float64 sum is a serial chain)
+  if (chunks <= 64)        return launch_warp<2, 4>(P, st);
+  else if (chunks <= 128)  return launch<128, 1>(P, st);
+  else if (chunks <= 256)  return launch<256, 1>(P, st);
+  else if (chunks <= 512)  return launch<512, 1>(P, st);
+  else if (chunks <= 1024) return launch<512, 2>(P, st);
+  else if (chunks <= 2048) return launch<512, 4>(P, st);
+  else if (chunks <= 4096) return launch<512, 8>(P, st);
+  else if (chunks <= 8192) return launch<1024, 8>(P, st);
   return cudaErrorInvalidValue;
 }
 
