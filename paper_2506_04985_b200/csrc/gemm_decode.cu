@@ -4,7 +4,7 @@
 //
 // The operands swap sides: 128 WEIGHT rows are the M side of the MMA and the (padded) tokens
 // are its N side, so one tcgen05.mma of shape 128 x {16,32,64} x 32 consumes 128 x 32 weight
-// codes.  Weights are widened nibble -> int8 in registers and written to tensor memory
+// codes in 9 .. 32 cycles.  Weights are widened nibble -> int8 in registers and written to tensor memory
 // (tcgen05.st), the MMA reads them from there; only the few token rows are widened into a
 // shared-memory tile.  Nothing of the weight stream is ever stored to shared memory twice.
 //
@@ -25,10 +25,8 @@
 // warps 4-7 token converters (with 64 tokens their tile is half as many bytes as the weights': two
 // warps were the slowest stage of the pipeline), warps 8-19 weight converters (three groups of four
 // warps, each group taking every third k-block: the chain load -> widen -> tcgen05.st -> wait -> arrive
-// is long, and one tcgen05.mma of 128 rows x 32 codes takes about 100 cycles whatever its width, so
-// several k-blocks in conversion are what keeps the tensor core's queue from running dry),
-// warps 20-23 epilogue.
-// Registers are traded between the warpgroups (setmaxnreg): the epilogue holds 64 accumulators per thread.
+// is long, so several k-blocks in conversion are what keeps the stream going), warps 20-23 epilogue.
+// Registers are traded between the warpgroups (setmaxnreg).
 #include <cuda.h>
 
 #include "fpt_internal.cuh"
@@ -45,6 +43,7 @@ constexpr int NPK = 4;                     // packed stages in flight from TMA
 constexpr int kGroups = 3;                 // weight-converter groups
 constexpr int kTokWarps = 4;               // token-converter warps
 constexpr int kMaxTok = 64;
+constexpr int kBatch = 16;                 // tokens an epilogue warp handles at a time
 constexpr int kAccCols = 64;               // per accumulator buffer (two of them)
 constexpr int kAStage0 = 2 * kAccCols;
 constexpr int kTmemCols = 512;
@@ -307,44 +306,36 @@ gemm_w4a4_decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
       // per-row constants, fetched while the matmul of the segment runs
       const float swn = n_ok ? load_scale(P.sw, P.scale_dtype, n) : 0.0f;
       const int zw = (P.wsum && n_ok) ? P.zero_point * __ldg(P.wsum + n) : 0;
-      if (!mbar_wait(acc_full(b), bph, abort_flag, P.status, 4)) break;
+      if (!__all_sync(0xffffffffu, mbar_wait(acc_full(b), bph, abort_flag, P.status, 4))) break;
       tc_fence_after();
-      uint32_t v[kMaxTok];
+      // Nothing below is unrolled further than a batch of sixteen tokens: this code runs once or twice a launch, and
+      // code that is entered for the first time comes at about 200 cycles per 128 bytes (64 unrolled stores of partial
+      // sums took 2.8 us, more than the loads of the whole tile; in batches 0.5 us).
       const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + b * kAccCols;
-      {
-        uint32_t t16[16];
+      const int32_t* sum = nullptr;                      // where the tile's other partial sums are, if this warp adds them
+      int c_first = 0, c_last = -1;
+      bool finalize = whole;
+      if (!whole) {
+        // raw partial sums -> this CTA's shared memory (cluster: the packed weight ring is free, every stage has been
+        // consumed once the accumulator is complete; finished after the cluster barrier below) or its scratch slot
+        // (the last contributor of the tile adds all slots up)
+        const int my_slot = (g == g_begin) ? 0 : 1;
+        int32_t* dst = D.cluster > 1 ? reinterpret_cast<int32_t*>(smem + L::kPkWOff) + quad * 32 + lane
+                                     : D.slots + ((size_t)(blockIdx.x * 2 + my_slot) * npad) * HR + quad * 32 + lane;
+#pragma unroll 1
+        for (int t0 = 0; t0 < npad; t0 += kBatch) {
+          uint32_t v[kBatch];
+          tmem_ld_32x16(taddr + t0, v);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          if (q * 16 < npad) {
-            tmem_ld_32x16(taddr + q * 16, t16);
-            tmem_wait_ld();
-#pragma unroll
-            for (int j = 0; j < 16; ++j) v[q * 16 + j] = t16[j];
-          }
+          for (int t = 0; t < kBatch; ++t) dst[(size_t)(t0 + t) * HR] = (int32_t)v[t];
         }
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(acc_empty(b));
-
-      bool finalize = whole;
-      if (!whole && D.cluster > 1) {
-        // raw partial sums -> this CTA's shared memory (the packed weight ring is free: every stage has been
-        // consumed once the accumulator is complete); finished after the cluster barrier below
-        int32_t* red = reinterpret_cast<int32_t*>(smem + L::kPkWOff) + quad * 32 + lane;
-#pragma unroll
-        for (int t = 0; t < kMaxTok; ++t) if (t < npad) red[t * HR] = (int32_t)v[t];
-      } else if (!whole) {
-        // raw partial sums -> this CTA's slot; the last contributor of the tile adds all slots up
-        const int my_slot = (g == g_begin) ? 0 : 1;
-        int32_t* slot = D.slots + ((size_t)(blockIdx.x * 2 + my_slot) * npad) * HR + quad * 32 + lane;
-#pragma unroll
-        for (int t = 0; t < kMaxTok; ++t) if (t < npad) slot[(size_t)t * HR] = (int32_t)v[t];
+      if (!whole && D.cluster <= 1) {
         __threadfence();
         __syncwarp();
         // contributors of this tile: every CTA whose range meets [tile*KB, (tile+1)*KB)
         const long long t_begin = (long long)tile * D.kblocks, t_end = t_begin + D.kblocks;
-        int c_first = blockIdx.x, c_last = blockIdx.x;
+        c_first = blockIdx.x; c_last = blockIdx.x;
         while (c_first > 0 && range_start(D, c_first, nctas) > t_begin) --c_first;
         while (c_last + 1 < nctas && range_start(D, c_last + 1, nctas) < t_end) ++c_last;
         const uint32_t expected = (uint32_t)(c_last - c_first + 1);
@@ -353,71 +344,70 @@ gemm_w4a4_decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
         old = __shfl_sync(0xffffffffu, old, 0);
         if (old == expected - 1) {
           __threadfence();
-#pragma unroll
-          for (int t = 0; t < kMaxTok; ++t) v[t] = 0;
-          // (sixteen loads in flight per batch: the four epilogue warps are alone on the SM by now, so
-          // nothing else hides the latency of a dependent chain)
-          for (int c = c_first; c <= c_last; ++c) {
-            const int cs = (range_start(D, c, nctas) >= t_begin) ? 0 : 1;
-            const int32_t* src = D.slots + ((size_t)(c * 2 + cs) * npad) * HR + quad * 32 + lane;
-#pragma unroll
-            for (int t0 = 0; t0 < kMaxTok; t0 += 16) {
-              if (t0 < npad) {
-                uint32_t w[16];
-#pragma unroll
-                for (int t = 0; t < 16; ++t) w[t] = (uint32_t)__ldcg(src + (size_t)(t0 + t) * HR);
-#pragma unroll
-                for (int t = 0; t < 16; ++t) v[t0 + t] += w[t];
-              }
-            }
-          }
           if (lane == 0) D.counters[tile * 4 + quad] = 0;      // ready for the next launch
+          sum = D.slots + quad * 32 + lane;
           finalize = true;
         }
       }
-      if (finalize && n_ok) {
+      if (finalize) {
         // (everything the loop needs from the parameter block is read once, here)
         const int m_tok = P.M;
         const size_t ldy = (size_t)P.N;
         int32_t* const acc_out = P.acc_out ? P.acc_out + n : nullptr;
         __nv_bfloat16* const yp = P.Y ? P.Y + n : nullptr;
         const __nv_bfloat16* const resp = P.residual ? P.residual + n : nullptr;
-        if (yp && !acc_out && !resp) {
-          // the usual case, straight-line: sixteen outputs computed, then sixteen stores
+#pragma unroll 1
+        for (int t0 = 0; t0 < npad; t0 += kBatch) {
+          uint32_t v[kBatch];
+          if (sum) {
+            // (sixteen loads in flight per batch: the four epilogue warps are alone on the SM by now, so
+            // nothing else hides the latency of a dependent chain)
 #pragma unroll
-          for (int t0 = 0; t0 < kMaxTok; t0 += 16) {
-            if (t0 < m_tok) {
-              __nv_bfloat16 y[16];
+            for (int t = 0; t < kBatch; ++t) v[t] = 0;
+            for (int c = c_first; c <= c_last; ++c) {
+              const int cs = (range_start(D, c, nctas) >= (long long)tile * D.kblocks) ? 0 : 1;
+              const int32_t* src = sum + ((size_t)(c * 2 + cs) * npad + t0) * HR;
+              uint32_t w[kBatch];
 #pragma unroll
-              for (int q = 0; q < 4; ++q) {
+              for (int t = 0; t < kBatch; ++t) w[t] = (uint32_t)__ldcg(src + (size_t)t * HR);
+#pragma unroll
+              for (int t = 0; t < kBatch; ++t) v[t] += w[t];
+            }
+          } else {
+            tmem_ld_32x16(taddr + t0, v);
+          }
+          if (n_ok) {
+            int a[kBatch];
+#pragma unroll
+            for (int t = 0; t < kBatch; ++t) a[t] = (((int)v[t]) >> 8) - zw;
+            if (acc_out) {
+#pragma unroll
+              for (int t = 0; t < kBatch; ++t) if (t0 + t < m_tok) acc_out[(size_t)(t0 + t) * ldy] = a[t];
+            }
+            if (yp) {
+              float y[kBatch];
+#pragma unroll
+              for (int q = 0; q < kBatch / 4; ++q) {
                 const float4 c4 = *reinterpret_cast<const float4*>(c_s + t0 + 4 * q);
                 const float cc[4] = {c4.x, c4.y, c4.z, c4.w};
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                  const int a = (((int)v[t0 + 4 * q + j]) >> 8) - zw;
-                  y[4 * q + j] = __float2bfloat16_rn(__fmul_rn(__fmul_rn((float)a, swn), cc[j]));
-                }
+                for (int j = 0; j < 4; ++j) y[4 * q + j] = __fmul_rn(__fmul_rn((float)a[4 * q + j], swn), cc[j]);
               }
-              __nv_bfloat16* o = yp + (size_t)t0 * ldy;
+              if (resp) {
 #pragma unroll
-              for (int t = 0; t < 16; ++t) if (t0 + t < m_tok) o[(size_t)t * ldy] = y[t];
+                for (int t = 0; t < kBatch; ++t)
+                  if (t0 + t < m_tok) y[t] = __fadd_rn(y[t], __fmul_rn(__bfloat162float(resp[(size_t)(t0 + t) * ldy]), rs_s[t0 + t]));
+              }
+#pragma unroll
+              for (int t = 0; t < kBatch; ++t) if (t0 + t < m_tok) yp[(size_t)(t0 + t) * ldy] = __float2bfloat16_rn(y[t]);
             }
           }
-        } else {
-#pragma unroll
-          for (int t = 0; t < kMaxTok; ++t) {
-            if (t < m_tok) {
-              const int a = (((int)v[t]) >> 8) - zw;
-              if (acc_out) acc_out[(size_t)t * ldy] = a;
-              if (yp) {
-                float y = __fmul_rn(__fmul_rn((float)a, swn), c_s[t]);
-                if (resp) y = __fadd_rn(y, __fmul_rn(__bfloat162float(resp[(size_t)t * ldy]), rs_s[t]));
-                yp[(size_t)t * ldy] = __float2bfloat16_rn(y);
-              }
-            }
-          }
+          __syncwarp();
         }
       }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(acc_empty(b));
       g += kb1 - kb0;
       ++seg;
     }
@@ -425,41 +415,40 @@ gemm_w4a4_decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
 
   if (D.cluster > 1) {
     // ---------------------------------------------------------------- split tiles: exchange inside the cluster
+    // Every thread of the CTA takes part (the other roles are done): this CTA finishes tokens
+    // [rank * tp, (rank + 1) * tp) of the tile, one (token, weight row) output per thread and pass, adding the partial
+    // sums of all CTAs of the cluster straight from their shared memory.  A thread keeps its weight row, whose
+    // constants it fetches in front of the barrier.
+    static_assert(kThreads % HR == 0, "a thread keeps its weight row");
+    const uint32_t rank = cluster_ctarank(), csize = cluster_nctarank();
+    const int tp = D.npad / (int)csize;
+    const int t_lo = (int)rank * tp;
+    const int nl = threadIdx.x % HR;
+    const int n = (int)(g_begin / D.kblocks) * HR + nl;
+    const bool n_ok = n < P.N;
+    const float swn = n_ok ? load_scale(P.sw, P.scale_dtype, n) : 0.0f;
+    const int zw = (P.wsum && n_ok) ? P.zero_point * __ldg(P.wsum + n) : 0;
+    const size_t ldy = (size_t)P.N;
+    const uint32_t red0 = sbase + L::kPkWOff;
     __syncwarp();
     cluster_sync_all();                                  // every CTA's partial sums are in its shared memory
     {
-      // Every thread of the CTA takes part (the other roles are done): this CTA finishes tokens
-      // [rank * tp, (rank + 1) * tp) of the tile, one (token, weight row) output per thread and pass,
-      // adding the partial sums of all CTAs of the cluster straight from their shared memory.
-      const uint32_t rank = cluster_ctarank(), csize = cluster_nctarank();
-      const int tp = D.npad / (int)csize;
-      const int t_lo = (int)rank * tp;
-      const int tile = (int)(g_begin / D.kblocks);
-      const int m_tok = P.M;
-      const size_t ldy = (size_t)P.N;
-      const uint32_t red0 = sbase + L::kPkWOff;
       uint32_t peer[8];
 #pragma unroll
       for (int c = 0; c < 8; ++c) peer[c] = map_to_cta(red0, (uint32_t)c < csize ? (uint32_t)c : 0u);
-      for (int idx = threadIdx.x; idx < tp * HR; idx += kThreads) {
-        const int tok = t_lo + idx / HR, nl = idx % HR;
-        const int n = tile * HR + nl;
+#pragma unroll 1
+      for (int tok = t_lo + threadIdx.x / HR; tok < t_lo + tp; tok += kThreads / HR) {
         const uint32_t off = 4u * (uint32_t)(tok * HR + nl);
         uint32_t w[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c) w[c] = (uint32_t)c < csize ? ld_shared_cluster_u32(peer[c] + off) : 0u;
         const int sum = (int)(((w[0] + w[1]) + (w[2] + w[3])) + ((w[4] + w[5]) + (w[6] + w[7])));
-        if (n < P.N && tok < m_tok) {
-          const int zw = P.wsum ? P.zero_point * __ldg(P.wsum + n) : 0;
+        if (n_ok && tok < P.M) {
           const int a = (sum >> 8) - zw;
           if (P.acc_out) P.acc_out[(size_t)tok * ldy + n] = a;
           if (P.Y) {
-            const float ct = P.post ? __fmul_rn(P.act_scale, __ldg(P.post + tok)) : P.act_scale;
-            float y = __fmul_rn(__fmul_rn((float)a, load_scale(P.sw, P.scale_dtype, n)), ct);
-            if (P.residual) {
-              const float rs = P.res_scale ? __ldg(P.res_scale + tok) : 1.0f;
-              y = __fadd_rn(y, __fmul_rn(__bfloat162float(P.residual[(size_t)tok * ldy + n]), rs));
-            }
+            float y = __fmul_rn(__fmul_rn((float)a, swn), c_s[tok]);
+            if (P.residual) y = __fadd_rn(y, __fmul_rn(__bfloat162float(P.residual[(size_t)tok * ldy + n]), rs_s[tok]));
             P.Y[(size_t)tok * ldy + n] = __float2bfloat16_rn(y);
           }
         }
@@ -533,10 +522,11 @@ int gemm_decode_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, co
     const int max_split = D.kblocks / 2 > 0 ? D.kblocks / 2 : 1;      // at least 2 k-blocks (512 codes) per range
     if (split > max_split) split = max_split;
     ctas = D.tiles * split;
-    // a power-of-two split up to 8 that keeps at least 85 % of those CTAs: the ranges of a tile become one cluster
+    // a power-of-two split up to 8: the ranges of a tile become one cluster.  (Also where that leaves SMs idle: 48
+    // tiles in 96 CTAs of clusters of two take 10.2 us at 37 tokens, in 144 ranges through scratch slots 17.2 us.)
     int pw = 1;
     while (pw * 2 <= split && pw * 2 <= 8) pw *= 2;
-    D.cluster = (pw > 1 && !D.whole_tiles && pw * 100 >= split * 85 && D.kblocks % pw == 0 && D.npad % pw == 0) ? pw : 0;
+    D.cluster = (pw > 1 && !D.whole_tiles && D.kblocks % pw == 0 && D.npad % pw == 0) ? pw : 0;
     if (D.cluster) ctas = D.tiles * pw;
     // (112 tiles stay on 112 SMs: cutting them into 148 equal ranges was measured slower, 19.4 against
     // 14.4 us at 64 tokens -- the partial sums of a split tile are 32 KB per range)
