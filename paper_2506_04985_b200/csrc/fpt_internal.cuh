@@ -58,6 +58,7 @@ int gemm_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, const Gem
 // gemm_decode.cu: the weight-streaming kernel for M <= 64 and the scratch it needs.
 size_t gemm_decode_scratch_bytes(int M);
 int gemm_decode_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, const GemmParams& P, void* scratch);
+bool gemm_decode_in_two(int N, int K);      // 65..128 tokens as two launches (which then need no scratch)
 inline size_t gemm_scratch_bytes(int M) { return M <= 64 ? gemm_decode_scratch_bytes(M) : 0; }
 
 // gemm_decode_small.cu: register-only weight streaming for M <= 16 (no scratch).

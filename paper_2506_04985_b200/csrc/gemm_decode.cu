@@ -484,12 +484,59 @@ static bool make_map(CUtensorMap* m, const void* base, int rows, int K, int box_
 
 static int num_sms() { return device_sm_count(); }
 
+// CTAs of one cluster that share a tile (2, 4 or 8), or 0: tiles too many for it, rows too short, k-blocks or tokens
+// that do not divide, or not all clusters resident at once.
+static int cluster_size(int tiles, int kblocks, int npad) {
+  const int sms = num_sms() < kDecodeMaxCtas ? num_sms() : kDecodeMaxCtas;
+  if (tiles > sms || tiles * 4 > kDecodeMaxCounters) return 0;
+  int split = sms / tiles;
+  if (split > kblocks / 2) split = kblocks / 2;                        // at least 2 k-blocks (512 codes) per range
+  int cl = 1, idx = 0;
+  while (cl * 2 <= split && cl * 2 <= 8) { cl *= 2; ++idx; }
+  if (cl < 2 || kblocks % cl != 0 || npad % cl != 0) return 0;
+  // the clusters must fit: with one CTA per SM a cluster needs that many free SMs in one GPC
+  static PerDeviceInt fits[4];                                         // cluster sizes 2, 4, 8 -> index 1, 2, 3
+  const int ok = fits[idx].get([&] {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cl, 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = Smem::kAlloc;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)cl; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, gemm_w4a4_decode_kernel, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+    return n > 0 ? n + 1 : 1;                                          // 1: does not fit (cached as such)
+  }) - 1;
+  return ok >= tiles ? cl : 0;
+}
+
 }  // namespace decode
 
 int decode_npad(int M) { return M <= 16 ? 16 : M <= 32 ? 32 : 64; }
 
 size_t gemm_decode_scratch_bytes(int M) {
   return (size_t)kDecodeMaxCtas * 2 * (size_t)decode_npad(M) * decode::HR * sizeof(int32_t);
+}
+
+// 65 .. 128 tokens: whether two launches of this kernel, 64 tokens and the rest, beat the CTA-pair kernel, whose tiles
+// of 256 x 208 leave most of the chip idle when N is small and K long.  Both sides as measured: the pair kernel takes
+// 0.33 us a k-block of 128 codes and round of tiles plus 5 us, this kernel 0.42 us a k-block of 256 codes of a CTA's
+// range plus 5.5 us a launch (the second finds the weights in L2); a tenth of margin.
+// 120 tokens, 4096x14336: 41.6 -> 24.0 us; 4096x4096 and 6144x4096 stay (16.9 and 17.1 us).
+bool gemm_decode_in_two(int N, int K) {
+  using namespace decode;
+  const int tiles = (N + HR - 1) / HR, kblocks = (K + BK - 1) / BK;
+  static PerDeviceInt attr_set;
+  if (!ensure_smem_attr(attr_set, gemm_w4a4_decode_kernel, Smem::kAlloc)) return false;
+  const int cl = cluster_size(tiles, kblocks, 16);                     // (16 to 64 padded tokens: any of them divides)
+  if (cl < 2) return false;
+  const int pairs = num_sms() >= 2 ? num_sms() / 2 : 1;
+  const int rounds = ((N + 207) / 208 + pairs - 1) / pairs;
+  const int pair_ns = rounds * (K / 128) * 330 + 5000;
+  const int two_ns = 2 * (kblocks / cl * 420 + 5500);
+  return two_ns * 10 < pair_ns * 9;
 }
 
 // Xq [M <= 64, K/2], Wq [N, K/2]; `scratch` holds gemm_decode_scratch_bytes(M) bytes; the counters
@@ -524,10 +571,8 @@ int gemm_decode_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, co
     ctas = D.tiles * split;
     // a power-of-two split up to 8: the ranges of a tile become one cluster.  (Also where that leaves SMs idle: 48
     // tiles in 96 CTAs of clusters of two take 10.2 us at 37 tokens, in 144 ranges through scratch slots 17.2 us.)
-    int pw = 1;
-    while (pw * 2 <= split && pw * 2 <= 8) pw *= 2;
-    D.cluster = (pw > 1 && !D.whole_tiles && D.kblocks % pw == 0 && D.npad % pw == 0) ? pw : 0;
-    if (D.cluster) ctas = D.tiles * pw;
+    D.cluster = cluster_size(D.tiles, D.kblocks, D.npad);
+    if (D.cluster) ctas = D.tiles * D.cluster;
     // (112 tiles stay on 112 SMs: cutting them into 148 equal ranges was measured slower, 19.4 against
     // 14.4 us at 64 tokens -- the partial sums of a split tile are 32 KB per range)
   }
@@ -535,26 +580,6 @@ int gemm_decode_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, co
   if (units < ctas) ctas = (int)units;
   D.per = (int)(D.total / ctas);
   D.rem = (int)(D.total % ctas);
-  if (D.cluster > 1) {
-    // the clusters must fit: with one CTA per SM a cluster needs that many free SMs in one GPC
-    static PerDeviceInt fits[4];                          // cluster sizes 2, 4, 8 -> index 1, 2, 3
-    const int idx = D.cluster == 2 ? 1 : D.cluster == 4 ? 2 : 3;
-    const int cl = D.cluster;
-    const int ok = fits[idx].get([&] {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(cl, 1, 1);
-      cfg.blockDim = dim3(kThreads, 1, 1);
-      cfg.dynamicSmemBytes = Smem::kAlloc;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = (unsigned)cl; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-      cfg.attrs = attr; cfg.numAttrs = 1;
-      int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, gemm_w4a4_decode_kernel, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
-      return n > 0 ? n + 1 : 1;                           // 1: does not fit (cached as such)
-    }) - 1;
-    if (ok * D.cluster < ctas) D.cluster = 0;             // not all clusters resident at once: use the slots instead
-  }
   const cudaError_t e = D.cluster > 1
       ? launch_kernel_cluster(gemm_w4a4_decode_kernel, dim3(ctas), dim3(kThreads), Smem::kAlloc, st, true, D.cluster, tmW, tmX, D)
       : launch_kernel(gemm_w4a4_decode_kernel, dim3(ctas), dim3(kThreads), Smem::kAlloc, st, true, tmW, tmX, D);

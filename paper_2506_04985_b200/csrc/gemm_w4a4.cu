@@ -313,6 +313,20 @@ int gemm_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, const Gem
   if (P.M <= 16) return gemm_decode_small_launch(st, Xq, Wq, P);
   if (P.M <= 64 && P.scratch) return gemm_decode_launch(st, Xq, Wq, P, P.scratch);
   if (P.M > 128 && P.N > 128) return gemm_pair_launch(st, Xq, Wq, P);
+  if (P.M > 64 && P.M <= 128 && P.N > 128 && gemm_decode_in_two(P.N, P.K)) {
+    GemmParams h = P;
+    h.M = 64;
+    const int rc = gemm_decode_launch(st, Xq, Wq, h, nullptr);
+    if (rc) return rc;
+    const size_t skip = (size_t)64 * (size_t)P.N;
+    h.M = P.M - 64;
+    if (h.post) h.post += 64;
+    if (h.residual) h.residual += skip;
+    if (h.res_scale) h.res_scale += 64;
+    if (h.Y) h.Y += skip;
+    if (h.acc_out) h.acc_out += skip;
+    return gemm_decode_launch(st, Xq + (size_t)64 * (size_t)(P.K / 2), Wq, h, nullptr);
+  }
   if (P.M > 64 && P.N > 128) {
     // 65..128 tokens: the CTA-pair kernel (half of its 256 activation rows empty) still beats the
     // one-CTA kernel per k-block (measured 0.5 against 0.68 us), unless it needs more rounds of tiles

@@ -100,3 +100,11 @@ def test_decode_split_tiles_cluster_and_slot_paths(M, N, K, what):
     ws = B.new_workspace(B.OP_GEMM, M, N, K)
     _run(M, N, K, seed=21, ws=ws, reps=2)
     _run(M, N, K, symmetric=False, z=9, seed=22, post=True, residual=True, f16=False, ws=ws, reps=2)
+
+
+@pytest.mark.parametrize("M", [65, 80, 113, 128])
+@pytest.mark.parametrize("N,K", [(1024, 8192), (4096, 14336)])
+def test_decode_65_to_128_tokens_in_two_launches(M, N, K):
+    """Few outputs and long rows: 64 tokens and the rest, the second launch on offset operands."""
+    _run(M, N, K, seed=31, f16=False)
+    _run(M, N, K, symmetric=False, z=9, seed=32, post=True, residual=True)
