@@ -237,7 +237,7 @@ extern "C" int fpt_decoder_mlp(void* stream, const void* X, int M, int d, int d_
   // X~ = RMSNorm(X) on the grid qp_in; S_n = S_{n-1} * r
   if (act_quant_launch(st, X, M, d, d, qp_in, FPT_RMSNORM, eps, nullptr, s_prev, Xq, sn, nullptr, r_ws) != cudaSuccess)
     return FPT_ERR_CUDA;
-  if (M > 128) {
+  if (M > 128 || (M <= 16 && !mid_hadamard)) {
     // gate || up in one matmul whose epilogue forms m = bf16(silu(g) * u) and quantises m * S_n:
     // the static grid and S_n are known before the matmul starts, so g and u never reach memory
     GemmParams P{};
@@ -254,7 +254,7 @@ extern "C" int fpt_decoder_mlp(void* stream, const void* X, int M, int d, int d_
     }
     P.status = reinterpret_cast<uint32_t*>(workspace);
     P.scratch = ws + kStatusBytes;
-    rc = gemm_pair_launch(st, Xq, Wgu_q, P);
+    rc = M > 128 ? gemm_pair_launch(st, Xq, Wgu_q, P) : gemm_decode_small_launch(st, Xq, Wgu_q, P);
     if (rc) return rc;
     if (mid_hadamard &&
         hadamard_quant_launch(st, GU, M, d_ff, d_ff, qp_mid, 0, sn, Mq) != cudaSuccess)

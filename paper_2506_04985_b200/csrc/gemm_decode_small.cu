@@ -16,6 +16,7 @@
 // eight token groups this form was measured 1.5 to 2.5 times slower than that kernel (registers,
 // re-widening the activations per group, legacy-MMA issue rate).
 #include "fpt_internal.cuh"
+#include "quant_math.cuh"
 
 namespace fpt {
 namespace decode_small {
@@ -53,7 +54,9 @@ __device__ __forceinline__ void gather_i8(const uint4& lo, const uint4& hi, uint
 
 // kA8: Xq holds int8 codes [M, K] instead of packed 4-bit codes [M, K/2] (signed, kBUnsigned = false).
 // U: 64-byte blocks in flight per warp; kMinCtas: CTAs per SM the register allocation must allow.
-template <int NW, int NT, bool kBUnsigned, bool kA8 = false, int U = 4, int kMinCtas = 768 / (NW * 32)>
+// kSwiglu: the rows are gate || up in groups of 64 + 64; a CTA takes eight gate rows and the matching up rows, and packed
+// codes of bf16(silu(g) * u) * S_n leave (P.Mq) instead of bf16 outputs: one word a token and CTA.
+template <int NW, int NT, bool kBUnsigned, bool kA8 = false, int U = 4, int kMinCtas = 768 / (NW * 32), bool kSwiglu = false>
 __global__ void __launch_bounds__(NW * 32, kMinCtas) gemm_w4a4_decode_small_kernel(const uint8_t* __restrict__ Xq,
                                                                           const uint8_t* __restrict__ Wq, const Params D) {
   __shared__ int part[NW][kRows][8 * NT];
@@ -62,10 +65,11 @@ __global__ void __launch_bounds__(NW * 32, kMinCtas) gemm_w4a4_decode_small_kern
   const GemmParams& P = D.g;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
-  const int n0 = blockIdx.x * kRows;
+  const int n0 = kSwiglu ? (int)(blockIdx.x >> 3) * 128 + (int)(blockIdx.x & 7) * 8 : (int)blockIdx.x * kRows;
+  constexpr int kSecond = kSwiglu ? 64 : 8;      // from a lane's first row to its second
   const size_t row_bytes = (size_t)P.K / 2;
   // rows past the end of the matrix and tokens past M are read from a valid row and masked to zero
-  const int ra = n0 + g, rb = n0 + g + 8;
+  const int ra = n0 + g, rb = n0 + g + kSecond;
   const bool ra_ok = ra < P.N, rb_ok = rb < P.N;
   const uint8_t* wa = Wq + (size_t)(ra_ok ? ra : 0) * row_bytes + 16 * t;
   const uint8_t* wb = Wq + (size_t)(rb_ok ? rb : 0) * row_bytes + 16 * t;
@@ -92,7 +96,7 @@ __global__ void __launch_bounds__(NW * 32, kMinCtas) gemm_w4a4_decode_small_kern
   for (int q = 0; q < kPer; ++q) {
     const int o = threadIdx.x + q * NW * 32;
     const int o_n = n0 + o % kRows, o_tok = o / kRows;
-    o_ok[q] = o < kOut && o_n < P.N && o_tok < P.M;
+    o_ok[q] = !kSwiglu && o < kOut && o_n < P.N && o_tok < P.M;
     o_sw[q] = 0.0f; o_ct[q] = P.act_scale; o_rs[q] = 1.0f; o_res[q] = 0.0f; o_zw[q] = 0;
     if (o_ok[q]) {
       o_sw[q] = load_scale(P.sw, P.scale_dtype, o_n);
@@ -103,6 +107,15 @@ __global__ void __launch_bounds__(NW * 32, kMinCtas) gemm_w4a4_decode_small_kern
         if (P.res_scale) o_rs[q] = __ldg(P.res_scale + o_tok);
       }
     }
+  }
+
+  // SwiGLU: thread (token, feature) = (tid / 8, tid % 8) finishes one product
+  const int s_tok = threadIdx.x >> 3, s_f = threadIdx.x & 7;
+  float s_gate = 0.0f, s_up = 0.0f, s_sn = 0.0f;
+  if (kSwiglu && s_tok < 8 * NT) {
+    s_gate = load_scale(P.sw, P.scale_dtype, n0 + s_f);
+    s_up = load_scale(P.sw, P.scale_dtype, n0 + kSecond + s_f);
+    if (s_tok < P.M) s_sn = __ldg(P.mid_scale + s_tok);
   }
 
   const uint4 zero = make_uint4(0, 0, 0, 0);
@@ -150,6 +163,19 @@ __global__ void __launch_bounds__(NW * 32, kMinCtas) gemm_w4a4_decode_small_kern
     part[warp][g + 8][nt * 8 + 2 * t + 1] = acc[nt][3];
   }
   __syncthreads();
+  if constexpr (kSwiglu) {
+    if (s_tok < 8 * NT) {                          // (whole warps)
+      int sg = 0, su = 0;
+#pragma unroll
+      for (int w = 0; w < NW; ++w) { sg += part[w][s_f][s_tok]; su += part[w][s_f + 8][s_tok]; }
+      const uint32_t code = swiglu_code(__fmul_rn(__fmul_rn((float)(sg >> 8), s_gate), P.act_scale),
+                                        __fmul_rn(__fmul_rn((float)(su >> 8), s_up), P.act_scale), s_sn, P.mid_inv_delta,
+                                        P.mid_qmax_minus_z, P.mid_flip);
+      const uint32_t word = pack_nibbles(code, lane);
+      if (s_f == 0 && s_tok < P.M) reinterpret_cast<uint32_t*>(P.Mq)[(size_t)s_tok * (size_t)(P.N >> 4) + blockIdx.x] = word;
+    }
+    return;
+  }
   // consecutive threads take consecutive weight rows of one token
 #pragma unroll
   for (int q = 0; q < kPer; ++q) {
@@ -174,7 +200,9 @@ template <int NW, int NT, int U = 4, int kMinCtas = 768 / (NW * 32)>
 static int launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, const Params& D) {
   const int grid = (D.g.N + kRows - 1) / kRows;
   cudaError_t e;
-  if (D.g.a_bits == 8)
+  if (D.g.Mq)
+    e = launch_kernel(gemm_w4a4_decode_small_kernel<NW, NT, false, false, U, kMinCtas, true>, dim3(grid), dim3(NW * 32), 0, st, true, Xq, Wq, D);
+  else if (D.g.a_bits == 8)
     e = launch_kernel(gemm_w4a4_decode_small_kernel<NW, NT, false, true>, dim3(grid), dim3(NW * 32), 0, st, true, Xq, Wq, D);
   else if (D.g.a_unsigned)
     e = launch_kernel(gemm_w4a4_decode_small_kernel<NW, NT, true, false, U, kMinCtas>, dim3(grid), dim3(NW * 32), 0, st, true, Xq, Wq, D);
@@ -185,7 +213,7 @@ static int launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, const P
 
 }  // namespace decode_small
 
-// Xq [M <= 16, K/2], Wq [N, K/2]; needs no scratch.
+// Xq [M <= 16, K/2], Wq [N, K/2]; needs no scratch.  With P.Mq the weight is gate || up (N % 128 == 0, symmetric codes).
 int gemm_decode_small_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, const GemmParams& P) {
   using namespace decode_small;
   Params D;

@@ -146,6 +146,22 @@ __device__ __forceinline__ uint32_t quant_word(const uint4& v, const QuantConsts
   return w ^ c.flip;
 }
 
+// One SwiGLU product on the grid of the down projection, from the float32 results of the two linears (rounded to bf16
+// here, like the product): the nibble of one code.
+__device__ __forceinline__ uint32_t swiglu_code(float gate, float up, float sn, float inv_delta, int qmax_minus_z, uint32_t flip) {
+  const float g = __bfloat162float(__float2bfloat16_rn(gate)), u = __bfloat162float(__float2bfloat16_rn(up));
+  const uint32_t m = f32_to_bf16_bits(__fmul_rn(silu_spec(g), u));
+  return (quant_pair(m, quant_consts(sn, inv_delta, qmax_minus_z, flip), 0u) ^ flip) & 15u;
+}
+// Eight consecutive lanes hold one nibble each -> their word, in each of the eight.  The whole warp takes part.
+__device__ __forceinline__ uint32_t pack_nibbles(uint32_t code, int lane) {
+  uint32_t w = code << (4 * (lane & 7));
+  w |= __shfl_xor_sync(0xffffffffu, w, 1);
+  w |= __shfl_xor_sync(0xffffffffu, w, 2);
+  w |= __shfl_xor_sync(0xffffffffu, w, 4);
+  return w;
+}
+
 // acc + the 8 squares of a chunk in float64.  The bf16 magnitude bits, moved to the top of a
 // float64's high word, are the value times 2^-896 for every finite input (normal, subnormal or
 // zero alike); one exact multiply by 2^896 restores it, the square is exact in float64 and the
