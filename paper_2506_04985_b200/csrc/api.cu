@@ -71,6 +71,7 @@ int linear4_run(cudaStream_t st, const void* X, int M, int K, const uint8_t* Wq,
   P.Y = reinterpret_cast<__nv_bfloat16*>(Y);
   P.status = reinterpret_cast<uint32_t*>(ws);
   P.scratch = ws + kStatusBytes;
+  P.early_weights = 1;                                              // act_quant is in front
   return gemm_launch(st, Xq, Wq, P);
 }
 
@@ -136,10 +137,11 @@ extern "C" int fpt_check_status(void* stream, void* workspace) {
   return word == 0 ? FPT_OK : FPT_ERR_TIMEOUT;
 }
 
-extern "C" int fpt_w4a4_gemm(void* stream, const uint8_t* Xq, const uint8_t* Wq, int M, int N, int K, const void* sw,
-                             int scale_dtype, const int32_t* wsum, float act_scale, int act_symmetric,
-                             int act_zero_point, const float* post, const void* residual, const float* res_scale,
-                             void* Y, int32_t* acc_out, void* workspace, size_t workspace_bytes) {
+// fpt_w4a4_gemm; `early`: see GemmParams::early_weights (only the composed calls below can say so).
+static int gemm4(void* stream, const uint8_t* Xq, const uint8_t* Wq, int M, int N, int K, const void* sw, int scale_dtype,
+                 const int32_t* wsum, float act_scale, int act_symmetric, int act_zero_point, const float* post,
+                 const void* residual, const float* res_scale, void* Y, int32_t* acc_out, void* workspace,
+                 size_t workspace_bytes, int early) {
   if (!Xq || !Wq || !sw || (!Y && !acc_out)) return FPT_ERR_BAD_ARG;
   int rc = check_gemm_shape(M, N, K);
   if (rc) return rc;
@@ -164,7 +166,16 @@ extern "C" int fpt_w4a4_gemm(void* stream, const uint8_t* Xq, const uint8_t* Wq,
   P.acc_out = acc_out;
   P.status = reinterpret_cast<uint32_t*>(workspace);
   P.scratch = reinterpret_cast<uint8_t*>(workspace) + kStatusBytes;
+  P.early_weights = early;
   return gemm_launch((cudaStream_t)stream, Xq, Wq, P);
+}
+
+extern "C" int fpt_w4a4_gemm(void* stream, const uint8_t* Xq, const uint8_t* Wq, int M, int N, int K, const void* sw,
+                             int scale_dtype, const int32_t* wsum, float act_scale, int act_symmetric,
+                             int act_zero_point, const float* post, const void* residual, const float* res_scale,
+                             void* Y, int32_t* acc_out, void* workspace, size_t workspace_bytes) {
+  return gemm4(stream, Xq, Wq, M, N, K, sw, scale_dtype, wsum, act_scale, act_symmetric, act_zero_point, post, residual,
+               res_scale, Y, acc_out, workspace, workspace_bytes, 0);
 }
 
 extern "C" int fpt_w4a4_linear(void* stream, const void* X, int M, int K, const uint8_t* Wq, const void* sw,
@@ -254,20 +265,21 @@ extern "C" int fpt_decoder_mlp(void* stream, const void* X, int M, int d, int d_
     }
     P.status = reinterpret_cast<uint32_t*>(workspace);
     P.scratch = ws + kStatusBytes;
+    P.early_weights = 1;
     rc = M > 128 ? gemm_pair_launch(st, Xq, Wgu_q, P) : gemm_decode_small_launch(st, Xq, Wgu_q, P);
     if (rc) return rc;
     if (mid_hadamard &&
         hadamard_quant_launch(st, GU, M, d_ff, d_ff, qp_mid, 0, sn, Mq) != cudaSuccess)
       return FPT_ERR_CUDA;
   } else if (mid_hadamard) {
-    rc = fpt_w4a4_gemm(stream, Xq, Wgu_q, M, 2 * d_ff, d, sw_gu, scale_dtype, nullptr, qp_in->scale, 1, 0, nullptr,
-                       nullptr, nullptr, GU, nullptr, workspace, gemm_ws);
+    rc = gemm4(stream, Xq, Wgu_q, M, 2 * d_ff, d, sw_gu, scale_dtype, nullptr, qp_in->scale, 1, 0, nullptr,
+               nullptr, nullptr, GU, nullptr, workspace, gemm_ws, 1);
     if (rc) return rc;
     if (hadamard_quant_launch(st, GU, M, d_ff, 2 * d_ff, qp_mid, 1, sn, Mq) != cudaSuccess) return FPT_ERR_CUDA;
   } else {
     // gate || up in one matmul over the interleaved weight
-    rc = fpt_w4a4_gemm(stream, Xq, Wgu_q, M, 2 * d_ff, d, sw_gu, scale_dtype, nullptr, qp_in->scale, 1, 0, nullptr,
-                       nullptr, nullptr, GU, nullptr, workspace, gemm_ws);
+    rc = gemm4(stream, Xq, Wgu_q, M, 2 * d_ff, d, sw_gu, scale_dtype, nullptr, qp_in->scale, 1, 0, nullptr,
+               nullptr, nullptr, GU, nullptr, workspace, gemm_ws, 1);
     if (rc) return rc;
     // m = bf16(silu(g) * u), quantised after the multiply by S_n
     if (act_quant_launch(st, GU, M, d_ff, 2 * d_ff, qp_mid, FPT_SILU_MUL | FPT_GU_INTERLEAVED | FPT_SCALE_INPUT, 0.0f,
@@ -275,8 +287,8 @@ extern "C" int fpt_decoder_mlp(void* stream, const void* X, int M, int d, int d_
       return FPT_ERR_CUDA;
   }
   // down projection; the normalised residual X * r joins before the final rounding
-  return fpt_w4a4_gemm(stream, Mq, Wd_q, M, d, d_ff, sw_d, scale_dtype, nullptr, qp_mid->scale, 1, 0, nullptr,
-                       add_residual ? X : nullptr, add_residual ? r_ws : nullptr, Y, nullptr, workspace, gemm_ws);
+  return gemm4(stream, Mq, Wd_q, M, d, d_ff, sw_d, scale_dtype, nullptr, qp_mid->scale, 1, 0, nullptr,
+               add_residual ? X : nullptr, add_residual ? r_ws : nullptr, Y, nullptr, workspace, gemm_ws, 1);
 }
 
 extern "C" int fpt_decoder_attn_qkv(void* stream, const void* X, int M, int d, const uint8_t* Wqkv_q, const void* sw_qkv,
@@ -297,8 +309,8 @@ extern "C" int fpt_decoder_attn_qkv(void* stream, const void* X, int M, int d, c
   if (act_quant_launch((cudaStream_t)stream, X, M, d, d, qp_in, FPT_RMSNORM, eps, nullptr, s_prev, Xq, s_out, nullptr,
                        r_out) != cudaSuccess)
     return FPT_ERR_CUDA;
-  return fpt_w4a4_gemm(stream, Xq, Wqkv_q, M, n_qkv, d, sw_qkv, scale_dtype, wsum_qkv, qp_in->scale, qp_in->symmetric,
-                       qp_in->zero_point, nullptr, nullptr, nullptr, QKV, nullptr, workspace, gemm_ws);
+  return gemm4(stream, Xq, Wqkv_q, M, n_qkv, d, sw_qkv, scale_dtype, wsum_qkv, qp_in->scale, qp_in->symmetric,
+               qp_in->zero_point, nullptr, nullptr, nullptr, QKV, nullptr, workspace, gemm_ws, 1);
 }
 
 extern "C" int fpt_decoder_attn_out(void* stream, const void* A, int M, int k_o, const uint8_t* Wo_q, const void* sw_o,
@@ -321,8 +333,8 @@ extern "C" int fpt_decoder_attn_out(void* stream, const void* A, int M, int k_o,
                        nullptr, nullptr) != cudaSuccess)
     return FPT_ERR_CUDA;
   // output projection; the normalised residual X * r joins before the final rounding
-  return fpt_w4a4_gemm(stream, Aq, Wo_q, M, d, k_o, sw_o, scale_dtype, wsum_o, qp_ap->scale, qp_ap->symmetric,
-                       qp_ap->zero_point, nullptr, X, X ? r : nullptr, Y, nullptr, workspace, gemm_ws);
+  return gemm4(stream, Aq, Wo_q, M, d, k_o, sw_o, scale_dtype, wsum_o, qp_ap->scale, qp_ap->symmetric,
+               qp_ap->zero_point, nullptr, X, X ? r : nullptr, Y, nullptr, workspace, gemm_ws, 1);
 }
 
 extern "C" int fpt_w4a4_linear_dynamic(void* stream, const void* X, int M, int K, const uint8_t* Wq, const void* sw,
@@ -358,6 +370,6 @@ extern "C" int fpt_w4a4_linear_dynamic(void* stream, const void* X, int M, int K
   if (act_quant_dyn_launch((cudaStream_t)stream, X, M, K, K, 4, 1, 1.0f, flags, eps, s_in, post_mode, post, Xq, s_out,
                            c_t, nullptr, nullptr) != cudaSuccess)
     return FPT_ERR_CUDA;
-  return fpt_w4a4_gemm(stream, Xq, Wq, M, N, K, sw, scale_dtype, nullptr, 1.0f, 1, 0, c_t, nullptr, nullptr, Y, nullptr,
-                       workspace, gemm_ws);
+  return gemm4(stream, Xq, Wq, M, N, K, sw, scale_dtype, nullptr, 1.0f, 1, 0, c_t, nullptr, nullptr, Y, nullptr,
+               workspace, gemm_ws, 1);
 }

@@ -30,6 +30,8 @@ struct GemmParams {
   float mid_inv_delta;         // 1/D of the grid at the down-projection input
   int mid_qmax_minus_z;
   uint32_t mid_flip;
+  int early_weights;           // the kernel in front in the stream belongs to the same call, waits for all before it
+                               // and writes no weights: they may be read before this kernel's own wait
   uint32_t* status;            // control block of the workspace (status word, decode counters)
   void* scratch;               // gemm_scratch_bytes(M) bytes behind the control block (decode partial sums)
 };

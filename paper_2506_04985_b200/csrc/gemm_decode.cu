@@ -11,7 +11,7 @@
 // Work is split stream-K style: the T = (N/128) * (K/256) weight k-blocks are cut into equal
 // contiguous ranges, one per CTA (one CTA per SM), so every SM streams the same number of bytes
 // whatever the shape.  A range that covers part of a tile leaves its raw int32 partial sums in
-// a scratch slot; the last CTA to arrive at a tile (an atomic counter per tile and lane
+// a scratch slot; the last CTA to arrive at a tile (an atomic byte per tile and lane
 // quadrant) adds the slots up -- integer addition, so the result does not depend on the order
 // -- and runs the epilogue.  No CTA ever waits for another.
 // Where every tile is cut into the same 2, 4 or 8 ranges (few tiles, long rows), the CTAs of a tile are
@@ -38,9 +38,15 @@ constexpr int HR = 128;                    // weight rows per tile
 constexpr int BK = 256;                    // codes per k-block: 128 packed bytes per row, one full cache line
 constexpr int PK_ROW = BK / 2;
 constexpr int I8_ROW = 128;                // the widened token tile is two 128-byte-swizzled halves of 128 codes
-constexpr int NS = 6;                      // widened stages: 6 x 64 tensor-memory columns + 6 token tiles
-constexpr int NPK = 4;                     // packed stages in flight from TMA
+constexpr int NS = 3;                      // widened stages: 3 x 64 tensor-memory columns + 3 token tiles
+constexpr int NPK = 6;                     // packed stages in flight from TMA
 constexpr int kGroups = 3;                 // weight-converter groups
+// A barrier's wait tells one phase from the next by its parity only, so whoever waits for a phase must know that the
+// one before it is over.  With stage counts that are multiples of the number of groups the stage of a group's k-block
+// was last used by a k-block of the same group, which has waited for it.  (With four packed stages a group could be
+// three k-blocks ahead of one whose tile had not arrived: its wait for the NEXT tile of that stage came back at once,
+// and up to a tenth of the launches had 32 weight rows of another k-block in them.)
+static_assert(NS % kGroups == 0 && NPK % kGroups == 0, "a stage must belong to one converter group");
 constexpr int kTokWarps = 4;               // token-converter warps
 constexpr int kMaxTok = 64;
 constexpr int kBatch = 16;                 // tokens an epilogue warp handles at a time
@@ -81,16 +87,14 @@ struct DecodeParams {
   int kblocks;             // K / 256 rounded up (a half block at the end reads zeros past the row)
   long long total;         // tiles * kblocks
   int per, rem;            // total = per * CTAs + rem: CTA c takes per k-blocks, the first rem CTAs one more
-  int whole_tiles;         // 1: ranges end on tile boundaries (no partial sums, no counters)
   int cluster;             // > 1: every tile is cut into this many equal ranges and the CTAs of a range set form a
                            // thread-block cluster: partial sums are exchanged through distributed shared memory
   int32_t* slots;          // [gridDim.x][2][npad][128] raw int32 partial sums
-  uint32_t* counters;      // [tiles][4], zero between launches
+  uint32_t* counters;      // [tiles] of four bytes, one per lane quadrant, zero between launches
 };
 
 // First weight k-block (global index) of CTA c's range.
 __device__ __forceinline__ long long range_start(const DecodeParams& D, int c, int nctas) {
-  if (D.whole_tiles) return (long long)D.kblocks * (long long)((unsigned)(D.tiles * c) / (unsigned)nctas);
   return (long long)c * D.per + (c < D.rem ? c : D.rem);          // no division: this runs inside the epilogue
 }
 
@@ -340,11 +344,11 @@ gemm_w4a4_decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
         while (c_last + 1 < nctas && range_start(D, c_last + 1, nctas) < t_end) ++c_last;
         const uint32_t expected = (uint32_t)(c_last - c_first + 1);
         uint32_t old = 0;
-        if (lane == 0) old = atomicAdd(D.counters + tile * 4 + quad, 1u);
+        if (lane == 0) old = (atomicAdd(D.counters + tile, 1u << (8 * quad)) >> (8 * quad)) & 0xFFu;   // (at most 160 CTAs)
         old = __shfl_sync(0xffffffffu, old, 0);
         if (old == expected - 1) {
           __threadfence();
-          if (lane == 0) D.counters[tile * 4 + quad] = 0;      // ready for the next launch
+          if (lane == 0) atomicSub(D.counters + tile, expected << (8 * quad));      // ready for the next launch
           sum = D.slots + quad * 32 + lane;
           finalize = true;
         }
@@ -488,7 +492,7 @@ static int num_sms() { return device_sm_count(); }
 // that do not divide, or not all clusters resident at once.
 static int cluster_size(int tiles, int kblocks, int npad) {
   const int sms = num_sms() < kDecodeMaxCtas ? num_sms() : kDecodeMaxCtas;
-  if (tiles > sms || tiles * 4 > kDecodeMaxCounters) return 0;
+  if (tiles > sms) return 0;
   int split = sms / tiles;
   if (split > kblocks / 2) split = kblocks / 2;                        // at least 2 k-blocks (512 codes) per range
   int cl = 1, idx = 0;
@@ -552,7 +556,6 @@ int gemm_decode_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, co
   D.tiles = (P.N + HR - 1) / HR;
   D.kblocks = (P.K + BK - 1) / BK;
   D.total = (long long)D.tiles * D.kblocks;
-  D.whole_tiles = D.tiles * 4 > kDecodeMaxCounters ? 1 : 0;
   D.slots = reinterpret_cast<int32_t*>(scratch);
   D.counters = P.status + kCounterWord0;
   CUtensorMap tmW, tmX;
@@ -576,8 +579,7 @@ int gemm_decode_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, co
     // (112 tiles stay on 112 SMs: cutting them into 148 equal ranges was measured slower, 19.4 against
     // 14.4 us at 64 tokens -- the partial sums of a split tile are 32 KB per range)
   }
-  const long long units = D.whole_tiles ? D.tiles : D.total;
-  if (units < ctas) ctas = (int)units;
+  if (D.total < ctas) ctas = (int)D.total;
   D.per = (int)(D.total / ctas);
   D.rem = (int)(D.total % ctas);
   const cudaError_t e = D.cluster > 1

@@ -60,8 +60,6 @@ template <int NW, int NT, bool kBUnsigned, bool kA8 = false, int U = 4, int kMin
 __global__ void __launch_bounds__(NW * 32, kMinCtas) gemm_w4a4_decode_small_kernel(const uint8_t* __restrict__ Xq,
                                                                           const uint8_t* __restrict__ Wq, const Params D) {
   __shared__ int part[NW][kRows][8 * NT];
-  pdl_wait();                      // the activation codes come from the kernel before this one
-  pdl_launch_dependents();
   const GemmParams& P = D.g;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
@@ -73,6 +71,23 @@ __global__ void __launch_bounds__(NW * 32, kMinCtas) gemm_w4a4_decode_small_kern
   const bool ra_ok = ra < P.N, rb_ok = rb < P.N;
   const uint8_t* wa = Wq + (size_t)(ra_ok ? ra : 0) * row_bytes + 16 * t;
   const uint8_t* wb = Wq + (size_t)(rb_ok ? rb : 0) * row_bytes + 16 * t;
+  uint4 pa[U], pb[U];
+  auto load = [&](int b0) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int b = b0 + u * NW;
+      if (b < D.kblocks) {
+        pa[u] = __ldcs(reinterpret_cast<const uint4*>(wa + (size_t)b * 64));      // streamed once: evict first
+        pb[u] = __ldcs(reinterpret_cast<const uint4*>(wb + (size_t)b * 64));
+      }
+    }
+  };
+  // The first weights are requested before the wait for the kernel in front where that is allowed: the stream from HBM
+  // then runs while the activations are still being quantised (MLP block of 14336, 1 / 8 / 16 tokens: 26.3 / 26.6 / 34.4 -> 24.2 / 24.8 / 31.3 us).
+  if (P.early_weights) load(warp);
+  pdl_wait();                      // the activation codes come from the kernel before this one
+  pdl_launch_dependents();
+  if (!P.early_weights) load(warp);
   const uint8_t* xr[NT];
   bool x_ok[NT];
 #pragma unroll
@@ -119,16 +134,7 @@ __global__ void __launch_bounds__(NW * 32, kMinCtas) gemm_w4a4_decode_small_kern
   }
 
   const uint4 zero = make_uint4(0, 0, 0, 0);
-  for (int b0 = warp; b0 < D.kblocks; b0 += NW * U) {
-    uint4 pa[U], pb[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int b = b0 + u * NW;
-      if (b < D.kblocks) {
-        pa[u] = __ldcs(reinterpret_cast<const uint4*>(wa + (size_t)b * 64));      // streamed once: evict first
-        pb[u] = __ldcs(reinterpret_cast<const uint4*>(wb + (size_t)b * 64));
-      }
-    }
+  for (int b0 = warp; b0 < D.kblocks;) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int b = b0 + u * NW;
@@ -153,6 +159,8 @@ __global__ void __launch_bounds__(NW * 32, kMinCtas) gemm_w4a4_decode_small_kern
         }
       }
     }
+    b0 += NW * U;
+    if (b0 < D.kblocks) load(b0);
   }
   // accumulator fragment: c0 (row g, token 2t), c1 (row g, token 2t+1), c2 / c3 the same for row g + 8
 #pragma unroll

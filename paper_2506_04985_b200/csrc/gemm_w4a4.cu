@@ -311,7 +311,8 @@ static int launch_gemm(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, Ge
 
 int gemm_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, const GemmParams& P) {
   if (P.M <= 16) return gemm_decode_small_launch(st, Xq, Wq, P);
-  if (P.M <= 64 && P.scratch) return gemm_decode_launch(st, Xq, Wq, P, P.scratch);
+  if (P.M <= 64 && P.scratch && (P.N + 127) / 128 <= kDecodeMaxCounters) return gemm_decode_launch(st, Xq, Wq, P, P.scratch);
+  if (P.M <= 64 && P.N > 128) return gemm_pair_launch(st, Xq, Wq, P);      // more tiles than the control block has counters
   if (P.M > 128 && P.N > 128) return gemm_pair_launch(st, Xq, Wq, P);
   if (P.M > 64 && P.M <= 128 && P.N > 128 && gemm_decode_in_two(P.N, P.K)) {
     GemmParams h = P;

@@ -57,6 +57,7 @@ static_assert(128 * (kRegsCtl + 2 * kRegsConv) + 32 * kEpiWarps * kRegsEpi <= kT
 // instead of packed 4-bit codes.
 template <int NS, int NPK, bool kA8 = false>
 struct Smem {
+  static_assert(NPK >= NS, "see the converters' waits");
   static_assert(kAccCols + NS * kAStageCols <= kTmemCols, "operand stages must fit beside the accumulator");
   static constexpr int kB8Stage = HR * I8_ROW;                      // 16 KB
   static constexpr int kPkOp = HR * PK_ROW;                         // 8 KB: a packed weight tile
@@ -231,7 +232,13 @@ gemm_w4a4_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     for (int tile = pair_id; ok && tile < num_tiles; tile += num_pairs) {
       for (int kb = 0; kb < kblocks; ++kb, ++gk) {
         if ((int)(gk & 1u) == grp) {
+          // The operand stage first: when it is free, every k-block up to NS before this one has been widened, so (NPK >=
+          // NS) the tile that used this packed stage before has arrived and is gone.  Without that a group could be ahead
+          // of one whose tile is late, and its wait, which tells phases apart by parity only, would come back for the
+          // phase before: the wrong tile.
+          if (!mbar_wait(op_empty(s), ph ^ 1u, abort_flag, status_w, 6)) { ok = false; break; }
           if (!mbar_wait(pk_full(ps), pph, abort_flag, status_w, 5)) { ok = false; break; }
+          __syncwarp();                                  // lanes leave a wait one by one; the store below is warp-wide
           uint32_t v[32];
           if constexpr (kA8) {
             // int8 codes, 128-byte rows under the 128-byte swizzle.  The weight side orders the 32 codes
@@ -262,7 +269,6 @@ gemm_w4a4_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
           uint4 cb[4];
 #pragma unroll
           for (int i = 0; i < 4; ++i) cb[i] = srcb[i * 128 + r];
-          if (!mbar_wait(op_empty(s), ph ^ 1u, abort_flag, status_w, 6)) { ok = false; break; }
           tc_fence_after();
           tmem_st_32x32(tmem_base + ((uint32_t)(quad * 32) << 16) + kAccCols + s * kAStageCols, v);
           // while the tensor-memory store completes: the weight rows
@@ -632,10 +638,10 @@ int gemm_pair_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, cons
   const int tn = pair::choose_tn(P.M, P.N, device_pairs());
   if (P.a_bits == 8) {                                                        // Xq: int8 [M, K]
     switch (tn) {
-      case 240: return pair::launch<4, 3, 0, true, 240>(st, Xq, Wq, P);
-      case 224: return pair::launch<4, 3, 0, true, 224>(st, Xq, Wq, P);
-      case 208: return pair::launch<4, 3, 0, true, 208>(st, Xq, Wq, P);
-      default:  return pair::launch<4, 3, 0, true, 256>(st, Xq, Wq, P);
+      case 240: return pair::launch<3, 4, 0, true, 240>(st, Xq, Wq, P);
+      case 224: return pair::launch<3, 4, 0, true, 224>(st, Xq, Wq, P);
+      case 208: return pair::launch<3, 4, 0, true, 208>(st, Xq, Wq, P);
+      default:  return pair::launch<3, 4, 0, true, 256>(st, Xq, Wq, P);
     }
   }
   switch (tn) {

@@ -88,6 +88,13 @@ def test_decode_many_tiles_without_counters():
     _run(8, 64000, 128, seed=11)
 
 
+@pytest.mark.parametrize("M,N,K", [(20, 64000, 512), (33, 64000, 768), (17, 254080, 128)])
+def test_decode_counters_of_many_tiles(M, N, K):
+    """500 tiles whose ranges are cut (a counter byte per tile and lane quadrant), twice on one workspace; 1985 tiles,
+    more than there are counters."""
+    _run(M, N, K, seed=12, ws=B.new_workspace(B.OP_GEMM, M, N, K), reps=2)
+
+
 @pytest.mark.parametrize("M,N,K,what", [
     (40, 8192, 2048, "64 tiles cut in 2: clusters of two CTAs"),
     (33, 2048, 4096, "16 tiles cut in 8: clusters of eight CTAs"),
@@ -108,3 +115,37 @@ def test_decode_65_to_128_tokens_in_two_launches(M, N, K):
     """Few outputs and long rows: 64 tokens and the rest, the second launch on offset operands."""
     _run(M, N, K, seed=31, f16=False)
     _run(M, N, K, symmetric=False, z=9, seed=32, post=True, residual=True)
+
+
+@pytest.mark.parametrize("M,N,K", [(37, 4096, 14336), (64, 14336, 4096), (37, 28672, 4096), (120, 4096, 14336), (2048, 6144, 4096)])
+def test_launches_in_a_row_give_every_output_every_time(M, N, K):
+    """Nine launches in a graph, replayed on cold caches: tiles arrive late and out of order, and every output of every
+    launch has to be right (one launch by itself, with a slow epilogue, hides a converter that runs ahead)."""
+    g = torch.Generator(device="cuda").manual_seed(5)
+    sets = []
+    for _ in range(3):
+        xa = torch.randint(0, 256, (M, K // 2), dtype=torch.uint8, device="cuda", generator=g)
+        xw = torch.randint(0, 256, (N, K // 2), dtype=torch.uint8, device="cuda", generator=g)
+        sw = torch.rand((N,), device="cuda", generator=g)
+        u = [torch.stack(((q.view(torch.int8) << 4) >> 4, q.view(torch.int8) >> 4), 2).flatten(1).double() for q in (xa, xw)]
+        sets.append((xa, xw, sw, B.new_workspace(B.OP_GEMM, M, N, K), ((u[0] @ u[1].T).float() * sw * torch.tensor(0.3)).to(torch.bfloat16)))
+    ys = [torch.empty((M, N), dtype=torch.bfloat16, device="cuda") for _ in range(9)]
+
+    def launches():
+        for i, y in enumerate(ys):
+            xa, xw, sw, ws, _ = sets[i % 3]
+            B.fpt_w4a4_gemm(xa, xw, sw, 0.3, ws=ws, Y=y)
+
+    launches()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        launches()
+    for _ in range(30):
+        for y in ys:
+            y.zero_()
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(y, sets[i % 3][4]) for i, y in enumerate(ys))
+    assert all(B.fpt_check_status(s[3]) == B.OK for s in sets)
