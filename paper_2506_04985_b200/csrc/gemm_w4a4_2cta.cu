@@ -13,13 +13,15 @@
 // Per k-block and CTA: TMA in 16 KB, converter loads 16 KB, int8 weight stores 16 KB, tensor-core
 // reads 16 KB = 512 transfers for 512 MMA cycles.
 //
-// Roles per CTA (20 warps):
+// Roles per CTA (24 warps):
 //   warp 0        TMA producer: packed tiles (128 rows x 64 bytes of each operand per k-block)
 //   warp 1        tensor-memory owner; in the leader CTA (rank 0) also the MMA issuer
-//   warps 4..11   converters, two groups of four warps that take the k-blocks in turns: a group widens
-//                 the CTA's activation rows (shared -> registers -> tcgen05.st, one row per thread) and,
-//                 while that store completes, its weight rows (-> 128-byte-swizzled K-major int8 tile)
-//   warps 12..19  epilogue: tcgen05.ld, >> 8, scales, bf16 into a swizzled shared-memory tile; the
+//   warps 4..15   converters, three groups of four warps that take the k-blocks in turns: a group widens the CTA's
+//                 activation rows (shared -> registers -> tcgen05.st, one row per thread) and, while those stores
+//                 complete, its weight rows (-> 128-byte-swizzled K-major int8 tile).  The chain of latencies of a
+//                 k-block is what sets the pace (twenty more instructions in it cost 5 %): with two groups
+//                 2048x6144x4096 took 44.6, 4096x28672x4096 363, 8192x57344x8192 2616 us, with three 40.7 / 326 / 2314
+//   warps 16..23  epilogue: tcgen05.ld, >> 8, scales, bf16 into a swizzled shared-memory tile; the
 //                 accumulator is released as soon as it has been read, the tile leaves by TMA store;
 //                 a residual tile is fetched by TMA into the same slabs while the tile's matmul runs
 // Both operands are widened as code*16 (see gemm_w4a4.cu), so the accumulator holds 256 * sum.
@@ -41,14 +43,15 @@ constexpr int I8_ROW = BK;                 // int8 bytes per row and k-block
 constexpr int kAccCols = 256;              // tensor-memory columns of the accumulator
 constexpr int kAStageCols = BK / 4;        // 32 columns hold 128 int8 per lane
 constexpr int kTmemCols = 512;
-constexpr int kThreads = 640;
-constexpr int kConvWarp0 = 4, kEpiWarp0 = 12, kEpiWarps = 8;
+constexpr int kGroups = 3;                 // converter groups of four warps
+constexpr int kConvWarp0 = 4, kEpiWarp0 = kConvWarp0 + 4 * kGroups, kEpiWarps = 8;
+constexpr int kThreads = 32 * (kEpiWarp0 + kEpiWarps);
 // Registers per thread: what the CTA is launched with, and what the roles trade it into (warps 0-3,
 // the two converter groups, epilogue).  A CTA can only redistribute what it owns: an
 // increase that the decreases do not cover would never return, so the sum is checked here.
-constexpr int kRegsLaunch = 96, kRegsCtl = 48, kRegsConv = 64, kRegsEpi = 152;
+constexpr int kRegsLaunch = 80, kRegsCtl = 32, kRegsConv = 48, kRegsEpi = 152;
 static_assert(kThreads * kRegsLaunch <= 65536, "launch allocation exceeds the register file");
-static_assert(128 * (kRegsCtl + 2 * kRegsConv) + 32 * kEpiWarps * kRegsEpi <= kThreads * kRegsLaunch,
+static_assert(128 * (kRegsCtl + kGroups * kRegsConv) + 32 * kEpiWarps * kRegsEpi <= kThreads * kRegsLaunch,
               "the warpgroups ask for more registers than the CTA was launched with: setmaxnreg.inc would never return");
 
 // NS: stages of widened operands (int8 weight tile in shared memory + activation columns in
@@ -57,7 +60,10 @@ static_assert(128 * (kRegsCtl + 2 * kRegsConv) + 32 * kEpiWarps * kRegsEpi <= kT
 // instead of packed 4-bit codes.
 template <int NS, int NPK, bool kA8 = false>
 struct Smem {
-  static_assert(NPK >= NS, "see the converters' waits");
+  // A barrier's wait tells one phase from the next by its parity only, so whoever waits for a phase must know that the
+  // one before it is over: the stage of a group's k-block was last used by a k-block of the same group.  (With five
+  // packed stages a group that was ahead of a late tile got the wrong one.)
+  static_assert(NS % kGroups == 0 && NPK % kGroups == 0, "a stage must belong to one converter group");
   static_assert(kAccCols + NS * kAStageCols <= kTmemCols, "operand stages must fit beside the accumulator");
   static constexpr int kB8Stage = HR * I8_ROW;                      // 16 KB
   static constexpr int kPkOp = HR * PK_ROW;                         // 8 KB: a packed weight tile
@@ -152,8 +158,8 @@ gemm_w4a4_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
 
   // Registers: the epilogue wants the 128 accumulators of its row in registers at once, the other
   // roles need few; the warpgroups trade.  A CTA can only redistribute what it was launched with
-  // (640 x 96 registers): 128 x (48 + 64 + 64) + 256 x 152 = 61440 <= 61440, so the request of the
-  // epilogue groups is always met once the three other groups have given theirs back.  Each role
+  // (768 x 80 registers): 128 x (32 + 3 x 48) + 256 x 152 = 61440 <= 61440, so the request of the
+  // epilogue groups is always met once the other groups have given theirs back.  Each role
   // branch starts with its own re-allocation (the compiler budgets registers per branch).
   if (warp < kConvWarp0) {
     reg_dec<kRegsCtl>();
@@ -214,12 +220,11 @@ gemm_w4a4_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     }
   } else if (warp < kEpiWarp0) {
     // ------------------------------------------------------------------ converters
-    // Two groups of four warps (4..7 and 8..11) take the k-blocks in turns, and a group widens a whole
-    // k-block: the CTA's 128 activation rows into tensor memory (one row per thread; warp % 4 selects
-    // the tensor-memory lanes the warp may touch) and the CTA's weight rows into the int8 tile in shared
-    // memory.  For one warp a k-block is a chain of long latencies (shared loads, the tensor-memory store
-    // and its wait, the proxy fence) that does not shrink with the tile; alternating groups give every
-    // chain two k-block periods.
+    // The groups take the k-blocks in turns, and a group widens a whole k-block: the CTA's 128 activation rows into
+    // tensor memory (one row per thread; warp % 4 selects the tensor-memory lanes the warp may touch) and the CTA's
+    // weight rows into the int8 tile in shared memory.  For one warp a k-block is a chain of long latencies (shared
+    // loads, the tensor-memory stores and their wait, the proxy fence) that does not shrink with the tile; alternating
+    // groups give every chain three k-block periods.
     reg_dec<kRegsConv>();
     const int grp = (warp - kConvWarp0) >> 2;
     const int quad = warp & 3;                           // the TMEM lanes this warp may touch
@@ -227,73 +232,78 @@ gemm_w4a4_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     const uint32_t swz = (uint32_t)((r >> 1) & 3);       // SWIZZLE_64B: 16-byte chunk index ^= (row / 2) % 4
     const uint32_t op_full_leader = map_to_cta(op_full(0), 0);
     int ps = 0, s = 0; uint32_t pph = 0, ph = 0;
-    uint32_t gk = 0;                                     // k-blocks since the start of the kernel
+    int turn = 0;                                        // the group whose k-block this is
     bool ok = true;
     for (int tile = pair_id; ok && tile < num_tiles; tile += num_pairs) {
-      for (int kb = 0; kb < kblocks; ++kb, ++gk) {
-        if ((int)(gk & 1u) == grp) {
-          // The operand stage first: when it is free, every k-block up to NS before this one has been widened, so (NPK >=
-          // NS) the tile that used this packed stage before has arrived and is gone.  Without that a group could be ahead
-          // of one whose tile is late, and its wait, which tells phases apart by parity only, would come back for the
-          // phase before: the wrong tile.
-          if (!mbar_wait(op_empty(s), ph ^ 1u, abort_flag, status_w, 6)) { ok = false; break; }
+      for (int kb = 0; kb < kblocks; ++kb) {
+        if (turn == grp) {
           if (!mbar_wait(pk_full(ps), pph, abort_flag, status_w, 5)) { ok = false; break; }
-          __syncwarp();                                  // lanes leave a wait one by one; the store below is warp-wide
-          uint32_t v[32];
-          if constexpr (kA8) {
-            // int8 codes, 128-byte rows under the 128-byte swizzle.  The weight side orders the 32 codes
-            // of a group as 16 even-k then 16 odd-k bytes (that is how the nibbles fall apart); the
-            // activation bytes are put into the same order.
-            const uint8_t* src = smem + L::kPkAOff + ps * L::kPkOpA + r * I8_ROW;
-#pragma unroll
-            for (int g = 0; g < 4; ++g) {
-              const uint4 c0 = *reinterpret_cast<const uint4*>(src + (((uint32_t)(2 * g) ^ (uint32_t)(r & 7)) << 4));
-              const uint4 c1 = *reinterpret_cast<const uint4*>(src + (((uint32_t)(2 * g + 1) ^ (uint32_t)(r & 7)) << 4));
-              const uint32_t a[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
-#pragma unroll
-              for (int w = 0; w < 4; ++w) {
-                v[8 * g + w] = __byte_perm(a[2 * w], a[2 * w + 1], 0x6420);
-                v[8 * g + 4 + w] = __byte_perm(a[2 * w], a[2 * w + 1], 0x7531);
-              }
-            }
-          } else {
-            const uint8_t* src = smem + L::kPkAOff + ps * L::kPkOpA + r * PK_ROW;
-            uint4 c[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) c[j] = *reinterpret_cast<const uint4*>(src + (((uint32_t)j ^ swz) << 4));
-#pragma unroll
-            for (int j = 0; j < 4; ++j) widen(c[j], v + 8 * j);
-          }
+          const uint8_t* src = smem + L::kPkAOff + ps * L::kPkOpA + r * (kA8 ? I8_ROW : PK_ROW);
           // the packed weight tile: 16-byte chunk i * 128 + r is row (i * 128 + r) / 4, chunk r % 4
           const uint4* srcb = reinterpret_cast<const uint4*>(smem + L::kPkBOff + ps * L::kPkOp);
-          uint4 cb[4];
+          const uint32_t a_tmem = tmem_base + ((uint32_t)(quad * 32) << 16) + kAccCols + s * kAStageCols;
+          // the activation row's 128 codes in two halves of 64 (16 tensor-memory columns each): fewer live registers
 #pragma unroll
-          for (int i = 0; i < 4; ++i) cb[i] = srcb[i * 128 + r];
-          tc_fence_after();
-          tmem_st_32x32(tmem_base + ((uint32_t)(quad * 32) << 16) + kAccCols + s * kAStageCols, v);
-          // while the tensor-memory store completes: the weight rows
+          for (int h = 0; h < 2; ++h) {
+            uint32_t v[16];
+            if constexpr (kA8) {
+              // int8 codes, 128-byte rows under the 128-byte swizzle.  The weight side orders the 32 codes
+              // of a group as 16 even-k then 16 odd-k bytes (that is how the nibbles fall apart); the
+              // activation bytes are put into the same order.
+#pragma unroll
+              for (int g = 0; g < 2; ++g) {
+                const uint4 c0 = *reinterpret_cast<const uint4*>(src + (((uint32_t)(4 * h + 2 * g) ^ (uint32_t)(r & 7)) << 4));
+                const uint4 c1 = *reinterpret_cast<const uint4*>(src + (((uint32_t)(4 * h + 2 * g + 1) ^ (uint32_t)(r & 7)) << 4));
+                const uint32_t a[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+#pragma unroll
+                for (int w = 0; w < 4; ++w) {
+                  v[8 * g + w] = __byte_perm(a[2 * w], a[2 * w + 1], 0x6420);
+                  v[8 * g + 4 + w] = __byte_perm(a[2 * w], a[2 * w + 1], 0x7531);
+                }
+              }
+            } else {
+              uint4 c[2];
+#pragma unroll
+              for (int j = 0; j < 2; ++j) c[j] = *reinterpret_cast<const uint4*>(src + (((uint32_t)(2 * h + j) ^ swz) << 4));
+#pragma unroll
+              for (int j = 0; j < 2; ++j) widen(c[j], v + 8 * j);
+            }
+            if (h == 0) {
+              if (!mbar_wait(op_empty(s), ph ^ 1u, abort_flag, status_w, 6)) { ok = false; break; }
+              __syncwarp();                              // lanes leave a wait one by one; the stores are warp-wide
+              tc_fence_after();
+            }
+            tmem_st_32x16(a_tmem + 16 * h, v);
+          }
+          if (!ok) break;
+          // while the tensor-memory stores complete: the weight rows
           uint8_t* dst = smem + L::kB8Off + s * L::kB8Stage;
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int br = (i * 128 + r) >> 2, ch = r & 3;
-            if (i == 3 && br >= hb) continue;            // a narrower tile has fewer weight rows
-            uint32_t w[8];
-            widen(cb[i], w);
-            uint8_t* rowp = dst + br * I8_ROW;
-            *reinterpret_cast<uint4*>(rowp + (((2 * ch) ^ (br & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
-            *reinterpret_cast<uint4*>(rowp + (((2 * ch + 1) ^ (br & 7)) << 4)) = make_uint4(w[4], w[5], w[6], w[7]);
+          for (int i0 = 0; i0 < 4; i0 += 2) {
+            uint4 cb[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) cb[i] = srcb[(i0 + i) * 128 + r];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              const int br = ((i0 + i) * 128 + r) >> 2, ch = r & 3;
+              if (i0 + i == 3 && br >= hb) continue;     // a narrower tile has fewer weight rows
+              uint32_t w[8];
+              widen(cb[i], w);
+              uint8_t* rowp = dst + br * I8_ROW;
+              *reinterpret_cast<uint4*>(rowp + (((2 * ch) ^ (br & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+              *reinterpret_cast<uint4*>(rowp + (((2 * ch + 1) ^ (br & 7)) << 4)) = make_uint4(w[4], w[5], w[6], w[7]);
+            }
           }
           tmem_wait_st();
           tc_fence_before();
           // One fence for both hand-overs: the widened tile becomes visible to the tensor core's async
           // proxy, and the reads of the packed tiles (consumed by the stores above) are ordered before
-          // the TMA writes that re-fill them.  The packed tiles go back to TMA only here: handing them
-          // back right after the loads, with nothing depending on them yet, let the next TMA write
-          // overtake reads still in flight (seen as wrong weight rows, rarely, under load).
+          // the TMA writes that re-fill them.
           fence_proxy_async_smem();
           __syncwarp();
           if (lane == 0) { mbar_arrive(pk_empty(ps)); mbar_arrive_cluster(op_full_leader + 8u * s); }
         }
+        if (++turn == kGroups) turn = 0;
         if (++ps == NPK) { ps = 0; pph ^= 1u; }
         if (++s == NS) { s = 0; ph ^= 1u; }
       }
@@ -361,8 +371,8 @@ gemm_w4a4_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
       const int* zws = zw_s + b * TN + half * 128;
       // all 128 accumulators of this thread's row -> registers, then the accumulator is free again
       uint32_t v[128];
-      tmem_ld_32x64(taddr, v);                           // each load and its wait in one statement
-      tmem_ld_32x64(taddr + 64, v + 64);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) tmem_ld_32x32(taddr + 32 * q, *reinterpret_cast<uint32_t(*)[32]>(v + 32 * q));
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(acc_empty_leader);
@@ -633,22 +643,22 @@ static int launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, GemmPar
 static int device_pairs() { const int sms = device_sm_count(); return sms >= 2 ? sms / 2 : 1; }
 
 int gemm_pair_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, const GemmParams& P) {
-  if (P.Mq) return pair::launch<4, 5, 1>(st, Xq, Wq, P);
-  if (P.swiglu_bf16) return pair::launch<4, 5, 2>(st, Xq, Wq, P);
+  if (P.Mq) return pair::launch<3, 6, 1>(st, Xq, Wq, P);
+  if (P.swiglu_bf16) return pair::launch<3, 6, 2>(st, Xq, Wq, P);
   const int tn = pair::choose_tn(P.M, P.N, device_pairs());
   if (P.a_bits == 8) {                                                        // Xq: int8 [M, K]
     switch (tn) {
-      case 240: return pair::launch<3, 4, 0, true, 240>(st, Xq, Wq, P);
-      case 224: return pair::launch<3, 4, 0, true, 224>(st, Xq, Wq, P);
-      case 208: return pair::launch<3, 4, 0, true, 208>(st, Xq, Wq, P);
-      default:  return pair::launch<3, 4, 0, true, 256>(st, Xq, Wq, P);
+      case 240: return pair::launch<3, 3, 0, true, 240>(st, Xq, Wq, P);
+      case 224: return pair::launch<3, 3, 0, true, 224>(st, Xq, Wq, P);
+      case 208: return pair::launch<3, 3, 0, true, 208>(st, Xq, Wq, P);
+      default:  return pair::launch<3, 3, 0, true, 256>(st, Xq, Wq, P);
     }
   }
   switch (tn) {
-    case 240: return pair::launch<4, 5, 0, false, 240>(st, Xq, Wq, P);
-    case 224: return pair::launch<4, 5, 0, false, 224>(st, Xq, Wq, P);
-    case 208: return pair::launch<4, 5, 0, false, 208>(st, Xq, Wq, P);
-    default:  return pair::launch<4, 5, 0, false, 256>(st, Xq, Wq, P);
+    case 240: return pair::launch<3, 6, 0, false, 240>(st, Xq, Wq, P);
+    case 224: return pair::launch<3, 6, 0, false, 224>(st, Xq, Wq, P);
+    case 208: return pair::launch<3, 6, 0, false, 208>(st, Xq, Wq, P);
+    default:  return pair::launch<3, 6, 0, false, 256>(st, Xq, Wq, P);
   }
 }
 
