@@ -84,7 +84,8 @@ struct Smem {
 
 // kFuse: 0 plain scale-factor epilogue; 1 SwiGLU product + quantiser (codes out); 2 SwiGLU product
 // (bf16 out).  Separate instantiations keep the plain epilogue's register budget free of the others.
-template <int NS, int NPK, int kFuse, bool kA8 = false, int kTN = TN>
+// kWide: accumulators may leave the range of the exponent trick (see `magic_ok`).
+template <int NS, int NPK, int kFuse, bool kA8 = false, int kTN = TN, bool kWide = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 gemm_w4a4_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                       const __grid_constant__ CUtensorMap tmY, const __grid_constant__ CUtensorMap tmYt,
@@ -319,9 +320,10 @@ gemm_w4a4_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     int* zw_s = reinterpret_cast<int*>(smem + L::kScaleOff + 2 * TN * 4);
     const int r = quad * 32 + lane;                      // row of the CTA's 128
     constexpr int kShift = kA8 ? 4 : 8;                  // both operands carry a factor 16, int8 activations none
-    // |acc| < 2^22: int -> float by the exponent trick.  With 4-bit activation codes that holds for every K
-    // the entry points accept (64 * 65408 < 2^22), so the conversion instruction is never even emitted.
-    const bool magic_ok = kA8 ? P.K < 4096 : true;
+    // |acc| < 2^22: int -> float by the exponent trick.  With symmetric 4-bit activation codes that holds for every
+    // K the entry points accept (64 * 65408 < 2^22); on an asymmetric grid |code - z| reaches 15 and 120 K passes 2^22
+    // from K = 34953 on, where the host launches the kWide form.  The others never emit the conversion instruction.
+    const bool magic_ok = kA8 ? P.K < 4096 : !kWide;
     const bool issuer = quad == 0 && lane == 0;          // issues the TMA stores (and residual loads) of its half
     const bool use_res = kFuse == 0 && residual_p != nullptr && y_out_p != nullptr;
     const bool has_z = P.wsum != nullptr;                // asymmetric activation grid: row-sum correction
@@ -590,10 +592,10 @@ static bool make_codes_map(CUtensorMap* m, const void* base, int M, int row_byte
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int NS, int NPK, int kFuse, bool kA8 = false, int kTN = TN>
+template <int NS, int NPK, int kFuse, bool kA8 = false, int kTN = TN, bool kWide = false>
 static int launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, GemmParams P) {
   using L = Smem<NS, NPK, kA8>;
-  auto kern = gemm_w4a4_pair_kernel<NS, NPK, kFuse, kA8, kTN>;
+  auto kern = gemm_w4a4_pair_kernel<NS, NPK, kFuse, kA8, kTN, kWide>;
   static PerDeviceInt pairs_cache;          // co-resident CTA pairs on the current device
   const int max_pairs = pairs_cache.get([&] {
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kAlloc) != cudaSuccess) return 0;
@@ -652,6 +654,14 @@ int gemm_pair_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, cons
       case 224: return pair::launch<3, 3, 0, true, 224>(st, Xq, Wq, P);
       case 208: return pair::launch<3, 3, 0, true, 208>(st, Xq, Wq, P);
       default:  return pair::launch<3, 3, 0, true, 256>(st, Xq, Wq, P);
+    }
+  }
+  if (P.a_unsigned && 15ll * 8 * P.K >= (1 << 22)) {
+    switch (tn) {
+      case 240: return pair::launch<3, 6, 0, false, 240, true>(st, Xq, Wq, P);
+      case 224: return pair::launch<3, 6, 0, false, 224, true>(st, Xq, Wq, P);
+      case 208: return pair::launch<3, 6, 0, false, 208, true>(st, Xq, Wq, P);
+      default:  return pair::launch<3, 6, 0, false, 256, true>(st, Xq, Wq, P);
     }
   }
   switch (tn) {

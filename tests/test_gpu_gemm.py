@@ -81,6 +81,24 @@ def test_gemm_extreme_codes_reach_the_accumulator_bound():
     assert np.all(acc[:, 0::2] == 64 * K) and np.all(acc[:, 1::2] == -56 * K)
 
 
+@pytest.mark.parametrize("M,N", [(130, 264), (66, 264), (130, 74 * 224), (130, 74 * 240), (130, 74 * 256)])
+@pytest.mark.parametrize("K", [34944, 35072, 65408])
+def test_gemm_asymmetric_outputs_at_the_accumulator_bound(M, N, K):
+    """Code - z = +-15 against weights of -8 and 7: from K = 34953 on |acc| passes 2^22, where the conversion of the
+    accumulators to float needs another form (every tile width of the CTA-pair kernel)."""
+    xw = torch.full((N, K // 2), 0x88, dtype=torch.uint8, device="cuda")
+    xw[1::2] = 0x77
+    qw = np.where(np.arange(N) % 2, 7, -8).astype(np.int64)
+    sw = (2.0 ** -20 * (1.0 + (np.arange(N) % 61) / 64.0)).astype(np.float32)
+    for z, code in ((0, 15), (15, 0)):
+        xa = torch.full((M, K // 2), code * 17, dtype=torch.uint8, device="cuda")
+        Y, acc = B.fpt_w4a4_gemm(xa, xw, dev(sw), 1.0, wsum=dev((qw * K).astype(np.int32)), act_symmetric=False,
+                                 act_zero_point=z, want_acc=True)
+        ref = np.broadcast_to((code - z) * qw * K, (M, N)).astype(np.int32)
+        assert np.array_equal(host(acc), ref)
+        assert assert_bf16_close(bf16_host(Y), dequant_epilogue(ref, sw, np.float32(1.0)), "Y") == 0
+
+
 def test_gemm_persistent_many_tiles_and_status_word():
     M, N, K = 1500, 2304, 512           # 12 x 9 tiles of 128 x 256: several per CTA is not reached on 148 SMs...
     _run(M, N, K, seed=5)
