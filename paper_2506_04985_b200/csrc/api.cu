@@ -28,6 +28,13 @@ static int check_gemm_shape(int M, int N, int K) {
   return FPT_OK;
 }
 
+// What the matmul refuses about a weight's scales (and row sums): for the composed entry points to say so before they
+// enqueue the quantiser in front of it.
+static int check_scales(const void* sw, int scale_dtype, const int32_t* wsum) {
+  if (scale_dtype != FPT_DTYPE_F32 && scale_dtype != FPT_DTYPE_F16) return FPT_ERR_BAD_ARG;
+  return (((uintptr_t)sw | (uintptr_t)wsum) & 15) ? FPT_ERR_ALIGNMENT : FPT_OK;
+}
+
 static int g_programmatic_launch = 1;
 int programmatic_launch_enabled() { return g_programmatic_launch; }
 
@@ -195,6 +202,9 @@ extern "C" int fpt_w4a4_linear(void* stream, const void* X, int M, int K, const 
   if (a8) {
     if (((uintptr_t)X | (uintptr_t)Wq | (uintptr_t)Y | (uintptr_t)workspace) & 15) return FPT_ERR_ALIGNMENT;
     if (!workspace || workspace_bytes < fpt_workspace_bytes(FPT_OP_LINEAR_A8, M, N, K)) return FPT_ERR_WORKSPACE;
+    if (K > kMaxKA8) return FPT_ERR_UNSUPPORTED;
+    rc = check_scales(sw, scale_dtype, nullptr);
+    if (rc) return rc;
     const size_t gemm_ws8 = fpt_workspace_bytes(FPT_OP_GEMM_A8, M, N, K);
     int8_t* Xq8 = reinterpret_cast<int8_t*>(workspace) + gemm_ws8;
     float* pinv = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(Xq8) + up256((size_t)M * K));
@@ -234,6 +244,10 @@ extern "C" int fpt_decoder_mlp(void* stream, const void* X, int M, int d, int d_
   if (!workspace ||
       workspace_bytes < fpt_workspace_bytes(mid_hadamard ? FPT_OP_MLP_HADAMARD : FPT_OP_MLP, M, d_ff, d))
     return FPT_ERR_WORKSPACE;
+  // (with more than 128 tokens sw_gu is read one value at a time and may lie anywhere)
+  rc = check_scales(M <= 128 ? sw_gu : nullptr, scale_dtype, nullptr);
+  if (!rc) rc = check_scales(sw_d, scale_dtype, nullptr);
+  if (rc) return rc;
   const size_t m = (size_t)M;
   uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
   const size_t gemm_ws = kStatusBytes + gemm_scratch_bytes(M);      // control block + matmul scratch
@@ -303,6 +317,8 @@ extern "C" int fpt_decoder_attn_qkv(void* stream, const void* X, int M, int d, c
   if (!qp_in->symmetric && !wsum_qkv) return FPT_ERR_BAD_ARG;
   if (((uintptr_t)X | (uintptr_t)Wqkv_q | (uintptr_t)QKV | (uintptr_t)workspace) & 15) return FPT_ERR_ALIGNMENT;
   if (!workspace || workspace_bytes < fpt_workspace_bytes(FPT_OP_LINEAR, M, n_qkv, d)) return FPT_ERR_WORKSPACE;
+  rc = check_scales(sw_qkv, scale_dtype, wsum_qkv);
+  if (rc) return rc;
   const size_t gemm_ws = kStatusBytes + gemm_scratch_bytes(M);
   uint8_t* Xq = reinterpret_cast<uint8_t*>(workspace) + gemm_ws;
   // X~ = RMSNorm(X) on the grid qp_in; S_n = S_{n-1} * r; r kept for the residual
@@ -326,6 +342,8 @@ extern "C" int fpt_decoder_attn_out(void* stream, const void* A, int M, int k_o,
   if (!qp_ap->symmetric && !wsum_o) return FPT_ERR_BAD_ARG;
   if (((uintptr_t)A | (uintptr_t)Wo_q | (uintptr_t)Y | (uintptr_t)X | (uintptr_t)workspace) & 15) return FPT_ERR_ALIGNMENT;
   if (!workspace || workspace_bytes < fpt_workspace_bytes(FPT_OP_LINEAR, M, d, k_o)) return FPT_ERR_WORKSPACE;
+  rc = check_scales(sw_o, scale_dtype, wsum_o);
+  if (rc) return rc;
   const size_t gemm_ws = kStatusBytes + gemm_scratch_bytes(M);
   uint8_t* Aq = reinterpret_cast<uint8_t*>(workspace) + gemm_ws;
   // the sequence scaler at the attention output: the grid sees A * S_n
@@ -352,6 +370,9 @@ extern "C" int fpt_w4a4_linear_dynamic(void* stream, const void* X, int M, int K
   if (((uintptr_t)X | (uintptr_t)Wq | (uintptr_t)Y | (uintptr_t)workspace) & 15) return FPT_ERR_ALIGNMENT;
   if (bits == 8) {
     if (!workspace || workspace_bytes < fpt_workspace_bytes(FPT_OP_LINEAR_A8, M, N, K)) return FPT_ERR_WORKSPACE;
+    if (K > kMaxKA8) return FPT_ERR_UNSUPPORTED;
+    rc = check_scales(sw, scale_dtype, nullptr);
+    if (rc) return rc;
     const size_t gemm_ws8 = fpt_workspace_bytes(FPT_OP_GEMM_A8, M, N, K);
     int8_t* Xq8 = reinterpret_cast<int8_t*>(workspace) + gemm_ws8;
     float* c8 = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(Xq8) + up256((size_t)M * K));
@@ -362,6 +383,8 @@ extern "C" int fpt_w4a4_linear_dynamic(void* stream, const void* X, int M, int K
                          gemm_ws8);
   }
   if (!workspace || workspace_bytes < fpt_workspace_bytes(FPT_OP_LINEAR, M, N, K)) return FPT_ERR_WORKSPACE;
+  rc = check_scales(sw, scale_dtype, nullptr);
+  if (rc) return rc;
   uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
   const size_t gemm_ws = kStatusBytes + gemm_scratch_bytes(M);
   uint8_t* Xq = ws + gemm_ws;

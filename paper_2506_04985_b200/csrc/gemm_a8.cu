@@ -93,7 +93,7 @@ extern "C" int fpt_w4a8_gemm(void* stream, const int8_t* Xq8, const uint8_t* Wq,
   if (!Xq8 || !Wq || !sw || (!Y && !acc_out)) return FPT_ERR_BAD_ARG;
   if (M <= 0 || N <= 0 || K <= 0) return FPT_ERR_BAD_ARG;
   if (K % 128 != 0 || N % 8 != 0) return FPT_ERR_UNSUPPORTED;
-  if (K > 16384) return FPT_ERR_UNSUPPORTED;               // keeps (float)acc exact: |acc| <= 1024 K < 2^24
+  if (K > kMaxKA8) return FPT_ERR_UNSUPPORTED;
   if (scale_dtype != FPT_DTYPE_F32 && scale_dtype != FPT_DTYPE_F16) return FPT_ERR_BAD_ARG;
   if (!(act_scale > 0.0f)) return FPT_ERR_BAD_ARG;
   if (((uintptr_t)Xq8 | (uintptr_t)Wq | (uintptr_t)Y | (uintptr_t)acc_out | (uintptr_t)residual | (uintptr_t)workspace |

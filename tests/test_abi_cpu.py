@@ -108,6 +108,40 @@ def test_argument_errors_are_reported_before_any_launch(B):
     assert L.fpt_check_status(None, None) == B.ERR_BAD_ARG
 
 
+def test_composed_calls_refuse_before_the_first_kernel(B):
+    """What the matmul inside would refuse is refused up front: without a device the quantiser in front of it would
+    otherwise be what fails, with another code (and with one it would already have written s_out)."""
+    L, p = B.lib(), ctypes.c_void_p
+    fake, odd, big = p(0x1000), p(0x1004), 1 << 40
+    q4, q8 = ctypes.byref(B.QParams(4, True, 0.5, 0)), ctypes.byref(B.QParams(8, True, 0.5, 0))
+    f32, bad = B.DTYPE_F32, 7
+
+    def mlp(M, sw_gu, sw_d, had=0):
+        return L.fpt_decoder_mlp(None, fake, M, 128, 256, fake, sw_gu, fake, sw_d, f32, q4, q4, 1e-5, None, None, 0, had,
+                                 fake, fake, big)
+
+    for M in (1, 16, 17, 64, 128, 129, 4096):
+        for had in (0, 1):
+            assert mlp(M, fake, odd, had) == B.ERR_ALIGNMENT
+            if M <= 128:
+                assert mlp(M, odd, fake, had) == B.ERR_ALIGNMENT
+        for wsum, sw, dt, want in ((None, odd, f32, B.ERR_ALIGNMENT), (odd, fake, f32, B.ERR_ALIGNMENT),
+                                   (None, fake, bad, B.ERR_BAD_ARG)):
+            assert L.fpt_decoder_attn_qkv(None, fake, M, 128, fake, sw, dt, wsum, 256, q4, 1e-5, None, fake, fake, fake,
+                                          fake, big) == want
+            assert L.fpt_decoder_attn_out(None, fake, M, 128, fake, sw, dt, wsum, 256, q4, fake, None, None, fake, fake,
+                                          big) == want
+        for sw, dt, K, want in ((odd, f32, 128, B.ERR_ALIGNMENT), (fake, bad, 128, B.ERR_BAD_ARG),
+                                (fake, f32, 16512, B.ERR_UNSUPPORTED)):
+            for bits in (4, 8):
+                if bits == 4 and K > 128:
+                    continue
+                assert L.fpt_w4a4_linear_dynamic(None, fake, M, K, fake, sw, dt, 256, bits, B.RMSNORM, 1e-5, None,
+                                                 B.POST_NONE, None, fake, None, fake, big) == want
+                assert L.fpt_w4a4_linear(None, fake, M, K, fake, sw, dt, None, 256, q4 if bits == 4 else q8, B.RMSNORM, 1e-5,
+                                         None, B.POST_NONE, None, fake, None, fake, big) == want
+
+
 def test_oracle_and_library_share_no_code():
     """The checker must not import the product and the product must not import the checker."""
     for dirpath, _, files in os.walk(os.path.join(ROOT, "oracle")):
