@@ -101,13 +101,20 @@ def lib():
 
 # What every call goes through.  A small linear spends more time here than on the GPU, so addresses and the stream are
 # passed as plain integers (the argument types turn them into pointers) and the stream handle comes without a
-# torch.cuda.Stream object around it: 128 tokens x 1024 -> 1024 in 19.2 -> 14.9 us a call.
+# torch.cuda.Stream object around it: 128 tokens x 1024 -> 1024 in 19.2 -> 14.9 us a call.  The two functions for that
+# are internal to torch: where one is missing, the public call serves.
 def _ptr(t):
     return None if t is None else t.data_ptr()
 
 
-def _stream():
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+_raw_stream, _device = (getattr(torch._C, name, None) for name in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+
+if _raw_stream is not None and _device is not None:
+    def _stream():
+        return _raw_stream(_device())
+else:
+    def _stream():
+        return torch.cuda.current_stream().cuda_stream
 
 
 def _check(code, where):

@@ -142,6 +142,20 @@ def test_composed_calls_refuse_before_the_first_kernel(B):
                                          None, B.POST_NONE, None, fake, None, fake, big) == want
 
 
+@pytest.mark.parametrize("gone", ["_cuda_getCurrentRawStream", "_cuda_getDevice"])
+def test_stream_handle_without_the_internals_of_torch(B, monkeypatch, gone):
+    import importlib.util
+    import types
+
+    import torch
+    monkeypatch.delattr(torch._C, gone, raising=False)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=0x1230))
+    spec = importlib.util.spec_from_file_location("binding_without", B.__file__)
+    mod = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(mod)
+    assert mod._stream() == 0x1230
+
+
 def test_oracle_and_library_share_no_code():
     """The checker must not import the product and the product must not import the checker."""
     for dirpath, _, files in os.walk(os.path.join(ROOT, "oracle")):
