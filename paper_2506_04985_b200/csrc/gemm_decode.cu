@@ -86,7 +86,7 @@ struct DecodeParams {
   int tiles;               // N / 128 rounded up
   int kblocks;             // K / 256 rounded up (a half block at the end reads zeros past the row)
   long long total;         // tiles * kblocks
-  int per, rem;            // total = per * CTAs + rem: CTA c takes per k-blocks, the first rem CTAs one more
+  int per, rem;            // CTA c takes per k-blocks, the first rem CTAs one more, the last what is left of `total`
   int cluster;             // > 1: every tile is cut into this many equal ranges and the CTAs of a range set form a
                            // thread-block cluster: partial sums are exchanged through distributed shared memory
   int32_t* slots;          // [gridDim.x][2][npad][128] raw int32 partial sums
@@ -125,7 +125,8 @@ gemm_w4a4_decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
   const int lane = threadIdx.x & 31;
   const int nctas = gridDim.x;
   const long long g_begin = range_start(D, blockIdx.x, nctas);
-  const long long g_end = range_start(D, blockIdx.x + 1, nctas);
+  long long g_end = range_start(D, blockIdx.x + 1, nctas);
+  if (g_end > D.total) g_end = D.total;              // (ranges of whole tiles: the last one may be shorter)
   const uint32_t pkx_bytes = (uint32_t)D.npad * PK_ROW;
 
   if (threadIdx.x == 0) {
@@ -582,6 +583,14 @@ int gemm_decode_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, co
   if (D.total < ctas) ctas = (int)D.total;
   D.per = (int)(D.total / ctas);
   D.rem = (int)(D.total % ctas);
+  if (D.tiles > kDecodeMaxCounters) {
+    // more tiles than the control block has counters: ranges of whole tiles, which leave no partial sums
+    // (17 / 37 / 64 tokens x 254080x1024: 33 / 40 / 45 us, in the CTA-pair kernel 72)
+    const int per = (D.tiles + sms - 1) / sms;
+    ctas = (D.tiles + per - 1) / per;
+    D.per = per * D.kblocks;
+    D.rem = 0;
+  }
   const cudaError_t e = D.cluster > 1
       ? launch_kernel_cluster(gemm_w4a4_decode_kernel, dim3(ctas), dim3(kThreads), Smem::kAlloc, st, true, D.cluster, tmW, tmX, D)
       : launch_kernel(gemm_w4a4_decode_kernel, dim3(ctas), dim3(kThreads), Smem::kAlloc, st, true, tmW, tmX, D);

@@ -311,8 +311,12 @@ static int launch_gemm(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, Ge
 
 int gemm_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, const GemmParams& P) {
   if (P.M <= 16) return gemm_decode_small_launch(st, Xq, Wq, P);
-  if (P.M <= 64 && P.scratch && (P.N + 127) / 128 <= kDecodeMaxCounters) return gemm_decode_launch(st, Xq, Wq, P, P.scratch);
-  if (P.M <= 64 && P.N > 128) return gemm_pair_launch(st, Xq, Wq, P);      // more tiles than the control block has counters
+  if (P.M <= 64 && P.scratch) {
+    // (more tiles than counters and a residual: its loads, a row of tokens at a time, make the epilogue of whole tiles
+    // the slow side beyond 32 tokens: 17 / 37 / 64 x 254080x1024 take 78 / 131 / 178 us, in the CTA-pair kernel 91 / 93 / 96)
+    const bool pair = P.M > 32 && P.residual && (P.N + 127) / 128 > kDecodeMaxCounters;
+    return pair ? gemm_pair_launch(st, Xq, Wq, P) : gemm_decode_launch(st, Xq, Wq, P, P.scratch);
+  }
   if (P.M > 128 && P.N > 128) return gemm_pair_launch(st, Xq, Wq, P);
   if (P.M > 64 && P.M <= 128 && P.N > 128 && gemm_decode_in_two(P.N, P.K)) {
     GemmParams h = P;

@@ -95,6 +95,14 @@ def test_decode_counters_of_many_tiles(M, N, K):
     _run(M, N, K, seed=12, ws=B.new_workspace(B.OP_GEMM, M, N, K), reps=2)
 
 
+@pytest.mark.parametrize("M,K,residual", [(17, 384, True), (37, 384, False), (64, 128, False), (40, 256, True)])
+def test_decode_more_tiles_than_counters(M, K, residual):
+    """Ranges of whole tiles, the last one shorter (1993 tiles in 143 ranges of 14), the last tile ragged."""
+    N = 255016
+    _run(M, N, K, symmetric=residual, z=0 if residual else 9, seed=13, post=True, residual=residual,
+         ws=B.new_workspace(B.OP_GEMM, M, N, K))
+
+
 @pytest.mark.parametrize("M,N,K,what", [
     (40, 8192, 2048, "64 tiles cut in 2: clusters of two CTAs"),
     (33, 2048, 4096, "16 tiles cut in 8: clusters of eight CTAs"),
