@@ -288,7 +288,8 @@ gemm_w4a4_decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     // ------------------------------------------------------------------ epilogue
     reg_inc<kRegsEpi>();
     const int quad = warp & 3;
-    const int npad = D.npad;
+    const int npad = D.npad, m_tok = P.M;
+    const int t_end = (m_tok + kBatch - 1) / kBatch * kBatch;      // (batches of padding alone, 33 .. 48 tokens have one, are left out)
     {
       // per-token factors of the epilogue, shared by the four epilogue warps
       const int t = threadIdx.x - kEpiWarp0 * 32;
@@ -328,7 +329,7 @@ gemm_w4a4_decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
         int32_t* dst = D.cluster > 1 ? reinterpret_cast<int32_t*>(smem + L::kPkWOff) + quad * 32 + lane
                                      : D.slots + ((size_t)(blockIdx.x * 2 + my_slot) * npad) * HR + quad * 32 + lane;
 #pragma unroll 1
-        for (int t0 = 0; t0 < npad; t0 += kBatch) {
+        for (int t0 = 0; t0 < t_end; t0 += kBatch) {
           uint32_t v[kBatch];
           tmem_ld_32x16(taddr + t0, v);
 #pragma unroll
@@ -356,13 +357,12 @@ gemm_w4a4_decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
       }
       if (finalize) {
         // (everything the loop needs from the parameter block is read once, here)
-        const int m_tok = P.M;
         const size_t ldy = (size_t)P.N;
         int32_t* const acc_out = P.acc_out ? P.acc_out + n : nullptr;
         __nv_bfloat16* const yp = P.Y ? P.Y + n : nullptr;
         const __nv_bfloat16* const resp = P.residual ? P.residual + n : nullptr;
 #pragma unroll 1
-        for (int t0 = 0; t0 < npad; t0 += kBatch) {
+        for (int t0 = 0; t0 < t_end; t0 += kBatch) {
           uint32_t v[kBatch];
           if (sum) {
             // (sixteen loads in flight per batch: the four epilogue warps are alone on the SM by now, so
