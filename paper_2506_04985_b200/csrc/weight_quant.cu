@@ -10,6 +10,7 @@
 // (the method's p) is two float64 multiplies; sums meet once per warp and candidate.
 // 14336 x 4096, p = 3, f16 scales: 38.6 -> 2.74 ms; min-max 95 -> 83 us (the row is read once, 16 bytes a load).
 #include "fpt_common.cuh"
+#include "fpt_host.cuh"
 
 namespace fpt {
 
@@ -82,9 +83,35 @@ __device__ __forceinline__ V block_reduce(V v, V* scratch, bool is_max) {
   return r;
 }
 
+// Sums of |w - D q|^p per candidate and warp over the values `from` .. `n` of a row, for a p that is not 3.  A power costs
+// hundreds of instructions, so no thread takes one for a value that is not there: the values (in L1) are dealt out one by
+// one, four at a time where a thread has that many.  p = 2, sixteen values held by each thread as below instead: 14336 x 96
+// 10.4 ms, now 1.14; 64 x 256 560 us, now 62; 4096 x 1056 5.9 ms, now 2.9.
+__device__ __forceinline__ float wload(const __nv_bfloat16* p) { return __bfloat162float(*p); }
+__device__ __forceinline__ float wload(const float* p) { return *p; }
+template <typename T, int NT>
+__device__ __forceinline__ void power_sums(const T* row, int from, int n, const Step* step, double (*part)[NT / 32], bool no_nan, double p) {
+  const int tid = threadIdx.x;
+  for (int i = 0; i < kLpCount; ++i) {
+    const Step s = step[i];
+    const bool fast = no_nan && s.inv != 0.0f;
+    auto error = [&](int k) {
+      const float w = wload(row + k);
+      return pow(fabs((double)w - (double)s.d * (double)quant_code(w, s, fast)), p);
+    };
+    double sum = 0.0;
+    int k = from + tid;
+    for (; k + 3 * NT < n; k += 4 * NT) sum += (error(k) + error(k + NT)) + (error(k + 2 * NT) + error(k + 3 * NT));
+    for (; k < n; k += NT) sum += error(k);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if ((tid & 31) == 0) part[i][tid >> 5] += sum;
+  }
+}
+
 // The search: the candidate with the least sum_k |w - D q|^p, equal sums to the larger scale, sums that are not
 // numbers left out; `fallback` where none is left.  Every thread returns the same step.
-template <typename T, int NT, bool kCube>
+template <typename T, int NT, int kRange>
 __device__ float lp_search(const T* row, int chunks, float a, bool no_nan, float p, int scale_dtype, float fallback) {
   __shared__ Step step[kLpCount];
   __shared__ double part[kLpCount][NT / 32];
@@ -97,7 +124,9 @@ __device__ float lp_search(const T* row, int chunks, float a, bool no_nan, float
   }
   for (int i = tid; i < kLpCount * (NT / 32); i += NT) (&part[0][0])[i] = 0.0;
   __syncthreads();
-  for (int c0 = 0; c0 < chunks; c0 += NT * (kLpHold / 8)) {
+  constexpr int kPass = NT * (kLpHold / 8);
+  int c0 = 0;
+  for (; kRange == 2 ? c0 < chunks : kRange == 3 && c0 + kPass <= chunks; c0 += kPass) {
     float w[kLpHold];
     double w64[kLpHold];
 #pragma unroll
@@ -133,7 +162,7 @@ __device__ float lp_search(const T* row, int chunks, float a, bool no_nan, float
         const double q = __hiloint2double(0x43300000, u[j]) - (4503599627370496.0 + 8.0);
         // |w - D q|: the product of a 24-bit and a 4-bit number is exact in float64
         const double e = fabs(fma(neg_d, q, w64[j]));
-        err[j & 1] = kCube ? fma(__dmul_rn(e, e), e, err[j & 1]) : err[j & 1] + pow(e, (double)p);
+        err[j & 1] = kRange == 2 ? fma(__dmul_rn(e, e), e, err[j & 1]) : err[j & 1] + pow(e, (double)p);
       }
       double sum = err[0] + err[1];
 #pragma unroll
@@ -141,6 +170,7 @@ __device__ float lp_search(const T* row, int chunks, float a, bool no_nan, float
       if (lane == 0) part[i][warp] += sum;
     }
   }
+  if constexpr (kRange != 2) power_sums<T, NT>(row, 8 * c0, 8 * chunks, step, part, no_nan, (double)p);
   __syncthreads();
   if (warp == 0) {
     double best = 1.0 / 0.0;
@@ -163,7 +193,8 @@ __device__ float lp_search(const T* row, int chunks, float a, bool no_nan, float
 }
 
 // NT threads; V > 0: the row (at most NT * 8 * V values) is held in registers; V = 0: it is read again (from L1 or
-// L2) in each pass.  kRange: 0 min-max, 1 L_p, 2 L_3; separate kernels, the search needs twice the registers of the rest.
+// L2) in each pass.  kRange: 0 min-max, 1 L_p, 2 L_3, 3 L_p with sixteen values held by a thread; separate kernels, the
+// searches need twice the registers of the rest.
 template <typename T, int NT, int V, int kRange>
 __global__ void __launch_bounds__(NT, kRange == 2 ? 768 / NT : 1) weight_quant_kernel(const T* __restrict__ W, int K, float p, int scale_dtype,
                                                           uint8_t* __restrict__ Wq, void* __restrict__ sw,
@@ -206,7 +237,7 @@ __global__ void __launch_bounds__(NT, kRange == 2 ? 768 / NT : 1) weight_quant_k
 
   float delta = store_round(__fdiv_rn(a, 7.0f), scale_dtype);
   if (a == 0.0f || delta == 0.0f) delta = 1.0f;
-  if constexpr (kRange != 0) delta = lp_search<T, NT, kRange == 2>(row, chunks, a, no_nan, p, scale_dtype, delta);
+  if constexpr (kRange != 0) delta = lp_search<T, NT, kRange>(row, chunks, a, no_nan, p, scale_dtype, delta);
   if (tid == 0) {
     if (scale_dtype == FPT_DTYPE_F16) reinterpret_cast<__half*>(sw)[n] = __float2half_rn(delta);
     else reinterpret_cast<float*>(sw)[n] = delta;
@@ -233,13 +264,20 @@ __global__ void __launch_bounds__(NT, kRange == 2 ? 768 / NT : 1) weight_quant_k
 }
 
 // Threads by the row's length: sixteen values a thread up to 4096 values, then more passes of the same CTA.  The
-// min-max kernel holds up to 8192 values in registers.
+// min-max kernel holds up to 8192 values in registers.  The search with a general power: one value a thread;
+// sixteen held ones where the rows are too few to fill the chip, so that as many chains of a thread hide the latency
+// (p = 2, 64 x 4096: 0.70 -> 0.61 ms, 8 x 131072: 26 -> 19 ms; 4096 x 4096 the other way round: 11.3 -> 10.9 ms).
 template <typename T, int kRange>
 static void launch_weight_quant(cudaStream_t st, const T* W, int N, int K, float p, int scale_dtype, uint8_t* Wq,
                                 void* sw, int32_t* wsum) {
   constexpr int V = kRange == 0 ? 2 : 0;
   auto go = [&](auto kern, int threads) { kern<<<N, threads, 0, st>>>(W, K, p, scale_dtype, Wq, sw, wsum); };
-  if (K <= 1024) go(weight_quant_kernel<T, 64, V, kRange>, 64);
+  if constexpr (kRange == 1) {
+    if (K >= 16 * kWqThreads && N <= 2 * device_sm_count()) go(weight_quant_kernel<T, kWqThreads, 0, 3>, kWqThreads);
+    else if (K > 128) go(weight_quant_kernel<T, kWqThreads, 0, 1>, kWqThreads);
+    else if (K > 64) go(weight_quant_kernel<T, 128, 0, 1>, 128);
+    else go(weight_quant_kernel<T, 64, 0, 1>, 64);
+  } else if (K <= 1024) go(weight_quant_kernel<T, 64, V, kRange>, 64);
   else if (K <= 2048) go(weight_quant_kernel<T, 128, V, kRange>, 128);
   else if (K <= 4096) go(weight_quant_kernel<T, kWqThreads, V, kRange>, kWqThreads);
   else if (K <= 8192) go(weight_quant_kernel<T, kWqThreads, 2 * V, kRange>, kWqThreads);

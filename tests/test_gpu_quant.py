@@ -143,6 +143,26 @@ def test_weight_quant_range_search_at_ties_and_odd_rows(K):
             assert host(wq)[6, 2] >> 4 == 8              # a NaN takes the lowest code
 
 
+@pytest.mark.parametrize("K", [32, 64, 96, 160, 1056, 4096, 4128, 8224])       # 1 to 33 values a thread, remainders
+@pytest.mark.parametrize("p", [2.0, 2.4, 0.7])
+def test_weight_quant_range_search_with_a_general_power(K, p):
+    rng = np.random.default_rng(K)
+    w = (rng.standard_normal((9, K)) * 0.02).astype(np.float32)
+    w[0] = rng.integers(-14, 15, K) * 0.5                # ties
+    w[1] = 0.0
+    w[2] *= 1e7                                          # float16 scales that overflow
+    w[3, 0] = 3.0                                        # one large value
+    for dt in (torch.bfloat16, torch.float32):
+        wd = torch.from_numpy(w).to(dt)
+        for sd, name in ((torch.float16, "fp16"), (torch.float32, "fp32")):
+            with np.errstate(all="ignore"):
+                codes, d, sums = OQ.quantize_weights(wd.float().numpy(), range_mode=OQ.RANGE_LP, p=p, scale_dtype=name)
+            wq, sw, wsum = B.fpt_quantize_weights(dev(wd), None, B.RANGE_LP, p, sd)
+            assert np.array_equal(host(sw.float()).view(np.uint32), d.view(np.uint32))
+            assert np.array_equal(host(wq), OQ.pack_int4(codes))
+            assert np.array_equal(host(wsum), sums)
+
+
 def test_interleave_gate_up_layout():
     d_ff, K = 384, 256
     rng = np.random.default_rng(0)
