@@ -95,43 +95,79 @@ __global__ void __launch_bounds__(T, V <= 4 ? 2048 / T : 1) act_quant_kernel(con
   }
 }
 
-// Without the RMSNorm nothing is reduced over a token (the multiplier is s_in or 1), so a thread takes one 16-byte
-// chunk of any token and the grid covers the chip whatever the number of tokens.  One CTA per token left 37 tokens
-// to 37 CTAs, which, started early behind a matmul that fills the SMs, pile up on the first few SMs to come free:
-// the SwiGLU pass of 37 x 14336 took 21 us there (5.8 us by itself), now 7 us.
-constexpr int kFlatThreads = 256;
-template <bool kSilu>
-__global__ void __launch_bounds__(kFlatThreads) act_quant_flat_kernel(const ActQuantParams P, int ctas_per_row) {
+// Without the RMSNorm nothing is reduced over a token (the multiplier is s_in or 1): the matrix is one stream of
+// 16-byte chunks, of which a thread takes U, and the grid covers the chip whatever the number of tokens and their
+// length.  One CTA per token left 37 tokens to 37 CTAs, which, started early behind a matmul that fills the SMs, pile up
+// on the first few SMs to come free: the SwiGLU pass of 37 x 14336 took 21 us there (5.8 us by itself), now 7 us.
+// T threads a CTA.
+struct FlatDiv { uint32_t mul, shift; };         // i / chunks = umulhi(i, mul) >> shift for every i below 2^31
+template <bool kSilu, int U, int T>
+__global__ void __launch_bounds__(T, 2048 / T) act_quant_flat_kernel(const ActQuantParams P, uint32_t total, FlatDiv div) {
   pdl_wait();
   pdl_launch_dependents();
-  const int chunks = P.K >> 3;
-  const int t = blockIdx.x / ctas_per_row;
-  const int c = (blockIdx.x - t * ctas_per_row) * kFlatThreads + threadIdx.x;
-  if (c >= chunks) return;
-  const uint4* row = P.X + (size_t)t * (size_t)(P.ldx >> 3);
-  uint4 v;
-  if constexpr (kSilu) {
-    const bool inter = (P.flags & FPT_GU_INTERLEAVED) != 0;
-    const int gc = inter ? ((c >> 3) << 4) + (c & 7) : c;          // groups of 8 chunks (64 columns), gate then up
-    const uint4 g = __ldg(row + gc);
-    const uint4 u = inter ? __ldg(row + gc + 8) : __ldg(P.X2 + (size_t)t * (size_t)(P.ldx >> 3) + c);
-    v = make_uint4(silu_mul_pair(g.x, u.x), silu_mul_pair(g.y, u.y), silu_mul_pair(g.z, u.z), silu_mul_pair(g.w, u.w));
-  } else {
-    v = __ldg(row + c);
+  const uint32_t chunks = (uint32_t)P.K >> 3;
+  const bool inter = kSilu && (P.flags & FPT_GU_INTERLEAVED) != 0;
+  const uint32_t i0 = blockIdx.x * (uint32_t)(T * U) + threadIdx.x;
+  uint4 v[U], v2[kSilu ? U : 1];
+  float s[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const uint32_t i = i0 + u * T;
+    if (i < total) {
+      const uint32_t t = __umulhi(i, div.mul) >> div.shift, c = i - t * chunks;
+      const size_t row = (size_t)t * (size_t)(P.ldx >> 3);
+      const uint32_t gc = inter ? ((c >> 3) << 4) + (c & 7) : c;   // groups of 8 chunks (64 columns), gate then up
+      v[u] = __ldg(P.X + row + gc);
+      if constexpr (kSilu) v2[u] = inter ? __ldg(P.X + row + gc + 8) : __ldg(P.X2 + row + c);
+      s[u] = P.s_in ? __ldg(P.s_in + t) : 1.0f;
+      if (c == 0) {
+        if (P.s_out) P.s_out[t] = s[u];
+        if (P.post_inv) P.post_inv[t] = __fdiv_rn(1.0f, (P.flags & FPT_SCALE_INPUT) ? s[u] : 1.0f);
+        if (P.r_out) P.r_out[t] = 1.0f;
+      }
+    }
   }
-  const float rs = P.s_in ? __ldg(P.s_in + t) : 1.0f;
-  const float p = (P.flags & FPT_SCALE_INPUT) ? rs : 1.0f;
-  if (c == 0) {
-    if (P.s_out) P.s_out[t] = rs;
-    if (P.post_inv) P.post_inv[t] = __fdiv_rn(1.0f, p);
-    if (P.r_out) P.r_out[t] = 1.0f;
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const uint32_t i = i0 + u * T;
+    if (i < total) {
+      if constexpr (kSilu)
+        v[u] = make_uint4(silu_mul_pair(v[u].x, v2[u].x), silu_mul_pair(v[u].y, v2[u].y), silu_mul_pair(v[u].z, v2[u].z),
+                          silu_mul_pair(v[u].w, v2[u].w));
+      const float p = (P.flags & FPT_SCALE_INPUT) ? s[u] : 1.0f;
+      P.Xq[i] = quant_word(v[u], quant_consts(p, P.inv_delta, P.qmax_minus_z, P.flip));
+    }
   }
-  P.Xq[(size_t)t * (size_t)chunks + c] = quant_word(v, quant_consts(p, P.inv_delta, P.qmax_minus_z, P.flip));
 }
 
-// RMSNorm, one warp per token for rows of up to 256 * V elements: the row lives in registers, the
+template <bool kSilu, int U, int T>
+static cudaError_t launch_flat(ActQuantParams P, cudaStream_t st) {
+  const uint32_t chunks = (uint32_t)P.K >> 3;
+  uint32_t log = 1;
+  while ((1u << log) < chunks) ++log;
+  const FlatDiv div = {(uint32_t)((1ull << (31 + log)) / chunks + 1), log - 1};
+  const int slice = (int)(0x7FFFFFFFu / chunks);                   // rows a launch can count in 31 bits
+  for (int left = P.M; left > 0; left -= slice) {
+    P.M = left < slice ? left : slice;
+    const uint32_t total = (uint32_t)P.M * chunks;
+    const cudaError_t e = launch_kernel(act_quant_flat_kernel<kSilu, U, T>, dim3((total + T * U - 1) / (T * U)), dim3(T), 0, st,
+                                        true, P, total, div);
+    if (e != cudaSuccess) return e;
+    const size_t n = (size_t)P.M;
+    P.X += n * (size_t)(P.ldx >> 3);
+    if (P.X2) P.X2 += n * (size_t)(P.ldx >> 3);
+    P.Xq += n * chunks;
+    if (P.s_in) P.s_in += n;
+    if (P.s_out) P.s_out += n;
+    if (P.post_inv) P.post_inv += n;
+    if (P.r_out) P.r_out += n;
+  }
+  return cudaSuccess;
+}
+
+// One warp per token for rows of up to 256 * V elements (kNorm: RMSNorm): the row lives in registers, the
 // reduction is a warp shuffle, no shared memory and no block-wide barrier.  W warps per CTA.
-template <int V, int W>
+template <int V, int W, bool kNorm>
 __global__ void __launch_bounds__(W * 32) act_quant_warp_kernel(const ActQuantParams P) {
   pdl_wait();
   pdl_launch_dependents();
@@ -146,26 +182,29 @@ __global__ void __launch_bounds__(W * 32) act_quant_warp_kernel(const ActQuantPa
     const int c = i * 32 + lane;
     if (c < chunks) v[i] = __ldg(row + c);
   }
-  double acc0 = 0.0, acc1 = 0.0;                 // two chains: the float64 adds are latency-bound otherwise
-#pragma unroll
-  for (int i = 0; i < V; ++i)
-    if (i * 32 + lane < chunks) { if (i & 1) acc1 = sumsq(v[i], acc1); else acc0 = sumsq(v[i], acc0); }
-  double acc = acc0 + acc1;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (!((float)acc <= 3.4028234e38f)) {          // Inf / NaN in the row (or a genuine overflow): by the definition
-    acc0 = 0.0;
+  float r = 1.0f;
+  if constexpr (kNorm) {
+    double acc0 = 0.0, acc1 = 0.0;                 // two chains: the float64 adds are latency-bound otherwise
 #pragma unroll
     for (int i = 0; i < V; ++i)
-      if (i * 32 + lane < chunks) acc0 = sumsq_exact(v[i], acc0);
-    acc = acc0;
+      if (i * 32 + lane < chunks) { if (i & 1) acc1 = sumsq(v[i], acc1); else acc0 = sumsq(v[i], acc0); }
+    double acc = acc0 + acc1;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (!((float)acc <= 3.4028234e38f)) {          // Inf / NaN in the row (or a genuine overflow): by the definition
+      acc0 = 0.0;
+#pragma unroll
+      for (int i = 0; i < V; ++i)
+        if (i * 32 + lane < chunks) acc0 = sumsq_exact(v[i], acc0);
+      acc = acc0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    }
+    const float ss = (float)acc;                   // one rounding to float32 (every lane holds the same sum)
+    const float ms = __fdiv_rn(ss, (float)P.K);
+    const float rho = __fsqrt_rn(__fadd_rn(ms, P.eps));
+    r = __fdiv_rn(1.0f, rho);
   }
-  const float ss = (float)acc;                   // one rounding to float32 (every lane holds the same sum)
-  const float ms = __fdiv_rn(ss, (float)P.K);
-  const float rho = __fsqrt_rn(__fadd_rn(ms, P.eps));
-  const float r = __fdiv_rn(1.0f, rho);
   const float s = P.s_in ? __ldg(P.s_in + t) : 1.0f;
   const float rs = P.s_in ? __fmul_rn(r, s) : r;
   const float p = (P.flags & FPT_SCALE_INPUT) ? rs : r;
@@ -290,9 +329,9 @@ static cudaError_t launch_stream(const ActQuantParams& P, cudaStream_t st) {
   return launch_kernel(act_quant_stream_kernel, dim3(grid), dim3(W * 32), smem, st, true, P, W, NB, row_bytes);
 }
 
-template <int V, int W>
+template <int V, int W, bool kNorm = true>
 static cudaError_t launch_warp(const ActQuantParams& P, cudaStream_t st) {
-  return launch_kernel(act_quant_warp_kernel<V, W>, dim3((P.M + W - 1) / W), dim3(W * 32), 0, st, true, P);
+  return launch_kernel(act_quant_warp_kernel<V, W, kNorm>, dim3((P.M + W - 1) / W), dim3(W * 32), 0, st, true, P);
 }
 
 template <int T, int V>
@@ -323,9 +362,19 @@ cudaError_t act_quant_launch(cudaStream_t st, const void* X, int M, int K, int l
   P.flip = qp->symmetric ? 0x77777777u : 0xFFFFFFFFu;
   const int chunks = K / 8;
   if (!(flags & FPT_RMSNORM)) {
-    const int per_row = (chunks + kFlatThreads - 1) / kFlatThreads;      // (a grid of 2^31 CTAs would read terabytes)
-    auto kern = (flags & FPT_SILU_MUL) ? act_quant_flat_kernel<true> : act_quant_flat_kernel<false>;
-    return launch_kernel(kern, dim3((unsigned)per_row * (unsigned)M), dim3(kFlatThreads), 0, st, true, P, per_row);
+    // By the number of chunks, in units of what the chip's threads hold at one each.  Below half of it small CTAs, which
+    // spread better (1024 x 512: 1.42 -> 1.29 us).  Far above it more chunks a thread and CTA: an SM starts a CTA in about
+    // 150 ns, and CTAs of 256 chunks are over sooner than the next ones come (8192 x 8192: 36.1 us, with 512 chunks 26.2;
+    // 32768 x 4096 70.2 / 49.8; 4096 x 4096 10.3 / 8.7; but 2048 x 2048 3.5 / 4.1).  A SwiGLU product is two loads and a
+    // longer computation: one chunk always (two: 4096 x 8192 51.3 -> 52.3 us).
+    const long long total = (long long)M * chunks, wave = (long long)device_sm_count() * 2048;
+    if (flags & FPT_SILU_MUL) return launch_flat<true, 1, 256>(P, st);
+    if (total >= wave && chunks > 48 && chunks <= 128)         // (32768 x 1024 in 13.8 us instead of 16.9, x 768 10.9 / 13.3)
+      return chunks <= 64 ? launch_warp<2, 4, false>(P, st) : launch_warp<4, 4, false>(P, st);
+    if (2 * total < wave) return launch_flat<false, 1, 128>(P, st);
+    if (total < 2 * wave) return launch_flat<false, 1, 256>(P, st);
+    if (total < 5 * wave) return launch_flat<false, 2, 256>(P, st);
+    return launch_flat<false, 4, 128>(P, st);
   }
   // Many tokens: long rows do best with one CTA per token and many CTAs per SM (measured: 2048 x 8192 in
   // 13 us against 19 us for the streaming kernel); short rows with the persistent streaming kernel

@@ -95,6 +95,44 @@ def test_silu_mul_quant_bit_exact(M, K, inter):
     assert np.array_equal(host(xq), OQ.pack_int4(codes))
 
 
+# Without the norm a CTA takes several short rows or a part of a long one, with one chunk a thread or more: ragged rows
+# a CTA, last CTAs that are nearly empty, rows that end inside a part.
+@pytest.mark.parametrize("M,K", [(1, 32), (63, 32), (65, 32), (90001, 32), (25, 96), (30001, 96), (5, 1024), (10007, 1056),
+                                 (3, 4064), (3300, 768), (801, 4128), (777, 8192), (301, 8256), (2, 65536), (70, 65536)])
+@pytest.mark.parametrize("form", ["plain", "scale_asym", "silu", "gate_up"])
+def test_act_quant_without_norm_short_and_long_rows(M, K, form):
+    if form == "gate_up" and K % 64:
+        pytest.skip("64-column groups")
+    g = torch.Generator(device="cuda").manual_seed(M + K)
+    x, x2 = (torch.randn((M, K), device="cuda", generator=g).to(torch.bfloat16) for _ in range(2))
+    x[M // 2, K // 3], x[M - 1, K - 1] = float("nan"), float("inf")
+    s_in = torch.rand((M,), device="cuda", generator=g) + 0.5
+    qp = B.QParams(4, form != "scale_asym", 0.31, 7)
+    if form == "plain":
+        xq, s_out = B.fpt_act_quant(x, qp, 0, s_in=s_in)
+    elif form == "scale_asym":
+        xq, s_out = B.fpt_act_quant(x, qp, B.SCALE_INPUT, s_in=s_in)
+    elif form == "silu":
+        xq, s_out = B.fpt_act_quant(x, qp, B.SILU_MUL | B.SCALE_INPUT, X2=x2, s_in=s_in)
+    else:
+        gu = torch.stack((x.view(M, K // 64, 64), x2.view(M, K // 64, 64)), 2).reshape(M, 2 * K)
+        xq, s_out = B.fpt_act_quant(gu, qp, B.SILU_MUL | B.GU_INTERLEAVED | B.SCALE_INPUT, s_in=s_in)
+    rows = np.unique(np.r_[0:min(M, 70), M // 2, max(0, M - 70):M])          # the oracle on the first, a middle and the last rows
+    xr, x2r, sr = synth.f32(x.cpu()[rows]), synth.f32(x2.cpu()[rows]), host(s_in)[rows]
+    with np.errstate(all="ignore"):
+        if form in ("silu", "gate_up"):
+            codes, _ = OQ.silu_mul_quant(xr, x2r, oqp(qp), sr)
+        else:
+            codes, _, _, _ = OQ.act_quant(xr, oqp(qp), rmsnorm=False, scale_input=form != "plain", s_in=sr)
+    assert np.array_equal(host(xq)[rows], OQ.pack_int4(codes))
+    assert torch.equal(s_out, s_in)
+    if form in ("plain", "scale_asym"):                                      # every row against torch's own operations
+        v = (x.float() * s_in[:, None] if form == "scale_asym" else x.float()) * float(np.float32(1.0) / np.float32(qp.scale))
+        lo, hi, z = (0, 15, 7) if form == "scale_asym" else (-8, 7, 0)
+        q = torch.where(v.isnan(), torch.full_like(v, lo), (v.round() + z).clamp(lo, hi)).to(torch.int32) & 15
+        assert torch.equal(xq.to(torch.int32), q[:, 0::2] | (q[:, 1::2] << 4))
+
+
 @pytest.mark.parametrize("N,K", [(64, 1024), (33, 4096), (8, 14336), (300, 128)])
 @pytest.mark.parametrize("mode", ["minmax32", "minmax16", "lp32", "lp16_f32in"])
 def test_weight_quant_bit_exact(N, K, mode):
