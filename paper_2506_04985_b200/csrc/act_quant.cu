@@ -380,6 +380,7 @@ cudaError_t act_quant_launch(cudaStream_t st, const void* X, int M, int K, int l
   // 13 us against 19 us for the streaming kernel); short rows with the persistent streaming kernel
   // (16384 x 2048: 20 us against 23 us).
   if (M >= 512) {
+    if (chunks > 64 && chunks < 128) return launch_warp<4, 4>(P, st);
     if (chunks >= 128 && chunks < 512) return launch_stream(P, st);
     if (chunks == 512) return launch<128, 4>(P, st);
     if (chunks > 512 && chunks <= 1024) return launch<256, 4>(P, st);

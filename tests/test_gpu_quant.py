@@ -34,7 +34,7 @@ def test_act_quant_codes_bit_exact(M, K, mode):
     assert len(np.unique(codes)) >= 8 or K < 64        # the grid is actually exercised
 
 
-@pytest.mark.parametrize("M,K,ld", [(600, 1024, 1024), (1500, 4096, 4096), (777, 8192, 8200), (513, 16384, 16384)])
+@pytest.mark.parametrize("M,K,ld", [(600, 768, 768), (513, 544, 552), (600, 1024, 1024), (1500, 4096, 4096), (777, 8192, 8200), (513, 16384, 16384)])
 @pytest.mark.parametrize("mode", ["norm", "scale", "asym"])
 def test_act_quant_many_tokens_streaming_kernel(M, K, ld, mode):
     """Enough tokens for the persistent double-buffered kernel: every warp walks over several rows,
