@@ -149,7 +149,7 @@ int fpt_interleave_gate_up(void* stream, const uint8_t* Wg_q, const uint8_t* Wu_
  *   X2     second operand of FPT_SILU_MUL, same layout as X; with FPT_GU_INTERLEAVED X2 is
  *          ignored, X is [M, 2K] (ldx >= 2K) and logical column k lives at
  *          gate: (k/64)*128 + k%64, up: gate + 64
- *   s_in   [M] f32 or NULL;  s_out [M] f32 or NULL
+ *   s_in   [M] f32 or NULL;  s_out [M] f32 or NULL, may be s_in (in place; so in every entry point with both)
  *   Xq     [M, K/2] packed codes out;  qp->bits == 8 (symmetric grid, no FPT_SILU_MUL): [M, K] int8 codes
  *          q = clamp(rne((x * p) * (1/D)), -128, 127)
  * silu(g) = g / (1 + 2^(-g*log2 e)) with a fixed float32 polynomial for 2^f (degree 6

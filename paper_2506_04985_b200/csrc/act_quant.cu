@@ -34,6 +34,8 @@ __global__ void __launch_bounds__(T, V <= 4 ? 2048 / T : 1) act_quant_kernel(con
   const int tid = threadIdx.x;
   const int chunks = P.K >> 3;                   // 16-byte chunks per row
   const size_t row = (size_t)t * (size_t)(P.ldx >> 3);
+  // read in front of the barriers below, and as memory that may be written: s_out may be s_in
+  const float s = P.s_in ? P.s_in[t] : 1.0f;
   uint4 v[V];
 #pragma unroll
   for (int i = 0; i < V; ++i) {
@@ -78,7 +80,6 @@ __global__ void __launch_bounds__(T, V <= 4 ? 2048 / T : 1) act_quant_kernel(con
   }
   __syncthreads();
   const float r = bcast;
-  const float s = P.s_in ? __ldg(P.s_in + t) : 1.0f;
   const float rs = P.s_in ? __fmul_rn(r, s) : r;
   const float p = (P.flags & FPT_SCALE_INPUT) ? rs : r;
   if (tid == 0) {
@@ -119,7 +120,7 @@ __global__ void __launch_bounds__(T, 2048 / T) act_quant_flat_kernel(const ActQu
       const uint32_t gc = inter ? ((c >> 3) << 4) + (c & 7) : c;   // groups of 8 chunks (64 columns), gate then up
       v[u] = __ldg(P.X + row + gc);
       if constexpr (kSilu) v2[u] = inter ? __ldg(P.X + row + gc + 8) : __ldg(P.X2 + row + c);
-      s[u] = P.s_in ? __ldg(P.s_in + t) : 1.0f;
+      s[u] = P.s_in ? P.s_in[t] : 1.0f;                            // (s_out may be s_in: the same value is stored)
       if (c == 0) {
         if (P.s_out) P.s_out[t] = s[u];
         if (P.post_inv) P.post_inv[t] = __fdiv_rn(1.0f, (P.flags & FPT_SCALE_INPUT) ? s[u] : 1.0f);
@@ -205,7 +206,8 @@ __global__ void __launch_bounds__(W * 32) act_quant_warp_kernel(const ActQuantPa
     const float rho = __fsqrt_rn(__fadd_rn(ms, P.eps));
     r = __fdiv_rn(1.0f, rho);
   }
-  const float s = P.s_in ? __ldg(P.s_in + t) : 1.0f;
+  const float s = P.s_in ? P.s_in[t] : 1.0f;
+  __syncwarp();                                  // every lane has its s: s_out may be s_in
   const float rs = P.s_in ? __fmul_rn(r, s) : r;
   const float p = (P.flags & FPT_SCALE_INPUT) ? rs : r;
   if (lane == 0) {
@@ -282,7 +284,8 @@ __global__ void __launch_bounds__(1024) act_quant_stream_kernel(const ActQuantPa
     const float ms = __fdiv_rn(ss, (float)P.K);
     const float rho = __fsqrt_rn(__fadd_rn(ms, P.eps));
     const float r = __fdiv_rn(1.0f, rho);
-    const float s = P.s_in ? __ldg(P.s_in + t) : 1.0f;
+    const float s = P.s_in ? P.s_in[t] : 1.0f;
+    __syncwarp();                                // every lane has its s: s_out may be s_in
     const float rs = P.s_in ? __fmul_rn(r, s) : r;
     const float p = (P.flags & FPT_SCALE_INPUT) ? rs : r;
     if (lane == 0) {

@@ -64,6 +64,8 @@ __global__ void __launch_bounds__(T, V <= 4 ? 2048 / T : 1) act_quant_dyn_kernel
   const int t = blockIdx.x, tid = threadIdx.x;
   const int chunks = P.K >> 3;
   const size_t row = (size_t)t * (size_t)(P.ldx >> 3);
+  // read in front of the barriers below, and as memory that may be written: s_out may be s_in
+  const float s = P.s_in ? P.s_in[t] : 1.0f;
   uint4 v[V];
 #pragma unroll
   for (int i = 0; i < V; ++i) {
@@ -117,7 +119,6 @@ __global__ void __launch_bounds__(T, V <= 4 ? 2048 / T : 1) act_quant_dyn_kernel
     __syncthreads();
     r = bcast;
   }
-  const float s = P.s_in ? __ldg(P.s_in + t) : 1.0f;
   const float rs = P.s_in ? __fmul_rn(r, s) : r;
   const float p = (P.flags & FPT_SCALE_INPUT) ? rs : r;
   constexpr float kQmax = BITS == 8 ? 127.0f : 7.0f;

@@ -1,5 +1,7 @@
 """GPU parity of the quantise kernels against the oracle: packed codes, scales and row
 sums must match bit for bit."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -199,6 +201,30 @@ def test_weight_quant_range_search_with_a_general_power(K, p):
             assert np.array_equal(host(sw.float()).view(np.uint32), d.view(np.uint32))
             assert np.array_equal(host(wq), OQ.pack_int4(codes))
             assert np.array_equal(host(wsum), sums)
+
+
+@pytest.mark.parametrize("M", [1, 37, 600])
+@pytest.mark.parametrize("K", [96, 256, 1024, 1536, 4096, 8192, 14336, 32768])
+def test_per_token_scale_in_place(M, K):
+    """s_out == s_in: every thread of a token has to see the scale as it was before the call."""
+    g = torch.Generator(device="cuda").manual_seed(K + M)
+    x = torch.randn((M, K), device="cuda", generator=g).to(torch.bfloat16)
+    s_in = torch.exp(torch.randn((M,), device="cuda", generator=g))
+    qp, q8, both = B.QParams(4, True, 0.3, 0), B.QParams(8, True, 0.02, 0), B.RMSNORM | B.SCALE_INPUT
+    ref = [B.fpt_act_quant(x, qp, both, s_in=s_in), B.fpt_act_quant(x, qp, B.SCALE_INPUT, s_in=s_in),
+           B.fpt_act_quant(x, q8, both, s_in=s_in), B.fpt_act_quant_dynamic(x, 4, both, s_in=s_in)]
+    L, delta = B.lib(), torch.empty((M,), device="cuda")
+    for _ in range(5):
+        for i, (codes, s_out) in enumerate(r[:2] for r in ref):
+            s, out = s_in.clone(), torch.empty_like(codes)
+            if i < 3:
+                rc = L.fpt_act_quant(B._stream(), B._ptr(x), M, K, K, ctypes.byref((qp, qp, q8)[i]), (both, B.SCALE_INPUT, both)[i],
+                                     1e-5, None, B._ptr(s), B._ptr(out), B._ptr(s))
+            else:
+                rc = L.fpt_act_quant_dynamic(B._stream(), B._ptr(x), M, K, K, 4, both, 1e-5, B._ptr(s), B._ptr(out), B._ptr(s),
+                                             B._ptr(delta))
+            assert rc == B.OK
+            assert torch.equal(s, s_out) and torch.equal(out, codes)
 
 
 def test_interleave_gate_up_layout():
