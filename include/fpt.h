@@ -367,10 +367,10 @@ int fpt_probe_mma(void* stream, int pair, int n, int n_acc, int a_in_tmem, int i
  * Self-test of the bounded device-side wait (the paper has no counterpart).  Every wait inside the
  * kernels gives up after a time limit, records a code in the status word of the workspace and lets
  * the kernel end normally (FPT_ERR_TIMEOUT from fpt_check_status).  This call runs that very wait
- * routine in a one-warp kernel on a barrier nothing ever arrives at, with a limit of limit_us
- * microseconds (1 .. 100000): the kernel ends by itself after that time.
+ * routine in a one-warp kernel, half of whose lanes wait on a barrier nothing ever arrives at, with a limit
+ * of limit_us microseconds (1 .. 100000): the kernel ends by itself after that time.
  *   workspace  device, 16-byte aligned, at least 8192 bytes, status word zero (fpt_reset_status)
- *   gave_up    device, may be NULL: 1 if the wait returned "gave up"
+ *   gave_up    device, may be NULL: 1 if the wait returned "gave up" in every lane
  * Afterwards fpt_check_status(stream, workspace) returns FPT_ERR_TIMEOUT until fpt_reset_status.
  */
 int fpt_selftest_wait_timeout(void* stream, void* workspace, unsigned int limit_us, unsigned int* gave_up);

@@ -140,6 +140,33 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
                                           uint32_t* status, uint32_t role) {
   return mbar_wait_limit(bar, parity, abort_flag, status, role, kWaitLimitNs);
 }
+// The same for a whole warp.  What follows a wait in the role loops is warp-wide (tcgen05.ld / st, __syncwarp, shuffles):
+// lanes that gave up one by one, where others just saw the phase complete, would never meet those again.  So the warp
+// polls, goes on and leaves as one.  (The phase after the one waited for cannot complete before this warp has gone on.)
+__device__ __forceinline__ bool mbar_wait_warp_limit(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag,
+                                                     uint32_t* status, uint32_t role, uint64_t limit_ns) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  uint64_t t0 = 0;
+  for (uint32_t it = 1;; ++it) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if ((it & 0xFFu) == 0) {
+      const uint64_t now = globaltimer_ns();
+      if (t0 == 0) t0 = now;
+      const bool late = now - t0 > limit_ns;
+      if (__any_sync(0xffffffffu, late || *abort_flag)) {
+        if (late) {
+          *abort_flag = 1u;
+          atomicCAS(status, 0u, kStatusTimeoutBase | role);
+        }
+        return false;
+      }
+    }
+  }
+}
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag,
+                                               uint32_t* status, uint32_t role) {
+  return mbar_wait_warp_limit(bar, parity, abort_flag, status, role, kWaitLimitNs);
+}
 
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

@@ -218,12 +218,12 @@ gemm_w4a4_decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     const int per_thread = D.npad * 8 / kTokThreads;     // 16-byte chunks per thread: 1, 2 or 4
     int ps = 0, s = 0; uint32_t pph = 0, ph = 0;
     for (long long g = g_begin; g < g_end; ++g) {
-      if (!mbar_wait(pk_full(ps), pph, abort_flag, P.status, 7)) break;
+      if (!mbar_wait_warp(pk_full(ps), pph, abort_flag, P.status, 7)) break;
       const uint4* src = reinterpret_cast<const uint4*>(smem + L::kPkXOff + ps * L::kPkX);
       uint4 c[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) if (i < per_thread) c[i] = src[i * kTokThreads + ctid];
-      if (!mbar_wait(op_empty(s), ph ^ 1u, abort_flag, P.status, 8)) break;
+      if (!mbar_wait_warp(op_empty(s), ph ^ 1u, abort_flag, P.status, 8)) break;
       uint8_t* dst = smem + L::kB8Off + s * L::kB8Stage;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -258,7 +258,7 @@ gemm_w4a4_decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     for (int kc = grp; kc < n_local; kc += kGroups) {    // kc: running k-block index of this CTA
       const int ps = kc % NPK; const uint32_t pph = (uint32_t)((kc / NPK) & 1);
       const int s = kc % NS;   const uint32_t ph = (uint32_t)((kc / NS) & 1);
-      if (!mbar_wait(pk_full(ps), pph, abort_flag, P.status, 5)) break;
+      if (!mbar_wait_warp(pk_full(ps), pph, abort_flag, P.status, 5)) break;
       const uint8_t* src = smem + L::kPkWOff + ps * L::kPkW + r * PK_ROW;
       const uint32_t a_tmem = tmem_base + ((uint32_t)(quad * 32) << 16) + kAStage0 + s * (BK / 4);
       bool ok = true;
@@ -272,7 +272,7 @@ gemm_w4a4_decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
 #pragma unroll
         for (int j = 0; j < 4; ++j) widen(c[j], v + 8 * j);
         if (h == 0) {
-          if (!mbar_wait(op_empty(s), ph ^ 1u, abort_flag, P.status, 6)) { ok = false; break; }
+          if (!mbar_wait_warp(op_empty(s), ph ^ 1u, abort_flag, P.status, 6)) { ok = false; break; }
           tc_fence_after();
         }
         tmem_st_32x32(a_tmem + 32 * h, v);
@@ -312,7 +312,7 @@ gemm_w4a4_decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
       // per-row constants, fetched while the matmul of the segment runs
       const float swn = n_ok ? load_scale(P.sw, P.scale_dtype, n) : 0.0f;
       const int zw = (P.wsum && n_ok) ? P.zero_point * __ldg(P.wsum + n) : 0;
-      if (!__all_sync(0xffffffffu, mbar_wait(acc_full(b), bph, abort_flag, P.status, 4))) break;
+      if (!mbar_wait_warp(acc_full(b), bph, abort_flag, P.status, 4)) break;
       tc_fence_after();
       // Nothing below is unrolled further than a batch of sixteen tokens: this code runs once or twice a launch, and
       // code that is entered for the first time comes at about 200 cycles per 128 bytes (64 unrolled stores of partial

@@ -171,8 +171,8 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(sw_full(as));
-      if (!mbar_wait(sw_full(as), aph, abort_flag, P.status, 7)) break;
-      if (!mbar_wait(acc_full(as), aph, abort_flag, P.status, 4)) break;
+      if (!mbar_wait_warp(sw_full(as), aph, abort_flag, P.status, 7)) break;
+      if (!mbar_wait_warp(acc_full(as), aph, abort_flag, P.status, 4)) break;
       tc_fence_after();
       const int row = m0 + quad * 32 + lane;
       const bool row_ok = row < P.M;
@@ -240,8 +240,8 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     bool ok = true;
     for (int tile = blockIdx.x; ok && tile < P.num_tiles; tile += gridDim.x) {
       for (int kb = 0; kb < P.kblocks; ++kb) {
-        if (!mbar_wait(pk_full(ps), pph, abort_flag, P.status, 5) ||
-            !mbar_wait(i8_empty(is), iph ^ 1u, abort_flag, P.status, 6)) { ok = false; break; }
+        if (!mbar_wait_warp(pk_full(ps), pph, abort_flag, P.status, 5) ||
+            !mbar_wait_warp(i8_empty(is), iph ^ 1u, abort_flag, P.status, 6)) { ok = false; break; }
         const uint4* src = reinterpret_cast<const uint4*>(smem + L::kPkOff + ps * L::kPkStage);
         uint8_t* dst = smem + L::kI8Off + is * L::kI8Stage;
 #pragma unroll

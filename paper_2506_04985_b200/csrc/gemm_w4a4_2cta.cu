@@ -238,7 +238,7 @@ gemm_w4a4_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     for (int tile = pair_id; ok && tile < num_tiles; tile += num_pairs) {
       for (int kb = 0; kb < kblocks; ++kb) {
         if (turn == grp) {
-          if (!mbar_wait(pk_full(ps), pph, abort_flag, status_w, 5)) { ok = false; break; }
+          if (!mbar_wait_warp(pk_full(ps), pph, abort_flag, status_w, 5)) { ok = false; break; }
           const uint8_t* src = smem + L::kPkAOff + ps * L::kPkOpA + r * (kA8 ? I8_ROW : PK_ROW);
           // the packed weight tile: 16-byte chunk i * 128 + r is row (i * 128 + r) / 4, chunk r % 4
           const uint4* srcb = reinterpret_cast<const uint4*>(smem + L::kPkBOff + ps * L::kPkOp);
@@ -270,8 +270,7 @@ gemm_w4a4_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
               for (int j = 0; j < 2; ++j) widen(c[j], v + 8 * j);
             }
             if (h == 0) {
-              if (!mbar_wait(op_empty(s), ph ^ 1u, abort_flag, status_w, 6)) { ok = false; break; }
-              __syncwarp();                              // lanes leave a wait one by one; the stores are warp-wide
+              if (!mbar_wait_warp(op_empty(s), ph ^ 1u, abort_flag, status_w, 6)) { ok = false; break; }
               tc_fence_after();
             }
             tmem_st_32x16(a_tmem + 16 * h, v);
@@ -348,9 +347,9 @@ gemm_w4a4_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
       const float sn = (kFuse == 1 && row_ok) ? __ldg(P.mid_scale + row) : 0.0f;
       __syncwarp();
       if (lane == 0) mbar_arrive(sc_full(b));
-      if (!mbar_wait(sc_full(b), bph, abort_flag, status_w, 9)) break;
+      if (!mbar_wait_warp(sc_full(b), bph, abort_flag, status_w, 9)) break;
       // the staging half must have been read by the TMA store of the previous tile
-      if ((y_out_p || kFuse == 1) && !mbar_wait(stg_empty(half), (it & 1) ^ 1u, abort_flag, status_w, 10)) break;
+      if ((y_out_p || kFuse == 1) && !mbar_wait_warp(stg_empty(half), (it & 1) ^ 1u, abort_flag, status_w, 10)) break;
       if constexpr (kFuse == 0) {
         // The residual tile of this half travels by TMA into the staging slabs, in the layout the output
         // will have there, while the matmul of the tile still runs; each thread later reads the 16 bytes
@@ -365,7 +364,7 @@ gemm_w4a4_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
           res_armed = it + 1;
         }
       }
-      if (!mbar_wait(acc_full, it & 1, abort_flag, status_w, 4)) break;
+      if (!mbar_wait_warp(acc_full, it & 1, abort_flag, status_w, 4)) break;
       tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + half * 128;
       const size_t rowoff = (size_t)row * (size_t)n_cols;
@@ -413,7 +412,7 @@ gemm_w4a4_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
           stg[1] = make_uint4(codes[4], codes[5], codes[6], codes[7]);
         }
       } else {
-      if (use_res && !mbar_wait(res_full(half), it & 1, abort_flag, status_w, 12)) break;
+      if (use_res && !mbar_wait_warp(res_full(half), it & 1, abort_flag, status_w, 12)) break;
       res_seen = it + 1;
 #pragma unroll
       for (int ch = 0; ch < 4; ++ch) {
@@ -482,8 +481,9 @@ gemm_w4a4_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
         fence_proxy_async_smem();                        // staged tile -> visible to the TMA engine
         __syncwarp();
         if (lane == 0) mbar_arrive(stg_full(half));
-        if (issuer) {
-          if (!mbar_wait(stg_full(half), it & 1, abort_flag, status_w, 11)) break;
+        bool staged = true;
+        if (issuer) staged = mbar_wait(stg_full(half), it & 1, abort_flag, status_w, 11);
+        if (issuer && staged) {
           const uint32_t s0 = sbase + L::kStgOff + (half * 2) * L::kStgSlab;
           if constexpr (kFuse == 1) {
             tma_store_2d(&tmY, s0, nt / 4 + half * 32, m0);            // 128 rows x 32 bytes of packed codes
@@ -497,7 +497,7 @@ gemm_w4a4_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
           tma_store_wait_read();
           mbar_arrive(stg_empty(half));
         }
-        __syncwarp();
+        if (!__all_sync(0xffffffffu, staged)) break;     // the warp leaves as one
       }
     }
     if (issuer) tma_store_wait_read();

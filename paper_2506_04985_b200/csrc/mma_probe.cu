@@ -114,23 +114,27 @@ __global__ void __launch_bounds__(kThreads, 1) mma_probe_kernel(const Params P) 
   }
 }
 
-// Self-test of the bounded wait every kernel of the library relies on: one thread waits on an
-// mbarrier on which nothing ever arrives, with a limit of `limit_ns`; the wait must give up, record
-// where in the status word, and the kernel must end normally.
+// Self-test of the bounded wait every kernel of the library relies on.  The upper half of the warp waits on an mbarrier
+// on which nothing ever arrives, with a limit of `limit_ns`, the lower half on one whose phase is complete: the wait
+// must give up, in all lanes alike, record where in the status word, and the kernel must end normally.
 __global__ void __launch_bounds__(32, 1) wait_timeout_kernel(uint32_t* status, unsigned long long limit_ns, uint32_t* gave_up) {
-  __shared__ __align__(8) unsigned long long bar_mem;
+  __shared__ __align__(8) unsigned long long bar_mem[2];
   __shared__ uint32_t abort_flag;
-  const uint32_t bar = smem_u32(&bar_mem);
+  const uint32_t bar = smem_u32(bar_mem);
   if (threadIdx.x == 0) {
     abort_flag = 0;
     mbar_init(bar, 1);
+    mbar_init(bar + 8, 1);
     fence_mbar_init();
+    mbar_arrive(bar + 8);
   }
   __syncwarp();
+  const bool ok = mbar_wait_warp_limit(threadIdx.x < 16 ? bar + 8 : bar, 0, &abort_flag, status, 14, limit_ns);
+  const uint32_t left = __ballot_sync(0xffffffffu, !ok);
   if (threadIdx.x == 0) {
-    const bool ok = mbar_wait_limit(bar, 0, &abort_flag, status, 14, limit_ns);
-    if (gave_up) *gave_up = ok ? 0u : 1u;
+    if (gave_up) *gave_up = left == 0xffffffffu ? 1u : 0u;
     mbar_inval(bar);
+    mbar_inval(bar + 8);
   }
 }
 
