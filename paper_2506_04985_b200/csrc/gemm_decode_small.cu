@@ -87,7 +87,12 @@ __global__ void __launch_bounds__(NW * 32, kMinCtas) gemm_w4a4_decode_small_kern
   if (P.early_weights) load(warp);
   pdl_wait();                      // the activation codes come from the kernel before this one
   pdl_launch_dependents();
-  if (!P.early_weights) load(warp);
+  // Otherwise the first weights come right behind the wait, and each further set behind the use of the one before.  Two
+  // forms do better with the rows' constants in front of the weights, as they stand below: unsigned activation codes, which
+  // come with row sums (8 x 28672x4096 with residual and post scale 17.3 -> 16.4 us), and sixteen warps with two token
+  // groups, which also want all loads at the head of the loop (16 x 8192x8192: 13.8 -> 13.1 us, 16 x 8192x28672 36.0 -> 35.2).
+  constexpr bool kHead = NW == 16 && NT == 2;
+  if (!kHead && !kBUnsigned && !P.early_weights) load(warp);
   const uint8_t* xr[NT];
   bool x_ok[NT];
 #pragma unroll
@@ -133,8 +138,10 @@ __global__ void __launch_bounds__(NW * 32, kMinCtas) gemm_w4a4_decode_small_kern
     if (s_tok < P.M) s_sn = __ldg(P.mid_scale + s_tok);
   }
 
+  if (!kHead && kBUnsigned && !P.early_weights) load(warp);
   const uint4 zero = make_uint4(0, 0, 0, 0);
   for (int b0 = warp; b0 < D.kblocks;) {
+    if (kHead && (!P.early_weights || b0 != warp)) load(b0);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int b = b0 + u * NW;
@@ -160,7 +167,7 @@ __global__ void __launch_bounds__(NW * 32, kMinCtas) gemm_w4a4_decode_small_kern
       }
     }
     b0 += NW * U;
-    if (b0 < D.kblocks) load(b0);
+    if (!kHead && b0 < D.kblocks) load(b0);
   }
   // accumulator fragment: c0 (row g, token 2t), c1 (row g, token 2t+1), c2 / c3 the same for row g + 8
 #pragma unroll
