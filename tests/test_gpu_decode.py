@@ -83,8 +83,8 @@ def test_decode_extreme_codes_and_long_k():
     assert np.all(acc[:, 0::2] == 64 * K) and np.all(acc[:, 1::2] == -56 * K)
 
 
-def test_decode_many_tiles_without_counters():
-    """More 128-row tiles than the control block has counters: ranges then end on tile boundaries."""
+def test_decode_few_tokens_and_many_rows():
+    """The kernel for up to 16 tokens, which has no tiles to count, at 4000 strips of sixteen rows."""
     _run(8, 64000, 128, seed=11)
 
 
@@ -125,35 +125,91 @@ def test_decode_65_to_128_tokens_in_two_launches(M, N, K):
     _run(M, N, K, symmetric=False, z=9, seed=32, post=True, residual=True)
 
 
-@pytest.mark.parametrize("M,N,K", [(37, 4096, 14336), (64, 14336, 4096), (37, 28672, 4096), (120, 4096, 14336), (2048, 6144, 4096)])
-def test_launches_in_a_row_give_every_output_every_time(M, N, K):
-    """Nine launches in a graph, replayed on cold caches: tiles arrive late and out of order, and every output of every
-    launch has to be right (one launch by itself, with a slow epilogue, hides a converter that runs ahead)."""
-    g = torch.Generator(device="cuda").manual_seed(5)
-    sets = []
-    for _ in range(3):
-        xa = torch.randint(0, 256, (M, K // 2), dtype=torch.uint8, device="cuda", generator=g)
-        xw = torch.randint(0, 256, (N, K // 2), dtype=torch.uint8, device="cuda", generator=g)
-        sw = torch.rand((N,), device="cuda", generator=g)
-        u = [torch.stack(((q.view(torch.int8) << 4) >> 4, q.view(torch.int8) >> 4), 2).flatten(1).double() for q in (xa, xw)]
-        sets.append((xa, xw, sw, B.new_workspace(B.OP_GEMM, M, N, K), ((u[0] @ u[1].T).float() * sw * torch.tensor(0.3)).to(torch.bfloat16)))
-    ys = [torch.empty((M, N), dtype=torch.bfloat16, device="cuda") for _ in range(9)]
-
-    def launches():
-        for i, y in enumerate(ys):
-            xa, xw, sw, ws, _ = sets[i % 3]
-            B.fpt_w4a4_gemm(xa, xw, sw, 0.3, ws=ws, Y=y)
-
-    launches()
+def _every_output_every_time(calls, outs, want, nbytes):
+    """`calls[i]` writes outs[i] from operands of its own; all of them in a graph, whose replays find nothing they need
+    in L2 (the operands are larger than twice that, `nbytes` in all): tiles arrive late and out of order."""
+    assert nbytes >= 2 * torch.cuda.get_device_properties(0).L2_cache_size
+    for c in calls:
+        c()
     torch.cuda.synchronize()
     graph = torch.cuda.CUDAGraph()
     with torch.cuda.graph(graph):
-        launches()
+        for c in calls:
+            c()
     for _ in range(30):
-        for y in ys:
+        for y in outs:
             y.zero_()
         torch.cuda.synchronize()
         graph.replay()
         torch.cuda.synchronize()
-        assert all(torch.equal(y, sets[i % 3][4]) for i, y in enumerate(ys))
-    assert all(B.fpt_check_status(s[3]) == B.OK for s in sets)
+        assert all(torch.equal(y, w) for y, w in zip(outs, want))
+
+
+def _sets_for(weight_bytes):
+    return max(9, 2 * torch.cuda.get_device_properties(0).L2_cache_size // weight_bytes + 1)
+
+
+def _signed(q):
+    return torch.stack(((q.view(torch.int8) << 4) >> 4, q.view(torch.int8) >> 4), 2).flatten(1).double()
+
+
+@pytest.mark.parametrize("M,N,K,form", [
+    (37, 4096, 14336, "sym"), (64, 14336, 4096, "sym"), (37, 28672, 4096, "sym"), (120, 4096, 14336, "sym"),
+    (2048, 6144, 4096, "sym"), (37, 6144, 4096, "asym"), (333, 6144, 4096, "asym"), (200, 6144, 4096, "a8"),
+    (777, 6144, 4096, "a8")])
+def test_launches_in_a_row_give_every_output_every_time(M, N, K, form):
+    """One launch by itself, with a slow epilogue, hides a converter that runs ahead."""
+    g = torch.Generator(device="cuda").manual_seed(5)
+    calls, outs, want, states = [], [], [], []
+    n = _sets_for(N * K // 2)
+    for _ in range(n):
+        xw = torch.randint(0, 256, (N, K // 2), dtype=torch.uint8, device="cuda", generator=g)
+        sw = torch.rand((N,), device="cuda", generator=g)
+        y = torch.empty((M, N), dtype=torch.bfloat16, device="cuda")
+        w = _signed(xw)
+        ws = B.new_workspace(B.OP_GEMM_A8 if form == "a8" else B.OP_GEMM, M, N, K)
+        if form == "a8":
+            xa = torch.randint(-128, 128, (M, K), dtype=torch.int8, device="cuda", generator=g)
+            a = xa.double()
+            calls.append(lambda xa=xa, xw=xw, sw=sw, ws=ws, y=y: B.fpt_w4a8_gemm(xa, xw, sw, 0.3, ws=ws, Y=y))
+        else:
+            xa = torch.randint(0, 256, (M, K // 2), dtype=torch.uint8, device="cuda", generator=g)
+            sym = form == "sym"
+            a = _signed(xa) if sym else torch.stack((xa & 15, xa >> 4), 2).flatten(1).double() - 8
+            wsum = None if sym else w.sum(1).to(torch.int32)
+            calls.append(lambda xa=xa, xw=xw, sw=sw, ws=ws, y=y, sym=sym, wsum=wsum: B.fpt_w4a4_gemm(
+                xa, xw, sw, 0.3, wsum=wsum, act_symmetric=sym, act_zero_point=0 if sym else 8, ws=ws, Y=y))
+        outs.append(y)
+        want.append(((a @ w.T).float() * sw * torch.tensor(0.3)).to(torch.bfloat16))
+        states.append(ws)
+    _every_output_every_time(calls, outs, want, n * N * K // 2)
+    assert all(B.fpt_check_status(ws) == B.OK for ws in states)
+
+
+@pytest.mark.parametrize("M,d,d_ff,hadamard", [(16, 4096, 3584, False), (520, 4096, 3584, False), (520, 4096, 3584, True)])
+def test_blocks_in_a_row_give_every_output_every_time(M, d, d_ff, hadamard):
+    """The same for the MLP block, whose gate||up matmul has the SwiGLU epilogues; against its parts, one by one."""
+    g = torch.Generator(device="cuda").manual_seed(6)
+    calls, outs, want, states = [], [], [], []
+    n = _sets_for(3 * d * d_ff // 2)
+    qi, qm = B.QParams(4, True, 0.4, 0), B.QParams(4, True, 0.3, 0)
+    for _ in range(n):
+        x = torch.randn((M, d), device="cuda", generator=g).to(torch.bfloat16)
+        wgu, wd = (torch.randint(0, 256, s, dtype=torch.uint8, device="cuda", generator=g) for s in ((2 * d_ff, d // 2), (d, d_ff // 2)))
+        sgu, sd = (torch.rand((k,), device="cuda", generator=g) * 0.01 for k in (2 * d_ff, d))
+        y = torch.empty((M, d), dtype=torch.bfloat16, device="cuda")
+        ws = B.new_workspace(B.OP_MLP_HADAMARD if hadamard else B.OP_MLP, M, d_ff, d)
+        xq, s_n = B.fpt_act_quant(x, qi, B.RMSNORM)
+        torch.cuda.synchronize()
+        gu = ((_signed(xq) @ _signed(wgu).T).float() * sgu * torch.tensor(0.4)).to(torch.bfloat16)
+        form = B.SILU_MUL | B.GU_INTERLEAVED | B.SCALE_INPUT
+        mq = B.fpt_hadamard_quant(gu, qm, form, s_in=s_n) if hadamard else B.fpt_act_quant(gu, qm, form, s_in=s_n)[0]
+        torch.cuda.synchronize()
+        want.append(((_signed(mq) @ _signed(wd).T).float() * sd * torch.tensor(0.3)).to(torch.bfloat16))
+        assert mq.unique().numel() >= 64
+        calls.append(lambda x=x, wgu=wgu, sgu=sgu, wd=wd, sd=sd, ws=ws, y=y: B.fpt_decoder_mlp(
+            x, wgu, sgu, wd, sd, qi, qm, want_s_out=False, ws=ws, Y=y, mid_hadamard=hadamard))
+        outs.append(y)
+        states.append(ws)
+    _every_output_every_time(calls, outs, want, n * 3 * d * d_ff // 2)
+    assert all(B.fpt_check_status(ws) == B.OK for ws in states)

@@ -49,7 +49,8 @@ def test_hadamard_quant_rejects_groups_it_cannot_do():
     assert e.value.code == B.ERR_UNSUPPORTED
 
 
-@pytest.mark.parametrize("M,d,d_ff,residual", [(96, 256, 512, True), (300, 1024, 3584, True), (130, 512, 1536, False)])
+@pytest.mark.parametrize("M,d,d_ff,residual", [(96, 256, 512, True), (300, 1024, 3584, True), (130, 512, 1536, False),
+                                                 (9, 1024, 3584, False), (16, 512, 3584, True)])
 def test_mlp_block_with_online_hadamard(M, d, d_ff, residual):
     seed = 9
     x = synth.activations(M, d, seed, "hmlp/x", law="student_t3", outlier_frac=0.005, outlier_gain=50.0)

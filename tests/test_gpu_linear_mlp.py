@@ -61,14 +61,15 @@ def test_linear_flag_and_post_combinations(flags, post_mode):
     assert assert_bf16_close(bf16_host(Y), ref["y"], "Y") == 0
 
 
-def _mlp_case(M, d, d_ff, seed, with_prev, residual):
+def _mlp_case(M, d, d_ff, seed, with_prev, residual, f16=False):
     x = synth.activations(M, d, seed, "mlp/x", law="student_t3", outlier_frac=0.005, outlier_gain=50.0)
     wg = synth.weights(d_ff, d, 0.02, seed, "mlp/wg")
     wu = synth.weights(d_ff, d, 0.02, seed, "mlp/wu")
     wd = synth.weights(d, d_ff, 0.02, seed, "mlp/wd")
     s_prev = synth.per_token_scale(M, seed, "mlp/s") if with_prev else None
     xf = synth.f32(x)
-    (cg, sg, _), (cu, su, _), (cd, sd, _) = (OQ.quantize_weights(synth.f32(w)) for w in (wg, wu, wd))
+    (cg, sg, _), (cu, su, _), (cd, sd, _) = (OQ.quantize_weights(synth.f32(w), scale_dtype="fp16" if f16 else "fp32")
+                                             for w in (wg, wu, wd))
     # static scales from the data itself (harness side, float64)
     r = OQ.rms_reciprocal(xf, 1e-5)
     d_in = float(OQ.calibrate_static_scale(xf[:64] * r[:64, None], OQ.QParams()))
@@ -78,9 +79,8 @@ def _mlp_case(M, d, d_ff, seed, with_prev, residual):
     sn = pre["s_out"]
     d_mid = float(OQ.calibrate_static_scale(pre["m"] * sn[:, None], OQ.QParams()))
     qp_mid = B.QParams(4, True, d_mid, 0)
-    gq, gs, _ = B.fpt_quantize_weights(dev(wg))
-    uq, us, _ = B.fpt_quantize_weights(dev(wu))
-    dq, ds, _ = B.fpt_quantize_weights(dev(wd))
+    (gq, gs, _), (uq, us, _), (dq, ds, _) = (B.fpt_quantize_weights(dev(w), scale_dtype=torch.float16 if f16 else torch.float32)
+                                             for w in (wg, wu, wd))
     wgu, swgu = B.fpt_interleave_gate_up(gq, uq, gs, us)
     Y, s_out = B.fpt_decoder_mlp(dev(x), wgu, swgu, dq, ds, qp_in, qp_mid, 1e-5,
                                  None if s_prev is None else dev(s_prev), residual)
@@ -97,6 +97,75 @@ def test_decoder_mlp_parity(M, d, d_ff, with_prev, residual):
     assert np.array_equal(host(s_out), ref["s_out"])
     assert len(np.unique(ref["mq"])) >= 8
     assert assert_bf16_close(bf16_host(Y), ref["y"], "mlp Y") == 0
+
+
+# At most 16 tokens: 8 or 16 token columns, many warps a strip below 600 strips (d_ff < 4800); one k-block (d = 128).
+@pytest.mark.parametrize("M,d,d_ff", [(1, 128, 128), (1, 1024, 3584), (2, 128, 4864), (7, 256, 4864), (8, 512, 1408),
+                                      (9, 256, 4864), (16, 1024, 3584)])
+@pytest.mark.parametrize("f16", [False, True])
+def test_decoder_mlp_parity_of_a_few_tokens(M, d, d_ff, f16):
+    Y, s_out, ref = _mlp_case(M, d, d_ff, 2, True, f16, f16)
+    assert np.array_equal(host(s_out), ref["s_out"])
+    assert len(np.unique(ref["mq"])) >= 8
+    assert assert_bf16_close(bf16_host(Y), ref["y"], "mlp Y") == 0
+
+
+@pytest.mark.parametrize("M", [1, 7, 8, 9, 16, 33, 130])
+@pytest.mark.parametrize("d_ff,hadamard", [(640, False), (4864, False), (4864, True)])
+def test_decoder_mlp_equals_its_parts_with_infinities_and_nans(M, d_ff, hadamard):
+    """Whichever kernel forms the products: the codes are those of the separate gate||up matmul and SwiGLU quantiser,
+    also where weight scales, per-token scales or activations are infinite, NaN, zero or at the ends of the range."""
+    d = 256
+    g = torch.Generator(device="cuda").manual_seed(M + d_ff)
+    wgu, wd = (torch.randint(0, 256, s, dtype=torch.uint8, device="cuda", generator=g) for s in ((2 * d_ff, d // 2), (d, d_ff // 2)))
+    sgu, sd = (torch.rand((n,), device="cuda", generator=g) * 0.05 for n in (2 * d_ff, d))
+    odd = torch.tensor([float("inf"), float("nan"), 0.0, 3e38, 1e-40, -0.02], device="cuda")
+    sgu[5::97] = odd.repeat(2 * d_ff)[: sgu[5::97].numel()]
+    s_prev = torch.rand((M,), device="cuda", generator=g) + 0.5
+    x = torch.randn((M, d), device="cuda", generator=g).to(torch.bfloat16)
+    for special in (False, True):
+        if special:
+            s_prev[M // 2:] = odd.repeat(M)[: M - M // 2]
+            x[M // 3, 3], x[M - 1, 5] = float("inf"), float("nan")
+        qi, qm = B.QParams(4, True, 0.4, 0), B.QParams(4, True, 0.7, 0)
+        Y, s_out = B.fpt_decoder_mlp(x, wgu, sgu, wd, sd, qi, qm, 1e-5, s_prev, mid_hadamard=hadamard)
+        xq, s_n = B.fpt_act_quant(x, qi, B.RMSNORM, 1e-5, s_in=s_prev)
+        gu, _ = B.fpt_w4a4_gemm(xq, wgu, sgu, qi.scale)
+        form = B.SILU_MUL | B.GU_INTERLEAVED | B.SCALE_INPUT
+        mq = B.fpt_hadamard_quant(gu, qm, form, s_in=s_n) if hadamard else B.fpt_act_quant(gu, qm, form, s_in=s_n)[0]
+        ref, _ = B.fpt_w4a4_gemm(mq, wd, sd, qm.scale)
+        assert torch.equal(s_out.view(torch.int32), s_n.view(torch.int32))
+        assert torch.equal(Y.view(torch.int16), ref.view(torch.int16))
+        assert special or mq.unique().numel() >= 16
+
+
+@pytest.mark.parametrize("M", [1, 8, 16, 37])
+def test_weights_written_by_the_kernel_in_front(M):
+    """The composed calls may request weights before they wait for the kernel in front of them: not before the kernel that
+    writes those weights, just before the call on the same stream, has finished."""
+    d, d_ff = 2048, 8192
+    g = torch.Generator(device="cuda").manual_seed(3)
+    x = torch.randn((M, d), device="cuda", generator=g).to(torch.bfloat16)
+    wgu, wd = (torch.randint(0, 256, s, dtype=torch.uint8, device="cuda", generator=g) for s in ((2 * d_ff, d // 2), (d, d_ff // 2)))
+    sgu, sd = torch.full((2 * d_ff,), 0.01, device="cuda"), torch.full((d,), 0.01, device="cuda")
+    qi, qm = B.QParams(4, True, 0.4, 0), B.QParams(4, True, 0.05, 0)
+    ws, wl = B.new_workspace(B.OP_MLP, M, d_ff, d), B.new_workspace(B.OP_LINEAR, M, 2 * d_ff, d)
+
+    outs = [(torch.empty((M, d), dtype=torch.bfloat16, device="cuda"), torch.empty((M, 2 * d_ff), dtype=torch.bfloat16, device="cuda"))
+            for _ in range(22)]
+    for i, (mlp, linear) in enumerate(outs):
+        wait = torch.cuda.synchronize if i < 2 else (lambda: None)       # the first two: what comes out with nothing running
+        for step in (lambda: wd.bitwise_xor_(0xA5), lambda: wgu.bitwise_xor_(0x5A),
+                     lambda: B.fpt_decoder_mlp(x, wgu, sgu, wd, sd, qi, qm, want_s_out=False, ws=ws, Y=mlp),
+                     lambda: wgu.bitwise_xor_(0x0F),
+                     lambda: B.fpt_w4a4_linear(x, wgu, sgu, qi, want_s_out=False, ws=wl, Y=linear),
+                     lambda: wgu.bitwise_xor_(0x0F)):
+            step()
+            wait()
+    torch.cuda.synchronize()
+    assert not any(torch.equal(a, b) for a, b in zip(*outs[:2]))
+    for i, out in enumerate(outs):
+        assert all(torch.equal(y, w) for y, w in zip(out, outs[i % 2])), i
 
 
 def test_config2_attention_projections_sampled():
@@ -141,7 +210,9 @@ def test_config2_attention_projections_sampled():
 
 @pytest.mark.parametrize("M,d,n_q,n_kv,with_prev,residual,symmetric",
                          [(96, 256, 256, 64, True, True, True), (300, 1024, 1024, 256, True, True, True),
-                          (33, 512, 512, 128, False, False, True), (513, 256, 256, 128, True, True, False)])
+                          (33, 512, 512, 128, False, False, True), (513, 256, 256, 128, True, True, False),
+                          (1, 1024, 1024, 256, True, True, False), (8, 1024, 1024, 256, True, True, True),
+                          (9, 512, 512, 128, False, False, True), (16, 512, 512, 128, True, True, False)])
 def test_decoder_attention_projections_parity(M, d, n_q, n_kv, with_prev, residual, symmetric):
     """fpt_decoder_attn_qkv -> (an attention stand-in on the host) -> fpt_decoder_attn_out against the
     oracle's two halves on the same values: codes-derived outputs, S_n and r bit-exact."""
