@@ -120,11 +120,11 @@ def test_decoder_mlp_equals_its_parts_with_infinities_and_nans(M, d_ff, hadamard
     wgu, wd = (torch.randint(0, 256, s, dtype=torch.uint8, device="cuda", generator=g) for s in ((2 * d_ff, d // 2), (d, d_ff // 2)))
     sgu, sd = (torch.rand((n,), device="cuda", generator=g) * 0.05 for n in (2 * d_ff, d))
     odd = torch.tensor([float("inf"), float("nan"), 0.0, 3e38, 1e-40, -0.02], device="cuda")
-    sgu[5::97] = odd.repeat(2 * d_ff)[: sgu[5::97].numel()]
     s_prev = torch.rand((M,), device="cuda", generator=g) + 0.5
     x = torch.randn((M, d), device="cuda", generator=g).to(torch.bfloat16)
     for special in (False, True):
         if special:
+            sgu[5::97] = odd.repeat(2 * d_ff)[: sgu[5::97].numel()]
             s_prev[M // 2:] = odd.repeat(M)[: M - M // 2]
             x[M // 3, 3], x[M - 1, 5] = float("inf"), float("nan")
         qi, qm = B.QParams(4, True, 0.4, 0), B.QParams(4, True, 0.7, 0)
