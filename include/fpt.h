@@ -207,8 +207,8 @@ int fpt_hadamard_quant(void* stream, const void* X, int M, int K, int ldx,
  *   acc_out [M, N] int32 or NULL: debugging aid, the raw accumulators.
  *   workspace: fpt_workspace_bytes(FPT_OP_GEMM, M, N, K) bytes; it starts with an 8 KiB control
  *   block (status word read by fpt_check_status, tile counters) that fpt_reset_status zeroes.
- * M >= 1; K % 128 == 0; N % 8 == 0.  For M <= 64 a weight-streaming kernel is used: it splits
- * the weight stream evenly over the SMs and adds the partial sums up as exact integers.
+ * M >= 1; K % 128 == 0; N % 8 == 0.  For M <= 64 weight-streaming kernels are used: beyond 16 tokens the
+ * weight stream is split evenly over the SMs and the partial sums are added up as exact integers.
  */
 int fpt_w4a4_gemm(void* stream, const uint8_t* Xq, const uint8_t* Wq, int M, int N, int K,
                   const void* sw, int scale_dtype, const int32_t* wsum,
@@ -307,7 +307,8 @@ int fpt_w4a4_linear_static(void* stream, const void* X, int M, int K,
  *   workspace: fpt_workspace_bytes(FPT_OP_MLP, M, d_ff, d) bytes, or (FPT_OP_MLP_HADAMARD, M, d_ff, d)
  *   with mid_hadamard = 1.  A 16-bit buffer between the two matmuls is part of it only where a route
  *   uses one: none with more than 128 tokens and no transform (the gate||up matmul quantises the
- *   products itself), the products [M, d_ff] with the transform, gate||up [M, 2 d_ff] up to 128 tokens.
+ *   products itself), the products [M, d_ff] with the transform, gate||up [M, 2 d_ff] up to 128 tokens
+ *   (reserved, not used, at up to 16 tokens without the transform).
  */
 int fpt_decoder_mlp(void* stream, const void* X, int M, int d, int d_ff,
                     const uint8_t* Wgu_q, const void* sw_gu, const uint8_t* Wd_q, const void* sw_d,

@@ -16,7 +16,8 @@ static int check_qp(const fpt_qparams* qp) {
 
 // bf16 buffer between the two matmuls of the MLP block: nothing when the gate||up matmul's epilogue
 // quantises the products itself (more than 128 tokens, no online transform), the products [M, d_ff]
-// when the transform needs whole rows of them, gate||up [M, 2 d_ff] on the unfused route.
+// when the transform needs whole rows of them, gate||up [M, 2 d_ff] on the unfused route (reserved up to 128 tokens,
+// although at most 16 tokens without the transform leave it alone: the size is part of the interface).
 static size_t mlp_gu_bytes(int M, int d_ff, bool hadamard) {
   if (M > 128) return hadamard ? (size_t)M * (size_t)d_ff * 2 : 0;
   return (size_t)M * 2 * (size_t)d_ff * 2;

@@ -31,7 +31,8 @@ struct GemmParams {
   int mid_qmax_minus_z;
   uint32_t mid_flip;
   int early_weights;           // the kernel in front in the stream belongs to the same call, waits for all before it
-                               // and writes no weights: they may be read before this kernel's own wait
+                               // and writes no weights: they may be read before this kernel's own wait (only the
+                               // kernel for at most 16 tokens does)
   uint32_t* status;            // control block of the workspace (status word, decode counters)
   void* scratch;               // gemm_scratch_bytes(M) bytes behind the control block (decode partial sums)
 };

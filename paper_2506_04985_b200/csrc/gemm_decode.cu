@@ -10,7 +10,8 @@
 //
 // Work is split stream-K style: the T = (N/128) * (K/256) weight k-blocks are cut into equal
 // contiguous ranges, one per CTA (one CTA per SM), so every SM streams the same number of bytes
-// whatever the shape.  A range that covers part of a tile leaves its raw int32 partial sums in
+// whatever the shape.  (More tiles than the control block has counters: ranges of whole tiles.)  A range that
+// covers part of a tile leaves its raw int32 partial sums in
 // a scratch slot; the last CTA to arrive at a tile (an atomic byte per tile and lane
 // quadrant) adds the slots up -- integer addition, so the result does not depend on the order
 // -- and runs the epilogue.  No CTA ever waits for another.
@@ -149,7 +150,7 @@ gemm_w4a4_decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
   pdl_wait();                      // nothing above touched memory another kernel may write
   pdl_launch_dependents();
 
-  // Registers: the epilogue wants the 64 accumulators of its row in registers at once, the other roles
+  // Registers: the epilogue holds sixteen partial sums and sixteen loads in flight at a time, the other roles
   // need few; the warpgroups trade (see the static_assert above: the requests are covered).
   if (warp < kConvBWarp0) reg_dec<kRegsCtl>();
   if (warp == 0) {

@@ -189,9 +189,8 @@ __global__ void __launch_bounds__(NW * 32, kMinCtas) gemm_w4a4_decode_small_kern
       const uint32_t word = pack_nibbles(code, lane);
       if (s_f == 0 && s_tok < P.M) reinterpret_cast<uint32_t*>(P.Mq)[(size_t)s_tok * (size_t)(P.N >> 4) + blockIdx.x] = word;
     }
-    return;
   }
-  // consecutive threads take consecutive weight rows of one token
+  // consecutive threads take consecutive weight rows of one token (SwiGLU: o_ok is false throughout)
 #pragma unroll
   for (int q = 0; q < kPer; ++q) {
     if (!o_ok[q]) continue;
