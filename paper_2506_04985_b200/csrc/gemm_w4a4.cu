@@ -333,12 +333,13 @@ int gemm_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, const Gem
     return gemm_decode_launch(st, Xq + (size_t)64 * (size_t)(P.K / 2), Wq, h, nullptr);
   }
   if (P.M > 64 && P.N > 128) {
-    // 65..128 tokens: the CTA-pair kernel (half of its 256 activation rows empty) still beats the
-    // one-CTA kernel per k-block (measured 0.5 against 0.68 us), unless it needs more rounds of tiles
+    // 65..128 tokens: the CTA-pair kernel (half of its 256 activation rows empty) takes half as long as the one-CTA
+    // kernel per round of tiles and k-block (0.27 against 0.54 us), so it is taken unless it needs twice the rounds or
+    // more (128 x 40960x4096, three against two: 38 against 49 us; 128 x 28672x4096, two against one: 28.1 against 28.7)
     const int sms = num_sms(), pairs = sms >= 2 ? sms / 2 : 1;
     const int rounds_1 = ((P.N + 255) / 256 + sms - 1) / sms;
     const int rounds_2 = ((P.N + 207) / 208 + pairs - 1) / pairs;
-    if (rounds_2 * 3 < rounds_1 * 4) return gemm_pair_launch(st, Xq, Wq, P);
+    if (rounds_2 < 2 * rounds_1) return gemm_pair_launch(st, Xq, Wq, P);
   }
   if (P.N <= 64) return launch_gemm<64, 4, 4, 8>(st, Xq, Wq, P);
   if (P.N <= 128) return launch_gemm<128, 4, 4, 8>(st, Xq, Wq, P);

@@ -70,6 +70,13 @@ def test_gemm_wide_outputs_ragged_column_tiles(M, N, K, extras):
     _run(M, N, K, seed=5, post=extras, residual=extras, symmetric=not extras, z=9 if extras else 0)
 
 
+@pytest.mark.parametrize("M", [65, 100, 128])
+@pytest.mark.parametrize("N", [37888, 38408, 40960, 46176])
+def test_gemm_65_to_128_tokens_either_side_of_a_round_of_tiles(M, N):
+    """One or two rounds of one-CTA tiles against two, three or four of CTA pairs."""
+    _run(M, N, 128, seed=6, post=True, residual=M == 100, symmetric=M != 128, z=9 if M == 128 else 0)
+
+
 def test_gemm_extreme_codes_reach_the_accumulator_bound():
     M, N, K = 130, 264, 28672
     qa = np.full((M, K), -8, dtype=np.int8)
