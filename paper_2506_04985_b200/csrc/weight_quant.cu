@@ -9,8 +9,11 @@
 // quotient lies so close to a tie that the two could round differently, one branch for the sixteen values; |e|^3
 // (the method's p) is two float64 multiplies; sums meet once per warp and candidate.
 // 14336 x 4096, p = 3, f16 scales: 38.6 -> 2.74 ms; min-max 72 -> 53 us (the row is read once, 16 bytes a load).
+#include <type_traits>
+
 #include "fpt_common.cuh"
 #include "fpt_host.cuh"
+#include "quant_math.cuh"
 
 namespace fpt {
 
@@ -109,6 +112,167 @@ __device__ __forceinline__ void power_sums(const T* row, int from, int n, const 
   }
 }
 
+// Screening of the candidates of an L_3 search in float32.  A candidate's sum there is within `kScreenEps` of the exact
+// one, relatively: a code can differ only where the quotient lies within 1e-6 of a tie, where both neighbours leave the
+// same |e| to 4e-6, so a term |e|^3 is right to 2e-5, and the additions (a chain of at most 203 terms, then of chunks)
+// add less than 3e-5.  So a candidate beyond (1 + 4 kScreenEps) times the least sum cannot be the answer; the ones that
+// are left (one to three of 81, as a rule) go through the float64 sums below, which decide as they always did.
+// The row is scaled by a power of two so that its largest magnitude lies in [1, 2): |e|^3 then underflows only below
+// 2^-42, which the absolute slack covers.
+//   * bf16 rows longer than kBins: what counts is how often a magnitude occurs.  Bins by bit pattern below the row's
+//     largest, 128 an octave: kTop for each sign (the grid's ends differ, -8 and 7), kBoth for the two together (no
+//     candidate clamps there, 0.19 a < 7.4 D), and from seven octaves down every candidate has the code 0 (a / 128 <
+//     0.49 D), the same error for all.  1216 magnitudes with a count each in place of K values.
+//   * otherwise the values themselves, kChunk at a time.
+// A thread takes a candidate and a third of the entries, which a warp then reads as broadcasts: nothing is reduced per
+// candidate but three numbers.  Two entries an instruction where the packed forms allow.
+constexpr float kScreenEps = 1e-4f;
+constexpr int kTop = 320, kBoth = 576, kBins = 2 * kTop + kBoth, kChunk = 1024, kThirds = 3;
+static_assert(kTop % 4 == 0 && kBoth % 4 == 0 && kChunk <= kBins, "four entries a load");
+
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+// Two entries: adds count * |D q - v|^3.  kClamp: 0 no code is clamped, 1 magnitudes, codes up to `hi`, 2 signed values.
+template <int kClamp>
+__device__ __forceinline__ uint64_t screen2(float v0, float v1, uint64_t count, uint64_t inv2, uint64_t neg_d2, float hi, uint64_t acc) {
+  constexpr float kMagic = 12582912.0f;                            // 1.5 * 2^23
+  const uint64_t v = pack_f32x2(v0, v1);
+  uint64_t q = fma_f32x2(v, inv2, pack_f32x2(kMagic, kMagic));
+  if constexpr (kClamp != 0) {
+    float r0, r1;
+    unpack_f32x2(q, r0, r1);
+    if constexpr (kClamp == 2) { r0 = fmaxf(r0, kMagic - 8.0f); r1 = fmaxf(r1, kMagic - 8.0f); }
+    q = pack_f32x2(fminf(r0, kMagic + hi), fminf(r1, kMagic + hi));
+  }
+  const uint64_t e = fma_f32x2(neg_d2, add_f32x2(q, pack_f32x2(-kMagic, -kMagic)), v);
+  float e0, e1, s0, s1;
+  unpack_f32x2(e, e0, e1);
+  unpack_f32x2(mul_f32x2(e, e), s0, s1);
+  return fma_f32x2(pack_f32x2(s0 * fabsf(e0), s1 * fabsf(e1)), count, acc);
+}
+
+// Finds the candidates that can be the answer: list[0 .. count), in ascending order.  False: not applicable, all can.
+template <typename T, int NT>
+__device__ bool lp_screen(const T* row, int chunks, float a, bool no_nan, const Step* step, unsigned char* list, int* count) {
+  __shared__ __align__(16) float val[kBins];
+  __shared__ __align__(16) union { unsigned n[kBins]; float f[kBins]; } cnt;   // (both read four at a time)
+  __shared__ float part[kThirds][kLpCount];
+  constexpr bool kBf16 = sizeof(T) == 2;
+  constexpr int kTasks = kThirds * kLpCount, kPer = (kTasks + NT - 1) / NT;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const float d_min = step[0].d;
+  // (steps grow with the candidate; a step of 0 has been replaced by 1, one beyond float16 has no reciprocal)
+  if (!no_nan || !(a > 0x1p-90f && a < 0x1p90f) || !(d_min < a * 0.03f) || step[0].inv == 0.0f || step[kLpCount - 1].inv == 0.0f) return false;
+  const int exponent = (int)(__float_as_uint(a) >> 23);
+  const float unit = __uint_as_float((uint32_t)(254 - exponent) << 23);       // a * unit in [1, 2)
+  const bool bins = kBf16 && 8 * chunks > kBins && 0.19f * a < 7.4f * d_min && a * (1.0f / 128) < 0.49f * d_min;
+  uint64_t acc[kPer];
+#pragma unroll
+  for (uint64_t& v : acc) v = 0;
+  if (bins) {
+    const int top = (int)(__float_as_uint(a) >> 16);               // pattern of the largest magnitude
+    for (int i = tid; i < kBins; i += NT) cnt.n[i] = 0;
+    __syncthreads();
+    for (int c = tid; c < chunks; c += NT) {
+      const uint4 x = *reinterpret_cast<const uint4*>(row + 8 * (size_t)c);
+      const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const uint32_t p = (w[j >> 1] >> (16 * (j & 1))) & 0xFFFFu;
+        const int idx = top - (int)(p & 0x7FFFu);
+        const int at = idx < kTop ? idx + ((p & 0x8000u) ? kTop : 0) : kTop + idx;
+        if (idx < kTop + kBoth) atomicAdd(&cnt.n[at], 1u);
+      }
+    }
+    __syncthreads();
+    for (int i = tid; i < kBins; i += NT) {
+      cnt.f[i] = (float)cnt.n[i];
+      val[i] = __uint_as_float((uint32_t)(top - (i < kTop ? i : i - kTop)) << 16) * unit;
+    }
+    __syncthreads();
+    int k = 0;
+    for (int task = tid; task < kTasks; task += NT, ++k) {
+      const int third = task / kLpCount;
+      const float d = step[task % kLpCount].d * unit, inv = __fdiv_rn(1.0f, d);
+      const uint64_t inv2 = pack_f32x2(inv, inv), nd2 = pack_f32x2(-d, -d);
+      uint64_t sum = 0;
+      auto run = [&](auto clamp, int from, int to, float hi) {
+#pragma unroll 4
+        for (int i = from + 4 * third; i < to; i += 4 * kThirds) {
+          const float4 v = *reinterpret_cast<const float4*>(val + i), n = *reinterpret_cast<const float4*>(cnt.f + i);
+          sum = screen2<decltype(clamp)::value>(v.x, v.y, pack_f32x2(n.x, n.y), inv2, nd2, hi, sum);
+          sum = screen2<decltype(clamp)::value>(v.z, v.w, pack_f32x2(n.z, n.w), inv2, nd2, hi, sum);
+        }
+      };
+      run(std::integral_constant<int, 1>(), 0, kTop, 7.0f);
+      run(std::integral_constant<int, 1>(), kTop, 2 * kTop, 8.0f);
+      run(std::integral_constant<int, 0>(), 2 * kTop, kBins, 0.0f);
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) if (q == k) acc[q] = sum;
+    }
+  } else {
+    for (int c0 = 0; c0 < chunks; c0 += kChunk / 8) {
+      __syncthreads();
+      for (int c = tid; c < kChunk / 8; c += NT) {
+        float x[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};        // a zero costs no error on any grid
+        if (c0 + c < chunks) wload8(row + 8 * (size_t)(c0 + c), x);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) val[8 * c + j] = x[j] * unit;
+      }
+      __syncthreads();
+      const int n = min(kChunk, 8 * (chunks - c0));
+      int k = 0;
+      for (int task = tid; task < kTasks; task += NT, ++k) {
+        const float d = step[task % kLpCount].d * unit, inv = __fdiv_rn(1.0f, d);
+        const uint64_t inv2 = pack_f32x2(inv, inv), nd2 = pack_f32x2(-d, -d), one = pack_f32x2(1.0f, 1.0f);
+        uint64_t sum = 0;
+#pragma unroll 4
+        for (int i = 4 * (task / kLpCount); i < n; i += 4 * kThirds) {
+          const float4 v = *reinterpret_cast<const float4*>(val + i);
+          sum = screen2<2>(v.x, v.y, one, inv2, nd2, 7.0f, sum);
+          sum = screen2<2>(v.z, v.w, one, inv2, nd2, 7.0f, sum);
+        }
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) if (q == k) acc[q] = add_f32x2(acc[q], sum);
+      }
+    }
+  }
+  int k = 0;
+  for (int task = tid; task < kTasks; task += NT, ++k) {
+    float lo = 0.0f, hi = 0.0f;
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) if (q == k) unpack_f32x2(acc[q], lo, hi);
+    part[task / kLpCount][task % kLpCount] = lo + hi;
+  }
+  __syncthreads();
+  if (tid < 32) {
+    float e[(kLpCount + 31) / 32], least = 3.4e38f;
+#pragma unroll
+    for (int j = 0; j < (kLpCount + 31) / 32; ++j) {
+      const int i = 32 * j + lane;
+      e[j] = i < kLpCount ? (part[0][i] + part[1][i]) + part[2][i] : 3.4e38f;
+      least = fminf(least, e[j]);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) least = fminf(least, __shfl_xor_sync(0xffffffffu, least, o));
+    const float limit = least * (1.0f + 4.0f * kScreenEps) + 0x1p-110f;
+    int n = 0;
+#pragma unroll
+    for (int j = 0; j < (kLpCount + 31) / 32; ++j) {
+      const bool keep = 32 * j + lane < kLpCount && e[j] <= limit;
+      const unsigned mask = __ballot_sync(0xffffffffu, keep);
+      if (keep) list[n + __popc(mask & ((1u << lane) - 1u))] = (unsigned char)(32 * j + lane);
+      n += __popc(mask);
+    }
+    if (lane == 0) *count = n;
+  }
+  __syncthreads();
+  return true;
+}
+
 // The search: the candidate with the least sum_k |w - D q|^p, equal sums to the larger scale, sums that are not
 // numbers left out; `fallback` where none is left.  Every thread returns the same step.
 template <typename T, int NT, int kRange>
@@ -116,6 +280,8 @@ __device__ float lp_search(const T* row, int chunks, float a, bool no_nan, float
   __shared__ Step step[kLpCount];
   __shared__ double part[kLpCount][NT / 32];
   __shared__ float found;
+  __shared__ unsigned char list[kLpCount];               // the candidates the float64 sums are taken for, ascending
+  __shared__ int count;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int i = tid; i < kLpCount; i += NT) {
     float d = store_round(__fdiv_rn(__fmul_rn(a, __fdiv_rn((float)(kLpFirst + i), 100.0f)), 7.0f), scale_dtype);
@@ -124,6 +290,9 @@ __device__ float lp_search(const T* row, int chunks, float a, bool no_nan, float
   }
   for (int i = tid; i < kLpCount * (NT / 32); i += NT) (&part[0][0])[i] = 0.0;
   __syncthreads();
+  bool screened = false;
+  if constexpr (kRange == 2) screened = lp_screen<T, NT>(row, chunks, a, no_nan, step, list, &count);
+  const int cands = screened ? count : kLpCount;
   constexpr int kPass = NT * (kLpHold / 8);
   int c0 = 0;
   for (; kRange == 2 ? c0 < chunks : kRange == 3 && c0 + kPass <= chunks; c0 += kPass) {
@@ -139,7 +308,8 @@ __device__ float lp_search(const T* row, int chunks, float a, bool no_nan, float
     }
 #pragma unroll
     for (int j = 0; j < kLpHold; ++j) w64[j] = (double)w[j];
-    for (int i = 0; i < kLpCount; ++i) {
+    for (int n = 0; n < cands; ++n) {
+      const int i = screened ? list[n] : n;
       const Step s = step[i];
       const double neg_d = -(double)s.d;
       const bool fast = no_nan && s.inv != 0.0f;
@@ -175,10 +345,11 @@ __device__ float lp_search(const T* row, int chunks, float a, bool no_nan, float
   if (warp == 0) {
     double best = 1.0 / 0.0;
     int at = -1;
-    for (int i = lane; i < kLpCount; i += 32) {
+    for (int n = lane; n < cands; n += 32) {
+      const int i = screened ? list[n] : n;
       double e = 0.0;
       for (int v = 0; v < NT / 32; ++v) e += part[i][v];
-      if (e <= best) { best = e; at = i; }                 // i grows: ties to the larger scale
+      if (e <= best) { best = e; at = i; }                 // i grows with n: ties to the larger scale
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {

@@ -183,6 +183,35 @@ def test_weight_quant_range_search_at_ties_and_odd_rows(K):
             assert host(wq)[6, 2] >> 4 == 8              # a NaN takes the lowest code
 
 
+@pytest.mark.parametrize("K", [992, 1216, 1248, 2080, 4096, 14336])     # either side of the rows whose magnitudes are counted
+def test_weight_quant_range_search_keeps_the_least_error(K):
+    """Rows on which the float32 screening of the candidates could go wrong: many equal errors, one sign, magnitudes at
+    the ends of what is counted, scales at the end of float16."""
+    rng = np.random.default_rng(K + 1)
+    w = rng.standard_normal((16, K)) * 0.02
+    w[0] = rng.choice([-1.0, 1.0], K)                    # one magnitude: the errors of many candidates are nearly alike
+    w[1] = np.abs(w[1])
+    w[2] = -np.abs(w[2])
+    w[3] = rng.integers(-8, 9, K) * 0.125                # a grid point of several candidates, both ends in use
+    w[4] = np.exp2(rng.uniform(-9, 0, K)) * rng.choice([-1.0, 1.0], K)      # every octave down to where all codes are 0
+    w[5], w[5, 7] = 0.0, 1.0                             # zeros but for one value
+    w[6, 11] = 40.0                                      # everything else far below the least step
+    w[7] = rng.uniform(-1, 1, K)
+    w[8] = -0.0 * w[8]
+    w[9] *= 0.004 / 0.08                                 # float16 scales around the least ordinary one
+    w[10] *= 1e-5
+    w[11] = rng.choice([-1.0, 1.0], K) * (1.0 + rng.integers(0, 128, K) / 128)      # one octave
+    w[12] = rng.integers(-14, 15, K) * 0.5
+    for dt in (torch.bfloat16, torch.float32):
+        wd = torch.from_numpy(w.astype(np.float32)).to(dt)
+        for sd, name in ((torch.float16, "fp16"), (torch.float32, "fp32")):
+            codes, d, sums = OQ.quantize_weights(wd.float().numpy(), range_mode=OQ.RANGE_LP, p=3.0, scale_dtype=name)
+            wq, sw, wsum = B.fpt_quantize_weights(dev(wd), None, B.RANGE_LP, 3.0, sd)
+            assert np.array_equal(host(sw.float()).view(np.uint32), d.view(np.uint32))
+            assert np.array_equal(host(wq), OQ.pack_int4(codes))
+            assert np.array_equal(host(wsum), sums)
+
+
 @pytest.mark.parametrize("K", [32, 64, 96, 160, 1056, 4096, 4128, 8224])       # 1 to 33 values a thread, remainders
 @pytest.mark.parametrize("p", [2.0, 2.4, 0.7])
 def test_weight_quant_range_search_with_a_general_power(K, p):
