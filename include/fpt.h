@@ -235,8 +235,9 @@ int fpt_w4a8_gemm(void* stream, const int8_t* Xq8, const uint8_t* Wq, int M, int
  * Steps (1)+(2)+(3): one W4A4 linear on bf16 activations.
  *   X [M, K] bf16; flags / eps / s_in / s_out as in fpt_act_quant (FPT_SILU_MUL not allowed);
  *   post_mode selects c_t (see FPT_POST_*); post [M] only for FPT_POST_VECTOR.
- *   workspace: fpt_workspace_bytes(FPT_OP_LINEAR, M, N, K) bytes (packed activations,
- *   the per-token vectors and the status word live there).
+ *   workspace: fpt_workspace_bytes(FPT_OP_LINEAR, M, N, K) bytes (activation codes, the per-token vectors and the
+ *   status word live there).  With more than 64 tokens that is room for codes of one byte each where a faster kernel
+ *   takes them; a workspace that holds them packed (M * K / 2 bytes less) is accepted too, with the same results.
  * act_qp->bits == 8 (symmetric grid only): int8 codes q = clamp(rne((x * p) * (1/D)), -128, 127) and
  *   the matmul of fpt_w4a8_gemm; workspace: fpt_workspace_bytes(FPT_OP_LINEAR_A8, M, N, K) bytes.
  */
@@ -274,7 +275,7 @@ int fpt_w4a4_linear_dynamic(void* stream, const void* X, int M, int K,
  * performs no device allocation or free of any kind.
  *
  * Arguments as fpt_w4a4_linear, minus workspace / workspace_bytes.
- * Limit: fpt_workspace_bytes(FPT_OP_LINEAR, M, N, K) <= FPT_STATIC_SCRATCH_BYTES (about
+ * Limit: the workspace of fpt_w4a4_linear with packed codes fits FPT_STATIC_SCRATCH_BYTES (about
  * M*K/2 + 4*M + 8 KiB, plus up to 10 MiB of matmul scratch when M <= 64), otherwise
  * FPT_ERR_WORKSPACE is returned and nothing is enqueued (e.g. 4096 tokens x 8192 features fit).
  * First call on a device: looks up the array's device address (cudaGetSymbolAddress, with that
@@ -309,6 +310,8 @@ int fpt_w4a4_linear_static(void* stream, const void* X, int M, int K,
  *   uses one: none with more than 128 tokens and no transform (the gate||up matmul quantises the
  *   products itself), the products [M, d_ff] with the transform, gate||up [M, 2 d_ff] up to 128 tokens
  *   (reserved, not used, at up to 16 tokens without the transform).
+ *   With more than 128 tokens Y may hold activation codes before it holds the result (unless it overlaps X, which is
+ *   allowed).
  */
 int fpt_decoder_mlp(void* stream, const void* X, int M, int d, int d_ff,
                     const uint8_t* Wgu_q, const void* sw_gu, const uint8_t* Wd_q, const void* sw_d,

@@ -21,7 +21,14 @@ struct ActQuantParams {
   float inv_delta;     // 1 / D, rounded once on the host
   int   qmax_minus_z;  // upper end of the grid minus the zero point
   uint32_t flip;       // see quant_word
+  int wide;            // codes leave widened, one byte each (see widen_word)
 };
+
+// Word i (8 codes) of the output.
+__device__ __forceinline__ void store_codes(const ActQuantParams& P, size_t i, uint32_t w) {
+  if (P.wide) reinterpret_cast<uint2*>(P.Xq)[i] = widen_word(w);
+  else P.Xq[i] = w;
+}
 
 // RMSNorm: T threads per token, up to V 16-byte chunks (8 elements) per thread held in registers.
 template <int T, int V>
@@ -87,12 +94,12 @@ __global__ void __launch_bounds__(T, V <= 4 ? 2048 / T : 1) act_quant_kernel(con
     if (P.post_inv) P.post_inv[t] = __fdiv_rn(1.0f, p);
     if (P.r_out) P.r_out[t] = r;
   }
-  uint32_t* out = P.Xq + (size_t)t * (size_t)chunks;
+  const size_t out = (size_t)t * (size_t)chunks;
   const QuantConsts qc = quant_consts(p, P.inv_delta, P.qmax_minus_z, P.flip);
 #pragma unroll
   for (int i = 0; i < V; ++i) {
     const int c = i * T + tid;
-    if (c < chunks) out[c] = quant_word(v[i], qc);
+    if (c < chunks) store_codes(P, out + c, quant_word(v[i], qc));
   }
 }
 
@@ -136,7 +143,7 @@ __global__ void __launch_bounds__(T, 2048 / T) act_quant_flat_kernel(const ActQu
         v[u] = make_uint4(silu_mul_pair(v[u].x, v2[u].x), silu_mul_pair(v[u].y, v2[u].y), silu_mul_pair(v[u].z, v2[u].z),
                           silu_mul_pair(v[u].w, v2[u].w));
       const float p = (P.flags & FPT_SCALE_INPUT) ? s[u] : 1.0f;
-      P.Xq[i] = quant_word(v[u], quant_consts(p, P.inv_delta, P.qmax_minus_z, P.flip));
+      store_codes(P, i, quant_word(v[u], quant_consts(p, P.inv_delta, P.qmax_minus_z, P.flip)));
     }
   }
 }
@@ -157,7 +164,7 @@ static cudaError_t launch_flat(ActQuantParams P, cudaStream_t st) {
     const size_t n = (size_t)P.M;
     P.X += n * (size_t)(P.ldx >> 3);
     if (P.X2) P.X2 += n * (size_t)(P.ldx >> 3);
-    P.Xq += n * chunks;
+    P.Xq += n * chunks * (P.wide ? 2 : 1);
     if (P.s_in) P.s_in += n;
     if (P.s_out) P.s_out += n;
     if (P.post_inv) P.post_inv += n;
@@ -215,12 +222,12 @@ __global__ void __launch_bounds__(W * 32) act_quant_warp_kernel(const ActQuantPa
     if (P.post_inv) P.post_inv[t] = __fdiv_rn(1.0f, p);
     if (P.r_out) P.r_out[t] = r;
   }
-  uint32_t* out = P.Xq + (size_t)t * (size_t)chunks;
+  const size_t out = (size_t)t * (size_t)chunks;
   const QuantConsts qc = quant_consts(p, P.inv_delta, P.qmax_minus_z, P.flip);
 #pragma unroll
   for (int i = 0; i < V; ++i) {
     const int c = i * 32 + lane;
-    if (c < chunks) out[c] = quant_word(v[i], qc);
+    if (c < chunks) store_codes(P, out + c, quant_word(v[i], qc));
   }
 }
 
@@ -293,10 +300,10 @@ __global__ void __launch_bounds__(1024) act_quant_stream_kernel(const ActQuantPa
       if (P.post_inv) P.post_inv[t] = __fdiv_rn(1.0f, p);
       if (P.r_out) P.r_out[t] = r;
     }
-    uint32_t* out = P.Xq + (size_t)t * (size_t)chunks;
+    const size_t out = (size_t)t * (size_t)chunks;
     const QuantConsts qc = quant_consts(p, P.inv_delta, P.qmax_minus_z, P.flip);
 #pragma unroll 4
-    for (int c = lane; c < chunks; c += 32) out[c] = quant_word(row[c], qc);
+    for (int c = lane; c < chunks; c += 32) store_codes(P, out + c, quant_word(row[c], qc));
     __syncwarp();                                  // every lane is done with the buffer
     const long long tn = t + NB * stride;
     if (lane == 0 && tn < P.M) {
@@ -346,8 +353,9 @@ static cudaError_t launch(const ActQuantParams& P, cudaStream_t st) {
 // composed calls).  All arguments already validated.
 cudaError_t act_quant_launch(cudaStream_t st, const void* X, int M, int K, int ldx, const fpt_qparams* qp,
                              int flags, float eps, const void* X2, const float* s_in, uint8_t* Xq,
-                             float* s_out, float* post_inv, float* r_out) {
+                             float* s_out, float* post_inv, float* r_out, int wide) {
   ActQuantParams P;
+  P.wide = wide;
   P.X = reinterpret_cast<const uint4*>(X);
   P.X2 = reinterpret_cast<const uint4*>(X2);
   P.s_in = s_in;
@@ -414,7 +422,7 @@ extern "C" int fpt_act_quant(void* stream, const void* X, int M, int K, int ldx,
     if (K % 32 != 0 || K > 65536) return FPT_ERR_UNSUPPORTED;
     if (ldx < K || ldx % 8 != 0 || (((uintptr_t)X | (uintptr_t)Xq) & 15)) return FPT_ERR_ALIGNMENT;
     cudaError_t e8 = fpt::act_quant_dyn_launch((cudaStream_t)stream, X, M, K, ldx, 8, 0, qp->scale, flags, eps, s_in,
-                                               FPT_POST_NONE, nullptr, Xq, s_out, nullptr, nullptr, nullptr);
+                                               FPT_POST_NONE, nullptr, Xq, s_out, nullptr, nullptr, nullptr, 0);
     return e8 == cudaSuccess ? FPT_OK : FPT_ERR_CUDA;
   }
   if (qp->bits != 4) return FPT_ERR_UNSUPPORTED;
@@ -432,6 +440,6 @@ extern "C" int fpt_act_quant(void* stream, const void* X, int M, int K, int ldx,
   if (ldx < need_ld || ldx % 8 != 0) return FPT_ERR_ALIGNMENT;
   if (((uintptr_t)X | (uintptr_t)Xq | (uintptr_t)X2) & 15) return FPT_ERR_ALIGNMENT;
   cudaError_t e = fpt::act_quant_launch((cudaStream_t)stream, X, M, K, ldx, qp, flags, eps, X2, s_in, Xq,
-                                        s_out, nullptr, nullptr);
+                                        s_out, nullptr, nullptr, 0);
   return e == cudaSuccess ? FPT_OK : FPT_ERR_CUDA;
 }

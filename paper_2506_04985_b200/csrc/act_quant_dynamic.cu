@@ -24,6 +24,7 @@ struct DynQuantParams {
   int flags, post_mode, dynamic;
   float eps;
   float inv_delta;       // static: 1 / D rounded once on the host
+  int wide;              // 4-bit codes leave widened, one byte each (see widen_word)
 };
 
 // Largest bf16 magnitude pattern of a chunk, per 16-bit half (patterns order like magnitudes; Inf and
@@ -147,7 +148,11 @@ __global__ void __launch_bounds__(T, V <= 4 ? 2048 / T : 1) act_quant_dyn_kernel
 #pragma unroll
     for (int i = 0; i < V; ++i) {
       const int c = i * T + tid;
-      if (c < chunks) out[c] = quant_word(v[i], qc);
+      if (c < chunks) {
+        const uint32_t w = quant_word(v[i], qc);
+        if (P.wide) reinterpret_cast<uint2*>(P.Xq)[(size_t)t * (size_t)chunks + c] = widen_word(w);
+        else out[c] = w;
+      }
     }
   } else {
     uint2* out = reinterpret_cast<uint2*>(P.Xq) + (size_t)t * (size_t)chunks;
@@ -170,8 +175,9 @@ static cudaError_t launch(const DynQuantParams& P, int bits, cudaStream_t st) {
 cudaError_t act_quant_dyn_launch(cudaStream_t st, const void* X, int M, int K, int ldx, int bits, int dynamic,
                                  float qp_scale, int flags, float eps, const float* s_in, int post_mode,
                                  const float* post, void* Xq, float* s_out, float* c_out, float* delta_out,
-                                 float* r_out) {
+                                 float* r_out, int wide) {
   DynQuantParams P;
+  P.wide = wide;
   P.X = reinterpret_cast<const uint4*>(X);
   P.s_in = s_in; P.post = post; P.Xq = Xq;
   P.s_out = s_out; P.c_out = c_out; P.delta_out = delta_out; P.r_out = r_out;
@@ -202,6 +208,6 @@ extern "C" int fpt_act_quant_dynamic(void* stream, const void* X, int M, int K, 
   if (ldx < K || ldx % 8 != 0) return FPT_ERR_ALIGNMENT;
   if (((uintptr_t)X | (uintptr_t)Xq) & 15) return FPT_ERR_ALIGNMENT;
   cudaError_t e = fpt::act_quant_dyn_launch((cudaStream_t)stream, X, M, K, ldx, bits, 1, 1.0f, flags, eps, s_in,
-                                            FPT_POST_NONE, nullptr, Xq, s_out, nullptr, delta_out, nullptr);
+                                            FPT_POST_NONE, nullptr, Xq, s_out, nullptr, delta_out, nullptr, 0);
   return e == cudaSuccess ? FPT_OK : FPT_ERR_CUDA;
 }

@@ -36,6 +36,15 @@ static int check_scales(const void* sw, int scale_dtype, const int32_t* wsum) {
   return (((uintptr_t)sw | (uintptr_t)wsum) & 15) ? FPT_ERR_ALIGNMENT : FPT_OK;
 }
 
+size_t linear4_bytes(int M, int N, int K, int wide) {
+  const size_t m = (size_t)M;
+  return kStatusBytes + gemm_scratch_bytes(M) + up256(m * (size_t)K / (wide ? 1 : 2)) + up256(m * 4);
+}
+// Whether the codes of a linear leave widened: the kernel that takes them serves the shape, and there is room for them.
+static int linear4_wide(int M, int N, int K, size_t workspace_bytes) {
+  return gemm_wt_serves(M, N, K) && workspace_bytes >= linear4_bytes(M, N, K, 1);
+}
+
 static int g_programmatic_launch = 1;
 int programmatic_launch_enabled() { return g_programmatic_launch; }
 
@@ -61,12 +70,12 @@ int linear4_check(const void* X, const uint8_t* Wq, const void* sw, int scale_dt
 
 int linear4_run(cudaStream_t st, const void* X, int M, int K, const uint8_t* Wq, const void* sw, int scale_dtype,
                 const int32_t* wsum, int N, const fpt_qparams* act_qp, int flags, float eps, const float* s_in,
-                int post_mode, const float* post, void* Y, float* s_out, uint8_t* ws) {
+                int post_mode, const float* post, void* Y, float* s_out, uint8_t* ws, int wide) {
   const size_t gemm_ws = kStatusBytes + gemm_scratch_bytes(M);      // control block + matmul scratch
   uint8_t* Xq = ws + gemm_ws;
-  float* post_inv = reinterpret_cast<float*>(Xq + up256((size_t)M * K / 2));
+  float* post_inv = reinterpret_cast<float*>(Xq + up256((size_t)M * K / (wide ? 1 : 2)));
   if (act_quant_launch(st, X, M, K, K, act_qp, flags, eps, nullptr, s_in, Xq, s_out,
-                       post_mode == FPT_POST_INVERSE_OF_PRE ? post_inv : nullptr, nullptr) != cudaSuccess)
+                       post_mode == FPT_POST_INVERSE_OF_PRE ? post_inv : nullptr, nullptr, wide) != cudaSuccess)
     return FPT_ERR_CUDA;
   GemmParams P{};
   P.M = M; P.N = N; P.K = K;
@@ -80,7 +89,7 @@ int linear4_run(cudaStream_t st, const void* X, int M, int K, const uint8_t* Wq,
   P.status = reinterpret_cast<uint32_t*>(ws);
   P.scratch = ws + kStatusBytes;
   P.early_weights = 1;                                              // act_quant is in front
-  return gemm_launch(st, Xq, Wq, P);
+  return wide ? gemm_wt_launch(st, reinterpret_cast<const int8_t*>(Xq), Wq, P) : gemm_launch(st, Xq, Wq, P);
 }
 
 }  // namespace fpt
@@ -115,7 +124,7 @@ extern "C" size_t fpt_workspace_bytes(int op, int M, int N, int K) {
     case FPT_OP_GEMM:
       return kStatusBytes + gemm_scratch_bytes(M);
     case FPT_OP_LINEAR:
-      return kStatusBytes + gemm_scratch_bytes(M) + up256(m * (size_t)K / 2) + up256(m * 4);
+      return linear4_bytes(M, N, K, gemm_wt_serves(M, N, K));
     case FPT_OP_GEMM_A8:
       return kStatusBytes + gemm_scratch_bytes(M) + gemm_a8_scratch_bytes(M, N, K);
     case FPT_OP_LINEAR_A8:
@@ -145,11 +154,12 @@ extern "C" int fpt_check_status(void* stream, void* workspace) {
   return word == 0 ? FPT_OK : FPT_ERR_TIMEOUT;
 }
 
-// fpt_w4a4_gemm; `early`: see GemmParams::early_weights (only the composed calls below can say so).
+// fpt_w4a4_gemm; `early`: see GemmParams::early_weights, `wide`: the codes are widened, [M, K] bytes (only the composed
+// calls below can say so).
 static int gemm4(void* stream, const uint8_t* Xq, const uint8_t* Wq, int M, int N, int K, const void* sw, int scale_dtype,
                  const int32_t* wsum, float act_scale, int act_symmetric, int act_zero_point, const float* post,
                  const void* residual, const float* res_scale, void* Y, int32_t* acc_out, void* workspace,
-                 size_t workspace_bytes, int early) {
+                 size_t workspace_bytes, int early, int wide) {
   if (!Xq || !Wq || !sw || (!Y && !acc_out)) return FPT_ERR_BAD_ARG;
   int rc = check_gemm_shape(M, N, K);
   if (rc) return rc;
@@ -175,7 +185,8 @@ static int gemm4(void* stream, const uint8_t* Xq, const uint8_t* Wq, int M, int 
   P.status = reinterpret_cast<uint32_t*>(workspace);
   P.scratch = reinterpret_cast<uint8_t*>(workspace) + kStatusBytes;
   P.early_weights = early;
-  return gemm_launch((cudaStream_t)stream, Xq, Wq, P);
+  return wide ? gemm_wt_launch((cudaStream_t)stream, reinterpret_cast<const int8_t*>(Xq), Wq, P)
+              : gemm_launch((cudaStream_t)stream, Xq, Wq, P);
 }
 
 extern "C" int fpt_w4a4_gemm(void* stream, const uint8_t* Xq, const uint8_t* Wq, int M, int N, int K, const void* sw,
@@ -183,7 +194,7 @@ extern "C" int fpt_w4a4_gemm(void* stream, const uint8_t* Xq, const uint8_t* Wq,
                              int act_zero_point, const float* post, const void* residual, const float* res_scale,
                              void* Y, int32_t* acc_out, void* workspace, size_t workspace_bytes) {
   return gemm4(stream, Xq, Wq, M, N, K, sw, scale_dtype, wsum, act_scale, act_symmetric, act_zero_point, post, residual,
-               res_scale, Y, acc_out, workspace, workspace_bytes, 0);
+               res_scale, Y, acc_out, workspace, workspace_bytes, 0, 0);
 }
 
 extern "C" int fpt_w4a4_linear(void* stream, const void* X, int M, int K, const uint8_t* Wq, const void* sw,
@@ -211,7 +222,7 @@ extern "C" int fpt_w4a4_linear(void* stream, const void* X, int M, int K, const 
     float* pinv = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(Xq8) + up256((size_t)M * K));
     if (act_quant_dyn_launch((cudaStream_t)stream, X, M, K, K, 8, 0, act_qp->scale, flags, eps, s_in, post_mode, post,
                              Xq8, s_out, post_mode == FPT_POST_INVERSE_OF_PRE ? pinv : nullptr, nullptr,
-                             nullptr) != cudaSuccess)
+                             nullptr, 0) != cudaSuccess)
       return FPT_ERR_CUDA;
     const float* pv8 = post_mode == FPT_POST_NONE ? nullptr : post_mode == FPT_POST_VECTOR ? post : pinv;
     return fpt_w4a8_gemm(stream, Xq8, Wq, M, N, K, sw, scale_dtype, act_qp->scale, pv8, nullptr, nullptr, Y, nullptr,
@@ -220,9 +231,9 @@ extern "C" int fpt_w4a4_linear(void* stream, const void* X, int M, int K, const 
   rc = linear4_check(X, Wq, sw, scale_dtype, wsum, Y, act_qp, M, N, K, flags, s_in, post_mode, post);
   if (rc) return rc;
   if ((uintptr_t)workspace & 15) return FPT_ERR_ALIGNMENT;
-  if (!workspace || workspace_bytes < fpt_workspace_bytes(FPT_OP_LINEAR, M, N, K)) return FPT_ERR_WORKSPACE;
+  if (!workspace || workspace_bytes < linear4_bytes(M, N, K, 0)) return FPT_ERR_WORKSPACE;
   return linear4_run((cudaStream_t)stream, X, M, K, Wq, sw, scale_dtype, wsum, N, act_qp, flags, eps, s_in, post_mode,
-                     post, Y, s_out, reinterpret_cast<uint8_t*>(workspace));
+                     post, Y, s_out, reinterpret_cast<uint8_t*>(workspace), linear4_wide(M, N, K, workspace_bytes));
 }
 
 extern "C" int fpt_decoder_mlp(void* stream, const void* X, int M, int d, int d_ff, const uint8_t* Wgu_q,
@@ -259,11 +270,24 @@ extern "C" int fpt_decoder_mlp(void* stream, const void* X, int M, int d, int d_
   uint8_t* Mq = GU + up256(mlp_gu_bytes(M, d_ff, mid_hadamard != 0));
   float* sn = s_out ? s_out : sn_ws;
   cudaStream_t st = (cudaStream_t)stream;
+  // Where the codes can leave widened, one byte each.  17 .. 128 tokens: the buffer between the matmuls, which the fused
+  // epilogue leaves free, holds those of the block's input and, from 65 tokens on, of the products (the kernel that streams
+  // the down projection for fewer takes packed codes).  More: Y, which nothing is written to before the down projection,
+  // holds those of the block's input, unless it is X, which the residual still needs; the products stay packed.
+  const uintptr_t xa = (uintptr_t)X, ya = (uintptr_t)Y, xy = (uintptr_t)(m * (size_t)d * 2);
+  const bool apart = xa + xy <= ya || ya + xy <= xa;
+  // (32 tokens or fewer of a block that is not large stream faster through the weight-streaming kernel: 17 x 2560x6912 26.3
+  // against 27.6 us, 17 x 4096x14336 36.6 against 33.5, 37 x 2560x6912 32.1 / 33.2, 64 x 2560x6912 37.1 / 35.9)
+  const int wide = M <= 16 || (M <= 48 && (long long)d * d_ff < (32ll << 20)) ? 0
+                   : M > 128 ? apart && gemm_wt_serves(M, 2 * d_ff, d) : !mid_hadamard && up256(m * (size_t)d_ff) + m * (size_t)d <= mlp_gu_bytes(M, d_ff, false);
+  const int wide_mid = wide && M <= 128 && gemm_wt_serves(M, d, d_ff);
+  if (wide) Xq = M <= 128 ? GU + up256(m * (size_t)d_ff) : reinterpret_cast<uint8_t*>(Y);
+  if (wide_mid) Mq = GU;
 
   // X~ = RMSNorm(X) on the grid qp_in; S_n = S_{n-1} * r
-  if (act_quant_launch(st, X, M, d, d, qp_in, FPT_RMSNORM, eps, nullptr, s_prev, Xq, sn, nullptr, r_ws) != cudaSuccess)
+  if (act_quant_launch(st, X, M, d, d, qp_in, FPT_RMSNORM, eps, nullptr, s_prev, Xq, sn, nullptr, r_ws, wide) != cudaSuccess)
     return FPT_ERR_CUDA;
-  if (M > 128 || (M <= 16 && !mid_hadamard)) {
+  if (M > 128 || wide || (M <= 16 && !mid_hadamard)) {
     // gate || up in one matmul whose epilogue forms m = bf16(silu(g) * u) and quantises m * S_n:
     // the static grid and S_n are known before the matmul starts, so g and u never reach memory
     GemmParams P{};
@@ -274,36 +298,37 @@ extern "C" int fpt_decoder_mlp(void* stream, const void* X, int M, int d, int d_
       P.swiglu_bf16 = 1;
       P.Y = reinterpret_cast<__nv_bfloat16*>(GU);
     } else {
-      P.Mq = Mq; P.mid_scale = sn;
+      P.Mq = Mq; P.mid_scale = sn; P.mq_wide = wide_mid;
       P.mid_inv_delta = 1.0f / qp_mid->scale;
       P.mid_qmax_minus_z = 7; P.mid_flip = 0x77777777u;
     }
     P.status = reinterpret_cast<uint32_t*>(workspace);
     P.scratch = ws + kStatusBytes;
     P.early_weights = 1;
-    rc = M > 128 ? gemm_pair_launch(st, Xq, Wgu_q, P) : gemm_decode_small_launch(st, Xq, Wgu_q, P);
+    rc = wide ? gemm_wt_launch(st, reinterpret_cast<const int8_t*>(Xq), Wgu_q, P)
+         : M > 128 ? gemm_pair_launch(st, Xq, Wgu_q, P) : gemm_decode_small_launch(st, Xq, Wgu_q, P);
     if (rc) return rc;
     if (mid_hadamard &&
         hadamard_quant_launch(st, GU, M, d_ff, d_ff, qp_mid, 0, sn, Mq) != cudaSuccess)
       return FPT_ERR_CUDA;
   } else if (mid_hadamard) {
     rc = gemm4(stream, Xq, Wgu_q, M, 2 * d_ff, d, sw_gu, scale_dtype, nullptr, qp_in->scale, 1, 0, nullptr,
-               nullptr, nullptr, GU, nullptr, workspace, gemm_ws, 1);
+               nullptr, nullptr, GU, nullptr, workspace, gemm_ws, 1, 0);
     if (rc) return rc;
     if (hadamard_quant_launch(st, GU, M, d_ff, 2 * d_ff, qp_mid, 1, sn, Mq) != cudaSuccess) return FPT_ERR_CUDA;
   } else {
     // gate || up in one matmul over the interleaved weight
     rc = gemm4(stream, Xq, Wgu_q, M, 2 * d_ff, d, sw_gu, scale_dtype, nullptr, qp_in->scale, 1, 0, nullptr,
-               nullptr, nullptr, GU, nullptr, workspace, gemm_ws, 1);
+               nullptr, nullptr, GU, nullptr, workspace, gemm_ws, 1, 0);
     if (rc) return rc;
     // m = bf16(silu(g) * u), quantised after the multiply by S_n
     if (act_quant_launch(st, GU, M, d_ff, 2 * d_ff, qp_mid, FPT_SILU_MUL | FPT_GU_INTERLEAVED | FPT_SCALE_INPUT, 0.0f,
-                         nullptr, sn, Mq, nullptr, nullptr, nullptr) != cudaSuccess)
+                         nullptr, sn, Mq, nullptr, nullptr, nullptr, 0) != cudaSuccess)
       return FPT_ERR_CUDA;
   }
   // down projection; the normalised residual X * r joins before the final rounding
   return gemm4(stream, Mq, Wd_q, M, d, d_ff, sw_d, scale_dtype, nullptr, qp_mid->scale, 1, 0, nullptr,
-               add_residual ? X : nullptr, add_residual ? r_ws : nullptr, Y, nullptr, workspace, gemm_ws, 1);
+               add_residual ? X : nullptr, add_residual ? r_ws : nullptr, Y, nullptr, workspace, gemm_ws, 1, wide_mid);
 }
 
 extern "C" int fpt_decoder_attn_qkv(void* stream, const void* X, int M, int d, const uint8_t* Wqkv_q, const void* sw_qkv,
@@ -317,17 +342,18 @@ extern "C" int fpt_decoder_attn_qkv(void* stream, const void* X, int M, int d, c
   if (rc) return rc;
   if (!qp_in->symmetric && !wsum_qkv) return FPT_ERR_BAD_ARG;
   if (((uintptr_t)X | (uintptr_t)Wqkv_q | (uintptr_t)QKV | (uintptr_t)workspace) & 15) return FPT_ERR_ALIGNMENT;
-  if (!workspace || workspace_bytes < fpt_workspace_bytes(FPT_OP_LINEAR, M, n_qkv, d)) return FPT_ERR_WORKSPACE;
+  if (!workspace || workspace_bytes < linear4_bytes(M, n_qkv, d, 0)) return FPT_ERR_WORKSPACE;
   rc = check_scales(sw_qkv, scale_dtype, wsum_qkv);
   if (rc) return rc;
   const size_t gemm_ws = kStatusBytes + gemm_scratch_bytes(M);
   uint8_t* Xq = reinterpret_cast<uint8_t*>(workspace) + gemm_ws;
+  const int wide = linear4_wide(M, n_qkv, d, workspace_bytes);
   // X~ = RMSNorm(X) on the grid qp_in; S_n = S_{n-1} * r; r kept for the residual
   if (act_quant_launch((cudaStream_t)stream, X, M, d, d, qp_in, FPT_RMSNORM, eps, nullptr, s_prev, Xq, s_out, nullptr,
-                       r_out) != cudaSuccess)
+                       r_out, wide) != cudaSuccess)
     return FPT_ERR_CUDA;
   return gemm4(stream, Xq, Wqkv_q, M, n_qkv, d, sw_qkv, scale_dtype, wsum_qkv, qp_in->scale, qp_in->symmetric,
-               qp_in->zero_point, nullptr, nullptr, nullptr, QKV, nullptr, workspace, gemm_ws, 1);
+               qp_in->zero_point, nullptr, nullptr, nullptr, QKV, nullptr, workspace, gemm_ws, 1, wide);
 }
 
 extern "C" int fpt_decoder_attn_out(void* stream, const void* A, int M, int k_o, const uint8_t* Wo_q, const void* sw_o,
@@ -342,18 +368,19 @@ extern "C" int fpt_decoder_attn_out(void* stream, const void* A, int M, int k_o,
   if (rc) return rc;
   if (!qp_ap->symmetric && !wsum_o) return FPT_ERR_BAD_ARG;
   if (((uintptr_t)A | (uintptr_t)Wo_q | (uintptr_t)Y | (uintptr_t)X | (uintptr_t)workspace) & 15) return FPT_ERR_ALIGNMENT;
-  if (!workspace || workspace_bytes < fpt_workspace_bytes(FPT_OP_LINEAR, M, d, k_o)) return FPT_ERR_WORKSPACE;
+  if (!workspace || workspace_bytes < linear4_bytes(M, d, k_o, 0)) return FPT_ERR_WORKSPACE;
   rc = check_scales(sw_o, scale_dtype, wsum_o);
   if (rc) return rc;
   const size_t gemm_ws = kStatusBytes + gemm_scratch_bytes(M);
   uint8_t* Aq = reinterpret_cast<uint8_t*>(workspace) + gemm_ws;
+  const int wide = linear4_wide(M, d, k_o, workspace_bytes);
   // the sequence scaler at the attention output: the grid sees A * S_n
   if (act_quant_launch((cudaStream_t)stream, A, M, k_o, k_o, qp_ap, FPT_SCALE_INPUT, 0.0f, nullptr, s_n, Aq, nullptr,
-                       nullptr, nullptr) != cudaSuccess)
+                       nullptr, nullptr, wide) != cudaSuccess)
     return FPT_ERR_CUDA;
   // output projection; the normalised residual X * r joins before the final rounding
   return gemm4(stream, Aq, Wo_q, M, d, k_o, sw_o, scale_dtype, wsum_o, qp_ap->scale, qp_ap->symmetric,
-               qp_ap->zero_point, nullptr, X, X ? r : nullptr, Y, nullptr, workspace, gemm_ws, 1);
+               qp_ap->zero_point, nullptr, X, X ? r : nullptr, Y, nullptr, workspace, gemm_ws, 1, wide);
 }
 
 extern "C" int fpt_w4a4_linear_dynamic(void* stream, const void* X, int M, int K, const uint8_t* Wq, const void* sw,
@@ -378,22 +405,23 @@ extern "C" int fpt_w4a4_linear_dynamic(void* stream, const void* X, int M, int K
     int8_t* Xq8 = reinterpret_cast<int8_t*>(workspace) + gemm_ws8;
     float* c8 = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(Xq8) + up256((size_t)M * K));
     if (act_quant_dyn_launch((cudaStream_t)stream, X, M, K, K, 8, 1, 1.0f, flags, eps, s_in, post_mode, post, Xq8, s_out,
-                             c8, nullptr, nullptr) != cudaSuccess)
+                             c8, nullptr, nullptr, 0) != cudaSuccess)
       return FPT_ERR_CUDA;
     return fpt_w4a8_gemm(stream, Xq8, Wq, M, N, K, sw, scale_dtype, 1.0f, c8, nullptr, nullptr, Y, nullptr, workspace,
                          gemm_ws8);
   }
-  if (!workspace || workspace_bytes < fpt_workspace_bytes(FPT_OP_LINEAR, M, N, K)) return FPT_ERR_WORKSPACE;
+  if (!workspace || workspace_bytes < linear4_bytes(M, N, K, 0)) return FPT_ERR_WORKSPACE;
   rc = check_scales(sw, scale_dtype, nullptr);
   if (rc) return rc;
   uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
   const size_t gemm_ws = kStatusBytes + gemm_scratch_bytes(M);
   uint8_t* Xq = ws + gemm_ws;
-  float* c_t = reinterpret_cast<float*>(Xq + up256((size_t)M * K / 2));
+  const int wide = linear4_wide(M, N, K, workspace_bytes);
+  float* c_t = reinterpret_cast<float*>(Xq + up256((size_t)M * K / (wide ? 1 : 2)));
   // per-token grid; the factor the epilogue needs (D_t, times whatever the post mode asks for) per token
   if (act_quant_dyn_launch((cudaStream_t)stream, X, M, K, K, 4, 1, 1.0f, flags, eps, s_in, post_mode, post, Xq, s_out,
-                           c_t, nullptr, nullptr) != cudaSuccess)
+                           c_t, nullptr, nullptr, wide) != cudaSuccess)
     return FPT_ERR_CUDA;
   return gemm4(stream, Xq, Wq, M, N, K, sw, scale_dtype, nullptr, 1.0f, 1, 0, c_t, nullptr, nullptr, Y, nullptr,
-               workspace, gemm_ws, 1);
+               workspace, gemm_ws, 1, wide);
 }

@@ -53,6 +53,10 @@ __device__ __forceinline__ void widen(const uint4& p, uint32_t* out) {
   out[3] = (p.w << 4) & 0xF0F0F0F0u;  out[7] = p.w & 0xF0F0F0F0u;
 }
 
+// The same for one word of eight codes, the even-k codes in front: the form in which the quantisers leave the codes for
+// the kernel that takes one byte a code (gemm_wt_pair.cu).
+__device__ __forceinline__ uint2 widen_word(uint32_t p) { return make_uint2((p << 4) & 0xF0F0F0F0u, p & 0xF0F0F0F0u); }
+
 // ----------------------------------------------------------------------------------
 // PTX wrappers
 // ----------------------------------------------------------------------------------

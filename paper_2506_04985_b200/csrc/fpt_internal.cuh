@@ -9,6 +9,7 @@ namespace fpt {
 struct GemmParams {
   int M, N, K;
   int tiles_m, num_tiles, kblocks;
+  int tn, ksplit;              // gemm_wt_pair.cu: tokens of a tile, CTA pairs that share one
   const void* sw;
   int scale_dtype;
   const int32_t* wsum;
@@ -26,6 +27,7 @@ struct GemmParams {
   // written, and m = bf16(silu(g) * u) is quantised with the per-token multiplier mid_scale[t]
   int swiglu_bf16;             // with Y set and Mq null: Y [M, N/2] receives m itself (bf16), nothing is quantised
   uint8_t* Mq;                 // [M, N/4] packed codes of the N/2 products, or nullptr
+  int mq_wide;                 // ... [M, N/2] widened codes instead (gemm_wt_pair.cu only)
   const float* mid_scale;      // [M] S_n
   float mid_inv_delta;         // 1/D of the grid at the down-projection input
   int mid_qmax_minus_z;
@@ -40,15 +42,16 @@ struct GemmParams {
 // gemm_a8.cu: scratch bytes fpt_w4a8_gemm needs behind the control block and the matmul scratch.
 size_t gemm_a8_scratch_bytes(int M, int N, int K);
 
-// act_quant.cu: validated arguments only; also fills 1/p_t and r_t for the composed calls.
+// act_quant.cu: validated arguments only; also fills 1/p_t and r_t for the composed calls.  wide: the codes leave widened,
+// [M, K] bytes.
 cudaError_t act_quant_launch(cudaStream_t st, const void* X, int M, int K, int ldx, const fpt_qparams* qp,
                              int flags, float eps, const void* X2, const float* s_in, uint8_t* Xq,
-                             float* s_out, float* post_inv, float* r_out);
+                             float* s_out, float* post_inv, float* r_out, int wide);
 // Dynamic (per-token grid) and 8-bit forms of the same step (act_quant_dynamic.cu).
 cudaError_t act_quant_dyn_launch(cudaStream_t st, const void* X, int M, int K, int ldx, int bits, int dynamic,
                                  float qp_scale, int flags, float eps, const float* s_in, int post_mode,
                                  const float* post, void* Xq, float* s_out, float* c_out, float* delta_out,
-                                 float* r_out);
+                                 float* r_out, int wide);
 
 // hadamard_quant.cu: block-wise Hadamard + per-token scale + quantise (validated arguments only).
 int hadamard_block(int K);
@@ -72,6 +75,11 @@ constexpr int kMaxKA8 = 16384;      // 8-bit activation codes: keeps (float)acc 
 // gemm_w4a4_2cta.cu: the CTA-pair kernel (256 x 256 tiles) behind gemm_launch for prefill sizes.
 int gemm_pair_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, const GemmParams& P);
 
+// gemm_wt_pair.cu: the CTA-pair kernel for activation codes of one byte (P.a_bits == 8: 8-bit codes, otherwise 4-bit codes
+// widened by the quantiser).
+int gemm_wt_launch(cudaStream_t st, const int8_t* X8, const uint8_t* Wq, const GemmParams& P);
+bool gemm_wt_serves(int M, int N, int K);   // whether the composed calls should leave widened codes for it
+
 // api.cu: argument checks and body of the 4-bit static linear on a workspace of
 // fpt_workspace_bytes(FPT_OP_LINEAR, M, N, K) bytes whose control block is zero (shared by
 // fpt_w4a4_linear and fpt_w4a4_linear_static).
@@ -80,6 +88,8 @@ int linear4_check(const void* X, const uint8_t* Wq, const void* sw, int scale_dt
                   const float* post);
 int linear4_run(cudaStream_t st, const void* X, int M, int K, const uint8_t* Wq, const void* sw, int scale_dtype,
                 const int32_t* wsum, int N, const fpt_qparams* act_qp, int flags, float eps, const float* s_in,
-                int post_mode, const float* post, void* Y, float* s_out, uint8_t* ws);
+                int post_mode, const float* post, void* Y, float* s_out, uint8_t* ws, int wide);
+// Workspace bytes of the linear with packed or widened codes (FPT_OP_LINEAR asks for the wider, the calls accept either).
+size_t linear4_bytes(int M, int N, int K, int wide);
 
 }  // namespace fpt

@@ -113,7 +113,7 @@ extern "C" int fpt_w4a8_gemm(void* stream, const int8_t* Xq8, const uint8_t* Wq,
     P.residual = reinterpret_cast<const __nv_bfloat16*>(residual); P.res_scale = res_scale;
     P.Y = reinterpret_cast<__nv_bfloat16*>(Y); P.acc_out = acc_out;
     if (M <= 16) return gemm_decode_small_launch(st, reinterpret_cast<const uint8_t*>(Xq8), Wq, P);
-    return gemm_pair_launch(st, reinterpret_cast<const uint8_t*>(Xq8), Wq, P);
+    return gemm_wt_launch(st, Xq8, Wq, P);
   }
   // a = 16 h + l through two 4-bit matmuls
   uint8_t* Hq = ws + kStatusBytes + gemm_scratch_bytes(M);

@@ -52,7 +52,8 @@ extern "C" int fpt_w4a4_linear_static(void* stream, const void* X, int M, int K,
   int rc = linear4_check(X, Wq, sw, scale_dtype, wsum, Y, act_qp, M, N, K, flags, s_in, post_mode, post);
   if (rc) return rc;
   // the same carving as fpt_w4a4_linear's workspace, inside the built-in array
-  if (fpt_workspace_bytes(FPT_OP_LINEAR, M, N, K) > kStaticScratchBytes) return FPT_ERR_WORKSPACE;
+  if (linear4_bytes(M, N, K, 0) > kStaticScratchBytes) return FPT_ERR_WORKSPACE;
+  const int wide = gemm_wt_serves(M, N, K) && linear4_bytes(M, N, K, 1) <= kStaticScratchBytes;
 
   unsigned char* base = nullptr;
   rc = static_scratch(&base);
@@ -61,5 +62,6 @@ extern "C" int fpt_w4a4_linear_static(void* stream, const void* X, int M, int K,
   // the array keeps whatever the last call left: the control block (status word, tile counters)
   // has to start at zero
   if (cudaMemsetAsync(base, 0, kStatusBytes, st) != cudaSuccess) return FPT_ERR_CUDA;
-  return linear4_run(st, X, M, K, Wq, sw, scale_dtype, wsum, N, act_qp, flags, eps, s_in, post_mode, post, Y, s_out, base);
+  return linear4_run(st, X, M, K, Wq, sw, scale_dtype, wsum, N, act_qp, flags, eps, s_in, post_mode, post, Y, s_out, base,
+                     wide);
 }

@@ -255,3 +255,43 @@ def test_decoder_attention_projections_parity(M, d, n_q, n_kv, with_prev, residu
                                ref1["r"] if residual else None)
     assert len(np.unique(ref2["aq"])) >= 6
     assert assert_bf16_close(bf16_host(Y), ref2["y"], "attn Y") == 0
+
+
+@pytest.mark.parametrize("M", [65, 96, 97, 129, 161, 250, 333, 900])     # tokens of a tile: 32 .. 256, the last one ragged
+@pytest.mark.parametrize("K,N", [(128, 264), (384, 1032), (1024, 4096), (4224, 520)])     # half a weight stage, odd k-blocks, two pairs a tile
+@pytest.mark.parametrize("sym", [True, False])
+def test_linear_with_widened_codes_equals_the_one_with_packed_codes(M, K, N, sym):
+    """A workspace of FPT_OP_LINEAR bytes has room for widened codes, one without that room takes the packed route: the same
+    exact integers, so the same bits.  Guard bands around every buffer (helpers) catch a store outside."""
+    g = torch.Generator(device="cuda").manual_seed(M + K + N)
+    x = torch.randn((M, K), device="cuda", generator=g).to(torch.bfloat16)
+    w = torch.randint(0, 256, (N, K // 2), device="cuda", generator=g, dtype=torch.uint8)
+    sw = (torch.rand((N,), device="cuda", generator=g) + 0.5).to(torch.float16)
+    codes = torch.stack(((w.view(torch.int8) << 4) >> 4, w.view(torch.int8) >> 4), 2)
+    wsum = codes.sum((1, 2), dtype=torch.int32)
+    qp = B.QParams(4, sym, 0.4, 0 if sym else 7)
+    wide = B.new_workspace(B.OP_LINEAR, M, N, K)
+    packed = 8192 + (M * K // 2 + 255) // 256 * 256 + (M * 4 + 255) // 256 * 256
+    assert wide.numel() > packed
+    out = []
+    for ws in (wide, wide[:packed].clone()):
+        assert B.lib().fpt_reset_status(B._stream(), B._ptr(ws)) == B.OK
+        out.append(B.fpt_w4a4_linear(x, w, sw, qp, B.RMSNORM, 1e-5, post_mode=B.POST_INVERSE_OF_PRE, wsum=wsum, ws=ws))
+        assert B.fpt_check_status(ws) == B.OK
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("M", [49, 64, 65, 100, 129, 300])
+def test_mlp_block_that_writes_over_its_input_equals_the_one_that_does_not(M):
+    """With Y apart from X the codes of the input may lie in Y until the down projection; with Y = X they may not."""
+    d, dff = 512, 1152
+    g = torch.Generator(device="cuda").manual_seed(M)
+    x = torch.randn((M, d), device="cuda", generator=g).to(torch.bfloat16)
+    wgu = torch.randint(0, 256, (2 * dff, d // 2), device="cuda", generator=g, dtype=torch.uint8)
+    wd = torch.randint(0, 256, (d, dff // 2), device="cuda", generator=g, dtype=torch.uint8)
+    sg, sd = torch.rand((2 * dff,), device="cuda", generator=g) * 0.02, torch.rand((d,), device="cuda", generator=g) * 0.02
+    qi, qm = B.QParams(4, True, 0.4, 0), B.QParams(4, True, 0.3, 0)
+    y, s = B.fpt_decoder_mlp(x, wgu, sg, wd, sd, qi, qm, 1e-5, None, True)
+    over = x.clone()
+    y2, s2 = B.fpt_decoder_mlp(over, wgu, sg, wd, sd, qi, qm, 1e-5, None, True, Y=over)
+    assert torch.equal(y, y2) and torch.equal(s, s2)
