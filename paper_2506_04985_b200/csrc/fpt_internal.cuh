@@ -15,7 +15,7 @@ struct GemmParams {
   const int32_t* wsum;
   int zero_point;              // 0 when the activation grid is symmetric
   int a_unsigned;              // activation codes are unsigned nibbles (asymmetric grid)
-  int a_bits;                  // 8: the activation operand is int8 [M, K] (CTA-pair kernel only); otherwise packed 4-bit
+  int a_bits;                  // 8: the activation operand is int8 [M, K] (gemm_wt_pair.cu, gemm_decode_small.cu); otherwise 4-bit
   float act_scale;
   const float* post;
   const __nv_bfloat16* residual;
@@ -72,7 +72,7 @@ int gemm_decode_small_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* 
 
 constexpr int kMaxKA8 = 16384;      // 8-bit activation codes: keeps (float)acc exact, |acc| <= 1024 K <= 2^24
 
-// gemm_w4a4_2cta.cu: the CTA-pair kernel (256 x 256 tiles) behind gemm_launch for prefill sizes.
+// gemm_w4a4_2cta.cu: the CTA-pair kernel (256 x 256 tiles) for packed codes, behind gemm_launch for prefill sizes.
 int gemm_pair_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, const GemmParams& P);
 
 // gemm_wt_pair.cu: the CTA-pair kernel for activation codes of one byte (P.a_bits == 8: 8-bit codes, otherwise 4-bit codes

@@ -25,8 +25,8 @@
 //                 accumulator is released as soon as it has been read, the tile leaves by TMA store;
 //                 a residual tile is fetched by TMA into the same slabs while the tile's matmul runs
 // Both operands are widened as code*16 (see gemm_w4a4.cu), so the accumulator holds 256 * sum.
-// Variants (template parameters): the two fused SwiGLU epilogues, int8 activation codes (the
-// activation tile then needs no widening and the shift is 4), output tiles of 208..256 columns.
+// Variants (template parameters): the two fused SwiGLU epilogues, output tiles of 208..256 columns.
+// (Activation codes of one byte: gemm_wt_pair.cu.)
 #include <cuda.h>
 
 #include "fpt_internal.cuh"
@@ -56,9 +56,7 @@ static_assert(128 * (kRegsCtl + kGroups * kRegsConv) + 32 * kEpiWarps * kRegsEpi
 
 // NS: stages of widened operands (int8 weight tile in shared memory + activation columns in
 // tensor memory); NPK: stages of packed tiles in flight from TMA.
-// kA8: the activation operand arrives as int8 codes (one byte each, 128-byte rows per k-block)
-// instead of packed 4-bit codes.
-template <int NS, int NPK, bool kA8 = false>
+template <int NS, int NPK>
 struct Smem {
   // A barrier's wait tells one phase from the next by its parity only, so whoever waits for a phase must know that the
   // one before it is over: the stage of a group's k-block was last used by a k-block of the same group.  (With five
@@ -66,11 +64,10 @@ struct Smem {
   static_assert(NS % kGroups == 0 && NPK % kGroups == 0, "a stage must belong to one converter group");
   static_assert(kAccCols + NS * kAStageCols <= kTmemCols, "operand stages must fit beside the accumulator");
   static constexpr int kB8Stage = HR * I8_ROW;                      // 16 KB
-  static constexpr int kPkOp = HR * PK_ROW;                         // 8 KB: a packed weight tile
-  static constexpr int kPkOpA = kA8 ? HR * I8_ROW : HR * PK_ROW;    // the activation tile of a stage
+  static constexpr int kPkOp = HR * PK_ROW;                         // 8 KB: a packed tile of either operand
   static constexpr int kB8Off = 0;
   static constexpr int kPkAOff = kB8Off + NS * kB8Stage;
-  static constexpr int kPkBOff = kPkAOff + NPK * kPkOpA;
+  static constexpr int kPkBOff = kPkAOff + NPK * kPkOp;
   static constexpr int kStgOff = kPkBOff + NPK * kPkOp;             // bf16 output tile: 4 slabs of 128 rows x 64 columns
   static constexpr int kStgSlab = HR * 128;                         // 16 KB, 128-byte rows, 128-byte swizzle
   static constexpr int kScaleOff = kStgOff + 4 * kStgSlab;          // 2 x 256 floats (sw) + 2 x 256 ints (z * wsum)
@@ -85,14 +82,13 @@ struct Smem {
 // kFuse: 0 plain scale-factor epilogue; 1 SwiGLU product + quantiser (codes out); 2 SwiGLU product
 // (bf16 out).  Separate instantiations keep the plain epilogue's register budget free of the others.
 // kWide: accumulators may leave the range of the exponent trick (see `magic_ok`).
-template <int NS, int NPK, int kFuse, bool kA8 = false, int kTN = TN, bool kWide = false>
+template <int NS, int NPK, int kFuse, int kTN = TN, bool kWide = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 gemm_w4a4_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                       const __grid_constant__ CUtensorMap tmY, const __grid_constant__ CUtensorMap tmYt,
                       const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmRt,
                       const GemmParams P) {
-  using L = Smem<NS, NPK, kA8>;
-  static_assert(!kA8 || kFuse == 0, "8-bit activations: plain epilogue only");
+  using L = Smem<NS, NPK>;
   extern __shared__ uint8_t smem_raw[];
   // aligned to 1024 bytes by an offset on the shared-memory array itself (a round trip through an
   // integer would leave a generic pointer: generic loads and stores, and no way for the compiler to
@@ -174,8 +170,8 @@ gemm_w4a4_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
         const int n0 = (tile / tiles_m) * tn + (int)rank * hb;
         for (int kb = 0; kb < kblocks; ++kb) {
           if (!mbar_wait(pk_empty(s), ph ^ 1u, abort_flag, status_w, 1)) { ok = false; break; }
-          mbar_arrive_expect_tx(pk_full(s), L::kPkOpA + (uint32_t)hb * PK_ROW);
-          tma_load_2d(sbase + L::kPkAOff + s * L::kPkOpA, &tmA, pk_full(s), kb * (kA8 ? I8_ROW : PK_ROW), m0);
+          mbar_arrive_expect_tx(pk_full(s), L::kPkOp + (uint32_t)hb * PK_ROW);
+          tma_load_2d(sbase + L::kPkAOff + s * L::kPkOp, &tmA, pk_full(s), kb * PK_ROW, m0);
           tma_load_2d(sbase + L::kPkBOff + s * L::kPkOp, &tmB, pk_full(s), kb * PK_ROW, n0);
           armed |= 1u << s;
           armed_par = (armed_par & ~(1u << s)) | (ph << s);
@@ -238,7 +234,7 @@ gemm_w4a4_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
       for (int kb = 0; kb < kblocks; ++kb) {
         if (turn == grp) {
           if (!mbar_wait_warp(pk_full(ps), pph, abort_flag, status_w, 5)) { ok = false; break; }
-          const uint8_t* src = smem + L::kPkAOff + ps * L::kPkOpA + r * (kA8 ? I8_ROW : PK_ROW);
+          const uint8_t* src = smem + L::kPkAOff + ps * L::kPkOp + r * PK_ROW;
           // the packed weight tile: 16-byte chunk i * 128 + r is row (i * 128 + r) / 4, chunk r % 4
           const uint4* srcb = reinterpret_cast<const uint4*>(smem + L::kPkBOff + ps * L::kPkOp);
           const uint32_t a_tmem = tmem_base + ((uint32_t)(quad * 32) << 16) + kAccCols + s * kAStageCols;
@@ -246,28 +242,11 @@ gemm_w4a4_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             uint32_t v[16];
-            if constexpr (kA8) {
-              // int8 codes, 128-byte rows under the 128-byte swizzle.  The weight side orders the 32 codes
-              // of a group as 16 even-k then 16 odd-k bytes (that is how the nibbles fall apart); the
-              // activation bytes are put into the same order.
+            uint4 c[2];
 #pragma unroll
-              for (int g = 0; g < 2; ++g) {
-                const uint4 c0 = *reinterpret_cast<const uint4*>(src + (((uint32_t)(4 * h + 2 * g) ^ (uint32_t)(r & 7)) << 4));
-                const uint4 c1 = *reinterpret_cast<const uint4*>(src + (((uint32_t)(4 * h + 2 * g + 1) ^ (uint32_t)(r & 7)) << 4));
-                const uint32_t a[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+            for (int j = 0; j < 2; ++j) c[j] = *reinterpret_cast<const uint4*>(src + (((uint32_t)(2 * h + j) ^ swz) << 4));
 #pragma unroll
-                for (int w = 0; w < 4; ++w) {
-                  v[8 * g + w] = __byte_perm(a[2 * w], a[2 * w + 1], 0x6420);
-                  v[8 * g + 4 + w] = __byte_perm(a[2 * w], a[2 * w + 1], 0x7531);
-                }
-              }
-            } else {
-              uint4 c[2];
-#pragma unroll
-              for (int j = 0; j < 2; ++j) c[j] = *reinterpret_cast<const uint4*>(src + (((uint32_t)(2 * h + j) ^ swz) << 4));
-#pragma unroll
-              for (int j = 0; j < 2; ++j) widen(c[j], v + 8 * j);
-            }
+            for (int j = 0; j < 2; ++j) widen(c[j], v + 8 * j);
             if (h == 0) {
               if (!mbar_wait_warp(op_empty(s), ph ^ 1u, abort_flag, status_w, 6)) { ok = false; break; }
               tc_fence_after();
@@ -317,11 +296,11 @@ gemm_w4a4_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     float* sw_s = reinterpret_cast<float*>(smem + L::kScaleOff);
     int* zw_s = reinterpret_cast<int*>(smem + L::kScaleOff + 2 * TN * 4);
     const int r = quad * 32 + lane;                      // row of the CTA's 128
-    constexpr int kShift = kA8 ? 4 : 8;                  // both operands carry a factor 16, int8 activations none
+    constexpr int kShift = 8;                            // both operands carry a factor 16
     // |acc| < 2^22: int -> float by the exponent trick.  With symmetric 4-bit activation codes that holds for every
     // K the entry points accept (64 * 65408 < 2^22); on an asymmetric grid |code - z| reaches 15 and 120 K passes 2^22
     // from K = 34953 on, where the host launches the kWide form.  The others never emit the conversion instruction.
-    const bool magic_ok = kA8 ? P.K < 4096 : !kWide;
+    constexpr bool magic_ok = !kWide;
     const bool issuer = quad == 0 && lane == 0;          // issues the TMA stores (and residual loads) of its half
     const bool use_res = kFuse == 0 && residual_p != nullptr && y_out_p != nullptr;
     const bool has_z = P.wsum != nullptr;                // asymmetric activation grid: row-sum correction
@@ -536,19 +515,6 @@ static bool make_map(CUtensorMap* m, const void* base, int rows, int K, CUtensor
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Tensor map over an int8 [rows, K]-byte matrix; one box = 128 rows of one k-block (128 bytes each).
-static bool make_map_i8(CUtensorMap* m, const void* base, int rows, int K) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn) return false;
-  const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
-  const cuuint64_t strides[1] = {(cuuint64_t)K};
-  const cuuint32_t box[2] = {(cuuint32_t)I8_ROW, (cuuint32_t)HR};
-  const cuuint32_t estr[2] = {1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(base), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 // Tensor map over the bf16 output [M, N]; one box = 128 rows x 64 columns, 128-byte swizzle in shared memory.
 // (box_cols < 64: the narrow last slab of a tile that is less than 256 columns wide; dense rows, no swizzle.)
 static bool make_out_map(CUtensorMap* m, const void* base, int M, int N, int box_cols = 64) {
@@ -593,10 +559,10 @@ static bool make_codes_map(CUtensorMap* m, const void* base, int M, int row_byte
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int NS, int NPK, int kFuse, bool kA8 = false, int kTN = TN, bool kWide = false>
+template <int NS, int NPK, int kFuse, int kTN = TN, bool kWide = false>
 static int launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, GemmParams P) {
-  using L = Smem<NS, NPK, kA8>;
-  auto kern = gemm_w4a4_pair_kernel<NS, NPK, kFuse, kA8, kTN, kWide>;
+  using L = Smem<NS, NPK>;
+  auto kern = gemm_w4a4_pair_kernel<NS, NPK, kFuse, kTN, kWide>;
   static PerDeviceInt pairs_cache;          // co-resident CTA pairs on the current device
   const int max_pairs = pairs_cache.get([&] {
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kAlloc) != cudaSuccess) return 0;
@@ -617,7 +583,7 @@ static int launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, GemmPar
   });
   if (max_pairs <= 0) return FPT_ERR_CUDA;
   CUtensorMap tmA, tmB, tmY, tmYt;
-  if (!(kA8 ? make_map_i8(&tmA, Xq, P.M, P.K) : make_map(&tmA, Xq, P.M, P.K, CU_TENSOR_MAP_SWIZZLE_64B)) ||
+  if (!make_map(&tmA, Xq, P.M, P.K, CU_TENSOR_MAP_SWIZZLE_64B) ||
       !make_map(&tmB, Wq, P.N, P.K, CU_TENSOR_MAP_SWIZZLE_NONE, kTN / 2))
     return FPT_ERR_CUDA;
   if (P.Mq) { if (!make_codes_map(&tmY, P.Mq, P.M, P.N / 4)) return FPT_ERR_CUDA; }
@@ -649,27 +615,19 @@ int gemm_pair_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, cons
   if (P.Mq) return pair::launch<3, 6, 1>(st, Xq, Wq, P);
   if (P.swiglu_bf16) return pair::launch<3, 6, 2>(st, Xq, Wq, P);
   const int tn = pair::choose_tn(P.M, P.N, device_pairs());
-  if (P.a_bits == 8) {                                                        // Xq: int8 [M, K]
-    switch (tn) {
-      case 240: return pair::launch<3, 3, 0, true, 240>(st, Xq, Wq, P);
-      case 224: return pair::launch<3, 3, 0, true, 224>(st, Xq, Wq, P);
-      case 208: return pair::launch<3, 3, 0, true, 208>(st, Xq, Wq, P);
-      default:  return pair::launch<3, 3, 0, true, 256>(st, Xq, Wq, P);
-    }
-  }
   if (P.a_unsigned && 15ll * 8 * P.K >= (1 << 22)) {
     switch (tn) {
-      case 240: return pair::launch<3, 6, 0, false, 240, true>(st, Xq, Wq, P);
-      case 224: return pair::launch<3, 6, 0, false, 224, true>(st, Xq, Wq, P);
-      case 208: return pair::launch<3, 6, 0, false, 208, true>(st, Xq, Wq, P);
-      default:  return pair::launch<3, 6, 0, false, 256, true>(st, Xq, Wq, P);
+      case 240: return pair::launch<3, 6, 0, 240, true>(st, Xq, Wq, P);
+      case 224: return pair::launch<3, 6, 0, 224, true>(st, Xq, Wq, P);
+      case 208: return pair::launch<3, 6, 0, 208, true>(st, Xq, Wq, P);
+      default:  return pair::launch<3, 6, 0, 256, true>(st, Xq, Wq, P);
     }
   }
   switch (tn) {
-    case 240: return pair::launch<3, 6, 0, false, 240>(st, Xq, Wq, P);
-    case 224: return pair::launch<3, 6, 0, false, 224>(st, Xq, Wq, P);
-    case 208: return pair::launch<3, 6, 0, false, 208>(st, Xq, Wq, P);
-    default:  return pair::launch<3, 6, 0, false, 256>(st, Xq, Wq, P);
+    case 240: return pair::launch<3, 6, 0, 240>(st, Xq, Wq, P);
+    case 224: return pair::launch<3, 6, 0, 224>(st, Xq, Wq, P);
+    case 208: return pair::launch<3, 6, 0, 208>(st, Xq, Wq, P);
+    default:  return pair::launch<3, 6, 0, 256>(st, Xq, Wq, P);
   }
 }
 

@@ -512,7 +512,7 @@ gemm_wt_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
             for (int i = 0; i < 4; ++i) {
               const int a0 = (((int)v[16 * (i >> 1) + 4 * j + 2 * (i & 1)]) >> kShift) - zw[i];
               const int a1 = (((int)v[16 * (i >> 1) + 4 * j + 2 * (i & 1) + 1]) >> kShift) - zw[i];
-              if constexpr (kNat) {                      // (a debugging aid; only fpt_w4a8_gemm asks this kernel for it)
+              if constexpr (kNat && !kHold) {            // (a debugging aid; only fpt_w4a8_gemm asks this kernel for it)
                 if (P.acc_out && nf + 8 * i < n_cols) {
                   int32_t* const out = P.acc_out + (size_t)(mh + t2) * n_cols + nf + 8 * i;
                   if (mh + t2 < m_rows) out[0] = a0;
@@ -735,7 +735,7 @@ static int launch(cudaStream_t st, const int8_t* X8, const uint8_t* Wq, GemmPara
   P.tn = cut.tn; P.ksplit = cut.ksplit;
   P.tiles_m = (P.M + P.tn - 1) / P.tn;
   P.num_tiles = P.tiles_m * ((P.N + RT - 1) / RT);
-  if (layout_of(P.tn).nbuf == 1 && P.ksplit == 1 && P.num_tiles > max_pairs)
+  if (layout_of(P.tn).nbuf == 1 && P.ksplit == 1 && P.num_tiles > max_pairs && !P.acc_out)
     return launch_cut<kFuse, kNat, kAsym, kWide, true>(st, X8, Wq, P, max_pairs);
   return launch_cut<kFuse, kNat, kAsym, kWide, false>(st, X8, Wq, P, max_pairs);
 }
