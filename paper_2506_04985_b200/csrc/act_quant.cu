@@ -24,14 +24,15 @@ struct ActQuantParams {
   int wide;            // codes leave widened, one byte each (see widen_word)
 };
 
-// Word i (8 codes) of the output.
-__device__ __forceinline__ void store_codes(const ActQuantParams& P, size_t i, uint32_t w) {
-  if (P.wide) reinterpret_cast<uint2*>(P.Xq)[i] = widen_word(w);
-  else P.Xq[i] = w;
+// Word i (8 codes) of the output.  (kWide is P.wide, in kernels of their own: tested for each word it cost 4 % of a pass.)
+template <bool kWide>
+__device__ __forceinline__ void store_codes(uint32_t* Xq, size_t i, uint32_t w) {
+  if constexpr (kWide) reinterpret_cast<uint2*>(Xq)[i] = widen_word(w);
+  else Xq[i] = w;
 }
 
 // RMSNorm: T threads per token, up to V 16-byte chunks (8 elements) per thread held in registers.
-template <int T, int V>
+template <int T, int V, bool kWide>
 __global__ void __launch_bounds__(T, V <= 4 ? 2048 / T : 1) act_quant_kernel(const ActQuantParams P) {
   __shared__ double warp_part[T / 32];
   __shared__ float  bcast;
@@ -94,12 +95,12 @@ __global__ void __launch_bounds__(T, V <= 4 ? 2048 / T : 1) act_quant_kernel(con
     if (P.post_inv) P.post_inv[t] = __fdiv_rn(1.0f, p);
     if (P.r_out) P.r_out[t] = r;
   }
-  const size_t out = (size_t)t * (size_t)chunks;
+  uint32_t* out = P.Xq + (size_t)t * (size_t)chunks * (kWide ? 2 : 1);
   const QuantConsts qc = quant_consts(p, P.inv_delta, P.qmax_minus_z, P.flip);
 #pragma unroll
   for (int i = 0; i < V; ++i) {
     const int c = i * T + tid;
-    if (c < chunks) store_codes(P, out + c, quant_word(v[i], qc));
+    if (c < chunks) store_codes<kWide>(out, c, quant_word(v[i], qc));
   }
 }
 
@@ -109,7 +110,7 @@ __global__ void __launch_bounds__(T, V <= 4 ? 2048 / T : 1) act_quant_kernel(con
 // on the first few SMs to come free: the SwiGLU pass of 37 x 14336 took 21 us there (5.8 us by itself), now 7 us.
 // T threads a CTA.
 struct FlatDiv { uint32_t mul, shift; };         // i / chunks = umulhi(i, mul) >> shift for every i below 2^31
-template <bool kSilu, int U, int T>
+template <bool kSilu, int U, int T, bool kWide>
 __global__ void __launch_bounds__(T, 2048 / T) act_quant_flat_kernel(const ActQuantParams P, uint32_t total, FlatDiv div) {
   pdl_wait();
   pdl_launch_dependents();
@@ -143,13 +144,14 @@ __global__ void __launch_bounds__(T, 2048 / T) act_quant_flat_kernel(const ActQu
         v[u] = make_uint4(silu_mul_pair(v[u].x, v2[u].x), silu_mul_pair(v[u].y, v2[u].y), silu_mul_pair(v[u].z, v2[u].z),
                           silu_mul_pair(v[u].w, v2[u].w));
       const float p = (P.flags & FPT_SCALE_INPUT) ? s[u] : 1.0f;
-      store_codes(P, i, quant_word(v[u], quant_consts(p, P.inv_delta, P.qmax_minus_z, P.flip)));
+      store_codes<kWide>(P.Xq, i, quant_word(v[u], quant_consts(p, P.inv_delta, P.qmax_minus_z, P.flip)));
     }
   }
 }
 
 template <bool kSilu, int U, int T>
 static cudaError_t launch_flat(ActQuantParams P, cudaStream_t st) {
+  const auto kern = P.wide ? act_quant_flat_kernel<kSilu, U, T, true> : act_quant_flat_kernel<kSilu, U, T, false>;
   const uint32_t chunks = (uint32_t)P.K >> 3;
   uint32_t log = 1;
   while ((1u << log) < chunks) ++log;
@@ -158,8 +160,7 @@ static cudaError_t launch_flat(ActQuantParams P, cudaStream_t st) {
   for (int left = P.M; left > 0; left -= slice) {
     P.M = left < slice ? left : slice;
     const uint32_t total = (uint32_t)P.M * chunks;
-    const cudaError_t e = launch_kernel(act_quant_flat_kernel<kSilu, U, T>, dim3((total + T * U - 1) / (T * U)), dim3(T), 0, st,
-                                        true, P, total, div);
+    const cudaError_t e = launch_kernel(kern, dim3((total + T * U - 1) / (T * U)), dim3(T), 0, st, true, P, total, div);
     if (e != cudaSuccess) return e;
     const size_t n = (size_t)P.M;
     P.X += n * (size_t)(P.ldx >> 3);
@@ -175,7 +176,7 @@ static cudaError_t launch_flat(ActQuantParams P, cudaStream_t st) {
 
 // One warp per token for rows of up to 256 * V elements (kNorm: RMSNorm): the row lives in registers, the
 // reduction is a warp shuffle, no shared memory and no block-wide barrier.  W warps per CTA.
-template <int V, int W, bool kNorm>
+template <int V, int W, bool kNorm, bool kWide>
 __global__ void __launch_bounds__(W * 32) act_quant_warp_kernel(const ActQuantParams P) {
   pdl_wait();
   pdl_launch_dependents();
@@ -222,12 +223,12 @@ __global__ void __launch_bounds__(W * 32) act_quant_warp_kernel(const ActQuantPa
     if (P.post_inv) P.post_inv[t] = __fdiv_rn(1.0f, p);
     if (P.r_out) P.r_out[t] = r;
   }
-  const size_t out = (size_t)t * (size_t)chunks;
+  uint32_t* out = P.Xq + (size_t)t * (size_t)chunks * (kWide ? 2 : 1);
   const QuantConsts qc = quant_consts(p, P.inv_delta, P.qmax_minus_z, P.flip);
 #pragma unroll
   for (int i = 0; i < V; ++i) {
     const int c = i * 32 + lane;
-    if (c < chunks) store_codes(P, out + c, quant_word(v[i], qc));
+    if (c < chunks) store_codes<kWide>(out, c, quant_word(v[i], qc));
   }
 }
 
@@ -238,6 +239,7 @@ __global__ void __launch_bounds__(W * 32) act_quant_warp_kernel(const ActQuantPa
 // A wait on a row that does not arrive within about two seconds makes the warp stop (its
 // remaining tokens stay unwritten); nothing can be reported from here, the entry point has no
 // status word.
+template <bool kWide>
 __global__ void __launch_bounds__(1024) act_quant_stream_kernel(const ActQuantParams P, int W, int NB, uint32_t row_bytes) {
   extern __shared__ __align__(128) uint8_t smem_aq[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -300,10 +302,10 @@ __global__ void __launch_bounds__(1024) act_quant_stream_kernel(const ActQuantPa
       if (P.post_inv) P.post_inv[t] = __fdiv_rn(1.0f, p);
       if (P.r_out) P.r_out[t] = r;
     }
-    const size_t out = (size_t)t * (size_t)chunks;
+    uint32_t* out = P.Xq + (size_t)t * (size_t)chunks * (kWide ? 2 : 1);
     const QuantConsts qc = quant_consts(p, P.inv_delta, P.qmax_minus_z, P.flip);
 #pragma unroll 4
-    for (int c = lane; c < chunks; c += 32) store_codes(P, out + c, quant_word(row[c], qc));
+    for (int c = lane; c < chunks; c += 32) store_codes<kWide>(out, c, quant_word(row[c], qc));
     __syncwarp();                                  // every lane is done with the buffer
     const long long tn = t + NB * stride;
     if (lane == 0 && tn < P.M) {
@@ -315,8 +317,9 @@ __global__ void __launch_bounds__(1024) act_quant_stream_kernel(const ActQuantPa
 }
 
 static cudaError_t launch_stream(const ActQuantParams& P, cudaStream_t st) {
-  static PerDeviceInt attr_set;
-  if (!ensure_smem_attr(attr_set, act_quant_stream_kernel, 220 * 1024)) return cudaErrorInvalidValue;
+  static PerDeviceInt attr_set[2];
+  const auto kern = P.wide ? act_quant_stream_kernel<true> : act_quant_stream_kernel<false>;
+  if (!ensure_smem_attr(attr_set[P.wide ? 1 : 0], kern, 220 * 1024)) return cudaErrorInvalidValue;
   const int sms = device_sm_count();
   // as many warps as row buffers fit (each warp needs at least one); two buffers per warp when
   // 32 warps leave room for them
@@ -336,17 +339,18 @@ static cudaError_t launch_stream(const ActQuantParams& P, cudaStream_t st) {
     if (eff > best + 0.1) { best = eff; W = w; }
   }
   const size_t smem = (size_t)W * NB * row_bytes + (size_t)W * 16;
-  return launch_kernel(act_quant_stream_kernel, dim3(grid), dim3(W * 32), smem, st, true, P, W, NB, row_bytes);
+  return launch_kernel(kern, dim3(grid), dim3(W * 32), smem, st, true, P, W, NB, row_bytes);
 }
 
 template <int V, int W, bool kNorm = true>
 static cudaError_t launch_warp(const ActQuantParams& P, cudaStream_t st) {
-  return launch_kernel(act_quant_warp_kernel<V, W, kNorm>, dim3((P.M + W - 1) / W), dim3(W * 32), 0, st, true, P);
+  return launch_kernel(P.wide ? act_quant_warp_kernel<V, W, kNorm, true> : act_quant_warp_kernel<V, W, kNorm, false>,
+                       dim3((P.M + W - 1) / W), dim3(W * 32), 0, st, true, P);
 }
 
 template <int T, int V>
 static cudaError_t launch(const ActQuantParams& P, cudaStream_t st) {
-  return launch_kernel(act_quant_kernel<T, V>, dim3(P.M), dim3(T), 0, st, true, P);
+  return launch_kernel(P.wide ? act_quant_kernel<T, V, true> : act_quant_kernel<T, V, false>, dim3(P.M), dim3(T), 0, st, true, P);
 }
 
 // Internal entry shared by the public functions (also fills post_inv / r_out for the

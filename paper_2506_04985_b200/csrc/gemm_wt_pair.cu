@@ -683,8 +683,6 @@ static Cut choose_cut(int M, int N, int K, int pairs, int quads) {
 template <int kFuse, bool kNat, bool kAsym, bool kWide, bool kHold>
 static int launch_cut(cudaStream_t st, const int8_t* X8, const uint8_t* Wq, GemmParams P, int max_pairs) {
   auto kern = gemm_wt_pair_kernel<kFuse, kNat, kAsym, kWide, kHold>;
-  static PerDeviceInt attr_set;
-  if (!ensure_smem_attr(attr_set, kern, most_shared())) return FPT_ERR_CUDA;
   const size_t k = (size_t)P.K, out_cols = (size_t)(kFuse == 2 ? P.N / 2 : P.N);
   CUtensorMap tmW, tmX, tmY, tmR;
   if (!make_map(&tmW, CU_TENSOR_MAP_DATA_TYPE_UINT8, Wq, k / 2, P.N, k / 2, W_ROW, HR, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -710,13 +708,17 @@ static int launch_cut(cudaStream_t st, const int8_t* X8, const uint8_t* Wq, Gemm
 
 template <int kFuse, bool kNat = false, bool kAsym = false, bool kWide = false>
 static int launch(cudaStream_t st, const int8_t* X8, const uint8_t* Wq, GemmParams P) {
-  // clusters of 2 and of 4 CTAs that are resident at once on the current device
-  static PerDeviceInt attr_set, resident[2];
-  auto kern = gemm_wt_pair_kernel<kFuse, kNat, kAsym, kWide, false>;
-  if (!ensure_smem_attr(attr_set, kern, most_shared())) return FPT_ERR_CUDA;
-  int clusters[2];
-  for (int i = 0; i < 2; ++i)
-    clusters[i] = resident[i].get([&] {
+  // Once a device: the kernels' attribute, and the clusters of 2 and of 4 CTAs that are resident at once (one look-up a
+  // call: each costs 0.1 us, which a small eager call notices).
+  static PerDeviceInt prepared;
+  const int found = prepared.get([] {
+    auto kern = gemm_wt_pair_kernel<kFuse, kNat, kAsym, kWide, false>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most_shared()) != cudaSuccess ||
+        cudaFuncSetAttribute(gemm_wt_pair_kernel<kFuse, kNat, kAsym, kWide, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             most_shared()) != cudaSuccess)
+      return 0;
+    int clusters[2];
+    for (int i = 0; i < 2; ++i) {
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(2 << i, 1, 1);
       cfg.blockDim = dim3(kThreads, 1, 1);
@@ -725,13 +727,14 @@ static int launch(cudaStream_t st, const int8_t* X8, const uint8_t* Wq, GemmPara
       attr[0].id = cudaLaunchAttributeClusterDimension;
       attr[0].val.clusterDim.x = 2 << i; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
       cfg.attrs = attr; cfg.numAttrs = 1;
-      int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
-      return n > 0 ? n + 1 : 1;                          // 1: none, or not known
-    }) - 1;
-  const int sms = device_sm_count();
-  const int max_pairs = clusters[0] > 0 ? clusters[0] : sms >= 2 ? sms / 2 : 1;
-  const Cut cut = choose_cut(P.M, P.N, P.K, max_pairs, clusters[1]);
+      if (cudaOccupancyMaxActiveClusters(&clusters[i], kern, &cfg) != cudaSuccess) { cudaGetLastError(); clusters[i] = 0; }
+    }
+    if (clusters[0] <= 0) clusters[0] = device_sm_count() >= 2 ? device_sm_count() / 2 : 1;      // (not known)
+    return (clusters[0] & 0x7FFF) | (clusters[1] > 0 ? clusters[1] & 0x7FFF : 0) << 15;
+  });
+  if (found <= 0) return FPT_ERR_CUDA;
+  const int max_pairs = found & 0x7FFF;
+  const Cut cut = choose_cut(P.M, P.N, P.K, max_pairs, found >> 15);
   P.tn = cut.tn; P.ksplit = cut.ksplit;
   P.tiles_m = (P.M + P.tn - 1) / P.tn;
   P.num_tiles = P.tiles_m * ((P.N + RT - 1) / RT);
