@@ -13,7 +13,7 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 LIB = os.path.join(HERE, "libfpt_b200.so")
 SRC = sorted(glob.glob(os.path.join(HERE, "csrc", "*.cu")))
-DEPS = SRC + sorted(glob.glob(os.path.join(HERE, "csrc", "*.cuh"))) + [
+DEPS = SRC + sorted(glob.glob(os.path.join(HERE, "csrc", "*.cuh")) + glob.glob(os.path.join(HERE, "csrc", "*.h"))) + [
     os.path.join(os.path.dirname(HERE), "include", "fpt.h")]
 
 

@@ -3,6 +3,7 @@
 
 #include "fpt_common.cuh"
 #include "fpt_host.cuh"
+#include "tile_rules.h"
 
 namespace fpt {
 

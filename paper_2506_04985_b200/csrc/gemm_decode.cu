@@ -527,7 +527,7 @@ size_t gemm_decode_scratch_bytes(int M) {
 }
 
 // 65 .. 128 tokens: whether two launches of this kernel, 64 tokens and the rest, beat the CTA-pair kernel, whose tiles
-// of 256 x 208 leave most of the chip idle when N is small and K long.  Both sides as measured: the pair kernel takes
+// of 256 x 224 leave most of the chip idle when N is small and K long.  Both sides as measured: the pair kernel takes
 // 0.33 us a k-block of 128 codes and round of tiles plus 5 us, this kernel 0.42 us a k-block of 256 codes of a CTA's
 // range plus 5.5 us a launch (the second finds the weights in L2); a tenth of margin.
 // 120 tokens, 4096x14336: 41.6 -> 24.0 us; 4096x4096 and 6144x4096 stay (16.9 and 17.1 us).
@@ -539,7 +539,7 @@ bool gemm_decode_in_two(int N, int K) {
   const int cl = cluster_size(tiles, kblocks, 16);                     // (16 to 64 padded tokens: any of them divides)
   if (cl < 2) return false;
   const int pairs = num_sms() >= 2 ? num_sms() / 2 : 1;
-  const int rounds = ((N + 207) / 208 + pairs - 1) / pairs;
+  const int rounds = ((N + kPairNarrow - 1) / kPairNarrow + pairs - 1) / pairs;
   const int pair_ns = rounds * (K / 128) * 330 + 5000;
   const int two_ns = 2 * (kblocks / cl * 420 + 5500);
   return two_ns * 10 < pair_ns * 9;

@@ -338,7 +338,7 @@ int gemm_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, const Gem
     // more (128 x 40960x4096, three against two: 38 against 49 us; 128 x 28672x4096, two against one: 28.1 against 28.7)
     const int sms = num_sms(), pairs = sms >= 2 ? sms / 2 : 1;
     const int rounds_1 = ((P.N + 255) / 256 + sms - 1) / sms;
-    const int rounds_2 = ((P.N + 207) / 208 + pairs - 1) / pairs;
+    const int rounds_2 = ((P.N + kPairNarrow - 1) / kPairNarrow + pairs - 1) / pairs;
     if (rounds_2 < 2 * rounds_1) return gemm_pair_launch(st, Xq, Wq, P);
   }
   if (P.N <= 64) return launch_gemm<64, 4, 4, 8>(st, Xq, Wq, P);

@@ -25,7 +25,7 @@
 //                 accumulator is released as soon as it has been read, the tile leaves by TMA store;
 //                 a residual tile is fetched by TMA into the same slabs while the tile's matmul runs
 // Both operands are widened as code*16 (see gemm_w4a4.cu), so the accumulator holds 256 * sum.
-// Variants (template parameters): the two fused SwiGLU epilogues, output tiles of 208..256 columns.
+// Variants (template parameters): the two fused SwiGLU epilogues, output tiles of 224 and 256 columns.
 // (Activation codes of one byte: gemm_wt_pair.cu.)
 #include <cuda.h>
 
@@ -35,7 +35,7 @@
 namespace fpt {
 namespace pair {
 
-constexpr int TM = 256, TN = 256;          // output tile of a CTA pair
+constexpr int TM = kPairRows, TN = kPairWidth;      // output tile of a CTA pair
 constexpr int HR = 128;                    // rows of each operand a CTA owns
 constexpr int BK = 128;                    // codes per k-block
 constexpr int PK_ROW = BK / 2;             // packed bytes per row and k-block
@@ -121,9 +121,9 @@ gemm_w4a4_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
   const uint32_t rank = cluster_ctarank();             // 0 = leader
   const int pair_id = blockIdx.x >> 1;
   const int num_pairs = gridDim.x >> 1;
-  // Width of the output tile.  The plain epilogue also exists for 208, 224 and 240 columns: the host
-  // picks the width that wastes the least of the last round of tiles (choose_tn).  The fused epilogues need 256.
-  static_assert(kTN == TN || (kFuse == 0 && kTN >= 208 && kTN % 16 == 0), "tile width");
+  // Width of the output tile.  The plain epilogue also exists for 224 columns: the host picks the width that wastes
+  // the least of the last round of tiles (pair_tile_width).  The fused epilogues need 256.
+  static_assert(kTN == TN || (kFuse == 0 && kTN > 192 && kTN < TN), "tile width");
   constexpr int tn = kTN;
   constexpr int hb = tn >> 1;                          // weight rows of the tile this CTA holds
 
@@ -529,23 +529,6 @@ static bool make_out_map(CUtensorMap* m, const void* base, int M, int N, int box
             CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Tile width for the plain epilogue: tiles are dealt out in rounds of `pairs`, and the width with the smallest
-// rounds x width wins; among equal costs the widest (fewest tiles, least activation traffic).  (A tile's time falls
-// less than its width, because the converters' chain per k-block does not shrink with the tile: one round of 256 / 240 /
-// 224 / 208 columns of 2048 tokens x 4096 takes 18.2 / 17.5 /
-// 17.2 / 16.7 us, x 14336 41.6 / 40.6 / 40.3 / 40.7.)
-static int choose_tn(int M, int N, int pairs) {
-  const int tiles_m = (M + TM - 1) / TM;
-  int best = TN;
-  long long best_cost = -1;
-  for (int tn = TN; tn >= 208; tn -= 16) {
-    const long long tiles = (long long)tiles_m * ((N + tn - 1) / tn);
-    const long long cost = ((tiles + pairs - 1) / pairs) * tn;
-    if (best_cost < 0 || cost * 100 < best_cost * 98) { best_cost = cost; best = tn; }
-  }
-  return best;
-}
-
 // Tensor map over the packed codes [M, N/4 bytes] the fused SwiGLU epilogue writes; one box = 128 rows x 32 bytes.
 static bool make_codes_map(CUtensorMap* m, const void* base, int M, int row_bytes) {
   EncodeTiledFn fn = encode_fn();
@@ -562,6 +545,7 @@ static bool make_codes_map(CUtensorMap* m, const void* base, int M, int row_byte
 template <int NS, int NPK, int kFuse, int kTN = TN, bool kWide = false>
 static int launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, GemmParams P) {
   using L = Smem<NS, NPK>;
+  static_assert(umma_i8_pair_width(kTN), "instruction shape");
   auto kern = gemm_w4a4_pair_kernel<NS, NPK, kFuse, kTN, kWide>;
   static PerDeviceInt pairs_cache;          // co-resident CTA pairs on the current device
   const int max_pairs = pairs_cache.get([&] {
@@ -614,21 +598,10 @@ static int device_pairs() { const int sms = device_sm_count(); return sms >= 2 ?
 int gemm_pair_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, const GemmParams& P) {
   if (P.Mq) return pair::launch<3, 6, 1>(st, Xq, Wq, P);
   if (P.swiglu_bf16) return pair::launch<3, 6, 2>(st, Xq, Wq, P);
-  const int tn = pair::choose_tn(P.M, P.N, device_pairs());
-  if (P.a_unsigned && 15ll * 8 * P.K >= (1 << 22)) {
-    switch (tn) {
-      case 240: return pair::launch<3, 6, 0, 240, true>(st, Xq, Wq, P);
-      case 224: return pair::launch<3, 6, 0, 224, true>(st, Xq, Wq, P);
-      case 208: return pair::launch<3, 6, 0, 208, true>(st, Xq, Wq, P);
-      default:  return pair::launch<3, 6, 0, 256, true>(st, Xq, Wq, P);
-    }
-  }
-  switch (tn) {
-    case 240: return pair::launch<3, 6, 0, 240>(st, Xq, Wq, P);
-    case 224: return pair::launch<3, 6, 0, 224>(st, Xq, Wq, P);
-    case 208: return pair::launch<3, 6, 0, 208>(st, Xq, Wq, P);
-    default:  return pair::launch<3, 6, 0, 256>(st, Xq, Wq, P);
-  }
+  const bool narrow = pair_tile_width(P.M, P.N, device_pairs()) == kPairNarrow;
+  if (P.a_unsigned && 15ll * 8 * P.K >= (1 << 22))
+    return narrow ? pair::launch<3, 6, 0, kPairNarrow, true>(st, Xq, Wq, P) : pair::launch<3, 6, 0, kPairWidth, true>(st, Xq, Wq, P);
+  return narrow ? pair::launch<3, 6, 0, kPairNarrow>(st, Xq, Wq, P) : pair::launch<3, 6, 0>(st, Xq, Wq, P);
 }
 
 }  // namespace fpt

@@ -96,6 +96,7 @@ constexpr int most_shared() {
   for (int tn = 32; tn <= TOK; tn += 32) n = layout_of(tn).alloc() > n ? layout_of(tn).alloc() : n;
   return n;
 }
+static_assert(umma_i8_pair_width(32) && umma_i8_pair_width(TOK), "a tile takes any multiple of 32 tokens up to TOK");
 static_assert(layouts_fit(), "rings and accumulators must fit; a place in a ring must keep its converter groups and its producer");
 
 // 32 tensor-memory lanes x 32 columns in the 16x256b form: v[16 * h + 4 * j + 2 * r + e] is lane 16 h + 8 r + lane / 4,
