@@ -359,7 +359,7 @@ int fpt_decoder_attn_out(void* stream, const void* A, int M, int k_o,
  * from tensor memory (a_in_tmem = 1) or from shared memory.  2 * rows * n * 32 * 4 * iters * CTAs
  * (pairs) integer operations per launch; the rate it reaches is the ceiling the matmul kernels
  * are compared with.
- *   n       multiple of 16 in [16, 256]
+ *   n       multiple of 16 in [16, 256]; with pair = 1 of 32, the shapes the instruction of a pair is specified for
  *   cycles  device [ctas] (pair: [ctas / 2]) out, may be NULL: SM clock ticks from the first issue
  *           to the completion of the last instruction
  *   workspace  device, 16-byte aligned, at least 8192 bytes: status block (fpt_check_status)

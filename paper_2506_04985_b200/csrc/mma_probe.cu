@@ -21,7 +21,7 @@ constexpr int kTmemCols = 512;
 constexpr int kAStageCol = 480;                    // 32 columns hold 128 int8 per lane
 
 struct Params {
-  int n;                   // columns of one instruction (multiple of 16, 16..256)
+  int n;                   // columns of one instruction (multiple of 16, of a CTA pair 32, up to 256)
   int n_acc;               // accumulators in rotation: n_acc * n <= 448 columns
   int iters;               // groups of four instructions
   uint32_t* status;
@@ -165,6 +165,7 @@ extern "C" int fpt_probe_mma(void* stream, int pair, int n, int n_acc, int a_in_
   using namespace probe;
   if (!workspace || iters <= 0 || ctas <= 0) return FPT_ERR_BAD_ARG;
   if (n < 16 || n > 256 || n % 16 != 0 || n_acc < 1 || n_acc * n > kAStageCol) return FPT_ERR_UNSUPPORTED;
+  if (pair && !umma_i8_pair_width(n)) return FPT_ERR_UNSUPPORTED;
   if (pair && (ctas & 1)) return FPT_ERR_BAD_ARG;
   if ((uintptr_t)workspace & 15) return FPT_ERR_ALIGNMENT;
   Params P;

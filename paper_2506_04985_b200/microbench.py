@@ -204,7 +204,7 @@ def main():
     if len(__import__("sys").argv) > 1 and __import__("sys").argv[1] == "mma_probe":
         B.lib()
         torch.cuda.set_device(0)
-        for pair, n, n_acc, atm in ((1, 256, 1, 1), (1, 256, 1, 0), (1, 240, 1, 1), (0, 256, 1, 1), (0, 256, 1, 0),
+        for pair, n, n_acc, atm in ((1, 256, 1, 1), (1, 256, 1, 0), (1, 224, 1, 1), (0, 256, 1, 1), (0, 256, 1, 0),
                                     (0, 64, 1, 1), (0, 64, 2, 1), (0, 64, 4, 1), (0, 64, 7, 1), (0, 64, 1, 0), (0, 64, 4, 0),
                                     (0, 32, 1, 1), (0, 32, 4, 1), (0, 32, 8, 1), (0, 16, 1, 1), (0, 16, 4, 1), (0, 16, 8, 1),
                                     (0, 128, 1, 1), (0, 128, 2, 1), (1, 64, 1, 1), (1, 64, 4, 1), (1, 128, 1, 1), (1, 128, 2, 1)):

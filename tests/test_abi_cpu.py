@@ -142,6 +142,13 @@ def test_composed_calls_refuse_before_the_first_kernel(B):
                                          None, B.POST_NONE, None, fake, None, fake, big) == want
 
 
+def test_rate_probe_refuses_shapes_the_instruction_is_not_specified_for(B):
+    L, fake = B.lib(), ctypes.c_void_p(0x1000)
+    for pair, bad in ((1, (0, 16, 48, 208, 240, 288)), (0, (0, 8, 24, 100, 272))):
+        for n in bad:
+            assert L.fpt_probe_mma(None, pair, n, 1, 1, 4, 2, None, fake) == B.ERR_UNSUPPORTED, (pair, n)
+
+
 @pytest.mark.parametrize("gone", ["_cuda_getCurrentRawStream", "_cuda_getDevice"])
 def test_stream_handle_without_the_internals_of_torch(B, monkeypatch, gone):
     import importlib.util
