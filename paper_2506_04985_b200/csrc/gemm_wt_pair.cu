@@ -181,8 +181,10 @@ __device__ __forceinline__ void st_shared_u32(uint32_t addr, uint32_t v) {
 // 4-bit codes.  kAsym: unsigned codes with a zero point.  kWide: accumulators may leave the range of the exponent trick
 // (see `magic_ok`).  kHold: a tile's only accumulator goes to registers as a whole, for the next tile's MMAs to start (more
 // than 128 tokens and several tiles a pair); otherwise 32 columns at a time, a quarter of the code, which the last tile of a
-// launch enters cold.  (Both in one kernel: 1 to 2 KB of spills.)
-template <int kFuse, bool kNat, bool kAsym, bool kWide, bool kHold>
+// launch enters cold.  (Both in one kernel: 1 to 2 KB of spills.)  kAcc: the accumulators leave too, a debugging aid of
+// fpt_w4a8_gemm, in a form of its own: tested for in the plain one it cost every call without it (8-bit codes, us, with the
+// test / without: 777x3072x1024 10.3 / 8.9, 2048x8192x1024 32.1 / 25.0, 8192x4096x128 53.0 / 39.2).
+template <int kFuse, bool kNat, bool kAsym, bool kWide, bool kHold, bool kAcc = false>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_wt_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
                     const __grid_constant__ CUtensorMap tmY, const __grid_constant__ CUtensorMap tmR,
@@ -513,8 +515,8 @@ gemm_wt_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
             for (int i = 0; i < 4; ++i) {
               const int a0 = (((int)v[16 * (i >> 1) + 4 * j + 2 * (i & 1)]) >> kShift) - zw[i];
               const int a1 = (((int)v[16 * (i >> 1) + 4 * j + 2 * (i & 1) + 1]) >> kShift) - zw[i];
-              if constexpr (kNat && !kHold) {            // (a debugging aid; only fpt_w4a8_gemm asks this kernel for it)
-                if (P.acc_out && nf + 8 * i < n_cols) {
+              if constexpr (kAcc) {
+                if (nf + 8 * i < n_cols) {
                   int32_t* const out = P.acc_out + (size_t)(mh + t2) * n_cols + nf + 8 * i;
                   if (mh + t2 < m_rows) out[0] = a0;
                   if (mh + t2 + 1 < m_rows) out[n_cols] = a1;
@@ -681,9 +683,9 @@ static Cut choose_cut(int M, int N, int K, int pairs, int quads) {
   return best;
 }
 
-template <int kFuse, bool kNat, bool kAsym, bool kWide, bool kHold>
+template <int kFuse, bool kNat, bool kAsym, bool kWide, bool kHold, bool kAcc = false>
 static int launch_cut(cudaStream_t st, const int8_t* X8, const uint8_t* Wq, GemmParams P, int max_pairs) {
-  auto kern = gemm_wt_pair_kernel<kFuse, kNat, kAsym, kWide, kHold>;
+  auto kern = gemm_wt_pair_kernel<kFuse, kNat, kAsym, kWide, kHold, kAcc>;
   const size_t k = (size_t)P.K, out_cols = (size_t)(kFuse == 2 ? P.N / 2 : P.N);
   CUtensorMap tmW, tmX, tmY, tmR;
   if (!make_map(&tmW, CU_TENSOR_MAP_DATA_TYPE_UINT8, Wq, k / 2, P.N, k / 2, W_ROW, HR, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -734,12 +736,19 @@ static int launch(cudaStream_t st, const int8_t* X8, const uint8_t* Wq, GemmPara
     return (clusters[0] & 0x7FFF) | (clusters[1] > 0 ? clusters[1] & 0x7FFF : 0) << 15;
   });
   if (found <= 0) return FPT_ERR_CUDA;
+  if constexpr (kNat) {
+    static PerDeviceInt acc_attr;
+    if (P.acc_out && !ensure_smem_attr(acc_attr, gemm_wt_pair_kernel<kFuse, kNat, kAsym, kWide, false, true>, most_shared()))
+      return FPT_ERR_CUDA;
+  }
   const int max_pairs = found & 0x7FFF;
   const Cut cut = choose_cut(P.M, P.N, P.K, max_pairs, found >> 15);
   P.tn = cut.tn; P.ksplit = cut.ksplit;
   P.tiles_m = (P.M + P.tn - 1) / P.tn;
   P.num_tiles = P.tiles_m * ((P.N + RT - 1) / RT);
-  if (layout_of(P.tn).nbuf == 1 && P.ksplit == 1 && P.num_tiles > max_pairs && !P.acc_out)
+  if constexpr (kNat)
+    if (P.acc_out) return launch_cut<kFuse, kNat, kAsym, kWide, false, true>(st, X8, Wq, P, max_pairs);
+  if (layout_of(P.tn).nbuf == 1 && P.ksplit == 1 && P.num_tiles > max_pairs)
     return launch_cut<kFuse, kNat, kAsym, kWide, true>(st, X8, Wq, P, max_pairs);
   return launch_cut<kFuse, kNat, kAsym, kWide, false>(st, X8, Wq, P, max_pairs);
 }

@@ -1,6 +1,7 @@
 """GPU parity of the W4A8 path (8-bit activation codes, 4-bit weights) against the oracle: integer
-accumulators and codes bit for bit, outputs within one bf16 ulp.  Both routes are covered: the
-CTA-pair kernel with an int8 activation tile and the split a = 16 (a >> 4) + (a & 15) for small shapes."""
+accumulators and codes bit for bit, outputs within one bf16 ulp.  All routes are covered: the kernel that streams
+weights for at most 16 tokens, the CTA-pair kernel for activation codes of one byte, and the split
+a = 16 (a >> 4) + (a & 15) where there are at most 128 outputs."""
 import numpy as np
 import pytest
 import torch
@@ -42,6 +43,22 @@ def test_w4a8_gemm_exact_accumulators_and_outputs(M, N, K, extras):
     resid = None if res is None else (synth.f32(res)[rows] * rs[rows, None]).astype(np.float32)
     ref_y = dequant_epilogue(ref_acc, sw, 0.031, None if post is None else post[rows], resid)
     assert assert_bf16_close(bf16_host(Y)[rows], ref_y, "w4a8 Y") == 0
+
+
+@pytest.mark.parametrize("M,N,K", [(40, 1024, 2048), (100, 512, 4096), (333, 264, 128), (777, 6144, 512), (1500, 3072, 256),
+                                   (2048, 8192, 1024)])      # two pairs a tile, one and several tiles a pair, both accumulator forms
+@pytest.mark.parametrize("extras", [False, True])
+def test_w4a8_gemm_outputs_do_not_depend_on_the_debugging_output(M, N, K, extras):
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    qa = torch.randint(-128, 128, (M, K), device="cuda", generator=g, dtype=torch.int8)
+    qw = torch.randint(0, 256, (N, K // 2), device="cuda", generator=g, dtype=torch.uint8)
+    sw, post, rs = (torch.rand((n,), device="cuda", generator=g) + 0.5 for n in (N, M, M))
+    res = torch.randn((M, N), device="cuda", generator=g).to(torch.bfloat16)
+    kw = dict(post=post, residual=res, res_scale=rs) if extras else {}
+    (Y, acc), (Y2, none) = (B.fpt_w4a8_gemm(qa, qw, sw, 0.031, want_acc=a, **kw) for a in (True, False))
+    assert torch.equal(Y, Y2) and none is None
+    want = (qa[-3:].double() @ torch.stack(((qw.view(torch.int8) << 4) >> 4, qw.view(torch.int8) >> 4), 2).flatten(1).double().T)
+    assert torch.equal(acc[-3:].double(), want)
 
 
 @pytest.mark.parametrize("M,K", [(128, 1024), (37, 4096), (5, 14336), (130, 128), (2, 32), (600, 2048)])
