@@ -236,8 +236,11 @@ int fpt_w4a8_gemm(void* stream, const int8_t* Xq8, const uint8_t* Wq, int M, int
  *   X [M, K] bf16; flags / eps / s_in / s_out as in fpt_act_quant (FPT_SILU_MUL not allowed);
  *   post_mode selects c_t (see FPT_POST_*); post [M] only for FPT_POST_VECTOR.
  *   workspace: fpt_workspace_bytes(FPT_OP_LINEAR, M, N, K) bytes (activation codes, the per-token vectors and the
- *   status word live there).  With more than 64 tokens that is room for codes of one byte each where a faster kernel
- *   takes them; a workspace that holds them packed (M * K / 2 bytes less) is accepted too, with the same results.
+ *   status word live there).  With more than 64 tokens that is room for codes of one byte each, for any N and on any
+ *   device, and grows with M: the size for the most tokens, more than 64, and the longest rows serves every call of 65 to
+ *   that many tokens and up to that K by its fastest route (up to 64 tokens there is matmul scratch in it as well, so ask
+ *   for both).  A workspace that holds the codes packed (M * K / 2 bytes less) is accepted too, with the same results by
+ *   a slower route.
  * act_qp->bits == 8 (symmetric grid only): int8 codes q = clamp(rne((x * p) * (1/D)), -128, 127) and
  *   the matmul of fpt_w4a8_gemm; workspace: fpt_workspace_bytes(FPT_OP_LINEAR_A8, M, N, K) bytes.
  */

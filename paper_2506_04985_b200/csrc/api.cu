@@ -124,7 +124,7 @@ extern "C" size_t fpt_workspace_bytes(int op, int M, int N, int K) {
     case FPT_OP_GEMM:
       return kStatusBytes + gemm_scratch_bytes(M);
     case FPT_OP_LINEAR:
-      return linear4_bytes(M, N, K, gemm_wt_serves(M, N, K));
+      return linear4_bytes(M, N, K, M > 64);       // (of no device and no N: one workspace serves several linears)
     case FPT_OP_GEMM_A8:
       return kStatusBytes + gemm_scratch_bytes(M) + gemm_a8_scratch_bytes(M, N, K);
     case FPT_OP_LINEAR_A8:

@@ -54,6 +54,18 @@ def test_workspace_sizes(B):
     assert B.fpt_workspace_bytes(B.OP_GEMM, 0, 8, 128) == 0
 
 
+def test_workspace_of_a_linear_serves_fewer_tokens_and_other_outputs(B):
+    """One workspace for a layer's linears: its size grows with the tokens and does not depend on N (nor on the device,
+    of which there is none here), so that no call finds less room than its own size asks for."""
+    for K in (128, 1024, 4096, 28672):
+        last = 0
+        for M in (65, 128, 129, 333, 899, 900, 901, 1003, 1100, 2048, 4096, 8192, 40000):
+            sizes = {B.fpt_workspace_bytes(B.OP_LINEAR, M, N, K) for N in (8, 128, 1024, 4096, 6144, 28672)}
+            assert len(sizes) == 1 and min(sizes) >= last, (M, K, sizes, last)
+            last = min(sizes)
+            assert last >= M * K + 4 * M
+
+
 def test_argument_errors_are_reported_before_any_launch(B):
     L = B.lib()
     qp = B.QParams(4, True, 0.5, 0)
