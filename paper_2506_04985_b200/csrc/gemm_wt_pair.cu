@@ -34,11 +34,11 @@
 namespace fpt {
 namespace wt {
 
-constexpr int RT = 256;                    // weight rows of a CTA pair's tile
+constexpr int RT = kWtRows;                // weight rows of a CTA pair's tile
 constexpr int HR = 128;                    // weight rows of a CTA
-constexpr int TOK = 256;                   // tokens of a tile at most
+constexpr int TOK = kWtTokens;             // tokens of a tile at most
 constexpr int BK = 128;                    // codes per k-block
-constexpr int WK = 2 * BK;                 // codes per weight stage: rows of 128 packed bytes (see Layout)
+constexpr int WK = kWtStage;               // codes per weight stage: rows of 128 packed bytes (see Layout)
 constexpr int W_ROW = WK / 2;
 constexpr int kWStageCols = BK / 4;        // 32 tensor-memory columns hold 128 int8 per lane
 constexpr int kTmemCols = 512;
@@ -81,7 +81,7 @@ struct Layout {
   __host__ __device__ constexpr int w_col(int s) const { return kTmemCols - (ns - s) * kWStageCols; }
 };
 __host__ __device__ constexpr Layout layout_of(int tn) {
-  return tn > 192 ? Layout{tn, 1, 6, 3} : tn > 128 ? Layout{tn, 1, 6, 6} : tn > 64 ? Layout{tn, 2, 6, 6} : Layout{tn, 2, 12, 6};
+  return tn > 192 ? Layout{tn, 1, 6, 3} : tn > kWtDouble ? Layout{tn, 1, 6, 6} : tn > 64 ? Layout{tn, 2, 6, 6} : Layout{tn, 2, 12, 6};
 }
 constexpr bool layouts_fit() {
   for (int tn = 32; tn <= TOK; tn += 32) {
@@ -97,6 +97,7 @@ constexpr int most_shared() {
   return n;
 }
 static_assert(umma_i8_pair_width(32) && umma_i8_pair_width(TOK), "a tile takes any multiple of 32 tokens up to TOK");
+static_assert(WK == 2 * BK && layout_of(kWtDouble).nbuf == 2 && layout_of(kWtDouble + 32).nbuf == 1, "what wt_cut takes for granted");
 static_assert(layouts_fit(), "rings and accumulators must fit; a place in a ring must keep its converter groups and its producer");
 
 // 32 tensor-memory lanes x 32 columns in the 16x256b form: v[16 * h + 4 * j + 2 * r + e] is lane 16 h + 8 r + lane / 4,
@@ -654,35 +655,6 @@ static bool make_map(CUtensorMap* m, CUtensorMapDataType type, const void* base,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// How a launch cuts its work: tokens of a tile, and whether two pairs share one.
-struct Cut { int tn, ksplit; };
-// The cut with the least time, by what was measured at 1.9 GHz (ns).  Tiles are dealt out in rounds of `pairs`; a k-block
-// takes what the hand-overs take up to 96 tokens (160), then more and more the MMAs (274 at 256 tokens); a tile with one
-// accumulator 1.2 us more, in which it is emptied.  Where the chip is full the power limit sets the pace instead, 95 a
-// k-block and 1.08 a token of it over all pairs.  Start and end of a launch 6500 and 14.5 a token of a tile; a shared tile
-// halves the k-blocks for 1.4 us.
-// (us, 32 / 64 / .. / 256 tokens: 2048x6144x4096 133 / 75 / 56 / 46 / 44 / 40 / 45 / 40; 777x6144x4096 58 / 36 / 26 / 26 / 22 /
-// 23.5 / 26 / 29; 512x4096x14336 81 / 44 / 45 / 32 / 30 / 33 / 37 / 41; 128x4096x14336, shared: 64 tokens 18.8, else 24.8.)
-static Cut choose_cut(int M, int N, int K, int pairs, int quads) {
-  const long long rows = (N + RT - 1) / RT, kblocks = 2 * ((K + WK - 1) / WK);
-  static constexpr int kBlockNs[TOK / 32] = {160, 160, 168, 176, 183, 203, 240, 274};
-  Cut best = {32, 1};
-  long long best_ns = -1;
-  for (int tn = TOK; tn >= 32; tn -= 32) {
-    const long long tiles = rows * ((M + tn - 1) / tn), block = kBlockNs[tn / 32 - 1];
-    const long long ends = 6500 + 29 * tn / 2;
-    const long long paced = (tiles + pairs - 1) / pairs * (kblocks * block + (tn > 128 ? 1200 : 100));
-    const long long power = tiles * kblocks * (9500 + 108 * tn) / (100ll * pairs);
-    const long long ns = (paced > power ? paced : power) + ends;
-    if (best_ns < 0 || ns < best_ns) { best_ns = ns; best = {tn, 1}; }
-    if (tiles <= quads && kblocks >= 8) {
-      const long long ns2 = (kblocks + 3) / 4 * 2 * block + 1400 + ends;
-      if (ns2 < best_ns) { best_ns = ns2; best = {tn, 2}; }
-    }
-  }
-  return best;
-}
-
 template <int kFuse, bool kNat, bool kAsym, bool kWide, bool kHold, bool kAcc = false>
 static int launch_cut(cudaStream_t st, const int8_t* X8, const uint8_t* Wq, GemmParams P, int max_pairs) {
   auto kern = gemm_wt_pair_kernel<kFuse, kNat, kAsym, kWide, kHold, kAcc>;
@@ -742,7 +714,7 @@ static int launch(cudaStream_t st, const int8_t* X8, const uint8_t* Wq, GemmPara
       return FPT_ERR_CUDA;
   }
   const int max_pairs = found & 0x7FFF;
-  const Cut cut = choose_cut(P.M, P.N, P.K, max_pairs, found >> 15);
+  const WtCut cut = wt_cut(P.M, P.N, P.K, max_pairs, found >> 15, kFuse == 0);
   P.tn = cut.tn; P.ksplit = cut.ksplit;
   P.tiles_m = (P.M + P.tn - 1) / P.tn;
   P.num_tiles = P.tiles_m * ((P.N + RT - 1) / RT);
