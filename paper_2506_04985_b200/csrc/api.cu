@@ -279,7 +279,7 @@ extern "C" int fpt_decoder_mlp(void* stream, const void* X, int M, int d, int d_
   // (32 tokens or fewer of a block that is not large stream faster through the weight-streaming kernel: 17 x 2560x6912 26.3
   // against 27.6 us, 17 x 4096x14336 36.6 against 33.5, 37 x 2560x6912 32.1 / 33.2, 64 x 2560x6912 37.1 / 35.9)
   const int wide = M <= 16 || (M <= 48 && (long long)d * d_ff < (32ll << 20)) ? 0
-                   : M > 128 ? apart && gemm_wt_serves(M, 2 * d_ff, d) : !mid_hadamard && up256(m * (size_t)d_ff) + m * (size_t)d <= mlp_gu_bytes(M, d_ff, false);
+                   : M > 128 ? apart && gemm_wt_serves_swiglu(M, 2 * d_ff, d) : !mid_hadamard && up256(m * (size_t)d_ff) + m * (size_t)d <= mlp_gu_bytes(M, d_ff, false);
   const int wide_mid = wide && M <= 128 && gemm_wt_serves(M, d, d_ff);
   if (wide) Xq = M <= 128 ? GU + up256(m * (size_t)d_ff) : reinterpret_cast<uint8_t*>(Y);
   if (wide_mid) Mq = GU;

@@ -47,6 +47,9 @@ inline int device_sm_count() {
   return n > 0 ? n : 1;
 }
 
+// CTA pairs of kernels that take a whole SM.
+inline int device_pairs() { const int sms = device_sm_count(); return sms >= 2 ? sms / 2 : 1; }
+
 // Raises the dynamic shared-memory limit of `kern` once per device.  `cache` is one object per kernel
 // (a function-local static of the launcher).
 template <class K>

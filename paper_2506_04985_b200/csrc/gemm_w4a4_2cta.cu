@@ -561,7 +561,7 @@ static int launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, GemmPar
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n <= 0) {
       cudaGetLastError();
-      n = device_sm_count() / 2;
+      n = device_pairs();
     }
     return n > 0 ? n : 1;
   });
@@ -592,8 +592,6 @@ static int launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, GemmPar
 }
 
 }  // namespace pair
-
-static int device_pairs() { const int sms = device_sm_count(); return sms >= 2 ? sms / 2 : 1; }
 
 int gemm_pair_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, const GemmParams& P) {
   if (P.Mq) return pair::launch<3, 6, 1>(st, Xq, Wq, P);

@@ -704,7 +704,7 @@ static int launch(cudaStream_t st, const int8_t* X8, const uint8_t* Wq, GemmPara
       cfg.attrs = attr; cfg.numAttrs = 1;
       if (cudaOccupancyMaxActiveClusters(&clusters[i], kern, &cfg) != cudaSuccess) { cudaGetLastError(); clusters[i] = 0; }
     }
-    if (clusters[0] <= 0) clusters[0] = device_sm_count() >= 2 ? device_sm_count() / 2 : 1;      // (not known)
+    if (clusters[0] <= 0) clusters[0] = device_pairs();      // (not known)
     return (clusters[0] & 0x7FFF) | (clusters[1] > 0 ? clusters[1] & 0x7FFF : 0) << 15;
   });
   if (found <= 0) return FPT_ERR_CUDA;
@@ -727,18 +727,8 @@ static int launch(cudaStream_t st, const int8_t* X8, const uint8_t* Wq, GemmPara
 
 }  // namespace wt
 
-// 4-bit codes: whether the quantiser should widen them for this kernel.  With many tokens and two to five rounds of 256 x
-// 256 tiles, or short rows, the kernel that widens both operands is level or up to 7 % (short rows 18 %) ahead: the quantiser writes twice
-// the bytes, and the end of a launch is longer (2048x4096x4096 35.7 against 37.5 us, 1003x10240x8192 69.4 / 72.1, 4096x1024x1024
-// 15.4 / 18.1; but 4096x28672x4096 312 against 282, 777x6144x4096 32.6 / 27.4, 120x4096x4096 17.9 / 13.3).
-bool gemm_wt_serves(int M, int N, int K) {
-  if (M <= 64) return false;
-  if (M <= 900) return true;
-  const int pairs = device_sm_count() >= 2 ? device_sm_count() / 2 : 1;
-  const long long tiles = (long long)((N + wt::RT - 1) / wt::RT) * ((M + wt::TOK - 1) / wt::TOK);
-  const long long rounds = (tiles + pairs - 1) / pairs;
-  return K >= 2048 && (rounds < 2 || rounds > 5);
-}
+bool gemm_wt_serves(int M, int N, int K) { return wt_ahead(M, N, K, device_pairs()); }
+bool gemm_wt_serves_swiglu(int M, int N, int K) { return wt_ahead_swiglu(M, N, K, device_pairs()); }
 
 int gemm_wt_launch(cudaStream_t st, const int8_t* X8, const uint8_t* Wq, const GemmParams& P) {
   if (P.Mq) return wt::launch<1>(st, X8, Wq, P);

@@ -59,4 +59,38 @@ inline WtCut wt_cut(int M, int N, int K, int pairs, int quads, bool plain = true
   return best;
 }
 
+// Whether the quantiser should leave 4-bit codes one byte each for that kernel, for a linear with the plain epilogue.  Both
+// sides measured (us with the quantise pass, packed / one byte) over 3500 shapes; the rule is 0.3 % behind the better side on
+// the average, 15 % at worst (2600x6144x8192 102 / 88.8, one round and a fifth of 256 tokens).
+//   * up to 128 tokens and more than 128 outputs: one byte, always (65x136x4096 12.0 / 9.1, 120x4096x4096 17.9 / 13.3);
+//   * up to 128 outputs the other side is the one-CTA kernel, whose tiles have 64 or 128 columns: 0.5 us a k-block, but
+//     2 us less start (65x8x128 4.4 / 5.9, 512x64x256 5.8 / 6.0, 900x64x512 6.7 / 6.6, 1280x8x1024 8.5 / 9.1, 2000x8x1024 9.5 / 10.2,
+//     2000x128x1024 11.8 / 9.6);
+//   * rows of 2048 codes and more: one byte, but where tokens by the thousand fill two to five rounds of 256 x 256 (224) tiles
+//     to 0.82 or more, since the quantiser writes twice the bytes (2048x8192x8192 93.5 / 96.6, 1280x6144x4096 33.6 / 35.4; but
+//     901x10240x8192 70.3 / 57.5, 1100x4096x4096 32.9 / 23.5, 8192x10240x8192 505 / 471);
+//   * shorter rows: the estimate above against the packed side's, a round 0.43 us a k-block and 2.06, or 0.146 and 4.2 where
+//     its epilogue sets the pace, and 5.5 us of start and end (6.05 up to 900 tokens, 7.0 there beyond 256 codes: with few
+//     tiles its last one is rarely full).  Up to 900 tokens from 640 codes on one byte is ahead all through (2300x8192x128
+//     22.5 / 25.9, 700x10240x256 14.5 / 15.8, 8192x14336x1024 136 / 145; 1100x1536x1024 12.5 / 10.3, 600x4096x256 9.4 / 8.5).
+inline bool wt_ahead(int M, int N, int K, int pairs) {
+  if (M <= 64) return false;
+  if (N <= 128) return K + 8 * N > (M <= 900 ? 768 : M <= 1500 ? 1152 : 1536);
+  if (M <= 128) return true;
+  const int tn = pair_tile_width(M, N, pairs);
+  const long long tiles = (long long)((M + kPairRows - 1) / kPairRows) * ((N + tn - 1) / tn), rounds = (tiles + pairs - 1) / pairs;
+  if (K >= 2048) return M <= 900 || rounds < 2 || rounds > 5 || 100ll * M * N < 82 * rounds * pairs * kPairRows * tn;
+  if (M <= 900 && K > 512) return true;
+  const long long kblocks = K / 128, round = kblocks > 7 ? 430 * kblocks + 2060 : 146 * kblocks + 4200;
+  return wt_cut(M, N, K, pairs, pairs * 4 / 9).ns <= rounds * round + (M > 900 ? 5500 : K <= 256 ? 6050 : 7000);
+}
+// The same for the gate||up matmul of a SwiGLU block of more than 128 tokens (N = 2 d_ff).  The packed side's epilogue is
+// slow with a ragged last tile, so that only many rounds of short rows are better there (blocks of tokens x d x d_ff, us:
+// 8192x1024x4096 183 / 203, 4096x1024x4096 99.7 / 108; but 2048x1024x4096 68.0 / 65.6, 1500x2048x5632 90.9 / 74.9, 3000x4096x14336
+// 390 / 359; 4096x2048x8192 215 / 221).
+inline bool wt_ahead_swiglu(int M, int N, int K, int pairs) {
+  const long long tiles = (long long)((M + kPairRows - 1) / kPairRows) * ((N + kPairWidth - 1) / kPairWidth);
+  return M <= 900 || K >= 2048 || tiles <= 6ll * pairs;
+}
+
 }  // namespace fpt

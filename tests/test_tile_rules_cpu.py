@@ -3,7 +3,7 @@ import glob
 import os
 import re
 
-from tile_rules import CSRC, rules, wt_cut
+from tile_rules import CSRC, rules, wt_ahead, wt_cut
 
 
 def test_widths_of_cta_pair_tiles_are_shapes_of_the_instruction():
@@ -44,3 +44,41 @@ def test_tiles_of_the_kernel_for_one_byte_codes_are_near_the_best_measured():
     for (M, N, K), us in MEASURED_CUTS.items():
         cut = wt_cut(M, N, K)
         assert not cut.shared and us[cut.tokens // 32 - 1] <= 1.06 * min(us), ((M, N, K), cut)
+
+
+# us of linears (quantise pass included) with packed codes and with codes of one byte
+MEASURED_SIDES = {
+    (65, 8, 256): (4.9, 5.8), (65, 14336, 4096): (19.5, 13.3), (100, 14336, 2048): (15.1, 10.9),
+    (129, 72, 14336): (48.3, 16.6), (256, 14336, 256): (9.5, 10.2), (333, 6144, 2048): (15.3, 11.9),
+    (333, 14336, 8192): (48.8, 39.8), (400, 1024, 512): (9.7, 6.6), (400, 8192, 256): (9.6, 10.3),
+    (512, 64, 256): (5.8, 5.9), (512, 128, 4096): (20.2, 10.7), (600, 1024, 256): (8.9, 7.1),
+    (600, 2560, 4096): (20.4, 16.9), (600, 4096, 256): (9.4, 8.4), (700, 2048, 512): (9.8, 8.4),
+    (700, 10240, 256): (14.5, 15.8), (777, 14336, 512): (25.2, 22.6), (900, 64, 512): (6.7, 6.6),
+    (900, 5120, 2048): (21.1, 18.4), (901, 5120, 2048): (21.1, 18.4), (901, 6144, 4096): (32.9, 28.8),
+    (901, 10240, 8192): (70.3, 57.5), (1003, 96, 512): (7.6, 6.7), (1003, 1024, 14336): (48.0, 27.2),
+    (1003, 2048, 1024): (12.6, 10.5), (1003, 6144, 1024): (17.6, 15.8), (1100, 4096, 4096): (32.8, 23.6),
+    (1100, 28672, 512): (44.5, 41.0), (1280, 64, 768): (8.2, 7.0), (1280, 96, 1024): (10.2, 8.9),
+    (1280, 1024, 256): (9.1, 7.6), (1280, 4096, 8192): (51.3, 39.9), (1280, 6144, 4096): (33.6, 35.4),
+    (1500, 8, 4096): (21.8, 15.1), (1500, 64, 1024): (9.6, 8.9), (1500, 2048, 8192): (34.3, 30.0),
+    (1650, 256, 4096): (21.6, 15.1), (1650, 256, 8192): (32.7, 20.3), (1650, 28672, 14336): (441.5, 414.2),
+    (1800, 6144, 1024): (23.5, 21.5), (2000, 128, 1024): (11.8, 9.6), (2048, 8192, 8192): (93.5, 96.6),
+    (2600, 2048, 2048): (23.0, 20.2), (2600, 2048, 14336): (92.4, 81.3), (3000, 256, 14336): (63.4, 44.1),
+    (3000, 2048, 2048): (23.3, 21.0), (4096, 96, 1536): (15.1, 13.5), (5000, 2048, 1024): (25.0, 23.4),
+    (6000, 28672, 512): (182.0, 194.7), (8192, 10240, 8192): (504.4, 470.4), (8192, 14336, 1024): (135.5, 145.4),
+}
+# us of SwiGLU blocks, tokens x d x d_ff, with packed and with one-byte codes in front of gate||up
+MEASURED_BLOCKS = {
+    (129, 256, 1024): (33.9, 17.5), (777, 4096, 14336): (182.7, 125.9), (1003, 4096, 14336): (181.0, 148.6),
+    (1500, 2048, 5632): (90.9, 74.9), (3000, 4096, 11008): (303.6, 276.8), (4096, 512, 8192): (169.6, 184.1),
+    (4096, 1024, 4096): (99.7, 107.8), (8192, 512, 2048): (91.4, 100.2), (8192, 1024, 4096): (183.3, 202.6),
+    (8192, 8192, 28672): (3676, 3362),
+}
+
+
+def test_route_of_the_codes_is_the_faster_one_measured():
+    """Either side of 900 tokens, few outputs, short rows, rounds of tiles that are filled and that are not."""
+    for (M, N, K), us in MEASURED_SIDES.items():
+        assert us[wt_ahead(M, N, K)] <= 1.06 * min(us), (M, N, K)
+    for (M, d, d_ff), us in MEASURED_BLOCKS.items():
+        assert us[wt_ahead(M, 2 * d_ff, d, swiglu=True)] <= 1.06 * min(us), (M, d, d_ff)
+    assert not any(wt_ahead(M, N, K) for M in (1, 17, 64) for N in (8, 4096) for K in (128, 4096))

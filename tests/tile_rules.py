@@ -12,6 +12,9 @@ SOURCE = """
 #include "tile_rules.h"
 extern "C" int mma_width(int n) { return fpt::umma_i8_pair_width(n); }
 extern "C" int pair_width(int M, int N, int pairs) { return fpt::pair_tile_width(M, N, pairs); }
+extern "C" int ahead(int M, int N, int K, int pairs, int swiglu) {
+  return swiglu ? fpt::wt_ahead_swiglu(M, N, K, pairs) : fpt::wt_ahead(M, N, K, pairs);
+}
 extern "C" void cut(int M, int N, int K, int pairs, int quads, long long* out) {
   const fpt::WtCut c = fpt::wt_cut(M, N, K, pairs, quads);
   out[0] = c.tn; out[1] = c.ksplit; out[2] = c.ns;
@@ -28,6 +31,11 @@ def rules():
             f.write(SOURCE)
         subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", CSRC, src, "-o", lib], check=True)
         return ctypes.CDLL(lib)
+
+
+def wt_ahead(M, N, K, swiglu=False, pairs=74):
+    """Whether a linear (swiglu: the gate||up matmul of a block of more than 128 tokens) takes the kernel for one-byte codes."""
+    return bool(rules().ahead(M, N, K, pairs, int(swiglu)))
 
 
 def wt_cut(M, N, K, pairs=74, quads=33):
