@@ -117,8 +117,8 @@ __device__ __forceinline__ void power_sums(const T* row, int from, int n, const 
 
 // Screening of the candidates of an L_3 search in float32.  A candidate's sum there is within `kScreenEps` of the exact
 // one, relatively: a code can differ only where the quotient lies within 1e-6 of a tie, where both neighbours leave the
-// same |e| to 4e-6, so a term |e|^3 is right to 2e-5, and the additions (a chain of at most 203 terms, then of chunks)
-// add less than 3e-5.  So a candidate beyond (1 + 4 kScreenEps) times the least sum cannot be the answer; the ones that
+// same |e| to 4e-6, so a term |e|^3 is right to 2e-5, and the additions (a chain of at most 203 terms; from chunk to chunk in
+// float64, a row has no end: in float32 33 million values lost 5e-4, and the answer with them) add less than 3e-5.  So a candidate beyond (1 + 4 kScreenEps) times the least sum cannot be the answer; the ones that
 // are left (one to three of 81, as a rule) go through the float64 sums below, which decide as they always did.
 // The row is scaled by a power of two so that its largest magnitude lies in [1, 2): |e|^3 then underflows only below
 // 2^-42, which the absolute slack covers.
@@ -172,9 +172,14 @@ __device__ bool lp_screen(const T* row, int chunks, float a, bool no_nan, const 
   const int exponent = (int)(__float_as_uint(a) >> 23);
   const float unit = __uint_as_float((uint32_t)(254 - exponent) << 23);       // a * unit in [1, 2)
   const bool bins = kBf16 && 8 * chunks > kBins && 0.19f * a < 7.4f * d_min && a * (1.0f / 128) < 0.49f * d_min;
-  uint64_t acc[kPer];
+  double acc[kPer];
 #pragma unroll
-  for (uint64_t& v : acc) v = 0;
+  for (double& v : acc) v = 0.0;
+  auto both = [](uint64_t v) {
+    float lo, hi;
+    unpack_f32x2(v, lo, hi);
+    return (double)lo + (double)hi;
+  };
   if (bins) {
     const int top = (int)(__float_as_uint(a) >> 16);               // pattern of the largest magnitude
     for (int i = tid; i < kBins; i += NT) cnt.n[i] = 0;
@@ -214,7 +219,7 @@ __device__ bool lp_screen(const T* row, int chunks, float a, bool no_nan, const 
       run(std::integral_constant<int, 1>(), kTop, 2 * kTop, 8.0f);
       run(std::integral_constant<int, 0>(), 2 * kTop, kBins, 0.0f);
 #pragma unroll
-      for (int q = 0; q < kPer; ++q) if (q == k) acc[q] = sum;
+      for (int q = 0; q < kPer; ++q) if (q == k) acc[q] = both(sum);
     }
   } else {
     for (int c0 = 0; c0 < chunks; c0 += kChunk / 8) {
@@ -239,16 +244,16 @@ __device__ bool lp_screen(const T* row, int chunks, float a, bool no_nan, const 
           sum = screen2<2>(v.z, v.w, one, inv2, nd2, 7.0f, sum);
         }
 #pragma unroll
-        for (int q = 0; q < kPer; ++q) if (q == k) acc[q] = add_f32x2(acc[q], sum);
+        for (int q = 0; q < kPer; ++q) if (q == k) acc[q] += both(sum);
       }
     }
   }
   int k = 0;
   for (int task = tid; task < kTasks; task += NT, ++k) {
-    float lo = 0.0f, hi = 0.0f;
+    double sum = 0.0;
 #pragma unroll
-    for (int q = 0; q < kPer; ++q) if (q == k) unpack_f32x2(acc[q], lo, hi);
-    part[task / kLpCount][task % kLpCount] = lo + hi;
+    for (int q = 0; q < kPer; ++q) if (q == k) sum = acc[q];
+    part[task / kLpCount][task % kLpCount] = (float)sum;
   }
   __syncthreads();
   if (tid < 32) {

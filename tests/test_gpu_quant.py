@@ -212,6 +212,20 @@ def test_weight_quant_range_search_keeps_the_least_error(K):
             assert np.array_equal(host(wsum), sums)
 
 
+def test_weight_quant_range_search_of_a_row_without_end():
+    """A row of 33 million values, a pattern of 1024 over and over, with two candidates whose errors differ by 1e-10: float32
+    sums from chunk to chunk are 5e-4 off, each in its own way, and the screening dropped the right one."""
+    pattern = np.random.default_rng(2).standard_normal(1024) * 0.02
+    pattern[:64] *= 1.463646882039535
+    pattern[100] = 0.08
+    pattern = pattern.astype(np.float32)
+    codes, d, sums = OQ.quantize_weights(pattern[None], range_mode=OQ.RANGE_LP, p=3.0)
+    times = 1 << 15
+    wq, sw, wsum = B.fpt_quantize_weights(dev(pattern).repeat(times)[None], None, B.RANGE_LP, 3.0)
+    assert np.array_equal(host(sw), d.astype(np.float32)) and int(host(wsum)[0]) == int(sums[0]) * times
+    assert torch.equal(wq.view(times, 512), dev(OQ.pack_int4(codes)).expand(times, 512))
+
+
 @pytest.mark.parametrize("K", [32, 64, 96, 160, 1056, 4096, 4128, 8224])       # 1 to 33 values a thread, remainders
 @pytest.mark.parametrize("p", [2.0, 2.4, 0.7])
 def test_weight_quant_range_search_with_a_general_power(K, p):
