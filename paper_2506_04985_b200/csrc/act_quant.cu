@@ -151,7 +151,9 @@ __global__ void __launch_bounds__(T, 2048 / T) act_quant_flat_kernel(const ActQu
 
 template <bool kSilu, int U, int T>
 static cudaError_t launch_flat(ActQuantParams P, cudaStream_t st) {
-  const auto kern = P.wide ? act_quant_flat_kernel<kSilu, U, T, true> : act_quant_flat_kernel<kSilu, U, T, false>;
+  auto kern = act_quant_flat_kernel<kSilu, U, T, false>;
+  if constexpr (!kSilu)                                            // (the products of a SwiGLU leave packed from here)
+    if (P.wide) kern = act_quant_flat_kernel<kSilu, U, T, true>;
   const uint32_t chunks = (uint32_t)P.K >> 3;
   uint32_t log = 1;
   while ((1u << log) < chunks) ++log;
