@@ -186,6 +186,31 @@ def test_launches_in_a_row_give_every_output_every_time(M, N, K, form):
     assert all(B.fpt_check_status(ws) == B.OK for ws in states)
 
 
+@pytest.mark.parametrize("M,N,K,sym", [(120, 4096, 4096, True), (333, 6144, 4096, False), (777, 6144, 4096, True), (777, 6144, 4096, False)])
+def test_output_projections_in_a_row_give_every_output_every_time(M, N, K, sym):
+    """The same for composed calls on one-byte codes with a residual: two pairs a tile, one tile a pair, several."""
+    g = torch.Generator(device="cuda").manual_seed(8)
+    calls, outs, want = [], [], []
+    n = _sets_for(N * K // 2)
+    qp = B.QParams(4, sym, 0.4, 0 if sym else 8)
+    ws = B.new_workspace(B.OP_LINEAR, M, N, K)
+    for _ in range(n):
+        a, x = (torch.randn((M, k), device="cuda", generator=g).to(torch.bfloat16) for k in (K, N))
+        s_n, r = (torch.rand((M,), device="cuda", generator=g) + 0.5 for _ in range(2))
+        xw = torch.randint(0, 256, (N, K // 2), dtype=torch.uint8, device="cuda", generator=g)
+        sw = torch.rand((N,), device="cuda", generator=g) * 0.01
+        y = torch.empty((M, N), dtype=torch.bfloat16, device="cuda")
+        w, aq = _signed(xw), B.fpt_act_quant(a, qp, B.SCALE_INPUT, s_in=s_n)[0]
+        codes = _signed(aq) if sym else torch.stack((aq & 15, aq >> 4), 2).flatten(1).double() - 8
+        want.append(((codes @ w.T).float() * sw * torch.tensor(0.4) + x.float() * r[:, None]).to(torch.bfloat16))
+        wsum = None if sym else w.sum(1).to(torch.int32)
+        calls.append(lambda a=a, x=x, s_n=s_n, r=r, xw=xw, sw=sw, y=y, wsum=wsum: B.fpt_decoder_attn_out(
+            a, xw, sw, qp, s_n, X=x, r=r, wsum=wsum, ws=ws, Y=y))
+        outs.append(y)
+    _every_output_every_time(calls, outs, want, n * N * K // 2)
+    assert B.fpt_check_status(ws) == B.OK
+
+
 @pytest.mark.parametrize("M,d,d_ff,hadamard", [(16, 4096, 3584, False), (520, 4096, 3584, False), (520, 4096, 3584, True)])
 def test_blocks_in_a_row_give_every_output_every_time(M, d, d_ff, hadamard):
     """The same for the MLP block, whose gate||up matmul has the SwiGLU epilogues; against its parts, one by one."""

@@ -9,6 +9,7 @@ from oracle.int_matmul import int_matmul
 from oracle.epilogue import dequant_epilogue
 from paper_2506_04985_b200 import binding as B, fold, synth
 from helpers import dev, host, oqp, bf16_host, assert_bf16_close
+from tile_rules import wt_ahead, wt_cut
 
 pytestmark = pytest.mark.gpu
 
@@ -139,7 +140,7 @@ def test_decoder_mlp_equals_its_parts_with_infinities_and_nans(M, d_ff, hadamard
         assert special or mq.unique().numel() >= 16
 
 
-@pytest.mark.parametrize("M", [1, 8, 16, 37])
+@pytest.mark.parametrize("M", [1, 8, 16, 37, 64, 100, 300])
 def test_weights_written_by_the_kernel_in_front(M):
     """The composed calls may request weights before they wait for the kernel in front of them: not before the kernel that
     writes those weights, just before the call on the same stream, has finished."""
@@ -257,7 +258,7 @@ def test_decoder_attention_projections_parity(M, d, n_q, n_kv, with_prev, residu
     assert assert_bf16_close(bf16_host(Y), ref2["y"], "attn Y") == 0
 
 
-@pytest.mark.parametrize("M", [65, 96, 97, 129, 161, 250, 333, 900])     # tokens of a tile: 32 .. 256, the last one ragged
+@pytest.mark.parametrize("M", [65, 96, 97, 129, 161, 250, 333, 900])     # tiles of 32 to 160 tokens, the last one ragged
 @pytest.mark.parametrize("K,N", [(128, 264), (384, 1032), (1024, 4096), (4224, 520)])     # half a weight stage, odd k-blocks, two pairs a tile
 @pytest.mark.parametrize("sym", [True, False])
 def test_linear_with_widened_codes_equals_the_one_with_packed_codes(M, K, N, sym):
@@ -279,6 +280,99 @@ def test_linear_with_widened_codes_equals_the_one_with_packed_codes(M, K, N, sym
         out.append(B.fpt_w4a4_linear(x, w, sw, qp, B.RMSNORM, 1e-5, post_mode=B.POST_INVERSE_OF_PRE, wsum=wsum, ws=ws))
         assert B.fpt_check_status(ws) == B.OK
     assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+
+
+def _signed(q):
+    return torch.stack(((q.view(torch.int8) << 4) >> 4, q.view(torch.int8) >> 4), 2).flatten(1)
+
+
+def _room(M, N, K, wide):
+    """A workspace of a linear with room for codes of one byte each, or for packed ones only."""
+    ws = B.new_workspace(B.OP_LINEAR, M, N, K)
+    if not wide:
+        ws = ws[:8192 + (M * K // 2 + 255) // 256 * 256 + (M * 4 + 255) // 256 * 256].clone()
+    return ws
+
+
+# tokens of a tile; whether two CTA pairs share a tile, a pair has one tile or several; every last tile is ragged
+@pytest.mark.parametrize("M,N,K,tokens,tiles", [
+    (65, 264, 384, 32, "one"), (65, 264, 4096, 32, "shared"), (100, 512, 4096, 32, "shared"), (130, 10248, 384, 64, "many"),
+    (517, 264, 4096, 64, "shared"), (65, 10248, 384, 96, "one"), (65, 20488, 384, 96, "many"), (517, 6152, 384, 128, "many"),
+    (97, 5128, 4096, 128, "shared"), (130, 14344, 384, 160, "one"), (130, 6152, 4096, 160, "shared"), (777, 6144, 4096, 160, "many"),
+    (333, 6152, 2176, 192, "one"), (517, 10248, 2048, 192, "many"), (400, 8200, 2048, 224, "one"), (400, 14344, 2048, 224, "many"),
+    (700, 5128, 4096, 256, "one"), (500, 14344, 4096, 256, "many"),
+    (70, 8, 1024, None, None), (300, 64, 2048, None, None), (1000, 128, 4096, None, None)])          # few outputs
+def test_every_tile_of_one_byte_codes_equals_the_packed_route(M, N, K, tokens, tiles):
+    """Both grids with a per-token factor, the dynamic grid, and the output projection with its residual, which the tiles of
+    a launch fetch and hand on to one another in the slabs that they leave through."""
+    cut = wt_cut(M, N, K)
+    assert wt_ahead(M, N, K)
+    assert tokens is None or (cut.tokens, "shared" if cut.shared else "one" if cut.tiles <= 74 else "many") == (tokens, tiles)
+    g = torch.Generator(device="cuda").manual_seed(M + K + N)
+    x = torch.randn((M, K), device="cuda", generator=g).to(torch.bfloat16)
+    res = torch.randn((M, N), device="cuda", generator=g).to(torch.bfloat16)
+    s_n, r = (torch.rand((M,), device="cuda", generator=g) + 0.5 for _ in range(2))
+    w = torch.randint(0, 256, (N, K // 2), device="cuda", generator=g, dtype=torch.uint8)
+    sw = torch.rand((N,), device="cuda", generator=g) * 0.01 + 0.005
+    wsum = _signed(w).sum(1, dtype=torch.int32)
+    for qp in (B.QParams(4, True, 0.4, 0), B.QParams(4, False, 0.4, 7)):
+        z = None if qp.symmetric else wsum
+        out = []
+        for wide in (True, False):
+            ws = _room(M, N, K, wide)
+            calls = [lambda: B.fpt_w4a4_linear(x, w, sw, qp, B.RMSNORM, 1e-5, post_mode=B.POST_INVERSE_OF_PRE, wsum=z, ws=ws)[0],
+                     lambda: B.fpt_w4a4_linear(x, w, sw, qp, B.RMSNORM, 1e-5, wsum=z, ws=ws)[0],
+                     lambda: B.fpt_decoder_attn_out(x, w, sw, qp, s_n, X=res, r=r, wsum=z, ws=ws)]
+            if qp.symmetric:
+                calls.append(lambda: B.fpt_w4a4_linear_dynamic(x, w, sw, 4, B.RMSNORM, 1e-5, ws=ws)[0])
+            out.append([c() for c in calls])
+            assert B.fpt_check_status(ws) == B.OK
+        assert all(torch.equal(a, b) for a, b in zip(*out))
+        assert all(float(y.float().abs().max()) > 0.01 for y in out[0])
+
+
+@pytest.mark.parametrize("M,N,K", [(66, 264, 34944), (66, 264, 35072), (66, 264, 65408), (130, 264, 35072), (130, 264, 65408),
+                                   (300, 14344, 35072)])         # the last: several tiles a pair, one accumulator
+def test_one_byte_codes_at_the_accumulator_bound(M, N, K):
+    """Code - z = +-15 against weights of -8 and 7: from K = 34953 on |acc| passes 2^22, where the conversion to float needs
+    another form; on the symmetric grid -8 and 7 against them stay below 2^22 up to the longest rows."""
+    assert wt_ahead(M, N, K)
+    w = torch.full((N, K // 2), 0x88, dtype=torch.uint8, device="cuda")
+    w[1::2] = 0x77
+    qw = np.where(np.arange(N) % 2, 7, -8).astype(np.int64)
+    sw = (2.0 ** -20 * (1.0 + (np.arange(N) % 61) / 64.0)).astype(np.float32)
+    one = torch.ones((M,), device="cuda")
+    sign = np.where(np.arange(M) % 3, 1, -1)
+    x = torch.from_numpy(np.tile(1000.0 * sign[:, None], (1, K)).astype(np.float32)).to(torch.bfloat16).cuda()
+    for z in (None, 0, 15):
+        qp = B.QParams(4, z is None, 1.0, z or 0)
+        ws = _room(M, N, K, True)
+        Y, _ = B.fpt_w4a4_linear(x, w, dev(sw), qp, B.SCALE_INPUT, 0.0, s_in=one,
+                                 wsum=None if z is None else dev((qw * K).astype(np.int32)), ws=ws)
+        assert B.fpt_check_status(ws) == B.OK
+        code = np.where(sign > 0, 7, -8) if z is None else np.where(sign > 0, 15, 0) - z
+        acc = code[:, None] * (qw * K)[None]
+        assert assert_bf16_close(bf16_host(Y), dequant_epilogue(acc.astype(np.int32), sw, np.float32(1.0)), "Y") == 0
+
+
+@pytest.mark.parametrize("M", [17, 33, 48, 49, 128])
+def test_large_block_of_17_to_128_tokens_equals_its_parts(M):
+    """From 32 Mi weights a matrix on, the products of 17 tokens and more are quantised in the epilogue of gate||up."""
+    d, d_ff = 4096, 8192
+    g = torch.Generator(device="cuda").manual_seed(M)
+    x = torch.randn((M, d), device="cuda", generator=g).to(torch.bfloat16)
+    wgu, wd = (torch.randint(0, 256, s, dtype=torch.uint8, device="cuda", generator=g) for s in ((2 * d_ff, d // 2), (d, d_ff // 2)))
+    sgu, sd = (torch.rand((n,), device="cuda", generator=g) * 0.01 for n in (2 * d_ff, d))
+    s_prev = torch.rand((M,), device="cuda", generator=g) + 0.5
+    qi, qm = B.QParams(4, True, 0.4, 0), B.QParams(4, True, 0.3, 0)
+    Y, s_out = B.fpt_decoder_mlp(x, wgu, sgu, wd, sd, qi, qm, 1e-5, s_prev, True)
+    xq, s_n = B.fpt_act_quant(x, qi, B.RMSNORM, 1e-5, s_in=s_prev)
+    _, r = B.fpt_act_quant(x, qi, B.RMSNORM, 1e-5)
+    gu = ((_signed(xq).double() @ _signed(wgu).double().T).float() * sgu * torch.tensor(0.4)).to(torch.bfloat16)
+    mq, _ = B.fpt_act_quant(gu, qm, B.SILU_MUL | B.GU_INTERLEAVED | B.SCALE_INPUT, s_in=s_n)
+    y = (_signed(mq).double() @ _signed(wd).double().T).float() * sd * torch.tensor(0.3) + x.float() * r[:, None]
+    assert torch.equal(s_out, s_n) and mq.unique().numel() >= 64
+    assert torch.equal(Y, y.to(torch.bfloat16))
 
 
 @pytest.mark.parametrize("M", [49, 64, 65, 100, 129, 300])
