@@ -312,7 +312,7 @@ int fpt_w4a4_linear_static(void* stream, const void* X, int M, int K,
  *   with mid_hadamard = 1.  A 16-bit buffer between the two matmuls is part of it only where a route
  *   uses one: none with more than 128 tokens and no transform (the gate||up matmul quantises the
  *   products itself), the products [M, d_ff] with the transform, gate||up [M, 2 d_ff] up to 128 tokens
- *   (reserved, not used, at up to 16 tokens without the transform).
+ *   (without the transform 17 tokens and more may keep activation codes there instead; up to 16 do not use it).
  *   With more than 128 tokens Y may hold activation codes before it holds the result (unless it overlaps X, which is
  *   allowed).
  */

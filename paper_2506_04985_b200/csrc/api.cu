@@ -16,8 +16,9 @@ static int check_qp(const fpt_qparams* qp) {
 
 // bf16 buffer between the two matmuls of the MLP block: nothing when the gate||up matmul's epilogue
 // quantises the products itself (more than 128 tokens, no online transform), the products [M, d_ff]
-// when the transform needs whole rows of them, gate||up [M, 2 d_ff] on the unfused route (reserved up to 128 tokens,
-// although at most 16 tokens without the transform leave it alone: the size is part of the interface).
+// when the transform needs whole rows of them, gate||up [M, 2 d_ff] up to 128 tokens: on the unfused route they lie there;
+// where the products are quantised in the epilogue, 17 tokens and more keep one-byte codes there (fpt_decoder_mlp), and at
+// most 16 leave it alone.  (The size is part of the interface.)
 static size_t mlp_gu_bytes(int M, int d_ff, bool hadamard) {
   if (M > 128) return hadamard ? (size_t)M * (size_t)d_ff * 2 : 0;
   return (size_t)M * 2 * (size_t)d_ff * 2;
@@ -276,8 +277,9 @@ extern "C" int fpt_decoder_mlp(void* stream, const void* X, int M, int d, int d_
   // holds those of the block's input, unless it is X, which the residual still needs; the products stay packed.
   const uintptr_t xa = (uintptr_t)X, ya = (uintptr_t)Y, xy = (uintptr_t)(m * (size_t)d * 2);
   const bool apart = xa + xy <= ya || ya + xy <= xa;
-  // (32 tokens or fewer of a block that is not large stream faster through the weight-streaming kernel: 17 x 2560x6912 26.3
-  // against 27.6 us, 17 x 4096x14336 36.6 against 33.5, 37 x 2560x6912 32.1 / 33.2, 64 x 2560x6912 37.1 / 35.9)
+  // (Up to 48 tokens of a block below 32 Mi weights a matrix stream faster through the weight-streaming kernel, us there / here:
+  // 17 x 2560x6912 26.3 / 27.6, 37 x 2560x6912 32.1 / 33.2; but 17 x 4096x14336 36.6 / 33.5, and with more tokens 49 x 512x1536
+  // 16.2 / 15.7, 49 x 1024x4096 20.1 / 16.7, 64 x 2560x6912 37.1 / 35.9)
   const int wide = M <= 16 || (M <= 48 && (long long)d * d_ff < (32ll << 20)) ? 0
                    : M > 128 ? apart && gemm_wt_serves_swiglu(M, 2 * d_ff, d) : !mid_hadamard && up256(m * (size_t)d_ff) + m * (size_t)d <= mlp_gu_bytes(M, d_ff, false);
   const int wide_mid = wide && M <= 128 && gemm_wt_serves(M, d, d_ff);

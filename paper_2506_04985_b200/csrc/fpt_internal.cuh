@@ -34,8 +34,8 @@ struct GemmParams {
   int mid_qmax_minus_z;
   uint32_t mid_flip;
   int early_weights;           // the kernel in front in the stream belongs to the same call, waits for all before it
-                               // and writes no weights: they may be read before this kernel's own wait (only the
-                               // kernel for at most 16 tokens does)
+                               // and writes no weights: they may be read before this kernel's own wait (the kernel for
+                               // at most 16 tokens and the one for one-byte codes do)
   uint32_t* status;            // control block of the workspace (status word, decode counters)
   void* scratch;               // gemm_scratch_bytes(M) bytes behind the control block (decode partial sums)
 };
@@ -84,9 +84,8 @@ int gemm_wt_launch(cudaStream_t st, const int8_t* X8, const uint8_t* Wq, const G
 bool gemm_wt_serves(int M, int N, int K);
 bool gemm_wt_serves_swiglu(int M, int N, int K);
 
-// api.cu: argument checks and body of the 4-bit static linear on a workspace of
-// fpt_workspace_bytes(FPT_OP_LINEAR, M, N, K) bytes whose control block is zero (shared by
-// fpt_w4a4_linear and fpt_w4a4_linear_static).
+// api.cu: argument checks and body of the 4-bit static linear on a workspace of linear4_bytes(M, N, K, wide) bytes whose
+// control block is zero (shared by fpt_w4a4_linear and fpt_w4a4_linear_static).
 int linear4_check(const void* X, const uint8_t* Wq, const void* sw, int scale_dtype, const int32_t* wsum, const void* Y,
                   const fpt_qparams* act_qp, int M, int N, int K, int flags, const float* s_in, int post_mode,
                   const float* post);

@@ -1,9 +1,9 @@
 // Steps (2)+(3) with 8-bit activation codes and 4-bit weights (the W4A8 setting of Sec. 4,
 // Table "4-8-8"): the same exact integer matmul and scale-factor epilogue (App. B, App. J).
 //
-// More than 16 tokens and 128 outputs: the CTA-pair kernel that takes one byte a code (gemm_wt_pair.cu); up to 16 tokens: the register kernel reading int8 codes.  What is left (17 to 128
-// tokens with at most 128 outputs, or more tokens with few outputs) takes a route that needs no kernel of its own: an int8 code is
-// a = 16 h + l with h = a >> 4 in [-8, 7] and l = a & 15 in [0, 15], so
+// More than 16 tokens and 128 outputs: the CTA-pair kernel that takes one byte a code (gemm_wt_pair.cu); up to 16 tokens: the
+// register kernel reading int8 codes.  What is left (more than 16 tokens with at most 128 outputs) takes a route that needs
+// no kernel of its own: an int8 code is a = 16 h + l with h = a >> 4 in [-8, 7] and l = a & 15 in [0, 15], so
 //   sum_k a w = 16 sum_k h w + sum_k l w,
 // two 4-bit matmuls (one signed, one unsigned activation operand) through the existing kernels,
 // their int32 results combined exactly before the scale factors.  Twice the matmul work: meant
