@@ -60,15 +60,17 @@ inline WtCut wt_cut(int M, int N, int K, int pairs, int quads, bool plain = true
 }
 
 // Whether the quantiser should leave 4-bit codes one byte each for that kernel, for a linear with the plain epilogue.  Both
-// sides measured (us with the quantise pass, packed / one byte) over 3500 shapes; the rule is 0.3 % behind the better side on
-// the average, 15 % at worst (2600x6144x8192 102 / 88.8, one round and a fifth of 256 tokens).
+// sides measured (us with the quantise pass, packed / one byte) over 3800 shapes; the rule is 0.25 % behind the better side on
+// the average, 13 % at worst (700x4096x512 10.3 / 11.7).
 //   * up to 128 tokens and more than 128 outputs: one byte, always (65x136x4096 12.0 / 9.1, 120x4096x4096 17.9 / 13.3);
 //   * up to 128 outputs the other side is the one-CTA kernel, whose tiles have 64 or 128 columns: 0.5 us a k-block, but
 //     2 us less start (65x8x128 4.4 / 5.9, 512x64x256 5.8 / 6.0, 900x64x512 6.7 / 6.6, 1280x8x1024 8.5 / 9.1, 2000x8x1024 9.5 / 10.2,
 //     2000x128x1024 11.8 / 9.6);
-//   * rows of 2048 codes and more: one byte, but where tokens by the thousand fill two to five rounds of 256 x 256 (224) tiles
-//     to 0.82 or more, since the quantiser writes twice the bytes (2048x8192x8192 93.5 / 96.6, 1280x6144x4096 33.6 / 35.4; but
-//     901x10240x8192 70.3 / 57.5, 1100x4096x4096 32.9 / 23.5, 8192x10240x8192 505 / 471);
+//   * rows of 2048 codes and more: one byte, but where tokens by the thousand fill two to five rounds of the packed side's
+//     tiles to 0.82 or more, since the quantiser writes twice the bytes; with 256 columns a tile that counts below 4096 codes
+//     only (tiles of 224: 2048x8192x8192 93.5 / 96.6, 1280x6144x4096 33.6 / 35.4; of 256: 1500x6144x2048 23.3 / 24.2, but
+//     2048x6144x4096 46.8 / 46.2, 2600x6144x8192 102 / 88.8; not filled: 901x10240x8192 70.3 / 57.5, 1100x4096x4096 32.9 / 23.5;
+//     more rounds: 8192x10240x8192 505 / 471);
 //   * shorter rows: the estimate above against the packed side's, a round 0.43 us a k-block and 2.06, or 0.146 and 4.2 where
 //     its epilogue sets the pace, and 5.5 us of start and end (6.05 up to 900 tokens, 7.0 there beyond 256 codes: with few
 //     tiles its last one is rarely full).  Up to 900 tokens from 640 codes on one byte is ahead all through (2300x8192x128
@@ -79,7 +81,8 @@ inline bool wt_ahead(int M, int N, int K, int pairs) {
   if (M <= 128) return true;
   const int tn = pair_tile_width(M, N, pairs);
   const long long tiles = (long long)((M + kPairRows - 1) / kPairRows) * ((N + tn - 1) / tn), rounds = (tiles + pairs - 1) / pairs;
-  if (K >= 2048) return M <= 900 || rounds < 2 || rounds > 5 || 100ll * M * N < 82 * rounds * pairs * kPairRows * tn;
+  if (K >= 2048)
+    return M <= 900 || rounds < 2 || rounds > 5 || (K >= 4096 && tn == kPairWidth) || 100ll * M * N < 82 * rounds * pairs * kPairRows * tn;
   if (M <= 900 && K > 512) return true;
   const long long kblocks = K / 128, round = kblocks > 7 ? 430 * kblocks + 2060 : 146 * kblocks + 4200;
   return wt_cut(M, N, K, pairs, pairs * 4 / 9).ns <= rounds * round + (M > 900 ? 5500 : K <= 256 ? 6050 : 7000);

@@ -62,6 +62,7 @@ MEASURED_SIDES = {
     (1500, 8, 4096): (21.8, 15.1), (1500, 64, 1024): (9.6, 8.9), (1500, 2048, 8192): (34.3, 30.0),
     (1650, 256, 4096): (21.6, 15.1), (1650, 256, 8192): (32.7, 20.3), (1650, 28672, 14336): (441.5, 414.2),
     (1800, 6144, 1024): (23.5, 21.5), (2000, 128, 1024): (11.8, 9.6), (2048, 8192, 8192): (93.5, 96.6),
+    (2600, 6144, 8192): (102.1, 88.8), (2048, 6144, 4096): (46.8, 46.2),
     (2600, 2048, 2048): (23.0, 20.2), (2600, 2048, 14336): (92.4, 81.3), (3000, 256, 14336): (63.4, 44.1),
     (3000, 2048, 2048): (23.3, 21.0), (4096, 96, 1536): (15.1, 13.5), (5000, 2048, 1024): (25.0, 23.4),
     (6000, 28672, 512): (182.0, 194.7), (8192, 10240, 8192): (504.4, 470.4), (8192, 14336, 1024): (135.5, 145.4),
