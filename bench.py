@@ -33,7 +33,7 @@ EPS = 1e-5
 NSETS = 4
 # dram__bytes_read.sum + dram__bytes_write.sum of one fused-QKV matmul launch, from the ncu capture
 # summarised in profiles/gemm_w4a4_pair_2048x6144x4096.md (set to None when the kernel changes)
-GEMM_QKV_DRAM_BYTES = 17.04e6
+GEMM_QKV_DRAM_BYTES = 16.90e6
 METRIC = "W4A4 linear TOPS (prefill, Llama-3-8B-shaped attention projections, 2048 tokens)"
 
 
@@ -434,7 +434,7 @@ def run_gpu(args):
     achieved_o = 2.0 * M_TOK * HID * N_O / (kern_us["gemm_o"] * 1e-6) / 1e12
     aq_bytes = M_TOK * HID * 2.5 + M_TOK * 4
     mhz = clocks.get("sm_mhz")
-    roofline = {"kernel": "gemm_w4a4_pair_kernel (fused QKV, 2048x6144x4096, CTA pairs)",
+    roofline = {"kernel": "gemm_w4a4_pair_kernel (fused QKV on packed codes, 2048x6144x4096, CTA pairs)",
                 "bound": "tensor", "achieved": achieved, "peak": int8_peak, "unit": "TOP/s",
                 "frac": achieved / int8_peak, "traffic": GEMM_QKV_DRAM_BYTES,
                 "peak_note": "measured in this run: bare int8 tcgen05.mma instructions on all SMs (fpt_probe_mma: CTA "
