@@ -41,9 +41,10 @@ size_t linear4_bytes(int M, int N, int K, int wide) {
   const size_t m = (size_t)M;
   return kStatusBytes + gemm_scratch_bytes(M) + up256(m * (size_t)K / (wide ? 1 : 2)) + up256(m * 4);
 }
-// Whether the codes of a linear leave widened: the kernel that takes them serves the shape, and there is room for them.
-static int linear4_wide(int M, int N, int K, size_t workspace_bytes) {
-  return gemm_wt_serves(M, N, K) && workspace_bytes >= linear4_bytes(M, N, K, 1);
+// Whether the codes of a linear leave widened: the kernel that takes them serves the shape with that epilogue (extras: see
+// wt_ahead), and there is room for them.
+static int linear4_wide(int M, int N, int K, size_t workspace_bytes, int extras) {
+  return gemm_wt_serves(M, N, K, extras) && workspace_bytes >= linear4_bytes(M, N, K, 1);
 }
 
 static int g_programmatic_launch = 1;
@@ -234,7 +235,8 @@ extern "C" int fpt_w4a4_linear(void* stream, const void* X, int M, int K, const 
   if ((uintptr_t)workspace & 15) return FPT_ERR_ALIGNMENT;
   if (!workspace || workspace_bytes < linear4_bytes(M, N, K, 0)) return FPT_ERR_WORKSPACE;
   return linear4_run((cudaStream_t)stream, X, M, K, Wq, sw, scale_dtype, wsum, N, act_qp, flags, eps, s_in, post_mode,
-                     post, Y, s_out, reinterpret_cast<uint8_t*>(workspace), linear4_wide(M, N, K, workspace_bytes));
+                     post, Y, s_out, reinterpret_cast<uint8_t*>(workspace),
+                     linear4_wide(M, N, K, workspace_bytes, !act_qp->symmetric || post_mode != FPT_POST_NONE));
 }
 
 extern "C" int fpt_decoder_mlp(void* stream, const void* X, int M, int d, int d_ff, const uint8_t* Wgu_q,
@@ -282,7 +284,7 @@ extern "C" int fpt_decoder_mlp(void* stream, const void* X, int M, int d, int d_
   // 16.2 / 15.7, 49 x 1024x4096 20.1 / 16.7, 64 x 2560x6912 37.1 / 35.9)
   const int wide = M <= 16 || (M <= 48 && (long long)d * d_ff < (32ll << 20)) ? 0
                    : M > 128 ? apart && gemm_wt_serves_swiglu(M, 2 * d_ff, d) : !mid_hadamard && up256(m * (size_t)d_ff) + m * (size_t)d <= mlp_gu_bytes(M, d_ff, false);
-  const int wide_mid = wide && M <= 128 && gemm_wt_serves(M, d, d_ff);
+  const int wide_mid = wide && M <= 128 && gemm_wt_serves(M, d, d_ff, add_residual ? 1 : 0);
   if (wide) Xq = M <= 128 ? GU + up256(m * (size_t)d_ff) : reinterpret_cast<uint8_t*>(Y);
   if (wide_mid) Mq = GU;
 
@@ -349,7 +351,7 @@ extern "C" int fpt_decoder_attn_qkv(void* stream, const void* X, int M, int d, c
   if (rc) return rc;
   const size_t gemm_ws = kStatusBytes + gemm_scratch_bytes(M);
   uint8_t* Xq = reinterpret_cast<uint8_t*>(workspace) + gemm_ws;
-  const int wide = linear4_wide(M, n_qkv, d, workspace_bytes);
+  const int wide = linear4_wide(M, n_qkv, d, workspace_bytes, !qp_in->symmetric);
   // X~ = RMSNorm(X) on the grid qp_in; S_n = S_{n-1} * r; r kept for the residual
   if (act_quant_launch((cudaStream_t)stream, X, M, d, d, qp_in, FPT_RMSNORM, eps, nullptr, s_prev, Xq, s_out, nullptr,
                        r_out, wide) != cudaSuccess)
@@ -375,7 +377,7 @@ extern "C" int fpt_decoder_attn_out(void* stream, const void* A, int M, int k_o,
   if (rc) return rc;
   const size_t gemm_ws = kStatusBytes + gemm_scratch_bytes(M);
   uint8_t* Aq = reinterpret_cast<uint8_t*>(workspace) + gemm_ws;
-  const int wide = linear4_wide(M, d, k_o, workspace_bytes);
+  const int wide = linear4_wide(M, d, k_o, workspace_bytes, !qp_ap->symmetric + (X != nullptr));
   // the sequence scaler at the attention output: the grid sees A * S_n
   if (act_quant_launch((cudaStream_t)stream, A, M, k_o, k_o, qp_ap, FPT_SCALE_INPUT, 0.0f, nullptr, s_n, Aq, nullptr,
                        nullptr, nullptr, wide) != cudaSuccess)
@@ -418,7 +420,7 @@ extern "C" int fpt_w4a4_linear_dynamic(void* stream, const void* X, int M, int K
   uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
   const size_t gemm_ws = kStatusBytes + gemm_scratch_bytes(M);
   uint8_t* Xq = ws + gemm_ws;
-  const int wide = linear4_wide(M, N, K, workspace_bytes);
+  const int wide = linear4_wide(M, N, K, workspace_bytes, 1);
   float* c_t = reinterpret_cast<float*>(Xq + up256((size_t)M * K / (wide ? 1 : 2)));
   // per-token grid; the factor the epilogue needs (D_t, times whatever the post mode asks for) per token
   if (act_quant_dyn_launch((cudaStream_t)stream, X, M, K, K, 4, 1, 1.0f, flags, eps, s_in, post_mode, post, Xq, s_out,

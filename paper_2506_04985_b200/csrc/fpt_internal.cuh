@@ -79,9 +79,9 @@ int gemm_pair_launch(cudaStream_t st, const uint8_t* Xq, const uint8_t* Wq, cons
 // gemm_wt_pair.cu: the CTA-pair kernel for activation codes of one byte (P.a_bits == 8: 8-bit codes, otherwise 4-bit codes
 // widened by the quantiser).
 int gemm_wt_launch(cudaStream_t st, const int8_t* X8, const uint8_t* Wq, const GemmParams& P);
-// Whether the composed calls should leave widened codes for it (wt_ahead on the current device), and so for the gate||up
+// Whether the composed calls should leave widened codes for it (wt_ahead on the current device, `extras` there), and so for the gate||up
 // matmul of a block of more than 128 tokens.
-bool gemm_wt_serves(int M, int N, int K);
+bool gemm_wt_serves(int M, int N, int K, int extras);
 bool gemm_wt_serves_swiglu(int M, int N, int K);
 
 // api.cu: argument checks and body of the 4-bit static linear on a workspace of linear4_bytes(M, N, K, wide) bytes whose

@@ -727,7 +727,7 @@ static int launch(cudaStream_t st, const int8_t* X8, const uint8_t* Wq, GemmPara
 
 }  // namespace wt
 
-bool gemm_wt_serves(int M, int N, int K) { return wt_ahead(M, N, K, device_pairs()); }
+bool gemm_wt_serves(int M, int N, int K, int extras) { return wt_ahead(M, N, K, device_pairs(), extras); }
 bool gemm_wt_serves_swiglu(int M, int N, int K) { return wt_ahead_swiglu(M, N, K, device_pairs()); }
 
 int gemm_wt_launch(cudaStream_t st, const int8_t* X8, const uint8_t* Wq, const GemmParams& P) {

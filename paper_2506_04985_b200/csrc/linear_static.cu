@@ -53,7 +53,8 @@ extern "C" int fpt_w4a4_linear_static(void* stream, const void* X, int M, int K,
   if (rc) return rc;
   // the same carving as fpt_w4a4_linear's workspace, inside the built-in array
   if (linear4_bytes(M, N, K, 0) > kStaticScratchBytes) return FPT_ERR_WORKSPACE;
-  const int wide = gemm_wt_serves(M, N, K) && linear4_bytes(M, N, K, 1) <= kStaticScratchBytes;
+  const int wide = gemm_wt_serves(M, N, K, !act_qp->symmetric || post_mode != FPT_POST_NONE) &&
+                   linear4_bytes(M, N, K, 1) <= kStaticScratchBytes;
 
   unsigned char* base = nullptr;
   rc = static_scratch(&base);

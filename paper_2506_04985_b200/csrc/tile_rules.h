@@ -75,17 +75,30 @@ inline WtCut wt_cut(int M, int N, int K, int pairs, int quads, bool plain = true
 //     its epilogue sets the pace, and 5.5 us of start and end (6.05 up to 900 tokens, 7.0 there beyond 256 codes: with few
 //     tiles its last one is rarely full).  Up to 900 tokens from 640 codes on one byte is ahead all through (2300x8192x128
 //     22.5 / 25.9, 700x10240x256 14.5 / 15.8, 8192x14336x1024 136 / 145; 1100x1536x1024 12.5 / 10.3, 600x4096x256 9.4 / 8.5).
-inline bool wt_ahead(int M, int N, int K, int pairs) {
+// All that is of the lightest epilogue.  `extras`: 1 with an asymmetric grid, factors of tokens or a residual, 2 with a residual
+// on an asymmetric grid.  They cost this kernel more, whose threads hold four features of two tokens each: where the packed
+// side's tiles are well filled, rows of up to 2048 codes (2: 3072; up to 900 tokens 512 and 1536) stay there (us: asymmetric
+// 8192x28672x1280 270 / 331, dynamic 2048x14336x2048 52.4 / 58.1, residual 8192x10240x256 125 / 149, both 8192x4096x2048 76.4 / 88.3;
+// not filled: asymmetric 1641x2776x3200 28.6 / 21.7, both 1003x1024x2048 14.5 / 10.5), and so do short rows that the estimates
+// speak clearly against (residual 5356x576x640 12.4 / 13.6).  5000 calls: 0.3 % behind the better side, 17 % at worst
+// (160x28672x128 with both 14.7 / 17.2).
+inline bool wt_ahead(int M, int N, int K, int pairs, int extras) {
   if (M <= 64) return false;
   if (N <= 128) return K + 8 * N > (M <= 900 ? 768 : M <= 1500 ? 1152 : 1536);
   if (M <= 128) return true;
   const int tn = pair_tile_width(M, N, pairs);
   const long long tiles = (long long)((M + kPairRows - 1) / kPairRows) * ((N + tn - 1) / tn), rounds = (tiles + pairs - 1) / pairs;
-  if (K >= 2048)
-    return M <= 900 || rounds < 2 || rounds > 5 || (K >= 4096 && tn == kPairWidth) || 100ll * M * N < 82 * rounds * pairs * kPairRows * tn;
-  if (M <= 900 && K > 512) return true;
+  auto filled = [&](int percent) { return 100ll * M * N >= percent * rounds * pairs * kPairRows * tn; };
   const long long kblocks = K / 128, round = kblocks > 7 ? 430 * kblocks + 2060 : 146 * kblocks + 4200;
-  return wt_cut(M, N, K, pairs, pairs * 4 / 9).ns <= rounds * round + (M > 900 ? 5500 : K <= 256 ? 6050 : 7000);
+  auto ahead = [&](int start, int percent) {             // of the packed side's estimate, to that much of it
+    return wt_cut(M, N, K, pairs, pairs * 4 / 9).ns * 100 <= (rounds * round + start) * percent;
+  };
+  if (extras > 0 && M > 900 && K <= (extras > 1 ? 3072 : 2048))
+    return !filled(extras > 1 || K <= 512 ? 70 : 75) && (K >= 2048 || ahead(5500, 107));
+  if (extras > 0 && M <= 900 && K <= (extras > 1 ? 1536 : 512) && filled(extras > 1 ? 60 : 65)) return false;
+  if (K >= 2048) return M <= 900 || rounds < 2 || rounds > 5 || (K >= 4096 && tn == kPairWidth) || !filled(82);
+  if (M <= 900 && K > 512) return true;
+  return ahead(M > 900 ? 5500 : K <= 256 ? 6050 : 7000, 100);
 }
 // The same for the gate||up matmul of a SwiGLU block of more than 128 tokens (N = 2 d_ff).  The packed side's epilogue is
 // slow with a ragged last tile, so that only many rounds of short rows are better there (blocks of tokens x d x d_ff, us:

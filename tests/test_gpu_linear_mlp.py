@@ -306,7 +306,7 @@ def test_every_tile_of_one_byte_codes_equals_the_packed_route(M, N, K, tokens, t
     """Both grids with a per-token factor, the dynamic grid, and the output projection with its residual, which the tiles of
     a launch fetch and hand on to one another in the slabs that they leave through."""
     cut = wt_cut(M, N, K)
-    assert wt_ahead(M, N, K)
+    assert all(wt_ahead(M, N, K, extras) for extras in (0, 1, 2))
     assert tokens is None or (cut.tokens, "shared" if cut.shared else "one" if cut.tiles <= 74 else "many") == (tokens, tiles)
     g = torch.Generator(device="cuda").manual_seed(M + K + N)
     x = torch.randn((M, K), device="cuda", generator=g).to(torch.bfloat16)
@@ -336,7 +336,7 @@ def test_every_tile_of_one_byte_codes_equals_the_packed_route(M, N, K, tokens, t
 def test_one_byte_codes_at_the_accumulator_bound(M, N, K):
     """Code - z = +-15 against weights of -8 and 7: from K = 34953 on |acc| passes 2^22, where the conversion to float needs
     another form; on the symmetric grid -8 and 7 against them stay below 2^22 up to the longest rows."""
-    assert wt_ahead(M, N, K)
+    assert wt_ahead(M, N, K, 1)
     w = torch.full((N, K // 2), 0x88, dtype=torch.uint8, device="cuda")
     w[1::2] = 0x77
     qw = np.where(np.arange(N) % 2, 7, -8).astype(np.int64)

@@ -12,8 +12,8 @@ SOURCE = """
 #include "tile_rules.h"
 extern "C" int mma_width(int n) { return fpt::umma_i8_pair_width(n); }
 extern "C" int pair_width(int M, int N, int pairs) { return fpt::pair_tile_width(M, N, pairs); }
-extern "C" int ahead(int M, int N, int K, int pairs, int swiglu) {
-  return swiglu ? fpt::wt_ahead_swiglu(M, N, K, pairs) : fpt::wt_ahead(M, N, K, pairs);
+extern "C" int ahead(int M, int N, int K, int pairs, int extras, int swiglu) {
+  return swiglu ? fpt::wt_ahead_swiglu(M, N, K, pairs) : fpt::wt_ahead(M, N, K, pairs, extras);
 }
 extern "C" void cut(int M, int N, int K, int pairs, int quads, long long* out) {
   const fpt::WtCut c = fpt::wt_cut(M, N, K, pairs, quads);
@@ -33,9 +33,9 @@ def rules():
         return ctypes.CDLL(lib)
 
 
-def wt_ahead(M, N, K, swiglu=False, pairs=74):
+def wt_ahead(M, N, K, extras=0, swiglu=False, pairs=74):
     """Whether a linear (swiglu: the gate||up matmul of a block of more than 128 tokens) takes the kernel for one-byte codes."""
-    return bool(rules().ahead(M, N, K, pairs, int(swiglu)))
+    return bool(rules().ahead(M, N, K, pairs, extras, int(swiglu)))
 
 
 def wt_cut(M, N, K, pairs=74, quads=33):
